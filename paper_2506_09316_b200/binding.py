@@ -1,4 +1,7 @@
-"""ctypes binding of ``libdsla.so``: argument marshalling only.
+"""Binding of ``libdsla.so``: argument marshalling only.
+
+The calls of a serving loop (prefill, decode step, their n-state forms, gate producer) go through the extension module
+``_native``; everything else through ctypes.
 
 Every function here has the name of the C entry point it forwards to (see
 ``include/dsla.h``).  Tensors are torch tensors (torch supplies device memory and
@@ -19,6 +22,7 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2506_09316_b200.build` "
                       "(there is no fallback path)")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _native  # noqa: E402  (needs libdsla.so and torch's libraries, both loaded above)
 
 DSLA_OK, DSLA_ERR_INVALID_ARG, DSLA_ERR_UNSUPPORTED, DSLA_ERR_CUDA, DSLA_ERR_OOM, DSLA_ERR_TIMEOUT = range(6)
 DSLA_ERR_SCRATCH_LIMIT = 6
@@ -156,6 +160,7 @@ class DslaState:
 
     def __init__(self, handle, tensor, num_slots, H, d_k, d_v):
         self.handle, self.tensor = handle, tensor
+        self.address = handle.value     # what _native takes; None once the store is freed
         self.num_slots, self.H, self.d_k, self.d_v = num_slots, H, d_k, d_v
 
     def __del__(self):
@@ -199,7 +204,7 @@ def dsla_state_alloc_n(num_slots: int, n_states: int, H: int, d_k: int, d_v: int
 
 def dsla_state_free(st: DslaState):
     if st.handle is not None and st.handle.value:
-        h, st.handle = st.handle, None
+        h, st.handle, st.address = st.handle, None, None
         _check(_lib.dsla_state_free(h), "dsla_state_free")
 
 
@@ -218,6 +223,18 @@ def dsla_state_last_error(st: DslaState) -> int:
 
 def dsla_selftest_bounded_wait(st: DslaState, max_polls: int = 2000, stream=None):
     _check(_lib.dsla_selftest_bounded_wait(st.handle, int(max_polls), _stream(stream)), "dsla_selftest_bounded_wait")
+
+
+def _stream_or_none(stream):
+    return stream if stream is None else stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+def _sequences(T_total, cu_seqlens, max_seqlen):
+    """(N, T, max_seqlen) of the C interface: dense batches have T tokens per sequence, packed ones T = 0."""
+    if cu_seqlens is None:
+        T = int(max_seqlen) if max_seqlen is not None else T_total
+        return (T_total // T if T > 0 else 0), T, T
+    return cu_seqlens.shape[0] - 1, 0, max_seqlen
 
 
 def _prefill_args(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, N, T, max_seqlen, chunk, scale,
@@ -258,14 +275,9 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
     """q, k, v: [T_total, H, d] device tensors (fp32 or bf16).  Dense batches pass ``cu_seqlens=None``
     with q shaped [B*T, H, d] and ``max_seqlen=T``.  Returns o; final states land in ``st``."""
     T_total = q.shape[0]
-    if cu_seqlens is None:
-        T = int(max_seqlen) if max_seqlen is not None else T_total
-        N = T_total // T if T > 0 else 0
-        max_seqlen = T
-    else:
-        N, T = cu_seqlens.numel() - 1, 0
-        if max_seqlen is None:
-            raise ValueError("max_seqlen is required with cu_seqlens")
+    N, T, max_seqlen = _sequences(T_total, cu_seqlens, max_seqlen)
+    if max_seqlen is None:
+        raise ValueError("max_seqlen is required with cu_seqlens")
     if o is None:
         o = torch.empty_like(v)
     if workspace is None:
@@ -274,9 +286,9 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
                                             dense_T=T if cu_seqlens is None else None)
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    a = _prefill_args(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, N, T, max_seqlen, chunk, scale,
-                      use_initial_state, impl, workspace)
-    _check(_lib.dsla_prefill(byref(a), st.handle, _stream(stream)), "dsla_prefill")
+    _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, int(max_seqlen), int(chunk),
+                           scale, 1 if use_initial_state else 0, _IMPLS[impl] if isinstance(impl, str) else int(impl),
+                           _stream_or_none(stream)), "dsla_prefill")
     return o
 
 
@@ -322,8 +334,8 @@ def dsla_decode_step(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, sl
     [B, H, d] per key channel.  ``row_mask`` (uint8 [B]): rows with 0 are not touched (state and o)."""
     if o is None:
         o = torch.empty_like(v)
-    a = _decode_args(q, k, v, o, g_hist, g_rec, gamma, slots, scale, row_mask)
-    _check(_lib.dsla_decode_step(byref(a), st.handle, _stream(stream)), "dsla_decode_step")
+    _check(_native.decode_step(q, k, v, o, g_hist, g_rec, gamma, slots, row_mask, st.address, scale, _stream_or_none(stream)),
+           "dsla_decode_step")
     return o
 
 
@@ -377,15 +389,8 @@ def dsla_nstate_decode_step(q, k, v, gates, weights, st: DslaState, *, o=None, s
     """n-state decode step: gates [n, B, H] (or [n, B, H, d] per key channel) fp32, weights [H, n] fp32."""
     if o is None:
         o = torch.empty_like(v)
-    B, H, d_k = q.shape
-    a = dsla_nstate_decode_args()
-    a.q, a.k, a.v, a.o = _ptr(q), _ptr(k), _ptr(v), _ptr(o)
-    a.gates, a.weights, a.slots, a.row_mask = _ptr(gates), _ptr(weights), _ptr(slots), _ptr(row_mask)
-    a.B, a.H, a.d_k, a.d_v, a.n_states = int(B), int(H), int(d_k), int(v.shape[2]), int(gates.shape[0])
-    a.dtype = _DTYPES[q.dtype]
-    a.scale = float(scale)
-    a.gate_layout = DSLA_GATE_PER_KEY_CHANNEL if gates.dim() == 4 else DSLA_GATE_SCALAR
-    _check(_lib.dsla_nstate_decode_step(byref(a), st.handle, _stream(stream)), "dsla_nstate_decode_step")
+    _check(_native.nstate_decode_step(q, k, v, o, gates, weights, slots, row_mask, st.address, scale, _stream_or_none(stream)),
+           "dsla_nstate_decode_step")
     return o
 
 
@@ -426,30 +431,27 @@ def dsla_nstate_prefill(q, k, v, gates, weights, st: DslaState, *, o=None, cu_se
     token-by-token CUDA-core kernel, which serves everything else)."""
     if o is None:
         o = torch.empty_like(v)
-    a = _nstate_prefill_args(q, k, v, o, gates, weights, cu_seqlens, slots, max_seqlen, scale, use_initial_state, impl)
+    T_total = q.shape[0]
+    N, T, longest = _sequences(T_total, cu_seqlens, max_seqlen)
+    if longest is None:
+        longest = T_total      # an upper bound is valid (the tighter the bound, the better the segment plan)
     if workspace is None:
-        need = int(_lib.dsla_nstate_prefill_workspace_bytes(byref(a)))
+        need = dsla_nstate_prefill_workspace_bytes(q, k, v, gates, weights, cu_seqlens=cu_seqlens, max_seqlen=max_seqlen, impl=impl)
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    a.workspace = _ptr(workspace)
-    a.workspace_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.dsla_nstate_prefill(byref(a), st.handle, _stream(stream)), "dsla_nstate_prefill")
+    _check(_native.nstate_prefill(q, k, v, o, gates, weights, cu_seqlens, slots, workspace, st.address, N, T, int(longest), scale,
+                                  1 if use_initial_state else 0, _IMPLS[impl], _stream_or_none(stream)), "dsla_nstate_prefill")
     return o
 
 
 def dsla_gate_project(x, w, bias=None, *, g_hist=None, g_rec=None, stream=None):
     """logistic(x W^T + bias) on the tensor cores: x [T, D_model] bf16, w [2 H, D_model] bf16, bias [2 H] fp32 or None.
     Returns (g_hist, g_rec), both [T, H] fp32."""
-    T, D_model = x.shape
-    H = w.shape[0] // 2
     if g_hist is None:
-        g_hist = torch.empty((T, H), dtype=torch.float32, device=x.device)
+        g_hist = torch.empty((x.shape[0], w.shape[0] // 2), dtype=torch.float32, device=x.device)
     if g_rec is None:
-        g_rec = torch.empty((T, H), dtype=torch.float32, device=x.device)
-    a = dsla_gate_project_args()
-    a.x, a.w, a.bias, a.g_hist, a.g_rec = _ptr(x), _ptr(w), _ptr(bias), _ptr(g_hist), _ptr(g_rec)
-    a.T, a.H, a.D_model = int(T), int(H), int(D_model)
-    _check(_lib.dsla_gate_project(byref(a), _stream(stream)), "dsla_gate_project")
+        g_rec = torch.empty((x.shape[0], w.shape[0] // 2), dtype=torch.float32, device=x.device)
+    _check(_native.gate_project(x, w, bias, g_hist, g_rec, _stream_or_none(stream)), "dsla_gate_project")
     return g_hist, g_rec
 
 
