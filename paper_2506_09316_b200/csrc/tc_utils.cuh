@@ -136,6 +136,14 @@ __device__ __forceinline__ void st_async_b32x4(uint32_t caddr, uint32_t a, uint3
                  "r"(c), "r"(d), "r"(cbar)
                  : "memory");
 }
+// Asynchronous copy of `bytes` (a multiple of 16) from this CTA's shared memory into that of a CTA of the cluster, counted
+// on an mbarrier of that CTA.  Writes of this thread (and, after a __syncwarp, of its warp) have to be behind a
+// fence_proxy_async_smem.
+__device__ __forceinline__ void bulk_copy_to_cta(uint32_t cdst, uint32_t ssrc, uint32_t bytes, uint32_t cbar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(cdst), "r"(ssrc), "r"(bytes),
+                 "r"(cbar)
+                 : "memory");
+}
 // Arrive on an mbarrier of another CTA without ordering anything (a "buffer is free" signal after its reads returned).
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t caddr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
