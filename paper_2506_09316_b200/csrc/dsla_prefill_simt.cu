@@ -8,7 +8,17 @@
 // Exponents are always differences b_j - b_s <= 0, so nothing overflows.  A gate that is exactly 0
 // is not pushed through log(): zero gates are counted (zc) and a factor is 0 whenever a zero gate
 // lies between the two tokens, which keeps tokens after the zero exact.
+//
+// CTA = (sequence, head, 32-column slab of d_v, segment of the sequence).  The chunks of a sequence are a serial chain,
+// and a layer of few heads has few slabs: one CTA per slab leaves most of the chip idle (4 heads of 64: 8 CTAs).  The
+// segments of a sequence therefore run on the 2, 4 or 8 CTAs of a thread-block cluster.  Every segment but the last
+// first accumulates its own state from zero (K and V only) and leaves it, with the product of its gates, in its
+// shared memory; after a cluster barrier the initial states are folded out of the summaries through distributed
+// shared memory and every CTA runs its chunks.  No scratch in global memory, no second launch.
+// 4 heads of 64, T = 512, fp32: 21 us, 106 us with one CTA per slab.  Bound by shared-memory wavefronts: the 4 x 4 tiles of
+// the update (2.6 us), the scores and their mask (5.8) and the outputs (3.0) do two FMAs per float read.
 #include "dsla_internal.cuh"
+#include "tc_utils.cuh"
 
 namespace dsla {
 
@@ -16,11 +26,16 @@ namespace {
 
 template <typename T> struct Vec4;
 template <> struct Vec4<float> {
-    static __device__ __forceinline__ float4 load(const float* p) { return *reinterpret_cast<const float4*>(p); }
+    using Raw = float4;
+    static __device__ __forceinline__ Raw zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+    static __device__ __forceinline__ Raw load(const float* p) { return *reinterpret_cast<const float4*>(p); }
+    static __device__ __forceinline__ float4 widen(Raw x) { return x; }
 };
 template <> struct Vec4<__nv_bfloat16> {
-    static __device__ __forceinline__ float4 load(const __nv_bfloat16* p) {
-        const uint2 u = *reinterpret_cast<const uint2*>(p);
+    using Raw = uint2;
+    static __device__ __forceinline__ Raw zero() { return make_uint2(0u, 0u); }
+    static __device__ __forceinline__ Raw load(const __nv_bfloat16* p) { return *reinterpret_cast<const uint2*>(p); }
+    static __device__ __forceinline__ float4 widen(Raw u) {
         const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&u.x);
         const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&u.y);
         return make_float4(__low2float(a), __high2float(a), __low2float(b), __high2float(b));
@@ -32,65 +47,64 @@ __device__ __forceinline__ void store2(__nv_bfloat16* p, float a, float b) {
     *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
 }
 
+constexpr int DVS = 32;      // d_v columns per CTA
+
+// Shared memory, in floats: Q, K [C][D], V [C][36], masked scores [C][C+4], states [2][D][36], per-token terms.  The 16-byte
+// pieces of a Q or K row are XORed with the row's group of four: in the score loop neighbouring lanes read rows four
+// apart, which a padded pitch would put on two banks.
+template <int D, int C> struct Layout {
+    static constexpr int VP = DVS + 4, CP = C + 4;
+    static constexpr int Q = 0, K = Q + C * D, V = K + C * D, P = V + C * VP, S = P + C * CP;
+    static constexpr int BB = S + 2 * D * VP;      // [2][C] cumulative log-gate (zeros skipped)
+    static constexpr int ROWF = BB + 2 * C;        // [2][C] weight_i * e^{b_j} (0 behind a zero gate)
+    static constexpr int WW = ROWF + 2 * C;        // [2][C] e^{b_last - b_s}
+    static constexpr int ZC = WW + 2 * C;          // [2][C] zero-gate count, inclusive (int)
+    static constexpr int END = ZC + 2 * C;
+    static __device__ __forceinline__ int qk(int row, int col) { return row * D + (col ^ (((row >> 2) & 7) << 2)); }      // col: a multiple of 4
+};
+
 }  // namespace
 
-// CTA = (sequence, head, 32-column slab of d_v); 256 threads.  The slab's two state slices live in
-// registers (4x4 tile per thread per state) across the chunk loop, with a copy in shared memory for
-// the readout.  Q K^T is recomputed per slab (D/32 times); acceptable for this fallback path.
+// 4 D threads.  In the state update a thread owns a 4 x 4 tile of one state (in registers across the chunk loop, with a
+// copy in shared memory for the readout); in the readout two neighbouring lanes share 4 rows x 2 columns of the
+// output, one lane per state when D = 128.  Q K^T is recomputed per slab (D / 32 times).
 template <int D, int C, typename T>
-__global__ void __launch_bounds__(256) prefill_simt_kernel(const PrefillParams p) {
-    constexpr int DVS = 32, SLABS = D / DVS, DP = D + 4, VP = DVS + 4, CP = C + 4, NT = 256;
+__global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams p, const int segs) {
+    using L = Layout<D, C>;
+    using V4 = Vec4<T>;
+    constexpr int SLABS = D / DVS, VP = L::VP, CP = L::CP, NT = 4 * D;
+    constexpr int SPLIT = D / 64;            // lanes that share a score tile or an output tile
     extern __shared__ __align__(16) float smem[];
-    float* Qs = smem;                 // [C][DP]
-    float* Ks = Qs + C * DP;          // [C][DP]
-    float* Vs = Ks + C * DP;          // [C][VP]
-    float* Ps = Vs + C * VP;          // [C][CP]  masked scores
-    float* Ss = Ps + C * CP;          // [2][D][VP]
-    float* bb = Ss + 2 * D * VP;      // [2][C] cumulative log-gate (zeros skipped)
-    float* rowf = bb + 2 * C;         // [2][C] weight_i * e^{b_j} (0 behind a zero gate)
-    float* ww = rowf + 2 * C;         // [2][C] e^{b_last - b_s}
-    int* zc = reinterpret_cast<int*>(ww + 2 * C);  // [2][C] zero-gate count, inclusive
-    __shared__ float a_dec[2];
+    float *Qs = smem + L::Q, *Ks = smem + L::K, *Vs = smem + L::V, *Ps = smem + L::P, *Ss = smem + L::S;
+    float *bb = smem + L::BB, *rowf = smem + L::ROWF, *ww = smem + L::WW;
+    int* zc = reinterpret_cast<int*>(smem + L::ZC);
+    __shared__ float a_dec[2], a_seg[2];
 
+    // The launch may overlap the tail of what precedes it in the stream; nothing is read or written before this wait.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x;
-    const int slab = blockIdx.x % SLABS;
-    const int h = (blockIdx.x / SLABS) % p.H;
-    const int n = blockIdx.x / (SLABS * p.H);
+    const int seg = blockIdx.x % segs;       // rank in the cluster
+    const int slab = (blockIdx.x / segs) % SLABS;
+    const int h = (blockIdx.x / (segs * SLABS)) % p.H;
+    const int n = blockIdx.x / (segs * SLABS * p.H);
     const int t_begin = p.cu_seqlens ? p.cu_seqlens[n] : n * p.T;
     const int t_end = p.cu_seqlens ? p.cu_seqlens[n + 1] : (n + 1) * p.T;
     const int len = t_end - t_begin;
     const int slot = p.slots ? p.slots[n] : n;
     if (slot < 0 || slot >= p.num_slots) return;
-    const int col0 = slab * DVS;
-
-    float* G1 = p.state + (((size_t)slot * 2 + 0) * p.H + h) * (size_t)(D * D);
-    float* G2 = G1 + (size_t)p.H * D * D;
-
-    // state tile of this thread: rows k0..k0+3, columns n0..n0+3 of the slab
-    const bool own = tid < (D / 4) * 8;
-    const int k0 = (tid >> 3) * 4, n0 = (tid & 7) * 4;
-    float s1[4][4], s2[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) s1[a][b] = s2[a][b] = 0.f;
-    if (own && p.use_initial_state) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float4 x = *reinterpret_cast<const float4*>(G1 + (size_t)(k0 + a) * D + col0 + n0);
-            const float4 y = *reinterpret_cast<const float4*>(G2 + (size_t)(k0 + a) * D + col0 + n0);
-            s1[a][0] = x.x; s1[a][1] = x.y; s1[a][2] = x.z; s1[a][3] = x.w;
-            s2[a][0] = y.x; s2[a][1] = y.y; s2[a][2] = y.z; s2[a][3] = y.w;
-        }
-    }
     if (len <= 0 && p.use_initial_state) return;  // nothing to do, slot untouched
-    if (own) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            *reinterpret_cast<float4*>(Ss + (k0 + a) * VP + n0) = make_float4(s1[a][0], s1[a][1], s1[a][2], s1[a][3]);
-            *reinterpret_cast<float4*>(Ss + D * VP + (k0 + a) * VP + n0) = make_float4(s2[a][0], s2[a][1], s2[a][2], s2[a][3]);
-        }
-    }
+    const int col0 = slab * DVS;
+    const int nchunks = (len + C - 1) / C, per = (nchunks + segs - 1) / segs;
+    const int c_begin = min(seg * per, nchunks), c_end = min(c_begin + per, nchunks);
+
+    // state tile of this thread
+    const int si = tid / (2 * D);
+    const int k0 = ((tid % (2 * D)) >> 3) * 4, n0 = (tid & 7) * 4;
+    float* G = p.state + (((size_t)slot * 2 + si) * p.H + h) * (size_t)(D * D) + (size_t)k0 * D + col0 + n0;
+    float* Sme = Ss + (si * D + k0) * VP + n0;
+    float s[4][4];
+
     const float gam = p.gamma[h];
     const float W1 = gam * p.scale, W2 = (1.f - gam) * p.scale;
     const T* qg = reinterpret_cast<const T*>(p.q);
@@ -98,41 +112,64 @@ __global__ void __launch_bounds__(256) prefill_simt_kernel(const PrefillParams p
     const T* vg = reinterpret_cast<const T*>(p.v);
     T* og = reinterpret_cast<T*>(p.o);
 
-    for (int c0 = 0; c0 < len; c0 += C) {
-        const int valid = min(C, len - c0);
-        __syncthreads();
-        // ---- stage Q, K, V (rows past the end of the sequence become zeros)
-        for (int idx = tid; idx < C * (D / 4); idx += NT) {
-            const int row = idx / (D / 4), c = idx % (D / 4);
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+    // One chunk ahead in registers: the loads of the next chunk are in flight while this one is computed.
+    constexpr int NQ = (C * (D / 4) + NT - 1) / NT, NV = (C * (DVS / 4) + NT - 1) / NT;
+    typename V4::Raw rq[NQ], rk[NQ], rv[NV];
+    float rg[C > 32 ? 2 : 1];
+    auto fetch = [&](int c, bool with_q) {
+        const int c0 = c * C, valid = min(C, len - c0);
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            const int idx = tid + i * NT, row = idx / (D / 4);
+            rq[i] = V4::zero(); rk[i] = V4::zero();
             if (row < valid) {
-                const size_t off = ((size_t)(t_begin + c0 + row) * p.H + h) * D + c * 4;
-                x = Vec4<T>::load(qg + off);
-                y = Vec4<T>::load(kg + off);
+                const size_t off = ((size_t)(t_begin + c0 + row) * p.H + h) * D + (idx % (D / 4)) * 4;
+                if (with_q) rq[i] = V4::load(qg + off);
+                rk[i] = V4::load(kg + off);
             }
-            *reinterpret_cast<float4*>(Qs + row * DP + c * 4) = x;
-            *reinterpret_cast<float4*>(Ks + row * DP + c * 4) = y;
         }
-        for (int idx = tid; idx < C * (DVS / 4); idx += NT) {
-            const int row = idx / (DVS / 4), c = idx % (DVS / 4);
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < valid) x = Vec4<T>::load(vg + ((size_t)(t_begin + c0 + row) * p.H + h) * D + col0 + c * 4);
-            *reinterpret_cast<float4*>(Vs + row * VP + c * 4) = x;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = tid + i * NT, row = idx / (DVS / 4);
+            rv[i] = V4::zero();
+            if (row < valid) rv[i] = V4::load(vg + ((size_t)(t_begin + c0 + row) * p.H + h) * D + col0 + (idx % (DVS / 4)) * 4);
+        }
+        if (tid < 64) {
+            constexpr int PER = C >= 32 ? C / 32 : 1;
+            const float* gp = (tid >> 5) == 0 ? p.g_hist : p.g_rec;
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+                const int j = (tid & 31) * PER + e;
+                rg[e] = j < valid ? gp[(size_t)(t_begin + c0 + j) * p.H + h] : 1.f;
+            }
+        }
+    };
+    // Registers -> shared memory (rows past the end of the sequence are zeros), then the per-token decay terms.
+    auto stage = [&](bool with_q) {
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            const int idx = tid + i * NT, row = idx / (D / 4), c = (idx % (D / 4)) * 4;
+            if (row < C) {
+                if (with_q) *reinterpret_cast<float4*>(Qs + L::qk(row, c)) = V4::widen(rq[i]);
+                *reinterpret_cast<float4*>(Ks + L::qk(row, c)) = V4::widen(rk[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int idx = tid + i * NT, row = idx / (DVS / 4);
+            if (row < C) *reinterpret_cast<float4*>(Vs + row * VP + (idx % (DVS / 4)) * 4) = V4::widen(rv[i]);
         }
         // ---- inclusive scan of log-gates (fp64 accumulation) and of the zero-gate count
         if (tid < 64) {
             constexpr int PER = C >= 32 ? C / 32 : 1;
             const int i = tid >> 5, lane = tid & 31;
-            const float* gp = i == 0 ? p.g_hist : p.g_rec;
             double lg[PER];
             int zz[PER];
             double run = 0.0;
             int zrun = 0;
 #pragma unroll
             for (int e = 0; e < PER; ++e) {
-                const int j = lane * PER + e;
-                float g = 1.f;
-                if (j < valid) g = gp[(size_t)(t_begin + c0 + j) * p.H + h];
+                const float g = rg[e];
                 const bool zero = !(g > 0.f);
                 run += zero ? 0.0 : (double)logf(g);
                 zrun += zero ? 1 : 0;
@@ -145,86 +182,222 @@ __global__ void __launch_bounds__(256) prefill_simt_kernel(const PrefillParams p
                 const int zup = __shfl_up_sync(0xffffffffu, zrun, off);
                 if (lane >= off) { run += up; zrun += zup; }
             }
-            const double excl = run - lg[PER - 1];
-            const int zexcl = zrun - zz[PER - 1];
+            const double excl = run - lg[PER - 1], last = __shfl_sync(0xffffffffu, run, 31);
+            const int zexcl = zrun - zz[PER - 1], zl = __shfl_sync(0xffffffffu, zrun, 31);
+            const float bl = (float)last, Wi = i == 0 ? W1 : W2;
 #pragma unroll
             for (int e = 0; e < PER; ++e) {
                 const int j = lane * PER + e;
                 if (j < C) {
-                    bb[i * C + j] = (float)(excl + lg[e]);
-                    zc[i * C + j] = zexcl + zz[e];
+                    const float b = (float)(excl + lg[e]);
+                    const int z = zexcl + zz[e];
+                    bb[i * C + j] = b;
+                    zc[i * C + j] = z;
+                    rowf[i * C + j] = z == 0 ? Wi * expf(b) : 0.f;
+                    ww[i * C + j] = z == zl ? expf(bl - b) : 0.f;
                 }
             }
+            if (lane == 0) a_dec[i] = zl == 0 ? expf(bl) : 0.f;
         }
-        __syncthreads();
-        if (tid < 2 * C) {
-            const int i = tid / C, j = tid % C;
-            const float bl = bb[i * C + C - 1];
-            const int zl = zc[i * C + C - 1];
-            const float b = bb[i * C + j];
-            const int z = zc[i * C + j];
-            rowf[i * C + j] = (z == 0) ? (i == 0 ? W1 : W2) * expf(b) : 0.f;
-            ww[i * C + j] = (z == zl) ? expf(bl - b) : 0.f;
-            if (j == 0) a_dec[i] = (zl == 0) ? expf(bl) : 0.f;
+    };
+    // S <- a S + (K (.) w)^T V on this thread's tile
+    auto update = [&]() {
+        float u[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) u[a][b] = 0.f;
+        const float* w = ww + si * C;
+#pragma unroll 4
+        for (int t = 0; t < C; ++t) {
+            const float4 kv = *reinterpret_cast<const float4*>(Ks + L::qk(t, k0));
+            const float4 vv = *reinterpret_cast<const float4*>(Vs + t * VP + n0);
+            const float wt = w[t];
+            const float ka[4] = {kv.x * wt, kv.y * wt, kv.z * wt, kv.w * wt};
+            const float va[4] = {vv.x, vv.y, vv.z, vv.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) u[a][b] = fmaf(ka[a], va[b], u[a][b]);
         }
+        const float ad = a_dec[si];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) s[a][b] = fmaf(ad, s[a][b], u[a][b]);
+    };
+    auto publish = [&]() {      // the tile -> its place in shared memory
+#pragma unroll
+        for (int a = 0; a < 4; ++a) *reinterpret_cast<float4*>(Sme + a * VP) = make_float4(s[a][0], s[a][1], s[a][2], s[a][3]);
+    };
+
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) s[a][b] = 0.f;
+    bool staged = false;      // the segment's only chunk is in shared memory already
+    if (segs > 1) {
+        // ---- summary of this segment, left in Ss and a_seg for the later segments
+        if (c_end < nchunks) {
+            const bool only = c_end - c_begin == 1;      // then Q is staged with it and the second pass starts from there
+            float as = 1.f;
+            fetch(c_begin, only);
+            for (int c = c_begin; c < c_end; ++c) {
+                stage(only);
+                __syncthreads();
+                if (c + 1 < c_end) fetch(c + 1, false);
+                update();
+                as *= a_dec[si];
+                __syncthreads();
+            }
+            staged = only;
+            publish();
+            if (tid % (2 * D) == 0) a_seg[si] = as;
+        }
+        tc::cluster_sync_all();
+        // ---- initial states: the slot (or zero) pushed through the earlier segments.  Each CTA does this for its share of the
+        // elements and for every segment: it reads the share out of all summaries and writes the initial states over them, so
+        // every CTA reads and writes 1 / segs of what a fold per segment would pull from the first CTAs of the cluster.
+        for (int f = seg * (2 * D * 8 / segs) + tid; f < (seg + 1) * (2 * D * 8 / segs); f += NT) {
+            const int fi = f / (D * 8), k = (f / 8) % D, c = (f & 7) * 4;
+            const float* slot_at = p.state + (((size_t)slot * 2 + fi) * p.H + h) * (size_t)(D * D) + (size_t)k * D + col0 + c;
+            float4 x = p.use_initial_state ? *reinterpret_cast<const float4*>(slot_at) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const uint32_t at = tc::smem_u32(Ss + (fi * D + k) * VP + c), a_at = tc::smem_u32(&a_seg[fi]);
+            float4 u[7];
+            float as[7];
+#pragma unroll
+            for (int e = 0; e < 7; ++e)
+                if (e < segs - 1) {
+                    u[e] = tc::ld_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e));
+                    as[e] = tc::ld_cluster_f32(tc::map_to_cta(a_at, (uint32_t)e));
+                }
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e < segs) {
+                    tc::st_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e), x.x, x.y, x.z, x.w);
+                    // (segments behind the sequence's last chunk have no summary, and nobody uses what they would start from)
+                    if (e < 7) { x.x = fmaf(as[e], x.x, u[e].x); x.y = fmaf(as[e], x.y, u[e].y); x.z = fmaf(as[e], x.z, u[e].z); x.w = fmaf(as[e], x.w, u[e].w); }
+                }
+        }
+        tc::cluster_sync_all();      // the initial states are in place; every read of the slot is done
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 x = *reinterpret_cast<const float4*>(Sme + a * VP);
+            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
+        }
+        if (c_begin >= c_end && !(seg == 0 && nchunks == 0)) return;
+    } else if (p.use_initial_state) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 x = *reinterpret_cast<const float4*>(G + (size_t)a * D);
+            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
+        }
+    }
+    if (!staged && c_begin < c_end) fetch(c_begin, true);
+    for (int c = c_begin; c < c_end; ++c) {
+        const int c0 = c * C, valid = min(C, len - c0);
+        publish();
+        if (!staged) stage(true);
         __syncthreads();
-        // ---- masked scores: 4x4 tiles of the lower triangle
-        for (int tile = tid; tile < (C / 4) * (C / 4); tile += NT) {
-            const int j0 = (tile / (C / 4)) * 4, s0 = (tile % (C / 4)) * 4;
+        if (c + 1 < c_end) fetch(c + 1, true);
+        // ---- masked scores: 4 x 4 tiles of the lower triangle, tile t of row group r is number r (r + 1) / 2 + t
+        constexpr int TILES = (C / 4) * (C / 4 + 1) / 2;
+        for (int it = tid; it < ((TILES * SPLIT + 31) & ~31); it += NT) {
+            const int tile = min(it / SPLIT, TILES - 1), part = it % SPLIT;
+            int r = (int)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);
+            if (r * (r + 1) / 2 > tile) --r;
+            if ((r + 1) * (r + 2) / 2 <= tile) ++r;
+            const int j0 = 4 * r, s0 = 4 * (tile - r * (r + 1) / 2);
             float acc[4][4];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-            if (s0 <= j0) {
-                for (int kk = 0; kk < D; kk += 4) {
-                    float4 qv[4], kv[4];
+#pragma unroll 2
+            for (int kk = 4 * part; kk < D; kk += 4 * SPLIT) {
+                float4 qv[4], kv[4];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + (j0 + a) * DP + kk);
+                for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + L::qk(j0 + a, kk));
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) kv[b] = *reinterpret_cast<const float4*>(Ks + (s0 + b) * DP + kk);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            acc[a][b] = fmaf(qv[a].x, kv[b].x, acc[a][b]);
-                            acc[a][b] = fmaf(qv[a].y, kv[b].y, acc[a][b]);
-                            acc[a][b] = fmaf(qv[a].z, kv[b].z, acc[a][b]);
-                            acc[a][b] = fmaf(qv[a].w, kv[b].w, acc[a][b]);
-                        }
-                }
+                for (int b = 0; b < 4; ++b) kv[b] = *reinterpret_cast<const float4*>(Ks + L::qk(s0 + b, kk));
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        const int j = j0 + a, s = s0 + b;
-                        float m = 0.f;
-                        if (s <= j) {
-                            const float d1 = (zc[j] == zc[s]) ? expf(bb[j] - bb[s]) : 0.f;
-                            const float d2 = (zc[C + j] == zc[C + s]) ? expf(bb[C + j] - bb[C + s]) : 0.f;
-                            m = W1 * d1 + W2 * d2;
-                        }
-                        acc[a][b] *= m;
+                        acc[a][b] = fmaf(qv[a].x, kv[b].x, acc[a][b]);
+                        acc[a][b] = fmaf(qv[a].y, kv[b].y, acc[a][b]);
+                        acc[a][b] = fmaf(qv[a].z, kv[b].z, acc[a][b]);
+                        acc[a][b] = fmaf(qv[a].w, kv[b].w, acc[a][b]);
                     }
             }
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-                *reinterpret_cast<float4*>(Ps + (j0 + a) * CP + s0) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+            for (int a = 0; a < 4; ++a) {
+                if (SPLIT > 1) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) acc[a][b] += __shfl_xor_sync(0xffffffffu, acc[a][b], 1);
+                }
+                if (part == 0) *reinterpret_cast<float4*>(Ps + (j0 + a) * CP + s0) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+            }
         }
         __syncthreads();
-        // ---- outputs: 4 rows x 2 columns per thread
-        for (int tile = tid; tile < (C / 4) * (DVS / 2); tile += NT) {
+        // ---- decay mask, one element per thread and round (the tiles above keep half of the threads busy, this all of them)
+#pragma unroll 2
+        for (int idx = tid; idx < C * C; idx += NT) {
+            const int j = idx / C, t = idx % C;
+            if (t <= (j | 3)) {
+                float m = 0.f;
+                if (t <= j) {
+                    const float d1 = (zc[j] == zc[t]) ? expf(bb[j] - bb[t]) : 0.f;
+                    const float d2 = (zc[C + j] == zc[C + t]) ? expf(bb[C + j] - bb[C + t]) : 0.f;
+                    m = W1 * d1 + W2 * d2;
+                }
+                Ps[j * CP + t] *= m;
+            }
+        }
+        __syncthreads();
+        // ---- outputs: 4 rows x 2 columns; with SPLIT = 2 lane `part` reads out state `part` and takes every other 4 columns of P
+        for (int it = tid; it < (C / 4) * (DVS / 2) * SPLIT; it += NT) {
+            const int part = it % SPLIT, tile = it / SPLIT;
             const int j0 = (tile / (DVS / 2)) * 4, m0 = (tile % (DVS / 2)) * 2;
-            float acc[4][2], r1[4][2], r2[4][2];
+            float acc[4][2];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) { acc[a][0] = acc[a][1] = r1[a][0] = r1[a][1] = r2[a][0] = r2[a][1] = 0.f; }
-            for (int s = 0; s < j0 + 4; s += 4) {  // masked scores are 0 beyond the diagonal tile
+            for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 2 / SPLIT; ++i) {
+                const int st = SPLIT > 1 ? part : i;
+                const float* S = Ss + st * D * VP + m0;
+                float r[4][2];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) r[a][0] = r[a][1] = 0.f;
+#pragma unroll 2
+                for (int kk = 0; kk < D; kk += 4) {
+                    float4 qv[4];
+                    float2 x[4];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + L::qk(j0 + a, kk));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float2*>(S + (kk + e) * VP);
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        r[a][0] = fmaf(qv[a].x, x[0].x, r[a][0]); r[a][1] = fmaf(qv[a].x, x[0].y, r[a][1]);
+                        r[a][0] = fmaf(qv[a].y, x[1].x, r[a][0]); r[a][1] = fmaf(qv[a].y, x[1].y, r[a][1]);
+                        r[a][0] = fmaf(qv[a].z, x[2].x, r[a][0]); r[a][1] = fmaf(qv[a].z, x[2].y, r[a][1]);
+                        r[a][0] = fmaf(qv[a].w, x[3].x, r[a][0]); r[a][1] = fmaf(qv[a].w, x[3].y, r[a][1]);
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float f = rowf[st * C + j0 + a];
+                    acc[a][0] = fmaf(f, r[a][0], acc[a][0]); acc[a][1] = fmaf(f, r[a][1], acc[a][1]);
+                }
+            }
+            for (int t = 4 * part; t < j0 + 4; t += 4 * SPLIT) {  // masked scores are 0 beyond the diagonal tile
                 float4 pv[4];
                 float2 vv[4];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) pv[a] = *reinterpret_cast<const float4*>(Ps + (j0 + a) * CP + s);
+                for (int a = 0; a < 4; ++a) pv[a] = *reinterpret_cast<const float4*>(Ps + (j0 + a) * CP + t);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) vv[e] = *reinterpret_cast<const float2*>(Vs + (s + e) * VP + m0);
+                for (int e = 0; e < 4; ++e) vv[e] = *reinterpret_cast<const float2*>(Vs + (t + e) * VP + m0);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
                     acc[a][0] = fmaf(pv[a].x, vv[0].x, acc[a][0]); acc[a][1] = fmaf(pv[a].x, vv[0].y, acc[a][1]);
@@ -233,100 +406,57 @@ __global__ void __launch_bounds__(256) prefill_simt_kernel(const PrefillParams p
                     acc[a][0] = fmaf(pv[a].w, vv[3].x, acc[a][0]); acc[a][1] = fmaf(pv[a].w, vv[3].y, acc[a][1]);
                 }
             }
-            for (int kk = 0; kk < D; kk += 4) {
-                float4 qv[4];
-                float2 x1[4], x2[4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + (j0 + a) * DP + kk);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    x1[e] = *reinterpret_cast<const float2*>(Ss + (kk + e) * VP + m0);
-                    x2[e] = *reinterpret_cast<const float2*>(Ss + D * VP + (kk + e) * VP + m0);
-                }
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    r1[a][0] = fmaf(qv[a].x, x1[0].x, r1[a][0]); r1[a][1] = fmaf(qv[a].x, x1[0].y, r1[a][1]);
-                    r1[a][0] = fmaf(qv[a].y, x1[1].x, r1[a][0]); r1[a][1] = fmaf(qv[a].y, x1[1].y, r1[a][1]);
-                    r1[a][0] = fmaf(qv[a].z, x1[2].x, r1[a][0]); r1[a][1] = fmaf(qv[a].z, x1[2].y, r1[a][1]);
-                    r1[a][0] = fmaf(qv[a].w, x1[3].x, r1[a][0]); r1[a][1] = fmaf(qv[a].w, x1[3].y, r1[a][1]);
-                    r2[a][0] = fmaf(qv[a].x, x2[0].x, r2[a][0]); r2[a][1] = fmaf(qv[a].x, x2[0].y, r2[a][1]);
-                    r2[a][0] = fmaf(qv[a].y, x2[1].x, r2[a][0]); r2[a][1] = fmaf(qv[a].y, x2[1].y, r2[a][1]);
-                    r2[a][0] = fmaf(qv[a].z, x2[2].x, r2[a][0]); r2[a][1] = fmaf(qv[a].z, x2[2].y, r2[a][1]);
-                    r2[a][0] = fmaf(qv[a].w, x2[3].x, r2[a][0]); r2[a][1] = fmaf(qv[a].w, x2[3].y, r2[a][1]);
-                }
-            }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
+                if (SPLIT > 1) {
+                    acc[a][0] += __shfl_xor_sync(0xffffffffu, acc[a][0], 1);
+                    acc[a][1] += __shfl_xor_sync(0xffffffffu, acc[a][1], 1);
+                }
                 const int j = j0 + a;
-                if (j < valid) {
-                    const float f1 = rowf[j], f2 = rowf[C + j];
-                    const float o0 = acc[a][0] + f1 * r1[a][0] + f2 * r2[a][0];
-                    const float o1 = acc[a][1] + f1 * r1[a][1] + f2 * r2[a][1];
-                    store2(og + ((size_t)(t_begin + c0 + j) * p.H + h) * D + col0 + m0, o0, o1);
-                }
+                if (a / (4 / SPLIT) == part && j < valid)
+                    store2(og + ((size_t)(t_begin + c0 + j) * p.H + h) * D + col0 + m0, acc[a][0], acc[a][1]);
             }
         }
-        // ---- state carry in registers: S <- a S + (K (.) w)^T V
-        if (own) {
-            float u1[4][4], u2[4][4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) u1[a][b] = u2[a][b] = 0.f;
-            for (int s = 0; s < C; ++s) {
-                const float4 kv = *reinterpret_cast<const float4*>(Ks + s * DP + k0);
-                const float4 vv = *reinterpret_cast<const float4*>(Vs + s * VP + n0);
-                const float w1 = ww[s], w2 = ww[C + s];
-                const float ka[4] = {kv.x, kv.y, kv.z, kv.w};
-                const float va[4] = {vv.x, vv.y, vv.z, vv.w};
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float k1 = ka[a] * w1, k2 = ka[a] * w2;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        u1[a][b] = fmaf(k1, va[b], u1[a][b]);
-                        u2[a][b] = fmaf(k2, va[b], u2[a][b]);
-                    }
-                }
-            }
-            const float a1 = a_dec[0], a2 = a_dec[1];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    s1[a][b] = fmaf(a1, s1[a][b], u1[a][b]);
-                    s2[a][b] = fmaf(a2, s2[a][b], u2[a][b]);
-                }
-        }
-        __syncthreads();  // every readout of the old state copy is done
-        if (own) {
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                *reinterpret_cast<float4*>(Ss + (k0 + a) * VP + n0) = make_float4(s1[a][0], s1[a][1], s1[a][2], s1[a][3]);
-                *reinterpret_cast<float4*>(Ss + D * VP + (k0 + a) * VP + n0) = make_float4(s2[a][0], s2[a][1], s2[a][2], s2[a][3]);
-            }
-        }
+        if (c_end < nchunks && c + 1 == c_end) break;      // not the last segment: its final state is nobody's
+        update();
+        __syncthreads();  // every read of this chunk's tiles and of the old state copy is done
     }
-    if (own) {
+    if (c_end == nchunks) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            *reinterpret_cast<float4*>(G1 + (size_t)(k0 + a) * D + col0 + n0) = make_float4(s1[a][0], s1[a][1], s1[a][2], s1[a][3]);
-            *reinterpret_cast<float4*>(G2 + (size_t)(k0 + a) * D + col0 + n0) = make_float4(s2[a][0], s2[a][1], s2[a][2], s2[a][3]);
-        }
+        for (int a = 0; a < 4; ++a) *reinterpret_cast<float4*>(G + (size_t)a * D) = make_float4(s[a][0], s[a][1], s[a][2], s[a][3]);
     }
+}
+
+// Segments per sequence: while a doubling still fits the SMs twice over (the extra pass over K and V for the summaries costs
+// less than idle SMs) and leaves every segment a chunk of the longest sequence.
+static int plan_segments(long long units, int max_chunks) {
+    int segs = 1;
+    while (segs < 8 && units * segs * 2 <= 2 * 148 && segs * 2 <= max_chunks) segs *= 2;
+    return segs;
 }
 
 template <int D, int C, typename T>
 static dsla_status launch_one(const PrefillParams& p, cudaStream_t s) {
-    constexpr int DVS = 32, DP = D + 4, VP = DVS + 4, CP = C + 4;
-    constexpr size_t smem = sizeof(float) * (2 * C * DP + C * VP + C * CP + 2 * D * VP + 6 * C) + sizeof(int) * 2 * C;
-    static bool configured = false;  // per process; the attribute is per function and device-wide enough here
-    cudaError_t e = cudaFuncSetAttribute(prefill_simt_kernel<D, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    (void)configured;
-    if (e != cudaSuccess) return DSLA_ERR_CUDA;
-    const long long blocks = (long long)p.N * p.H * (D / DVS);
-    if (blocks > 0x7fffffffLL) return DSLA_ERR_UNSUPPORTED;
-    prefill_simt_kernel<D, C, T><<<dim3((unsigned)blocks), dim3(256), smem, s>>>(p);
+    constexpr size_t smem = sizeof(float) * Layout<D, C>::END;
+    if (cudaFuncSetAttribute(prefill_simt_kernel<D, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DSLA_ERR_CUDA;
+    const long long units = (long long)p.N * p.H * (D / DVS);
+    const int segs = plan_segments(units, p.max_chunks);
+    if (units * segs > 0x7fffffffLL) return DSLA_ERR_UNSUPPORTED;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(units * segs));
+    cfg.blockDim = dim3(4 * D);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)segs;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = segs > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, prefill_simt_kernel<D, C, T>, p, segs) != cudaSuccess) return DSLA_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DSLA_OK : DSLA_ERR_CUDA;
 }

@@ -31,3 +31,24 @@ def test_gate_project_cluster_splits(T, H, D_model):
     assert np.max(np.abs(got - ref)) <= 2e-5
     assert bool((gh[:T] <= 1.0).all()) and bool((gr[:T] <= 1.0).all())      # every row written
     assert bool((gh[T:] == 7.0).all()) and bool((gr[T:] == 7.0).all())      # and none past the end
+
+
+# CUDA-core chunkwise prefill: 8, 4, 2 and 1 segments per sequence (one cluster each), segments of one chunk and of several, a last
+# segment of one token, segments without a chunk (a packed batch's short sequences), and an empty sequence in a cluster
+@pytest.mark.parametrize("lens,H,d,dtype,chunk", [
+    ((512,), 4, 64, torch.float32, 64), ((513,), 2, 128, torch.float32, 64), ((1100,), 9, 64, torch.float32, 64),
+    ((1025,), 18, 64, BF, 32), ((260,), 80, 64, torch.float32, 64), ((700, 0, 65, 1), 2, 64, torch.float32, 64),
+    ((129, 64, 300), 1, 128, BF, 16)])
+@pytest.mark.parametrize("resume", [False, True])
+def test_simt_prefill_segments(lens, H, d, dtype, chunk, resume):
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, gpu_prefill, oracle_prefill, rel_err
+    inp = gen.make_packed(5200 + sum(lens) + H, lens, H, d, dtype)
+    inp.g_rec[::37] = 0.0                   # exact zeros inside and at the edges of segments
+    inp.g_hist[100::211] = 0.0
+    slots = np.random.default_rng(1).permutation(len(lens) + 1)[:len(lens)].astype(np.int32)
+    state0 = gen.make_states(5201, len(lens) + 1, H, d, d, std=0.5).numpy() if resume else None
+    o, S = gpu_prefill(inp, num_slots=len(lens) + 1, state0=state0, slots=slots, chunk=chunk, impl="simt", scale=0.8)
+    start = np.zeros(S.shape) if state0 is None else state0.astype(np.float64)
+    o_ref, S_ref = oracle_prefill(inp, state0=start, slots=slots, scale=0.8)
+    assert rel_err(o, o_ref) <= TOL[dtype] and rel_err(S[slots], S_ref[slots]) <= TOL[torch.float32]
