@@ -47,11 +47,11 @@ prefill_tc_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const int h = (blockIdx.x / nsum) % p.H;
     const int rank = blockIdx.x / (nsum * p.H);
     const int n = tp.order ? tp.order[rank] : rank;
-    const SeqInfo sq = seq_info(p, n, g, tp.nseg, tp.cps, tp.skew8);
+    const SeqInfo sq = seq_info(p, n, g, tp);
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (sq.len <= 0 || g >= sq.last_seg) return;      // only segments that have a successor
-    const int nc = sq.c_end - sq.c_begin;             // full chunks only (not the sequence's last segment)
-    const int t0 = sq.t_begin + sq.c_begin * C;
+    const int nc = (sq.c_end - sq.c_begin) * (tp.chunk / C);      // full chunks only (not the sequence's last segment)
+    const int t0 = sq.t_begin + sq.c_begin * tp.chunk;
     float* out = tp.ws + ((size_t)(n * p.H + h) * tp.nseg + g) * (SUMMARY_STRIDE / 4);
 
     if (tid == 0) {
@@ -270,14 +270,14 @@ EncodeFn get_encode() {
 }  // namespace
 
 // [T_total, H, 128] bf16 seen as (x: 64 elements, t, half: the two 64-element halves of a row, h) so that one
-// copy of box {64, 64 tokens, 2, 1} lands as two consecutive 8 KB tiles [half][token][64], each in the 128-byte
+// copy of box {64, box_tokens, 2, 1} lands as two consecutive tiles [half][token][64], each in the 128-byte
 // swizzle the MMA descriptors expect.
-bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H) {
+bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H, int box_tokens) {
     EncodeFn fn = get_encode();
     if (!fn) return false;
     cuuint64_t dims[4] = {64, (cuuint64_t)T_total, 2, (cuuint64_t)H};
     cuuint64_t strides[3] = {(cuuint64_t)H * D * 2, 128, (cuuint64_t)D * 2};
-    cuuint32_t box[4] = {64, 64, 2, 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)box_tokens, 2, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

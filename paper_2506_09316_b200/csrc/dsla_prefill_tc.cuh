@@ -1,4 +1,4 @@
-// Pieces shared by the translation units of the tensor-core prefill (bf16, d = 128, chunk C = 64):
+// Pieces shared by the translation units of the tensor-core prefill (bf16, d = 128):
 // launch parameters, the split of a sequence into segments along T, the layout of the segment
 // summaries in the workspace, and the cold-path helpers that move a state between global memory and
 // TMEM.  Functions here are inline or static.
@@ -10,7 +10,7 @@ namespace dsla {
 
 using namespace tc;
 
-constexpr int C = 64;                 // tokens per chunk
+constexpr int C = 64;                 // tokens per chunk of the cluster variant and the summaries
 constexpr int D = 128;                // head size
 // One summary per (sequence, head, segment): U (both states, fp32 [2][D][D]) followed by the two
 // segment decays A[2], padded to a multiple of 256 bytes.
@@ -23,6 +23,7 @@ struct TcParams {
     const float* init;  // initial states the segments start from: the slots themselves, or a snapshot of them
                         // [(n*H + h)][2][D][D] taken before the main grid when a sequence is split (the CTA of the
                         // last segment overwrites the slot while CTAs of earlier segments may not have read it yet)
+    int chunk;          // tokens per chunk of the main grid (a multiple of C): the unit of cps
     int nseg;           // segments per sequence (grid dimension)
     int cps;            // chunks per segment (mean)
     int skew8;          // eighths of a chunk by which consecutive segments get shorter (later segments start later: they
@@ -62,13 +63,14 @@ struct SeqInfo {
 // chunks longer than the mean.  seg_begin(0) = 0 and seg_begin(nseg) = nseg cps.
 __host__ __device__ __forceinline__ int seg_begin(int g, int nseg, int cps, int skew8) { return g * cps + (skew8 * g * (nseg - g)) / 8; }
 
-__device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g, int nseg, int cps, int skew8) {
+__device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g, const TcParams& tp) {
+    const int nseg = tp.nseg, cps = tp.cps, skew8 = tp.skew8;
     SeqInfo s;
     s.t_begin = p.cu_seqlens ? p.cu_seqlens[n] : n * p.T;
     const int t_end = p.cu_seqlens ? p.cu_seqlens[n + 1] : (n + 1) * p.T;
     s.len = t_end - s.t_begin;
     s.slot = p.slots ? p.slots[n] : n;
-    s.nchunks = (s.len + C - 1) / C;
+    s.nchunks = (s.len + tp.chunk - 1) / tp.chunk;
     s.c_begin = seg_begin(g, nseg, cps, skew8);
     s.c_end = min(s.nchunks, seg_begin(g + 1, nseg, cps, skew8));
     s.last_seg = 0;     // the last segment that holds a chunk of this sequence
@@ -123,7 +125,7 @@ static __device__ __noinline__ void store_state(float* dst, int v, uint32_t s_ad
 }
 
 // dsla_prefill_summary.cu: helper launches of the tensor-core prefill (all enqueue on s and count themselves)
-bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H);
+bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H, int box_tokens);
 void launch_seq_order(const int32_t* cu, int N, int* order, cudaStream_t s);
 void launch_state_snapshot(const PrefillParams& p, float* snap, cudaStream_t s);
 dsla_status launch_summary(const CUtensorMap& mk, const CUtensorMap& mv, const TcParams& tp, cudaStream_t s);

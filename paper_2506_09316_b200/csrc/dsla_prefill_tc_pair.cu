@@ -105,7 +105,7 @@ prefill_tc_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const int h = (u % units) % p.H;
     const int seq_rank = (u % units) / p.H;
     const int n = tp.order ? tp.order[seq_rank] : seq_rank;
-    const SeqInfo sq = seq_info(p, n, g, tp.nseg, tp.cps, tp.skew8);
+    const SeqInfo sq = seq_info(p, n, g, tp);
     // Every early exit below depends only on values both CTAs of the cluster share, and comes before any cluster
     // operation.
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
@@ -270,7 +270,7 @@ prefill_tc_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     } else if (warp == WARP_GATE) {
         // ------------------------------------------------------------------ gate warp
         // Everything a chunk needs from the gates comes from the cumulative log-gates
-        //     L^i_j = sum_{t <= j} log2 g^i_t      (inclusive, from the chunk start; a zero gate counts as -200, so any
+        //     L^i_j = sum_{t <= j} log2 g^i_t      (inclusive, from the chunk start; a zero gate counts as -130, so any
         //                                           product that contains one flushes to an exact zero)
         // through independent exponentials.  Lane l holds tokens l and l + 32.  The chunk decay a that carries the state
         // is the plain product of the gates.

@@ -74,7 +74,7 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 }
 // Gives up after `limit` parked waits or about a second, whichever comes first.
 template <bool CLUSTER>
-__device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, uint32_t limit) {
+__device__ __forceinline__ bool mbar_wait_loop(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, uint32_t limit) {
     const uint64_t t0 = global_timer_ns();
     for (uint32_t i = 0; i < limit; ++i) {
         if (mbar_try_wait_t<CLUSTER>(bar, parity)) return true;
@@ -87,10 +87,18 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, vola
     atomicExch(status, 5 /* DSLA_ERR_TIMEOUT */);
     return false;
 }
+template <bool CLUSTER>
+__device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, uint32_t limit) {
+    return mbar_wait_loop<CLUSTER>(bar, parity, abort_flag, status, limit);
+}
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           uint32_t limit = MBAR_WAIT_LIMIT) {
     if (mbar_test_wait_t<false>(bar, parity)) return true;
     return mbar_wait_slow<false>(bar, parity, abort_flag, status, limit);
+}
+// The same without a call: for a wait across which a warp holds many registers (a call would spill them).
+__device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    return mbar_wait_loop<false>(bar, parity, abort_flag, status, MBAR_WAIT_LIMIT);
 }
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                   uint32_t limit = MBAR_WAIT_LIMIT) {
@@ -163,6 +171,11 @@ __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t saddr) {
     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(saddr));
     return (uint32_t)v;
 }
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t saddr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(saddr));
+    return v;
+}
 __device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -181,6 +194,15 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
                  "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
                  : "memory");
 }
+// Tile store: rows of this CTA's shared memory (written before a fence_proxy_async_smem) to global memory.
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, const void* smem_src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(map), "r"(smem_u32(smem_src)), "r"(c0),
+                 "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }      // the sources have been read
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
     asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
                  : "memory");
@@ -209,6 +231,14 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// True in one thread of the warp.  Behind this test (and not behind lane == 0) the compiler keeps the operands of the
+// MMAs in uniform registers: an MMA with A in TMEM takes 32 cycles to issue instead of 51.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+    return p != 0;
+}
 
 // ---- descriptors ---------------------------------------------------------------------------------
 // Shared-memory matrix descriptor, 128-byte swizzle.  Addresses and offsets in bytes (multiples of 16).
@@ -244,6 +274,25 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The same with only the low words of the descriptors (address and lbo) passed: the high word is that of smem_desc_sw128
+// with 1024 bytes between 8-row groups, which every operand of the single-CTA prefill has.
+constexpr uint32_t DESC_HI_SW128 = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo) { return ((saddr & 0x3FFFFu) >> 4) | (((lbo >> 4) & 0x3FFFu) << 16); }
+__device__ __forceinline__ void mma_ss_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(DESC_HI_SW128)
+        : "memory");
+}
+__device__ __forceinline__ void mma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 db;\n setp.ne.b32 p, %4, 0;\n mov.b64 db, {%2, %5};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(blo), "r"(idesc), "r"(accumulate), "r"(DESC_HI_SW128)
         : "memory");
 }
 
@@ -293,6 +342,13 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t saddr, uint32_t r0, u
 __device__ __forceinline__ void tmem_st_16x128b(uint32_t taddr, uint32_t a, uint32_t b) {
     asm volatile("tcgen05.st.sync.aligned.16x128b.x1.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
 }
+// Eight of them side by side: 16 lanes x 32 columns, v[2 i] and v[2 i + 1] are a and b of columns 4 i .. 4 i + 3.
+__device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_t* v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x128b.x8.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::DSLA_W8(v, 0), DSLA_W8(v, 8),
+        "r"(taddr)
+        : "memory");
+}
 // Four 8x8 matrices of 16-bit elements, transposed: thread t supplies the address of row t % 8 of matrix t / 8 and
 // receives, per matrix, the elements (rows 2 (t % 4), 2 (t % 4) + 1; column t / 4) in the low / high half of a register.
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -333,12 +389,12 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// log2 of a gate in [0, 1]; zero (and anything below the smallest normal) maps to a finite, very negative
-// value so that sums of logs stay finite and 2^(sum) still flushes to an exact zero
+// log2 of a gate in [0, 1]; zero (and anything below the smallest normal) maps to -130: sums of logs stay finite (and small
+// enough to keep the differences of later tokens precise) and 2^(sum) still flushes to an exact zero
 __device__ __forceinline__ float lg2_gate(float g) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(g));
-    return g >= 1.17549435e-38f ? y : -200.f;
+    return g >= 1.17549435e-38f ? y : -130.f;
 }
 // inclusive prefix sum over the lanes of a warp
 __device__ __forceinline__ float warp_prefix_sum(float x, int lane) {
@@ -350,6 +406,14 @@ __device__ __forceinline__ float warp_prefix_sum(float x, int lane) {
     return x;
 }
 
+// products of the two bf16 halves
+__device__ __forceinline__ uint32_t hmul2_u32(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 r = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+// the two bf16 halves of a word, widened
+__device__ __forceinline__ float2 unpack_bf16(uint32_t x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
+__device__ __forceinline__ uint32_t word_of(const uint4& x, int i) { return i == 0 ? x.x : i == 1 ? x.y : i == 2 ? x.z : x.w; }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // .x (low 16 bits) = lo
     return *reinterpret_cast<uint32_t*>(&h);
