@@ -136,8 +136,10 @@ typedef struct {
     void* workspace;            /* scratch of dsla_prefill_workspace_bytes(); may be NULL if 0    */
     size_t workspace_bytes;
     dsla_gate_layout gate_layout; /* SCALAR (0): g_hist, g_rec are [T_total, H].  PER_KEY_CHANNEL: [T_total, H, d_k];
-                                   served by a token-by-token CUDA-core kernel (impl AUTO or SIMT; the tensor-core
-                                   kernels take scalar gates only: DSLA_ERR_UNSUPPORTED)                        */
+                                   impl AUTO takes the tensor-core kernel for vector gates (bf16, d = 128, gates on 16-byte
+                                   boundaries; it needs no workspace, but with one -- the size dsla_prefill_workspace_bytes
+                                   gives for scalar gates -- it splits long sequences), else, and for impl SIMT, a token-by-token
+                                   CUDA-core kernel.  impl TENSOR and TENSOR_PAIR take scalar gates only: DSLA_ERR_UNSUPPORTED */
 } dsla_prefill_args;
 
 /* Scratch the chosen kernel needs for these sizes (0 for the SIMT kernel): the segment summaries of

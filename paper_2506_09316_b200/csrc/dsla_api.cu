@@ -222,6 +222,7 @@ static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cu
     p.max_chunks = (a->max_seqlen + chunk - 1) / chunk;
     p.scale = a->scale; p.use_initial_state = a->use_initial_state ? 1 : 0;
     p.weights = nullptr; p.n_total = 2; p.state_first = 0; p.single = 0;
+    if (a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL && a->impl == DSLA_IMPL_AUTO && prefill_vec_applies(a)) return launch_prefill_vec(p, a, s);
     if (a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL) {
         // the dual state as two states whose weights the kernel derives from gamma: (gamma, 1 - gamma)
         RecurrentParams r{};

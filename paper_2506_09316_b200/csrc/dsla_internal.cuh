@@ -75,6 +75,9 @@ dsla_status gate_project_last_error();
 // dsla_prefill_recurrent.cu: gates[i] is the gate tensor of state i (n_states of them)
 dsla_status launch_prefill_recurrent(const RecurrentParams& p, const float* const* gates, int n_states, int d, dsla_dtype dt,
                                      cudaStream_t s);
+// dsla_prefill_vec.cu: gates per key channel on the tensor cores
+bool prefill_vec_applies(const dsla_prefill_args* a);
+dsla_status launch_prefill_vec(const PrefillParams& p, const dsla_prefill_args* a, cudaStream_t s);
 // dsla_prefill_simt.cu
 dsla_status launch_prefill_simt(const PrefillParams& p, int d, int chunk, dsla_dtype dt, cudaStream_t s);
 // dsla_prefill_summary.cu: one warp waits, with the given poll limit, on a barrier nobody arrives at

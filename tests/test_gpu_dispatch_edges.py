@@ -52,3 +52,31 @@ def test_simt_prefill_segments(lens, H, d, dtype, chunk, resume):
     start = np.zeros(S.shape) if state0 is None else state0.astype(np.float64)
     o_ref, S_ref = oracle_prefill(inp, state0=start, slots=slots, scale=0.8)
     assert rel_err(o, o_ref) <= TOL[dtype] and rel_err(S[slots], S_ref[slots]) <= TOL[torch.float32]
+
+
+# Gates per key channel on the tensor cores: whole and ragged chunks of 32 tokens, one token past a block, several segments (with the
+# workspace dsla_prefill brings) and one (impl="auto" without room), exact zeros and ones, sequences shorter than a segment
+@pytest.mark.parametrize("lens,H,resume", [((1,), 2, False), ((16,), 1, True), ((17,), 3, False), ((32,), 2, True), ((33, 31, 0, 64), 2, True),
+                                           ((257,), 2, False), ((515, 40, 260), 1, True), ((1030,), 37, False), ((300,), 80, True)])
+@pytest.mark.parametrize("pattern", ["mix", "zeros", "ones"])
+def test_channel_prefill_tensor(lens, H, resume, pattern):
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, gpu_prefill, oracle_prefill, rel_err
+    if pattern != "mix" and sum(lens) > 300:
+        pytest.skip("the long cases run with mixed gates")
+    inp = gen.make_packed(5300 + sum(lens) + H, lens, H, 128, BF)
+    rng = np.random.default_rng(5301)
+    shape = (inp.T_total, H, 128)
+    for name, mu in (("g_hist", 5.0), ("g_rec", 1.0)):
+        g = 1.0 / (1.0 + np.exp(-rng.normal(mu, 2.0, size=shape)))
+        u = rng.uniform(size=shape)
+        g = np.where(u < 0.02, 0.0, np.where(u > 0.98, 1.0, g)) if pattern == "mix" else np.full(shape, 0.0 if pattern == "zeros" else 1.0)
+        setattr(inp, name, torch.from_numpy(g.astype(np.float32)))
+    slots = rng.permutation(len(lens) + 1)[:len(lens)].astype(np.int32)
+    state0 = gen.make_states(5302, len(lens) + 1, H, 128, 128, std=0.5).numpy() if resume else None
+    start = np.zeros((len(lens) + 1, 2, H, 128, 128)) if state0 is None else state0.astype(np.float64)
+    o_ref, S_ref = oracle_prefill(inp, state0=start, slots=slots, scale=0.7)
+    o, S = gpu_prefill(inp, num_slots=len(lens) + 1, state0=state0, slots=slots, scale=0.7)
+    # states: fp32 sums of exact products (three bf16 terms of an fp32 factor); outputs: one bf16 rounding (2^-9 of the value)
+    assert rel_err(S[slots], S_ref[slots]) <= 1e-5
+    assert rel_err(o, o_ref) <= 4e-3
