@@ -273,15 +273,19 @@ EncodeFn get_encode() {
 // copy of box {64, box_tokens, 2, 1} lands as two consecutive tiles [half][token][64], each in the 128-byte
 // swizzle the MMA descriptors expect.
 bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H, int box_tokens) {
-    EncodeFn fn = get_encode();
-    if (!fn) return false;
     cuuint64_t dims[4] = {64, (cuuint64_t)T_total, 2, (cuuint64_t)H};
     cuuint64_t strides[3] = {(cuuint64_t)H * D * 2, 128, (cuuint64_t)D * 2};
     cuuint32_t box[4] = {64, (cuuint32_t)box_tokens, 2, 1};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tile_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+bool encode_tile_map(CUtensorMap* m, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                     const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
+    EncodeFn fn = get_encode();
+    if (!fn) return false;
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    return fn(m, type, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 void launch_bounded_wait_selftest(int* status, unsigned max_polls, cudaStream_t s) {

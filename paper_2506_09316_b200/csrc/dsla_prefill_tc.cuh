@@ -126,6 +126,8 @@ static __device__ __noinline__ void store_state(float* dst, int v, uint32_t s_ad
 
 // dsla_prefill_summary.cu: helper launches of the tensor-core prefill (all enqueue on s and count themselves)
 bool make_tile_map(CUtensorMap* m, const void* base, int T_total, int H, int box_tokens);
+bool encode_tile_map(CUtensorMap* m, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                     const cuuint32_t* box, CUtensorMapSwizzle swizzle);
 void launch_seq_order(const int32_t* cu, int N, int* order, cudaStream_t s);
 void launch_state_snapshot(const PrefillParams& p, float* snap, cudaStream_t s);
 dsla_status launch_summary(const CUtensorMap& mk, const CUtensorMap& mv, const TcParams& tp, cudaStream_t s);

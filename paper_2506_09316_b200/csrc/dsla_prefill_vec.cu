@@ -12,17 +12,15 @@
 // 16-token block are fp32 on CUDA cores, those between the chunk's two blocks are products of two-term operands scaled
 // to the block boundary.
 //
-// CTA = (sequence, head, segment), 16 warps, no fixed roles: the chunk loop alternates between the two states.
-//   phase A: pass over S_1 (two bf16 terms of it for the readout, then S_1 diag(A_1)) | MMAs of state 1 | operands of state 2
-//   phase B: pass over S_2, P~                                                        | MMAs of state 2 | operands of state 1, next chunk
-// so the operands of one state are built while the tensor core works on the other and nothing is double-buffered but
-// the raw Q, K and V.  Bound by instruction issue: about 85 slots per token and SM sub-partition for the operands and scores and
-// 40 for the passes over the states.
+// CTA = (sequence, head, segment), 16 warps in step: each step takes one state through its pass (two bf16 terms of it for the
+// readout, then S_i diag(A_i)) and its MMAs, and meanwhile builds the operands of the other state for its next turn, so
+// nothing but the raw inputs is double-buffered.  Bound by instruction issue: 7000 warp instructions per chunk and SM
+// sub-partition, half of them for the operands, a quarter for the scores; 15.8 k cycles per chunk.
 //
 // A sequence is split into segments when there are few (sequence, head) pairs and the caller's workspace has room: a first
 // grid accumulates each segment's state from zero, walking the chunks backwards with the product of all later gates (no pass
-// over the states), an elementwise kernel turns these summaries into initial states, the main grid starts from them.
-// T = 4096, 32 heads: 540 us (413 of them this file's main grid); 2490 us with the token-by-token kernel.
+// over the states), and the main grid folds the summaries of the earlier segments into its initial states.
+// T = 4096, 32 heads: 321 us (of them 68 for the summaries); 2490 us with the token-by-token kernel.
 #include "dsla_prefill_tc.cuh"
 
 namespace dsla {
@@ -42,14 +40,15 @@ constexpr int OFF_QB = OFF_PT + 2 * VC * 128;        // Q of block 1 scaled from
 constexpr int OFF_KB = OFF_QB + 2 * V_BTILE;         // K of block 0 scaled to its end, two terms
 constexpr int OFF_RAW = OFF_KB + 2 * V_BTILE;        // raw Q, K: [buffer][32][128] bf16
 constexpr int OFF_RAWK = OFF_RAW + 2 * V_TILE;
-constexpr int OFF_G = OFF_RAWK + 2 * V_TILE;         // gates: [state][32][128] fp32
-constexpr int OFF_SC = OFF_G + 2 * VC * D * 4;       // scores: [state][32][32] fp32
-constexpr int OFF_A = OFF_SC + 2 * VC * VC * 4;      // chunk decays: [state][128] fp32
+constexpr int V_GBYTES = 2 * VC * D * 4;
+constexpr int OFF_G = OFF_RAWK + 2 * V_TILE;         // gates: [buffer][state][32][128] fp32
+constexpr int OFF_SC = OFF_G + 2 * V_GBYTES;         // blended scores [buffer][32][32] fp32
+constexpr int OFF_A = OFF_SC + 2 * VC * VC * 4;          // chunk decays: [state][128] fp32
 constexpr int V_SMEM = OFF_A + 2 * D * 4 + 1024;
 // summaries reuse the front: V buffers, then K~ [parity][state][term]
 constexpr int OFF_SKT = 2 * V_TILE;
 constexpr int OFF_SG = OFF_SKT + 12 * V_TILE;        // gates [parity][state][32][128] fp32
-constexpr int OFF_SK = OFF_SG + 4 * VC * D * 4;      // raw K [parity]
+constexpr int OFF_SK = OFF_SG + 2 * V_GBYTES;        // raw K [parity]
 constexpr int V_SMEM_SUM = OFF_SK + 2 * V_TILE + 1024;
 // TMEM columns
 constexpr uint32_t VCOL_S = 0, VCOL_SB = 256, VCOL_O = 384;      // fp32 states 2 x 128, bf16 terms of one state 2 x 64, O^T 32
@@ -62,25 +61,24 @@ struct VecParams {
 };
 
 struct alignas(16) VecShared {
-    uint64_t raw_full[2], g2_full, done[2];
+    uint64_t raw_full[2], done[2];
     uint32_t tmem_base;
     int abort_flag;
-    short pair[2][72];   // score pair numbers -> row * 32 + column inside a block
 };
 
 // bf16 terms of a pair of fp32 values; x is left with what the term does not hold
 __device__ __forceinline__ uint32_t take_term(float2& x) {
     const uint32_t t = pack_bf16(x.x, x.y);
     const float2 f = unpack_bf16(t);
-    x = __fadd2_rn(x, make_float2(-f.x, -f.y));
+    x = __ffma2_rn(f, make_float2(-1.f, -1.f), x);      // exact
     return t;
 }
-__device__ __forceinline__ float2 clamp0(float2 g) { return make_float2(fmaxf(g.x, 0.f), fmaxf(g.y, 0.f)); }
 
-// Sum over the lanes of 32 values per lane: lane l is left with the total of v[l] (31 exchanges).
-__device__ __forceinline__ float transpose_sum(float (&v)[32], int lane) {
+// Sums over the lanes of N values per lane (a power of two): lane l is left with the total of v[l % N].
+template <int N>
+__device__ __forceinline__ float transpose_sum(float* v, int lane) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = N / 2; off > 0; off >>= 1) {
         const bool up = lane & off;
 #pragma unroll
         for (int i = 0; i < off; ++i) {
@@ -88,6 +86,8 @@ __device__ __forceinline__ float transpose_sum(float (&v)[32], int lane) {
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
+#pragma unroll
+    for (int off = N; off < 32; off <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
     return v[0];
 }
 
@@ -109,49 +109,53 @@ __device__ __forceinline__ VecUnit vec_unit(const VecParams& vp, int block, int 
     return u;
 }
 
-// One score block of 16 tokens: pairs (j, s < j) with s in [S0, S1), this lane's four channels, all pairs of a batch of 32 reduced
-// together.  q, k: raw rows of the block; g: gates.
-template <int S0, int S1>
-__device__ __forceinline__ void block_scores(const uint8_t* q, const uint8_t* k, const float* g, int valid, int lane, const short* pair, float* out) {
-    float2 kd[S1 - S0][2];
+// Blended scores of a block of 16 tokens: keys s0 .. s0 + 3 with tokens j_begin .. j_end - 1 (the current token, undecayed, included), four
+// channels per lane, four tokens per round.  Both states share the product with q and the sums over the lanes: their
+// decayed copies of k are added first.
+// (A loop over the tokens, not unrolled code: every role of this kernel passes through its code once per phase, and when that
+// does not fit the instruction cache all of them wait for it.  Unrolled to all pairs: twice the time per phase.)
+__device__ __forceinline__ void block_scores(const uint8_t* q, const uint8_t* k, const uint8_t* g, int s0, int j_begin, int j_end, float W1, float W2, int lane, float* out) {
+    float2 k1[4][2], k2[4][2];
 #pragma unroll
-    for (int s = S0; s < S1; ++s) {
-        const uint2 x = *reinterpret_cast<const uint2*>(k + s * 256 + lane * 8);
-        kd[s - S0][0] = s < valid ? unpack_bf16(x.x) : make_float2(0.f, 0.f);
-        kd[s - S0][1] = s < valid ? unpack_bf16(x.y) : make_float2(0.f, 0.f);
+    for (int e = 0; e < 4; ++e) {
+        const uint2 x = *reinterpret_cast<const uint2*>(k + (s0 + e) * 256 + lane * 8);
+        const float2 a = unpack_bf16(x.x), b = unpack_bf16(x.y);
+        k1[e][0] = __fmul2_rn(a, make_float2(W1, W1)); k1[e][1] = __fmul2_rn(b, make_float2(W1, W1));
+        k2[e][0] = __fmul2_rn(a, make_float2(W2, W2)); k2[e][1] = __fmul2_rn(b, make_float2(W2, W2));
     }
-    float v[32];
-    int at = 0;      // (compile-time: every loop below is unrolled)
+#pragma unroll 1
+    for (int j = s0 + 1; j < j_begin; ++j) {      // decays up to the first token of this warp's part
+        const float4 g1 = *reinterpret_cast<const float4*>(g + j * 512 + lane * 16), g2 = *reinterpret_cast<const float4*>(g + V_GBYTES / 2 + j * 512 + lane * 16);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = 0.f;
+        for (int e = 0; e < 4; ++e)
+            if (s0 + e < j) {
+                k1[e][0] = __fmul2_rn(k1[e][0], make_float2(g1.x, g1.y)); k1[e][1] = __fmul2_rn(k1[e][1], make_float2(g1.z, g1.w));
+                k2[e][0] = __fmul2_rn(k2[e][0], make_float2(g2.x, g2.y)); k2[e][1] = __fmul2_rn(k2[e][1], make_float2(g2.z, g2.w));
+            }
+    }
+#pragma unroll 1
+    for (int j0 = j_begin; j0 < j_end; j0 += 4) {
+        float v[16];
 #pragma unroll
-    for (int j = S0 + 1; j < VB; ++j) {
-        const uint2 x = *reinterpret_cast<const uint2*>(q + j * 256 + lane * 8);
-        const float4 gg = *reinterpret_cast<const float4*>(g + j * D + lane * 4);
-        const float2 q0 = unpack_bf16(x.x), q1 = unpack_bf16(x.y);
-        const float2 g0 = clamp0(make_float2(gg.x, gg.y)), g1 = clamp0(make_float2(gg.z, gg.w));
+        for (int r = 0; r < 4; ++r) {
+            const int j = j0 + r;
+            const uint2 x = *reinterpret_cast<const uint2*>(q + j * 256 + lane * 8);
+            const float4 g1 = *reinterpret_cast<const float4*>(g + j * 512 + lane * 16), g2 = *reinterpret_cast<const float4*>(g + V_GBYTES / 2 + j * 512 + lane * 16);
+            const float2 q0 = unpack_bf16(x.x), q1 = unpack_bf16(x.y);
 #pragma unroll
-        for (int s = S0; s < S1; ++s) {
-            if (s >= j) continue;
-            float2(&w)[2] = kd[s - S0];
-            w[0] = __fmul2_rn(w[0], g0);
-            w[1] = __fmul2_rn(w[1], g1);
-            const float2 y = __ffma2_rn(q1, w[1], __fmul2_rn(q0, w[0]));
-            v[at % 32] = y.x + y.y;
-            if (++at % 32 == 0) {
-                const float total = transpose_sum(v, lane);
-                out[pair[at - 32 + lane]] = total;
-#pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = 0.f;
+            for (int e = 0; e < 4; ++e) {
+                if (e < r || j0 > s0) {      // key s0 + e is earlier than token j
+                    k1[e][0] = __fmul2_rn(k1[e][0], make_float2(g1.x, g1.y)); k1[e][1] = __fmul2_rn(k1[e][1], make_float2(g1.z, g1.w));
+                    k2[e][0] = __fmul2_rn(k2[e][0], make_float2(g2.x, g2.y)); k2[e][1] = __fmul2_rn(k2[e][1], make_float2(g2.z, g2.w));
+                }
+                const float2 y = __ffma2_rn(q1, __fadd2_rn(k1[e][1], k2[e][1]), __fmul2_rn(q0, __fadd2_rn(k1[e][0], k2[e][0])));
+                v[4 * r + e] = y.x + y.y;
             }
         }
-    }
-    if (at % 32) {
-        const float total = transpose_sum(v, lane);
-        if (lane < at % 32) out[pair[at - at % 32 + lane]] = total;
+        const float total = transpose_sum<16>(v, lane);
+        if (lane < 16) out[(j0 + (lane >> 2)) * VC + s0 + (lane & 3)] = total;      // (above the diagonal: never read)
     }
 }
-constexpr int SPLIT_S = 5;      // keys 0..4 of a block: 65 pairs, keys 5..14: 55
 
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -171,71 +175,80 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint
 __device__ __forceinline__ uint32_t pair_at(int row, int hh, int lane, int half) {
     return (uint32_t)(hh * half + row * 128 + ((((lane >> 2) ^ (row & 7)) << 4) | ((lane & 3) << 2)));
 }
+__device__ __forceinline__ float2 gate_pair(const uint8_t* g, int t) { return *reinterpret_cast<const float2*>(g + t * 512); }
 
-// Q~ of one state: rows 16 b .. 16 b + 15, channels 64 hh ..; block 1 also leaves its copy scaled from the block's start.
-__device__ __forceinline__ void build_q(uint8_t* tiles, const uint8_t* qraw, const uint8_t* graw, int i, int hh, int b, int valid, float W, int lane) {
-    const uint8_t* q = qraw + hh * 128 + lane * 4;
-    const uint8_t* g = graw + hh * 256 + lane * 8;
-    uint8_t* qt = tiles + OFF_QT + 2 * i * V_TILE;
-    float2 first = make_float2(W, W);          // weight times the decay before this block
+// The four builders below take the raw rows and gates of one channel half (a channel pair per lane).
+// Q~ of one state, two terms: rows 16 b .. 16 b + 15 of Q scaled from the chunk's start.
+__device__ __forceinline__ void build_q(uint8_t* qt, const uint8_t* q, const uint8_t* g, int hh, int b, float W, int lane) {
+    float2 pr = make_float2(W, W);
     if (b == 1) {
-#pragma unroll 4
-        for (int t = 0; t < VB; ++t) first = __fmul2_rn(first, clamp0(*reinterpret_cast<const float2*>(g + t * 512)));      // (valid > 16, or the rows do not matter)
+#pragma unroll 8
+        for (int t = 0; t < VB; ++t) pr = __fmul2_rn(pr, gate_pair(g, t));
     }
-    float2 pr = make_float2(1.f, 1.f);
+    q += b * VB * 256; g += b * VB * 512; qt += b * VB * 128;
 #pragma unroll 4
-    for (int t = VB * b; t < VB * b + VB; ++t) {
-        const float2 gg = clamp0(*reinterpret_cast<const float2*>(g + t * 512));
-        if (t < valid) pr = __fmul2_rn(pr, gg);
-        float2 x = __fmul2_rn(unpack_bf16(*reinterpret_cast<const uint32_t*>(q + t * 256)), pr);
-        float2 y = __fmul2_rn(x, first);
+    for (int t = 0; t < VB; ++t) {
+        pr = __fmul2_rn(pr, gate_pair(g, t));
+        float2 y = __fmul2_rn(unpack_bf16(*reinterpret_cast<const uint32_t*>(q + t * 256)), pr);
         const uint32_t at = pair_at(t, hh, lane, V_HALF);
         *reinterpret_cast<uint32_t*>(qt + at) = take_term(y);
         *reinterpret_cast<uint32_t*>(qt + V_TILE + at) = pack_bf16(y.x, y.y);
-        if (b == 1) {
-            const uint32_t bt = pair_at(t - VB, hh, lane, V_BHALF);
-            *reinterpret_cast<uint32_t*>(tiles + OFF_QB + bt) = take_term(x);
-            *reinterpret_cast<uint32_t*>(tiles + OFF_QB + V_BTILE + bt) = pack_bf16(x.x, x.y);
-        }
     }
 }
-
-// K~ of one state in three terms (kt), rows 16 b .. 16 b + 15, weighted to the end of the chunk times `carry`; block 0 also leaves its
-// copy scaled to the block's end (kb, unless null).  Returns the product of the chunk's gates.
-__device__ __forceinline__ float2 build_k(uint8_t* kt, uint8_t* kb, const uint8_t* kraw, const uint8_t* graw, int hh, int b, int valid, float2 carry, int lane) {
-    const uint8_t* k = kraw + hh * 128 + lane * 4;
-    const uint8_t* g = graw + hh * 256 + lane * 8;
-    float2 other = make_float2(1.f, 1.f);      // product of the other block's gates
+// Rows 16..31 of Q scaled from their block's start, two terms.
+__device__ __forceinline__ void build_qb(uint8_t* qb, const uint8_t* q, const uint8_t* g, int hh, float W, int lane) {
+    float2 pr = make_float2(W, W);
+    q += VB * 256; g += VB * 512;
 #pragma unroll 4
-    for (int t = VB * (1 - b); t < VB * (1 - b) + VB; ++t) {
-        const float2 gg = clamp0(*reinterpret_cast<const float2*>(g + t * 512));
-        if (t < valid) other = __fmul2_rn(other, gg);
+    for (int t = 0; t < VB; ++t) {
+        pr = __fmul2_rn(pr, gate_pair(g, t));
+        float2 y = __fmul2_rn(unpack_bf16(*reinterpret_cast<const uint32_t*>(q + t * 256)), pr);
+        const uint32_t at = pair_at(t, hh, lane, V_BHALF);
+        *reinterpret_cast<uint32_t*>(qb + at) = take_term(y);
+        *reinterpret_cast<uint32_t*>(qb + V_BTILE + at) = pack_bf16(y.x, y.y);
     }
-    const float2 behind = b == 0 ? __fmul2_rn(other, carry) : carry;      // decay behind this block
+}
+// Rows 0..15 of K scaled to their block's end, two terms.
+__device__ __forceinline__ void build_kb(uint8_t* kb, const uint8_t* k, const uint8_t* g, int hh, int lane) {
     float2 sf = make_float2(1.f, 1.f);
 #pragma unroll 4
-    for (int t = VB * b + VB - 1; t >= VB * b; --t) {
-        const float2 kk = t < valid ? unpack_bf16(*reinterpret_cast<const uint32_t*>(k + t * 256)) : make_float2(0.f, 0.f);
-        float2 x = __fmul2_rn(kk, sf);
-        float2 y = __fmul2_rn(x, behind);
-        const uint32_t at = pair_at(t, hh, lane, V_HALF);
+    for (int t = VB - 1; t >= 0; --t) {
+        float2 y = __fmul2_rn(unpack_bf16(*reinterpret_cast<const uint32_t*>(k + t * 256)), sf);
+        const uint32_t at = pair_at(t, hh, lane, V_BHALF);
+        *reinterpret_cast<uint32_t*>(kb + at) = take_term(y);
+        *reinterpret_cast<uint32_t*>(kb + V_BTILE + at) = pack_bf16(y.x, y.y);
+        sf = __fmul2_rn(sf, gate_pair(g, t));
+    }
+}
+// K~ of one state, three terms: rows t_begin .. t_begin + ROWS - 1 of K scaled to the chunk's end times `carry`.  Returns the
+// product of the gates from row t_begin on, times carry.
+template <int ROWS, bool CLAMP>
+__device__ __forceinline__ float2 build_k(uint8_t* kt, const uint8_t* k, const uint8_t* g, int hh, int t_begin, float2 carry, int lane) {
+    auto gate = [&](int t) {
+        const float2 x = gate_pair(g, t);
+        return CLAMP ? make_float2(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f)) : x;
+    };
+    float2 sf = carry;
+#pragma unroll 8
+    for (int t = VC - 1; t >= t_begin + ROWS; --t) sf = __fmul2_rn(sf, gate(t));
+    k += t_begin * 256; g += t_begin * 512; kt += t_begin * 128;
+#pragma unroll 4
+    for (int t = ROWS - 1; t >= 0; --t) {
+        float2 y = __fmul2_rn(unpack_bf16(*reinterpret_cast<const uint32_t*>(k + t * 256)), sf);
+        const uint32_t at = pair_at(t, hh, lane, V_HALF);      // (t_begin is a multiple of 8)
         *reinterpret_cast<uint32_t*>(kt + at) = take_term(y);
         *reinterpret_cast<uint32_t*>(kt + V_TILE + at) = take_term(y);
         *reinterpret_cast<uint32_t*>(kt + 2 * V_TILE + at) = pack_bf16(y.x, y.y);
-        if (b == 0 && kb) {
-            const uint32_t bt = pair_at(t, hh, lane, V_BHALF);
-            *reinterpret_cast<uint32_t*>(kb + bt) = take_term(x);
-            *reinterpret_cast<uint32_t*>(kb + V_BTILE + bt) = pack_bf16(x.x, x.y);
-        }
-        const float2 gg = clamp0(*reinterpret_cast<const float2*>(g + t * 512));
-        if (t < valid) sf = __fmul2_rn(sf, gg);
+        sf = __fmul2_rn(sf, gate(t));
     }
-    return __fmul2_rn(sf, other);
+    return sf;
 }
 
 // Scores between the blocks, rows 16..31 x columns 8 nt .. 8 nt + 7: two-term operands, the product of the two low terms left out.
-__device__ __forceinline__ void cross_scores(const uint8_t* tiles, int nt, int lane, float* out) {
+__device__ __forceinline__ void cross_scores(const uint8_t* tiles, int nt, int lane, bool add, float* out) {
+    float* o = out + (VB + (lane >> 2)) * VC + 8 * nt + 2 * (lane & 3);
     float c[4] = {0.f, 0.f, 0.f, 0.f};
+    if (add) { c[0] = o[0]; c[1] = o[1]; c[2] = o[8 * VC]; c[3] = o[8 * VC + 1]; }
     const uint32_t qb = smem_u32(tiles + OFF_QB), kb = smem_u32(tiles + OFF_KB);
     const int arow = lane & 15, brow = 8 * nt + (lane & 7);
 #pragma unroll 2
@@ -258,60 +271,46 @@ __device__ __forceinline__ void cross_scores(const uint8_t* tiles, int nt, int l
             mma16816(c, a[0], b[0][2 * s], b[0][2 * s + 1]);
         }
     }
-    float* o = out + (VB + (lane >> 2)) * VC + 8 * nt + 2 * (lane & 3);
     *reinterpret_cast<float2*>(o) = make_float2(c[0], c[1]);
     *reinterpret_cast<float2*>(o + 8 * VC) = make_float2(c[2], c[3]);
 }
 
-// Everything state i needs of a chunk from its raw Q, K and gates.
-__device__ __forceinline__ void build_operands(uint8_t* tiles, const VecShared& sh, int i, int buf, int valid, float W, int warp, int lane) {
+// The operands of state i of a chunk, and half of its scores: block i of 16 tokens and this state's share between the blocks.
+__device__ __forceinline__ void build_operands(uint8_t* tiles, int i, int buf, float W1, float W2, int warp, int lane) {
     const uint8_t* qraw = tiles + OFF_RAW + buf * V_TILE;
     const uint8_t* kraw = tiles + OFF_RAWK + buf * V_TILE;
-    const uint8_t* graw = tiles + OFF_G + i * VC * D * 4;
-    float* sc = reinterpret_cast<float*>(tiles + OFF_SC) + i * VC * VC;
+    const uint8_t* graw = tiles + OFF_G + buf * V_GBYTES;
+    float* sc = reinterpret_cast<float*>(tiles + OFF_SC) + buf * VC * VC;
+    const int hh = warp & 1;
+    const float W = i == 0 ? W1 : W2;
+    const uint8_t *qh = qraw + hh * 128 + lane * 4, *kh = kraw + hh * 128 + lane * 4, *gh = graw + i * (V_GBYTES / 2) + hh * 256 + lane * 8;
     if (warp < 4) {
-        build_q(tiles, qraw, graw, i, warp & 1, warp >> 1, valid, W, lane);
-        if (warp >= 2) asm volatile("bar.arrive 1, 192;" ::: "memory");
+        build_q(tiles + OFF_QT + 2 * i * V_TILE, qh, gh, hh, warp >> 1, W, lane);
     } else if (warp < 8) {
-        const int hh = warp & 1, b = (warp - 4) >> 1;
-        const float2 a = build_k(tiles + OFF_KT + 3 * i * V_TILE, tiles + OFF_KB, kraw, graw, hh, b, valid, make_float2(1.f, 1.f), lane);
-        if (b == 0) {
-            asm volatile("bar.arrive 1, 192;" ::: "memory");
-            reinterpret_cast<float2*>(tiles + OFF_A)[i * (D / 2) + 32 * hh + lane] = a;
-        }
+        const int b = (warp - 4) >> 1;
+        const float2 a = build_k<VB, false>(tiles + OFF_KT + 3 * i * V_TILE, kh, gh, hh, b * VB, make_float2(1.f, 1.f), lane);
+        if (b == 0) reinterpret_cast<float2*>(tiles + OFF_A)[i * (D / 2) + 32 * hh + lane] = a;
     } else if (warp < 12) {
-        const int b = (warp - 8) >> 1;
-        const uint8_t *q = qraw + b * VB * 256, *k = kraw + b * VB * 256;
-        const float* g = reinterpret_cast<const float*>(graw) + b * VB * D;
-        float* out = sc + b * (VB * VC + VB);
-        if (warp & 1) block_scores<SPLIT_S, VB - 1>(q, k, g, valid - b * VB, lane, sh.pair[1], out);
-        else block_scores<0, SPLIT_S>(q, k, g, valid - b * VB, lane, sh.pair[0], out);
-    } else if (warp < 14) {
-        asm volatile("bar.sync 1, 192;" ::: "memory");
-        cross_scores(tiles, warp - 12, lane, sc);
-    } else if (warp == 14 && i == 0) {
-        // the current token is undecayed: its score is the same for both states
-        float v[32];
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            const uint2 x = *reinterpret_cast<const uint2*>(qraw + t * 256 + lane * 8), y = *reinterpret_cast<const uint2*>(kraw + t * 256 + lane * 8);
-            const float2 z = __ffma2_rn(unpack_bf16(x.y), unpack_bf16(y.y), __fmul2_rn(unpack_bf16(x.x), unpack_bf16(y.x)));
-            v[t] = t < valid ? z.x + z.y : 0.f;
+        // ten rounds of 4 x 4 tokens and keys: 2 + 1, 3, 2 and 2 (behind eight tokens' decays)
+        const uint8_t *q = qraw + i * VB * 256, *k = kraw + i * VB * 256, *g = graw + i * VB * 512;
+#pragma unroll 1
+        for (int part = 0; part < (warp == 8 ? 2 : 1); ++part) {
+            const int s0 = warp == 8 ? 12 * part : warp == 11 ? 0 : 4 * (warp - 8);
+            block_scores(q, k, g, s0, warp == 11 ? 8 : s0, warp == 8 && part == 0 ? 8 : VB, W1, W2, lane, sc + i * (VB * VC + VB));
         }
-        const float total = transpose_sum(v, lane);
-        sc[lane * (VC + 1)] = total;
-        sc[VC * VC + lane * (VC + 1)] = total;
-    } else if (warp == 15 && i == 0) {
-        // V rows past the end belong to the next sequence: they meet only zero weights, but 0 * inf is not 0
-        for (int t = VC - 1; t >= valid; --t)
-            if (lane < 16) *reinterpret_cast<uint4*>(tiles + OFF_V + buf * V_TILE + (lane >> 3) * V_HALF + t * 128 + (lane & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+    } else if (warp < 14) {
+        build_qb(tiles + OFF_QB, qh, gh, hh, W, lane);
+        asm volatile("bar.arrive 1, 128;" ::: "memory");
+    } else {
+        build_kb(tiles + OFF_KB, kh, gh, hh, lane);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        cross_scores(tiles, hh, lane, i == 1, sc);
     }
 }
 
 __device__ __forceinline__ void vec_setup(VecShared& sh, int tid, int warp, int mma_warp) {
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) { mbar_init(&sh.raw_full[i], 1); mbar_init(&sh.done[i], 1); }
-        mbar_init(&sh.g2_full, 1);
         sh.abort_flag = 0;
         fence_barrier_init();
     }
@@ -321,7 +320,8 @@ __device__ __forceinline__ void vec_setup(VecShared& sh, int tid, int warp, int 
 // ============================================================================================
 // Main kernel
 // ============================================================================================
-__global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid_constant__ CUtensorMap map_v, const VecParams vp) {
+__global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                                                                   const __grid_constant__ CUtensorMap map_g1, const __grid_constant__ CUtensorMap map_g2, const VecParams vp) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ VecShared sh;
     const PrefillParams& p = vp.p;
@@ -340,16 +340,6 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
     const int nc = u.c_end - u.c_begin, tok0 = u.c_begin * VC, t0 = u.t_begin + tok0;
     const bool last = u.c_end == u.nchunks;
     vec_setup(sh, tid, warp, 0);
-    if (tid >= 64 && tid < 96) {      // (row, column) of every score pair, in the order block_scores produces them; a row per lane
-        const int j = lane + 1;
-        for (int part = 0; part < 2; ++part) {
-            const int s0 = part ? SPLIT_S : 0, s1 = part ? VB - 1 : SPLIT_S;
-            int at = 0;
-            for (int r = s0 + 1; r < j; ++r) at += min(r, s1) - s0;
-            if (j < VB)
-                for (int s = s0; s < min(j, s1); ++s, ++at) sh.pair[part][at] = (short)(j * VC + s);
-        }
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -358,29 +348,37 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
     const uint32_t lane_addr = (uint32_t)(32 * q) << 16;      // (all of TMEM is allocated: column 0 is its base)
     const int v = 32 * q + lane;
     const float W1 = p.gamma[u.h] * p.scale, W2 = (1.f - p.gamma[u.h]) * p.scale;
-    const __nv_bfloat16* qg = reinterpret_cast<const __nv_bfloat16*>(p.q);
-    const __nv_bfloat16* kg = reinterpret_cast<const __nv_bfloat16*>(p.k);
     __nv_bfloat16* og = reinterpret_cast<__nv_bfloat16*>(p.o);
 #define WAIT(bar, ph) mbar_wait(bar, (uint32_t)(ph), abortp, p.status)
 
-    // one warp, a row per lane
-    auto load_raw = [&](int c) {
-        const int valid = min(VC, u.len - tok0 - c * VC), b = c & 1;
-        if (lane == 0) mbar_arrive_expect_tx(&sh.raw_full[b], (uint32_t)(valid * (256 + 256 + 512) + V_TILE));
-        __syncwarp();
-        if (lane < valid) {
-            const size_t off = ((size_t)(t0 + c * VC + lane) * p.H + u.h) * D;
-            bulk_load(tiles + OFF_RAW + b * V_TILE + lane * 256, qg + off, 256, &sh.raw_full[b]);
-            bulk_load(tiles + OFF_RAWK + b * V_TILE + lane * 256, kg + off, 256, &sh.raw_full[b]);
-            bulk_load(tiles + OFF_G + lane * 512, p.g_hist + off, 512, &sh.raw_full[b]);
-        }
-        if (lane == 0) tma_load_4d(tiles + OFF_V + b * V_TILE, &map_v, &sh.raw_full[b], 0, t0 + c * VC, 0, u.h);
+    auto load_raw = [&](int c) {      // by one thread
+        const int b = c & 1, t = t0 + c * VC;
+        mbar_arrive_expect_tx(&sh.raw_full[b], 3 * V_TILE + V_GBYTES);
+        tma_load_3d(tiles + OFF_G + b * V_GBYTES, &map_g1, &sh.raw_full[b], 0, u.h, t);
+        tma_load_3d(tiles + OFF_G + b * V_GBYTES + V_GBYTES / 2, &map_g2, &sh.raw_full[b], 0, u.h, t);
+        tma_load_3d(tiles + OFF_RAW + b * V_TILE, &map_q, &sh.raw_full[b], 0, u.h, t);
+        tma_load_3d(tiles + OFF_RAWK + b * V_TILE, &map_k, &sh.raw_full[b], 0, u.h, t);
+        tma_load_4d(tiles + OFF_V + b * V_TILE, &map_v, &sh.raw_full[b], 0, t, 0, u.h);
     };
-    auto load_g2 = [&](int c) {
-        const int valid = min(VC, u.len - tok0 - c * VC);
-        if (lane == 0) mbar_arrive_expect_tx(&sh.g2_full, (uint32_t)(valid * 512));
-        __syncwarp();
-        if (lane < valid) bulk_load(tiles + OFF_G + VC * D * 4 + lane * 512, p.g_rec + ((size_t)(t0 + c * VC + lane) * p.H + u.h) * D, 512, &sh.g2_full);
+    // Gates below 0 count as 0; past the end of the sequence gates are 1 and the other rows 0 (what landed there belongs to the next
+    // sequence: it would meet only zero weights, but 0 * inf is not 0).
+    auto clean = [&](int c) {
+        const int b = c & 1, valid = u.len - tok0 - c * VC;
+        float4* g = reinterpret_cast<float4*>(tiles + OFF_G + b * V_GBYTES);
+#pragma unroll
+        for (int m = 0; m < V_GBYTES / 16 / V_NTHREADS; ++m) {
+            const int idx = tid + m * V_NTHREADS;
+            const float4 x = g[idx];
+            g[idx] = ((idx >> 5) & (VC - 1)) < valid ? make_float4(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f), fmaxf(x.z, 0.f), fmaxf(x.w, 0.f)) : make_float4(1.f, 1.f, 1.f, 1.f);
+        }
+        if (valid < VC) {
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            if ((tid >> 4) >= valid) {
+                reinterpret_cast<uint4*>(tiles + OFF_RAW + b * V_TILE)[tid] = zero;
+                reinterpret_cast<uint4*>(tiles + OFF_RAWK + b * V_TILE)[tid] = zero;
+            }
+            if (((tid >> 3) & (VC - 1)) >= valid) reinterpret_cast<uint4*>(tiles + OFF_V + b * V_TILE)[tid] = zero;
+        }
     };
     // S_i -> two bf16 terms for the readout, then S_i diag(A_i); 32 columns (key channels) of one lane quadrant per warp
     auto pass = [&](int i) {
@@ -432,72 +430,88 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
         tc_commit(&sh.done[i]);
     };
 
-    if (warp == 15) { load_raw(0); load_g2(0); }
-    {   // initial states: the slot, what the summaries were folded into, or zero
+    if (warp == 15 && lane == 0) load_raw(0);
+    // Initial states: the slot (or zero) pushed through the summaries of the earlier segments, S <- diag(A_j) S + U_j.  The summary
+    // of the first one holds the slot's share already, and the entry of the last segment, which has no summary, a copy of the
+    // slot for the first (the CTA of the last segment overwrites the slot itself).
+    if (vp.ws) asm volatile("griddepcontrol.wait;" ::: "memory");
+    {
         const int i = warp >> 3, half = (warp >> 2) & 1;
+        const float* unit = vp.ws ? vp.ws + (size_t)(u.n * p.H + u.h) * vp.nseg * (VEC_STRIDE / 4) : nullptr;
+        const float* first = (u.g == 0 && last) ? slot1 + (size_t)i * state_stride : u.g == 0 ? unit + (size_t)(vp.nseg - 1) * (VEC_STRIDE / 4) + (size_t)i * D * D : unit + (size_t)i * D * D;
         const bool load = u.g > 0 || p.use_initial_state;
-        const float* base = vp.ws ? vp.ws + ((size_t)(u.n * p.H + u.h) * vp.nseg + u.g) * (VEC_STRIDE / 4) + (size_t)i * D * D : slot1 + (size_t)i * state_stride;
 #pragma unroll 1
         for (int bt = 2 * half; bt < 2 * half + 2; ++bt) {
+            float acc[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) acc[k] = load ? first[(size_t)(32 * bt + k) * D + v] : 0.f;
+#pragma unroll 1
+            for (int jg = 1; jg < u.g; ++jg) {
+                const float* U = unit + (size_t)jg * (VEC_STRIDE / 4);
+                const float4* A = reinterpret_cast<const float4*>(U + 2 * D * D + i * D + 32 * bt);
+                float x[32];
+#pragma unroll
+                for (int k = 0; k < 32; ++k) x[k] = U[(size_t)i * D * D + (size_t)(32 * bt + k) * D + v];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float4 a = A[k];
+                    acc[4 * k] = fmaf(a.x, acc[4 * k], x[4 * k]); acc[4 * k + 1] = fmaf(a.y, acc[4 * k + 1], x[4 * k + 1]);
+                    acc[4 * k + 2] = fmaf(a.z, acc[4 * k + 2], x[4 * k + 2]); acc[4 * k + 3] = fmaf(a.w, acc[4 * k + 3], x[4 * k + 3]);
+                }
+            }
             uint32_t r[32];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) r[k] = load ? __float_as_uint(base[(size_t)(32 * bt + k) * D + v]) : 0u;
+            for (int k = 0; k < 32; ++k) r[k] = __float_as_uint(acc[k]);
             tmem_st32(lane_addr + VCOL_S + 128 * i + 32 * bt, r);
         }
         tc_wait_st();
         tc_fence_before();
     }
     WAIT(&sh.raw_full[0], 0);
-    build_operands(tiles, sh, 0, 0, min(VC, u.len - tok0), W1, warp, lane);
-    fence_proxy_async_smem();
+    clean(0);
+    tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // Step hs = 2 c + i: pass over state i, its MMAs for chunk c, the operands of the other state.  One body for both phases (and for the
+    // first operands, hs = -1): the code has to stay in the instruction cache.
 #pragma unroll 1
-    for (int c = 0; c < nc; ++c) {
-        const int b = c & 1, valid = min(VC, u.len - tok0 - c * VC);
-        // ---- phase A
-        if (c > 0) {
-            WAIT(&sh.done[1], (c - 1) & 1);
-            tc_fence_after();
+    for (int hs = -1; hs < 2 * nc; ++hs) {
+        const int i = hs & 1, c = hs >> 1, b = c & 1;
+        if (hs >= 0) {
+            if (hs > 0) {
+                WAIT(&sh.done[i ^ 1], ((hs - 1) >> 1) & 1);
+                tc_fence_after();
+            }
+            if (i == 0) {
+                if (warp == 15 && lane == 0 && c + 1 < nc) load_raw(c + 1);
+                __syncwarp();
+                if (c > 0) outputs(c - 1);
+            } else {      // P~: two columns of one row per thread
+                const int j = tid >> 4, s = (tid & 15) * 2;
+                const float2 x = *reinterpret_cast<const float2*>(tiles + OFF_SC + (b * VC * VC + j * VC + s) * 4);
+                float2 z = make_float2(s <= j ? x.x : 0.f, s + 1 <= j ? x.y : 0.f);
+                uint8_t* at = tiles + OFF_PT + j * 128 + (((s >> 3) ^ (j & 7)) << 4) + (s & 7) * 2;
+                *reinterpret_cast<uint32_t*>(at) = take_term(z);
+                *reinterpret_cast<uint32_t*>(at + VC * 128) = pack_bf16(z.x, z.y);
+                fence_proxy_async_smem();
+            }
+            pass(i);
+            tc_fence_before();
+            if (warp == 1) {      // only the issuing warp waits for the others
+                asm volatile("bar.sync 2, 512;" ::: "memory");
+                if (elect_one()) {
+                    tc_fence_after();
+                    issue(i, b);
+                }
+                __syncwarp();
+            } else {
+                asm volatile("bar.arrive 2, 512;" ::: "memory");
+            }
         }
-        if (warp == 15 && c + 1 < nc) load_raw(c + 1);
-        if (c > 0) outputs(c - 1);
-        pass(0);
-        tc_fence_before();
-        __syncthreads();
-        if (warp == 0 && elect_one()) {
-            tc_fence_after();
-            issue(0, b);
-        }
-        __syncwarp();
-        WAIT(&sh.g2_full, c & 1);
-        build_operands(tiles, sh, 1, b, valid, W2, warp, lane);
-        fence_proxy_async_smem();
-        __syncthreads();
-        // ---- phase B
-        if (warp == 15 && c + 1 < nc) load_g2(c + 1);
-        WAIT(&sh.done[0], c & 1);
-        tc_fence_after();
-        pass(1);
-        {   // P~: two columns of one row per thread
-            const int j = tid >> 4, s = (tid & 15) * 2;
-            const float2 x = *reinterpret_cast<const float2*>(tiles + OFF_SC + (j * VC + s) * 4), y = *reinterpret_cast<const float2*>(tiles + OFF_SC + (VC * VC + j * VC + s) * 4);
-            float2 z = make_float2(s <= j ? fmaf(W2, y.x, W1 * x.x) : 0.f, s + 1 <= j ? fmaf(W2, y.y, W1 * x.y) : 0.f);
-            uint8_t* at = tiles + OFF_PT + j * 128 + (((s >> 3) ^ (j & 7)) << 4) + (s & 7) * 2;
-            *reinterpret_cast<uint32_t*>(at) = take_term(z);
-            *reinterpret_cast<uint32_t*>(at + VC * 128) = pack_bf16(z.x, z.y);
-        }
-        tc_fence_before();
-        fence_proxy_async_smem();
-        __syncthreads();
-        if (warp == 0 && elect_one()) {
-            tc_fence_after();
-            issue(1, b);
-        }
-        __syncwarp();
-        if (c + 1 < nc) {
+        if (hs + 1 < 2 * nc) build_operands(tiles, i ^ 1, i == 0 ? b : b ^ 1, W1, W2, warp, lane);
+        if (i == 0 && c + 1 < nc) {
             WAIT(&sh.raw_full[b ^ 1], ((c + 1) >> 1) & 1);
-            build_operands(tiles, sh, 0, b ^ 1, min(VC, u.len - tok0 - (c + 1) * VC), W1, warp, lane);
+            clean(c + 1);
         }
         fence_proxy_async_smem();
         __syncthreads();
@@ -512,65 +526,69 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
 }
 
 // ============================================================================================
-// Segments: summaries and initial states
+// Segment summaries
 // ============================================================================================
-// U_g (both states, accumulated from zero) and A_g (products of the segment's gates) of a segment that has a successor.  Warps 0..7
-// build K~ (state, channel half, block), warp 8 loads and issues.
-constexpr int VS_NTHREADS = 288;
-__global__ void __launch_bounds__(VS_NTHREADS, 1) prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_v, const VecParams vp) {
+// U_g (both states, accumulated from zero) and A_g (products of the segment's gates) of a segment that has a successor.  Warps 0..15
+// build K~ (state, channel half, eight rows each), warp 16 loads and issues.  The first segment of a sequence that continues
+// from its slot also pushes that through its summary, and leaves a copy of it in the entry of the last segment.
+constexpr int VS_NTHREADS = 17 * 32;
+__global__ void __launch_bounds__(VS_NTHREADS, 1)
+prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g1,
+                           const __grid_constant__ CUtensorMap map_g2, const VecParams vp) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ VecShared sh;
+    __shared__ float2 carries[2][2][D / 2];      // [parity][state]: product of the gates of all later chunks
     const PrefillParams& p = vp.p;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const VecUnit u = vec_unit(vp, blockIdx.x, vp.nseg - 1);
     if (u.slot < 0 || u.slot >= p.num_slots || u.len <= 0 || u.c_end >= u.nchunks) return;      // (c_end < nchunks: whole chunks only)
     const int nc = u.c_end - u.c_begin, t0 = u.t_begin + u.c_begin * VC;
-    float* out = vp.ws + ((size_t)(u.n * p.H + u.h) * vp.nseg + u.g) * (VEC_STRIDE / 4);
-    vec_setup(sh, tid, warp, 8);
+    float* unit = vp.ws + (size_t)(u.n * p.H + u.h) * vp.nseg * (VEC_STRIDE / 4);
+    float* out = unit + (size_t)u.g * (VEC_STRIDE / 4);
+    vec_setup(sh, tid, warp, 16);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     volatile int* abortp = &sh.abort_flag;
-    const __nv_bfloat16* kg = reinterpret_cast<const __nv_bfloat16*>(p.k);
     const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int i = warp >> 2, hh = warp & 1, b = (warp >> 1) & 1;
-    float2 carry = make_float2(1.f, 1.f);
+    const int i = warp >> 3, hh = warp & 1, rows = 8 * ((warp >> 1) & 3);
+    float2 after = make_float2(1.f, 1.f);
     // step it = chunk nc - 1 - it; buffers by the parity of it
-    auto load = [&](int it) {
+    auto load = [&](int it) {      // by one thread
         const int par = it & 1, t = t0 + (nc - 1 - it) * VC;
-        const size_t off = ((size_t)(t + lane) * p.H + u.h) * D;
-        if (lane == 0) mbar_arrive_expect_tx(&sh.raw_full[par], VC * (256 + 1024) + V_TILE);
-        __syncwarp();
-        bulk_load(tiles + OFF_SK + par * V_TILE + lane * 256, kg + off, 256, &sh.raw_full[par]);
-        bulk_load(tiles + OFF_SG + par * 2 * VC * D * 4 + lane * 512, p.g_hist + off, 512, &sh.raw_full[par]);
-        bulk_load(tiles + OFF_SG + (par * 2 + 1) * VC * D * 4 + lane * 512, p.g_rec + off, 512, &sh.raw_full[par]);
-        if (lane == 0) tma_load_4d(tiles + OFF_V + par * V_TILE, &map_v, &sh.raw_full[par], 0, t, 0, u.h);
+        mbar_arrive_expect_tx(&sh.raw_full[par], 2 * V_TILE + V_GBYTES);
+        tma_load_3d(tiles + OFF_SG + par * V_GBYTES, &map_g1, &sh.raw_full[par], 0, u.h, t);
+        tma_load_3d(tiles + OFF_SG + par * V_GBYTES + V_GBYTES / 2, &map_g2, &sh.raw_full[par], 0, u.h, t);
+        tma_load_3d(tiles + OFF_SK + par * V_TILE, &map_k, &sh.raw_full[par], 0, u.h, t);
+        tma_load_4d(tiles + OFF_V + par * V_TILE, &map_v, &sh.raw_full[par], 0, t, 0, u.h);
     };
-    if (warp == 8) load(0);
+    if (warp == 16 && lane == 0) load(0);
 #pragma unroll 1
     for (int it = 0; it < nc; ++it) {
         const int par = it & 1;
-        if (warp == 8) {
+        if (warp == 16) {
             if (it + 1 < nc) {
                 if (it >= 1) WAIT(&sh.done[par ^ 1], ((it - 1) >> 1) & 1);      // the MMAs of step it - 1 have read V
-                load(it + 1);
+                if (lane == 0) load(it + 1);
             }
         } else {
+            if (it > 0) after = carries[par][i][32 * hh + lane];
             WAIT(&sh.raw_full[par], (it >> 1) & 1);
             if (it >= 2) WAIT(&sh.done[par], ((it >> 1) - 1) & 1);              // ... and those of step it - 2 this K~
-            const float2 a = build_k(tiles + OFF_SKT + (par * 6 + 3 * i) * V_TILE, nullptr, tiles + OFF_SK + par * V_TILE,
-                                     tiles + OFF_SG + (par * 2 + i) * VC * D * 4, hh, b, VC, carry, lane);
-            carry = __fmul2_rn(carry, a);
+            const float2 a = build_k<8, true>(tiles + OFF_SKT + (par * 6 + 3 * i) * V_TILE, tiles + OFF_SK + par * V_TILE + hh * 128 + lane * 4,
+                                              tiles + OFF_SG + par * V_GBYTES + i * (V_GBYTES / 2) + hh * 256 + lane * 8, hh, rows, after, lane);
+            if (rows == 0) carries[par ^ 1][i][32 * hh + lane] = a;
             fence_proxy_async_smem();
         }
         __syncthreads();
-        if (warp == 8 && elect_one()) {
+        if (warp == 16 && elect_one()) {
             constexpr uint32_t ID_U = idesc_bf16(128, 128, 1, 1);
-            WAIT(&sh.raw_full[par], (it >> 1) & 1);
             tc_fence_after();
             const uint32_t vd = smem_desc_lo(sa + OFF_V + par * V_TILE, V_HALF), kd = smem_desc_lo(sa + OFF_SKT + par * 6 * V_TILE, V_HALF);
-#pragma unroll 1
+            WAIT(&sh.raw_full[par], (it >> 1) & 1);
+#pragma unroll
             for (int m = 0; m < 6; ++m) {       // (state, term)
                 const uint32_t d = VCOL_S + (m >= 3 ? 128 : 0), k = kd + (uint32_t)(m * (V_TILE >> 4)), fresh = (it == 0 && (m == 0 || m == 3)) ? 0u : 1u;
                 mma_ss_lo(d, vd, k, ID_U, fresh);
@@ -582,40 +600,42 @@ __global__ void __launch_bounds__(VS_NTHREADS, 1) prefill_vec_summary_kernel(con
     }
     WAIT(&sh.done[(nc - 1) & 1], ((nc - 1) >> 1) & 1);
     tc_fence_after();
-    if (warp < 8) {
-        store_state(out + (size_t)i * D * D, 32 * (warp & 3) + lane, ((uint32_t)(32 * (warp & 3)) << 16) + VCOL_S + 128 * i, 0, 4);
-        if (b == 0) reinterpret_cast<float2*>(out + 2 * D * D)[i * (D / 2) + 32 * hh + lane] = carry;
+    if (warp < 16) {
+        const float* A = reinterpret_cast<const float*>(carries[nc & 1][i]);
+        const int q = warp & 3, v = 32 * q + lane;
+        const bool from_slot = u.g == 0 && p.use_initial_state;
+        const float* slot = p.state + (((size_t)u.slot * 2 + i) * p.H + u.h) * (size_t)(D * D) + v;
+        float* copy = unit + (size_t)(vp.nseg - 1) * (VEC_STRIDE / 4) + (size_t)i * D * D + v;
+        float* dst = out + (size_t)i * D * D + v;
+#pragma unroll 1
+        for (int k0 = 64 * ((warp >> 2) & 1), end = k0 + 64; k0 < end; k0 += 32) {
+            uint32_t r[32];
+            float x[32];
+            tmem_ld32(((uint32_t)(32 * q) << 16) + VCOL_S + 128 * i + k0, r);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) x[k] = from_slot ? slot[(size_t)(k0 + k) * D] : 0.f;
+            tc_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                if (from_slot) copy[(size_t)(k0 + k) * D] = x[k];
+                dst[(size_t)(k0 + k) * D] = fmaf(A[k0 + k], x[k], __uint_as_float(r[k]));
+            }
+        }
+        if (tid < 64) reinterpret_cast<float4*>(out + 2 * D * D)[tid] = reinterpret_cast<const float4*>(&carries[nc & 1][0][0])[tid];
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 8) tmem_dealloc(0, 512);
+    if (warp == 16) tmem_dealloc(0, 512);
 }
 #undef WAIT
 
-// Summaries -> initial states, in place: S_g = fold over earlier segments of (S <- diag(A_j) S + U_j), from the slot or zero.  Four
-// elements of one state row per thread.
-__global__ void __launch_bounds__(256) prefill_vec_fold_kernel(const VecParams vp) {
-    const PrefillParams& p = vp.p;
-    const int part = blockIdx.x % (2 * 16), unit = blockIdx.x / (2 * 16), i = part >> 4;
-    const int e = ((part & 15) * 256 + threadIdx.x) * 4, row = e / D;
-    const int n = unit / p.H, h = unit % p.H;
-    const int slot = p.slots ? p.slots[n] : n;
-    if (slot < 0 || slot >= p.num_slots) return;
-    const int len = p.cu_seqlens ? p.cu_seqlens[n + 1] - p.cu_seqlens[n] : p.T;
-    if (len <= 0) return;
-    const int last = min(vp.nseg - 1, ((len + VC - 1) / VC - 1) / vp.cps);
-    float* at = vp.ws + (size_t)unit * vp.nseg * (VEC_STRIDE / 4) + (size_t)i * D * D + e;
-    const float* A = vp.ws + (size_t)unit * vp.nseg * (VEC_STRIDE / 4) + 2 * D * D + i * D + row;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (p.use_initial_state) s = *reinterpret_cast<const float4*>(p.state + (((size_t)slot * 2 + i) * p.H + h) * (size_t)(D * D) + e);
-#pragma unroll 4
-    for (int g = 0; g <= last; ++g, at += VEC_STRIDE / 4, A += VEC_STRIDE / 4) {
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        float a = 0.f;
-        if (g < last) { x = *reinterpret_cast<const float4*>(at); a = *A; }
-        *reinterpret_cast<float4*>(at) = s;
-        s.x = fmaf(a, s.x, x.x); s.y = fmaf(a, s.y, x.y); s.z = fmaf(a, s.z, x.z); s.w = fmaf(a, s.w, x.w);
-    }
+// [T_total, H, 128] of 2- or 4-byte elements, a chunk of one head per copy, rows as they are
+bool make_row_map(CUtensorMap* m, const void* base, bool f32, int T_total, int H) {
+    const cuuint64_t es = f32 ? 4 : 2;
+    cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T_total};
+    cuuint64_t strides[2] = {D * es, (cuuint64_t)H * D * es};
+    cuuint32_t box[3] = {D, 1, VC};
+    return encode_tile_map(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 }  // namespace
@@ -631,7 +651,7 @@ dsla_status launch_prefill_vec(const PrefillParams& p, const dsla_prefill_args* 
     vp.p = p;
     const long long units = (long long)p.N * p.H;
     const int max_chunks = (a->max_seqlen + VC - 1) / VC;
-    // Segments: as many as keep every SM at one CTA, at least eight chunks each (below that the two extra launches cost more than the
+    // Segments: as many as keep every SM at one CTA, at least eight chunks each (below that the extra launch costs more than the
     // shorter chains save), and no more than the workspace holds (these calls need none: without one a sequence is one segment).
     int ns = (int)(148 / units);
     if (ns > 16) ns = 16;
@@ -641,16 +661,27 @@ dsla_status launch_prefill_vec(const PrefillParams& p, const dsla_prefill_args* 
     vp.cps = ns > 1 ? (max_chunks + ns - 1) / ns : max_chunks;
     vp.ws = ns > 1 ? static_cast<float*>(a->workspace) : nullptr;
     if (units * ns > 0x7fffffffLL / 32) return DSLA_ERR_UNSUPPORTED;
-    CUtensorMap mv;
-    if (!make_tile_map(&mv, p.v, a->T_total, p.H, VC)) return DSLA_ERR_CUDA;
+    CUtensorMap mq, mk, mv, m1, m2;
+    if (!make_row_map(&mq, p.q, false, a->T_total, p.H) || !make_row_map(&mk, p.k, false, a->T_total, p.H) || !make_tile_map(&mv, p.v, a->T_total, p.H, VC) ||
+        !make_row_map(&m1, p.g_hist, true, a->T_total, p.H) || !make_row_map(&m2, p.g_rec, true, a->T_total, p.H))
+        return DSLA_ERR_CUDA;
     if (ns > 1) {
         if (cudaFuncSetAttribute(prefill_vec_summary_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, V_SMEM_SUM) != cudaSuccess) return DSLA_ERR_CUDA;
-        prefill_vec_summary_kernel<<<dim3((unsigned)(units * (ns - 1))), dim3(VS_NTHREADS), V_SMEM_SUM, s>>>(mv, vp);
-        prefill_vec_fold_kernel<<<dim3((unsigned)(units * 2 * 16)), dim3(256), 0, s>>>(vp);
-        count_launch(2);
+        prefill_vec_summary_kernel<<<dim3((unsigned)(units * (ns - 1))), dim3(VS_NTHREADS), V_SMEM_SUM, s>>>(mk, mv, m1, m2, vp);
+        count_launch();
     }
     if (cudaFuncSetAttribute(prefill_vec_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, V_SMEM) != cudaSuccess) return DSLA_ERR_CUDA;
-    prefill_vec_kernel<<<dim3((unsigned)(units * ns)), dim3(V_NTHREADS), V_SMEM, s>>>(mv, vp);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(units * ns));
+    cfg.blockDim = dim3(V_NTHREADS);
+    cfg.dynamicSmemBytes = V_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ns > 1 ? 1 : 0;      // its prologue under the summaries' tail
+    if (cudaLaunchKernelEx(&cfg, prefill_vec_kernel, mq, mk, mv, m1, m2, vp) != cudaSuccess) return DSLA_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DSLA_OK : DSLA_ERR_CUDA;
 }
