@@ -20,21 +20,6 @@ __global__ void zero_slots_kernel(float* data, const int32_t* slots, int num_slo
         base[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// o += t over n8 pieces of eight bf16 (fp32 sum, one rounding): the share of a later pair of states of the n-state prefill
-__global__ void __launch_bounds__(256) add_bf16_kernel(uint4* __restrict__ o, const uint4* __restrict__ t, size_t n8) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
-        uint4 a = o[i];
-        const uint4 b = __ldcs(t + i);
-        __nv_bfloat162* pa = reinterpret_cast<__nv_bfloat162*>(&a);
-        const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 x = __bfloat1622float2(pa[e]), y = __bfloat1622float2(pb[e]);
-            pa[e] = __floats2bfloat162_rn(x.x + y.x, x.y + y.y);
-        }
-        o[i] = a;
-    }
-}
 }  // namespace dsla
 
 using namespace dsla;
@@ -333,15 +318,10 @@ static bool nstate_tensor_applies(const dsla_nstate_prefill_args* a) {
     return a->dtype == DSLA_BF16 && a->d_k == 128 && a->gate_layout == DSLA_GATE_SCALAR && prefill_tc_available();
 }
 
-// pairs after the first write their share of o to a scratch tensor that is then added to o
-static size_t nstate_o_scratch_bytes(const dsla_nstate_prefill_args* a) {
-    return a->n_states > 2 ? (((size_t)a->T_total * a->H * a->d_v * 2 + 255) & ~(size_t)255) : 0;
-}
-
 size_t dsla_nstate_prefill_workspace_bytes(const dsla_nstate_prefill_args* a) {
     if (check_nstate_prefill_sizes(a) != DSLA_OK || a->impl == DSLA_IMPL_SIMT || !nstate_tensor_applies(a)) return 0;
     const dsla_prefill_args b = nstate_as_prefill_args(a);
-    return prefill_tc_workspace_bytes(&b, false) + nstate_o_scratch_bytes(a);
+    return prefill_tc_workspace_bytes(&b, false);
 }
 
 dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* st, void* cuda_stream) {
@@ -360,11 +340,9 @@ dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* s
     }
     if (a->impl != DSLA_IMPL_SIMT && nstate_tensor_applies(a) && a->T_total > 0) {
         const dsla_prefill_args b = nstate_as_prefill_args(a);
-        const size_t need_tc = prefill_tc_workspace_bytes(&b, false), need = need_tc + nstate_o_scratch_bytes(a);
+        const size_t need = prefill_tc_workspace_bytes(&b, false);
         if (need > 0 && (!a->workspace || a->workspace_bytes < need || !aligned(a->workspace, 256))) return DSLA_ERR_INVALID_ARG;
         if (!aligned(a->gates, 4)) return DSLA_ERR_INVALID_ARG;
-        void* o_scratch = static_cast<char*>(a->workspace) + need_tc;
-        const size_t n8 = (size_t)a->T_total * a->H * a->d_v / 8;
         cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
         PrefillParams p{};
         p.q = a->q; p.k = a->k; p.v = a->v; p.o = a->o;
@@ -380,16 +358,9 @@ dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* s
             p.single = a->n_states == 1;
             p.g_rec = a->gates + (size_t)(p.single ? first : first + 1) * gs;
             p.state_first = first;
-            p.o = first == 0 ? a->o : o_scratch;
+            p.accumulate = first > 0;      // later pairs add their share of o
             const dsla_status rc = launch_prefill_tc(p, &b, false, s);
             if (rc != DSLA_OK) return rc;
-            if (first > 0) {
-                const size_t blocks = (n8 + 255) / 256;
-                add_bf16_kernel<<<dim3((unsigned)(blocks < 148 * 8 ? blocks : 148 * 8)), dim3(256), 0, s>>>(
-                    static_cast<uint4*>(a->o), static_cast<const uint4*>(o_scratch), n8);
-                count_launch();
-                if (cudaGetLastError() != cudaSuccess) return DSLA_ERR_CUDA;
-            }
         }
         return DSLA_OK;
     }

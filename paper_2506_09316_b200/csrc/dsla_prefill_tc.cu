@@ -16,11 +16,15 @@
 // chunks of 128 tokens (half the passes of 64-token chunks), the update's A operand in TMEM, raw K and V as
 // operands, and Q the only tile that is copied.
 //
-// A sequence may be split into segments along T so that few (sequence, head) pairs still fill the
-// GPU (dsla_prefill_summary.cu computes the segment summaries); the main kernel, launched as the
-// summary grid's programmatic dependent, folds the summaries of earlier segments into its initial
-// state.  Packed batches are visited longest sequence first.  This file also holds the host side
-// of both tensor-core variants (segment plan, workspace layout, launches).
+// A sequence may be split into segments along T so that few (sequence, head) pairs still fill the GPU.  The segments of a
+// sequence are the CTAs of a thread-block cluster: each first accumulates the state its own tokens leave behind, from
+// zero (its summary), the initial states are folded out of the summaries through distributed shared memory, then each runs
+// its chunks.  (As a kernel of its own the summaries took 21 of 68 us at T = 4096, 32 heads: launch, fill and drain of a second
+// pipeline, and 131 KB per segment through global memory and back.)
+// Packed batches are visited longest sequence first.  This file also holds the host side of both tensor-core variants (segment
+// plan, workspace layout, launches).
+#include <atomic>
+
 #include "dsla_prefill_tc.cuh"
 
 namespace dsla {
@@ -47,6 +51,11 @@ constexpr uint32_t COL_S = 0;      // fp32 S1^T [0,128), S2^T [128,256)
 constexpr uint32_t COL_SB = 256;   // per state 64 columns: the bf16 copy of S^T (readout), then the weighted V~^T (update)
 constexpr uint32_t COL_R = 384;    // P (scores, tokens x tokens), then O^T (d_v x tokens): 128 columns
 
+// Where the summaries of the two states (fp32 [d_k][d_v], 64 KB each) wait for the fold, and the initial states for their owner: slots
+// that the first chunk's Q and K do not land in.
+__device__ constexpr int summary_off(int i) { return i == 0 ? TILE_BYTES : OFF_K + TILE_BYTES; }
+constexpr int SUM_STAGES = 3;        // K and V tiles of the summaries: two slots each, in order
+
 // Per-token terms of one chunk; the first index is the state.
 struct alignas(16) GateSmem {
     float L[2][CM];                  // cumulative log2-gate from the chunk start, inclusive
@@ -58,9 +67,11 @@ struct alignas(16) GateSmem {
 
 struct alignas(16) Shared {
     uint64_t kq_full[2], v_full[2], p_full, prep_ready, sb_ready[2], ro_done, vt_ready[2], o_full, o_free, o_staged, u_full[2], g_ready[2], g_free[2], init_done;
+    uint64_t s_full[SUM_STAGES], s_empty[SUM_STAGES], sw_ready[2], sw_free[2], svt_ready[2], svt_free[2], s_done;      // summaries
     uint32_t tmem_base;
     int abort_flag;
     GateSmem gs[2];
+    float a_seg[16][2];                   // products of the gates of every segment of the cluster
 };
 
 // Four MMAs whose operands advance by a constant.
@@ -86,69 +97,129 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const PrefillParams& p = tp.p;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // Blocks are handed out in index order: the last segments first.  When this grid starts as a programmatic dependent
-    // of the summary grid, the blocks that fit next to it are then the ones with the longest fold of summaries ahead of
-    // them, and their prologue (TMEM, first tiles, first scores) is hidden behind the summary grid's tail.
-    const int units = p.N * p.H;
-    const int g = tp.nseg - 1 - (int)(blockIdx.x / units);
-    const int h = (blockIdx.x % units) % p.H;
-    const int rank = (blockIdx.x % units) / p.H;
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // the launch may overlap the tail of what precedes it in the stream
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int nseg = tp.nseg;
+    const int g = blockIdx.x % nseg;             // rank in the cluster
+    const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
     const int n = tp.order ? tp.order[rank] : rank;
     const SeqInfo sq = seq_info(p, n, g, tp);
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (tid == 0 && g == 0 && sq.nchunks > seg_begin(tp.nseg, tp.nseg, tp.cps, tp.skew8)) atomicExch(p.status, (int)DSLA_ERR_INVALID_ARG);
     float* slot1 = p.state + (((size_t)sq.slot * p.n_total + p.state_first) * p.H + h) * (size_t)(D * D);
     const size_t state_stride = (size_t)p.H * D * D;
-    // where the initial state is read: the slot, or the snapshot taken before this grid (split sequences)
-    const float* init1 = tp.init ? tp.init + (size_t)(n * p.H + h) * 2 * (size_t)(D * D) : slot1;
-    const size_t init_stride = tp.init ? (size_t)(D * D) : state_stride;
     if (sq.len <= 0) {  // empty sequence: a fresh start leaves zero states, a resume leaves the slot alone
         if (g == 0 && !p.use_initial_state)
             for (int i = tid; i < (p.single ? 1 : 2) * D * D; i += NTHREADS) slot1[(size_t)(i / (D * D)) * state_stride + i % (D * D)] = 0.f;
         return;
     }
-    if (sq.c_begin >= sq.c_end) return;
-    const int nc = sq.c_end - sq.c_begin;
+    const int nc = max(0, sq.c_end - sq.c_begin);  // 0: a segment behind the end of its sequence, here only for its share of the fold
     const int t0 = sq.t_begin + sq.c_begin * CM;  // first token of this segment
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
     const bool last = g == sq.last_seg;           // the final state is kept; other segments skip the last chunk's update
-    const bool init_shared = (g > 0 && tp.ws) || p.use_initial_state;   // the initial state is loaded, not just zero
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a dependent launch behind this grid (the decode step) may be scheduled early
+    const bool split = nseg > 1, summarize = g < sq.last_seg;
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh.kq_full[i], 1); mbar_init(&sh.v_full[i], 1);
-            mbar_init(&sh.sb_ready[i], 4); mbar_init(&sh.vt_ready[i], 4); mbar_init(&sh.u_full[i], 1);
+            mbar_init(&sh.sb_ready[i], 4); mbar_init(&sh.vt_ready[i], 8); mbar_init(&sh.u_full[i], 1);
             mbar_init(&sh.g_ready[i], 2); mbar_init(&sh.g_free[i], 16);
         }
         mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
         mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8);
-        mbar_init(&sh.init_done, 8);     // the tile warps' share of the initial state
+        mbar_init(&sh.init_done, 16);
+        for (int i = 0; i < SUM_STAGES; ++i) { mbar_init(&sh.s_full[i], 1); mbar_init(&sh.s_empty[i], 9); }      // eight V~ warps + the MMAs on K
+        for (int i = 0; i < 2; ++i) { mbar_init(&sh.sw_ready[i], 2); mbar_init(&sh.sw_free[i], 8); mbar_init(&sh.svt_ready[i], 8); mbar_init(&sh.svt_free[i], 1); }
+        mbar_init(&sh.s_done, 1);
         sh.abort_flag = 0;
         fence_barrier_init();
     }
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
-    __syncthreads();
+    if (split) cluster_sync_all();      // (nothing is sent to a CTA that has not started)
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tb = 0;      // all 512 columns are allocated: the base is column 0
     volatile int* abortp = &sh.abort_flag;
 #define WAIT(bar, ph) mbar_wait(bar, (uint32_t)(ph), abortp, p.status)
 
+    // Tile and state warps (t = 0..511): the slot (or zero) pushed through the summaries of the earlier segments.  Each CTA does this
+    // for its share of the elements and for every segment: it reads the share out of all summaries and writes the initial
+    // states over them, so that every CTA moves 1 / nseg of what a fold per segment would pull from the first ones.
+    auto initial_state_from_cluster = [&](int t) {
+        __syncwarp();
+        cluster_sync_all();       // the summaries are in place
+        const int nsum = sq.last_seg, begin = g * 8192 / nseg, end = (g + 1) * 8192 / nseg;      // 16-byte pieces of [2][D][D]
+#pragma unroll 2
+        for (int f = begin + t; f < end; f += 512) {
+            const int i = f >> 12, e = f & 4095;
+            const uint32_t at = smem_u32(tiles + summary_off(i) + e * 16);
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p.use_initial_state && !(p.single && i == 1)) x = *reinterpret_cast<const float4*>(slot1 + (size_t)i * state_stride + (size_t)e * 4);
+#pragma unroll 1
+            for (int s0 = 0; s0 <= nsum; s0 += 3) {      // three segments' loads in flight
+                float4 u[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (s0 + k < nsum) u[k] = ld_cluster_f32x4(map_to_cta(at, (uint32_t)(s0 + k)));
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int r = s0 + k;
+                    if (r > nsum) break;
+                    if (r > 0 || p.use_initial_state) st_cluster_f32x4(map_to_cta(at, (uint32_t)r), x.x, x.y, x.z, x.w);
+                    if (r < nsum) {
+                        const float a = sh.a_seg[r][i];
+                        x.x = fmaf(a, x.x, u[k].x); x.y = fmaf(a, x.y, u[k].y); x.z = fmaf(a, x.z, u[k].z); x.w = fmaf(a, x.w, u[k].w);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();       // the initial states are in place; every read of the slot is done
+    };
+    // d_k rows 64 part .. 64 part + 63 of state i, one d_v lane per thread: the bf16 copy for the readout and a_0 S for the first update
+    auto start_state = [&](int i, int part, uint32_t lane_addr, int v, float a) {
+        const float* src = split ? reinterpret_cast<const float*>(tiles + summary_off(i)) : slot1 + (size_t)i * state_stride;
+        init_state_pass(src, (split && g > 0) || (p.use_initial_state && !(p.single && i == 1)), nullptr, 0, i, v, a, lane_addr + COL_S + 128 * i, lane_addr + COL_SB + 64 * i,
+                        2 * part, 2 * part + 2);
+        tc_wait_st();
+        tc_fence_before();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&sh.init_done);
+    };
+
     if (warp == WARP_TMA) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
-            auto load_kq = [&](int c, int q3) {
-                mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
-                tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-                tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-            };
-            auto load_v = [&](int c, int v3) {
-                mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
-                tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
-            };
-            load_kq(0, 0);
+        }
+        auto load_kq = [&](int c, int q3) {
+            mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
+            tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+            tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+        };
+        auto load_v = [&](int c, int v3) {
+            mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
+            tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
+        };
+        if (lane == 0) {
+            if (summarize) {      // step it = chunk nc - 1 - it
+                for (int it = 0; it < nc; ++it) {
+                    const int st = it % SUM_STAGES, t = t0 + (nc - 1 - it) * CM;
+                    if (it >= SUM_STAGES) WAIT(&sh.s_empty[st], (it / SUM_STAGES - 1) & 1);
+                    mbar_arrive_expect_tx(&sh.s_full[st], 2 * TILE_BYTES);
+                    tma_load_4d(tiles + (2 * st + 1) * TILE_BYTES, &map_v, &sh.s_full[st], 0, t, 0, h);
+                    tma_load_4d(tiles + 2 * st * TILE_BYTES, &map_k, &sh.s_full[st], 0, t, 0, h);
+                }
+                WAIT(&sh.s_done, 0);
+            }
+            if (nc > 0) load_kq(0, 0);
+        }
+        __syncwarp();
+        if (split) { cluster_sync_all(); cluster_sync_all(); }
+        if (lane == 0 && nc > 0) {
+            if (split) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
             load_v(0, 2);
             if (nc > 1) load_kq(1, 1);
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
@@ -164,7 +235,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
                 if (c < nfull) {
                     WAIT(&sh.o_staged, c & 1);             // the outputs of chunk c are in the slot of its V
-                    tma_store_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);
+                    if (p.accumulate) tma_add_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);      // bf16 sums, one rounding each
+                    else tma_store_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);
                     bulk_commit();
                     bulk_wait_read();
                 }
@@ -185,23 +257,46 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // Per chunk:  O^T = S1^T Q~1^T + S2^T Q~2^T,  O^T += V^T P~^T,  S1^T += V~1^T K,  P of the next chunk,  S2^T += V~2^T K.
         // The readout of a state starts as soon as its bf16 copy is there; V~ is stored under the P~ part, O^T is read out under
         // the first update, the next scores are masked under the second.
+        const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
+        constexpr uint32_t ID_KK = idesc_bf16(128, 128, 0, 0);     // both operands K-major (scores; readout with A in TMEM)
+        constexpr uint32_t ID_V128 = idesc_bf16(128, 128, 1, 0), ID_V64 = idesc_bf16(128, 64, 1, 0);
+        constexpr uint32_t ID_U = idesc_bf16(128, 128, 0, 1);      // A in TMEM, B = raw K, MN-major
+        constexpr uint32_t T_STEP = TILE_BYTES >> 4, H_STEP = HALF_BYTES >> 4;
+        const uint32_t dq0 = smem_desc_lo(sa, 16), dq2 = smem_desc_lo(sa + OFF_Q2, 16), dkk = smem_desc_lo(sa + OFF_K, 16);
+        const uint32_t dkn = smem_desc_lo(sa + OFF_K, HALF_BYTES), dv0 = smem_desc_lo(sa, HALF_BYTES), dp0 = smem_desc_lo(sa + OFF_PT, 16);
+        auto scores = [&](int c, int q3) {
+            WAIT(&sh.kq_full[c & 1], (c >> 1) & 1);
+            tc_fence_after();
+            const uint32_t a = dq0 + (uint32_t)q3 * T_STEP, b = dkk + (uint32_t)(c & 1) * T_STEP;
+            issue4_ss<2, 2>(COL_R, a, b, ID_KK, 0u);
+            issue4_ss<2, 2>(COL_R, a + H_STEP, b + H_STEP, ID_KK, 1u);
+            tc_commit(&sh.p_full);
+        };
         if (elect_one()) {
-            const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
-            constexpr uint32_t ID_KK = idesc_bf16(128, 128, 0, 0);     // both operands K-major (scores; readout with A in TMEM)
-            constexpr uint32_t ID_V128 = idesc_bf16(128, 128, 1, 0), ID_V64 = idesc_bf16(128, 64, 1, 0);
-            constexpr uint32_t ID_U = idesc_bf16(128, 128, 0, 1);      // A in TMEM, B = raw K, MN-major
-            constexpr uint32_t T_STEP = TILE_BYTES >> 4, H_STEP = HALF_BYTES >> 4;
-            const uint32_t dq0 = smem_desc_lo(sa, 16), dq2 = smem_desc_lo(sa + OFF_Q2, 16), dkk = smem_desc_lo(sa + OFF_K, 16);
-            const uint32_t dkn = smem_desc_lo(sa + OFF_K, HALF_BYTES), dv0 = smem_desc_lo(sa, HALF_BYTES), dp0 = smem_desc_lo(sa + OFF_PT, 16);
-            auto scores = [&](int c, int q3) {
-                WAIT(&sh.kq_full[c & 1], (c >> 1) & 1);
-                tc_fence_after();
-                const uint32_t a = dq0 + (uint32_t)q3 * T_STEP, b = dkk + (uint32_t)(c & 1) * T_STEP;
-                issue4_ss<2, 2>(COL_R, a, b, ID_KK, 0u);
-                issue4_ss<2, 2>(COL_R, a + H_STEP, b + H_STEP, ID_KK, 1u);
-                tc_commit(&sh.p_full);
-            };
-            scores(0, 0);
+            if (summarize) {
+#pragma unroll 1
+                for (int it = 0; it < nc; ++it) {
+                    const int st = it % SUM_STAGES, b = it & 1;
+                    WAIT(&sh.s_full[st], (it / SUM_STAGES) & 1);
+                    WAIT(&sh.svt_ready[b], (it >> 1) & 1);
+                    tc_fence_after();
+                    const uint32_t bk = dv0 + (uint32_t)(2 * st) * T_STEP;      // K in slot 2 st, MN-major like V
+#pragma unroll 1
+                    for (int i = 0; i < 2; ++i) {
+                        const uint32_t a = (b ? COL_R : COL_SB) + 64 * i;
+                        issue4_ts<128>(COL_S + 128 * i, a, bk, ID_U, it ? 1u : 0u);
+                        issue4_ts<128>(COL_S + 128 * i, a + 32, bk + 512, ID_U, 1u);
+                    }
+                    tc_commit(&sh.s_empty[st]);
+                    tc_commit(&sh.svt_free[b]);
+                }
+                tc_commit(&sh.s_done);
+            }
+            if (nc > 0) scores(0, 0);
+        }
+        __syncwarp();
+        if (split) { cluster_sync_all(); cluster_sync_all(); }
+        if (elect_one()) {
             int c3 = 0;
 #pragma unroll 1
             for (int c = 0; c < nc; ++c) {
@@ -250,18 +345,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first] : p.gamma[h]) * p.scale;
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
 
-        if (init_shared) {
-            // d_k rows 64..127 of the initial state of state `half` for this lane quadrant, while the first tiles are in flight
+        if (split) initial_state_from_cluster(tid - TILE_W0 * 32);
+        if (nc > 0) {
             WAIT(&sh.g_ready[0], 0);
-            if (g > 0 && tp.ws) asm volatile("griddepcontrol.wait;" ::: "memory");
-            init_state_pass(init1 + (size_t)half * init_stride, p.use_initial_state && !(p.single && half == 1),
-                            tp.ws ? tp.ws + ((size_t)(n * p.H + h) * tp.nseg) * (SUMMARY_STRIDE / 4) : nullptr, g, half, j, sh.gs[0].a[half],
-                            lane_addr + COL_S + 128 * half, lane_addr + COL_SB + 64 * half, 2, 4);
-            tc_wait_st();
-            tc_fence_before();
+            start_state(half, 1, lane_addr, j, sh.gs[0].a[half]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.init_done);
         // The ten 32 x 32 blocks of the lower triangle: a quadrant's q + 1 blocks are split between its two warps (the second one
         // has the diagonal block).  The two blocks above the diagonal that the MMAs read are zeroed once.
         const int blk0 = half == 0 ? 0 : (q == 1 ? 1 : 2), nblk = q == 0 ? 1 - half : (q == 3 || (q == 2 && half == 0)) ? 2 : 1;
@@ -348,39 +436,68 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float* gsrc = i == 0 ? p.g_hist : p.g_rec;
         const float Wi = (p.weights ? (i == 1 && p.single ? 0.f : p.weights[(size_t)h * p.n_total + p.state_first + i])
                                     : (i == 0 ? p.gamma[h] : 1.f - p.gamma[h])) * p.scale;
+        auto decays = [&](const float (&x)[4], float (&L)[4], float& pr, float& incl) {      // L: inclusive from the chunk start; incl: of the lane's last token
+            float run = 0.f;
+            pr = 1.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float y = fmaxf(x[e], 0.f);
+                pr *= y;
+                run += lg2_gate(y);
+                L[e] = run;
+            }
+            incl = warp_prefix_sum(run, lane);
+            float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+            if (lane == 0) excl = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) L[e] = e == 3 ? incl : excl + L[e];      // (`incl` is what other lanes see: keep the two consistent)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) pr *= __shfl_xor_sync(0xffffffffu, pr, off);
+        };
         float nx[4];
         auto fetch = [&](int c) {      // raw values: nothing may consume them here, or the warp would sit out the load latency in every chunk
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int j = c * CM + 4 * lane + e;
-                nx[e] = load_gate(gsrc, t0 + j, p.H, h, c < nc && tok0 + j < sq.len);
+                nx[e] = load_gate(gsrc, t0 + j, p.H, h, c >= 0 && c < nc && tok0 + j < sq.len);
             }
         };
+        if (summarize) {      // weights to the end of the segment, chunks from the last to the first
+            float after = 0.f, A = 1.f;      // log2 and product of the gates of all later chunks
+            fetch(nc - 1);
+            for (int it = 0; it < nc; ++it) {
+                const int b = it & 1;
+                const float x[4] = {nx[0], nx[1], nx[2], nx[3]};
+                fetch(nc - 2 - it);
+                float L[4], pr, incl;
+                decays(x, L, pr, incl);
+                const float end = __shfl_sync(0xffffffffu, incl, 31);
+                if (it >= 2) WAIT(&sh.sw_free[b], ((it >> 1) - 1) & 1);
+                *reinterpret_cast<uint2*>(&sh.gs[b].w[i][4 * lane]) = make_uint2(pack_bf16(ex2(end - L[0] + after), ex2(end - L[1] + after)),
+                                                                               pack_bf16(ex2(end - L[2] + after), ex2(end - L[3] + after)));
+                after += end;
+                A *= pr;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.sw_ready[b]);
+            }
+            if (lane < nseg) st_cluster_f32(map_to_cta(smem_u32(&sh.a_seg[g][i]), (uint32_t)lane), A);      // to every CTA of the cluster
+            for (int it = max(0, nc - 2); it < nc; ++it) WAIT(&sh.sw_free[it & 1], (it >> 1) & 1);      // the ring is reused for the chunks below
+        }
         fetch(0);
+        if (nc == 0 && split) { cluster_sync_all(); cluster_sync_all(); }
         for (int c = 0; c < nc; ++c) {
             const int s = c & 1;
             GateSmem& gs = sh.gs[s];
-            float L[4], pr = 1.f, run = 0.f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float x = fmaxf(nx[e], 0.f);
-                pr *= x;
-                run += lg2_gate(x);
-                L[e] = run;
-            }
+            const float x[4] = {nx[0], nx[1], nx[2], nx[3]};
             fetch(c + 1);
-            const float incl = warp_prefix_sum(run, lane);
-            float excl = __shfl_up_sync(0xffffffffu, incl, 1);
-            if (lane == 0) excl = 0.f;
+            float L[4], pr, incl;
+            decays(x, L, pr, incl);
             const float block_end = __shfl_sync(0xffffffffu, incl, lane | 7), end = __shfl_sync(0xffffffffu, incl, 31);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) pr *= __shfl_xor_sync(0xffffffffu, pr, off);
             const int valid = min(CM, sq.len - tok0 - c * CM);
             if (c >= 2) WAIT(&sh.g_free[s], ((c >> 1) - 1) & 1);
             float f[4], E[4], w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                L[e] = e == 3 ? incl : excl + L[e];      // (block_end is some lane's incl: keep the two consistent)
                 f[e] = Wi * ex2(L[e]);
                 E[e] = ex2(block_end - L[e]);
                 w[e] = 4 * lane + e < valid ? ex2(end - L[e]) : 0.f;
@@ -392,6 +509,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0) gs.a[i] = pr;
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.g_ready[s]);
+            if (c == 0 && split) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }
         }
     } else {
         // ------------------------------------------------------------------ state warps 10..17
@@ -403,6 +521,51 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         __nv_bfloat16* og = reinterpret_cast<__nv_bfloat16*>(p.o);
         // ldmatrix: this thread addresses row mr of matrix mk; matrices (tokens 0..7 | 8..15) x (d_v 0..7 | 8..15)
         const int mk = lane >> 3, mr = lane & 7;
+        // V~_i^T[v][s] = w^i_s V[s][v] of both states, for the 16 lanes 16 hi .. of this quadrant: ldmatrix.trans hands out the element
+        // pairs a 16x128b TMEM store takes.  `wait` runs between the arithmetic and the stores.
+        auto weighted_v = [&](const uint8_t* vtile, const GateSmem& gs, uint32_t col, auto wait) {
+            const int d = 32 * q + 16 * hi + 8 * (mk & 1);            // first d_v column of the matrix this thread addresses
+            const uint32_t row0 = smem_u32(vtile) + (uint32_t)((8 * (mk >> 1) + mr) * 128) + (uint32_t)(d >> 6) * HALF_BYTES +
+                                  (((uint32_t)((d & 63) >> 3) ^ (uint32_t)mr) << 4);
+            uint32_t r[32], y[32];
+#pragma unroll
+            for (int t16 = 0; t16 < 8; ++t16) ldmatrix_x4_trans(row0 + (uint32_t)(t16 * 16 * 128), r[4 * t16], r[4 * t16 + 1], r[4 * t16 + 2], r[4 * t16 + 3]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t wp = smem_u32(&gs.w[i][2 * (lane & 3)]);
+                uint32_t* o = i == 0 ? y : r;
+#pragma unroll
+                for (int t16 = 0; t16 < 8; ++t16) {
+                    const uint32_t w0 = ld_shared_u32(wp + 32 * t16), w1 = ld_shared_u32(wp + 32 * t16 + 16);
+                    o[4 * t16] = hmul2_u32(r[4 * t16], w0); o[4 * t16 + 1] = hmul2_u32(r[4 * t16 + 1], w0);
+                    o[4 * t16 + 2] = hmul2_u32(r[4 * t16 + 2], w1); o[4 * t16 + 3] = hmul2_u32(r[4 * t16 + 3], w1);
+                }
+            }
+            wait();
+            const uint32_t at = lane_addr + ((uint32_t)(16 * hi) << 16) + col;
+            tmem_st_16x128b_x8(at, y); tmem_st_16x128b_x8(at + 32, y + 16);
+            tmem_st_16x128b_x8(at + 64, r); tmem_st_16x128b_x8(at + 96, r + 16);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+        };
+        if (summarize) {
+#pragma unroll 1
+            for (int it = 0; it < nc; ++it) {
+                const int st = it % SUM_STAGES, b = it & 1;
+                WAIT(&sh.sw_ready[b], (it >> 1) & 1);
+                WAIT(&sh.s_full[st], (it / SUM_STAGES) & 1);
+                weighted_v(tiles + (2 * st + 1) * TILE_BYTES, sh.gs[b], b ? COL_R : COL_SB, [&] {
+                    if (it >= 2) WAIT(&sh.svt_free[b], ((it >> 1) - 1) & 1);
+                    tc_fence_after();
+                });
+                if (lane == 0) { mbar_arrive(&sh.svt_ready[b]); mbar_arrive(&sh.s_empty[st]); mbar_arrive(&sh.sw_free[b]); }
+            }
+            WAIT(&sh.s_done, 0);
+            tc_fence_after();
+            store_state(reinterpret_cast<float*>(tiles + summary_off(hi)), v, s_addr, 0, 4);
+        }
+        if (split) initial_state_from_cluster(256 + tid - STATE_W0 * 32);
         int v3 = 2;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
@@ -411,13 +574,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
             const float a = gs.a[hi];
             if (c == 0) {
-                // With programmatic dependent launch this grid may start while the summary grid is still running;
-                // everything up to here (and all of chunk 0's operand work in the other warps) is independent of it.
-                if (g > 0 && tp.ws) asm volatile("griddepcontrol.wait;" ::: "memory");
-                init_state_pass(init1 + (size_t)hi * init_stride, p.use_initial_state && !(p.single && hi == 1),
-                                tp.ws ? tp.ws + ((size_t)(n * p.H + h) * tp.nseg) * (SUMMARY_STRIDE / 4) : nullptr, g, hi, v, a, s_addr, sb_addr,
-                                0, init_shared ? 2 : 4);
-                WAIT(&sh.init_done, 0);     // the other half (or nothing) from the tile warps
+                start_state(hi, 0, lane_addr, v, a);
+                WAIT(&sh.init_done, 0);     // the tile warps' half
             } else {
                 WAIT(&sh.u_full[hi], (c - 1) & 1);
                 tc_fence_after();
@@ -443,44 +601,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.sb_ready[hi]);
-            // ---- V~^T[v][s] = w_s V[s][v] of this state and quadrant: built in registers under the readout, stored over the bf16 copy as
-            // soon as that has been read; the P~ part of the outputs, which follows, leaves shared memory no room for other reads (ldmatrix.trans hands out the element pairs a 16x128b TMEM store takes)
+            // ---- V~ of both states: built in registers under the readout, stored over the bf16 copies as soon as those have been read; the
+            // P~ part of the outputs, which follows, leaves shared memory no room for other reads
             WAIT(&sh.v_full[s], (c >> 1) & 1);
             WAIT(&sh.prep_ready, c & 1);      // (under the readout: before it the tile warps need the issue slots and shared memory)
-            {
-                const uint32_t vrow = smem_u32(tiles + v3 * TILE_BYTES) + (uint32_t)((8 * (mk >> 1) + mr) * 128);
-                const uint32_t wp = smem_u32(&gs.w[hi][2 * (lane & 3)]);
-                uint32_t vt[2][32];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {       // the two 16-lane halves of this warp's TMEM quadrant
-                    const int d = 32 * q + 16 * hh + 8 * (mk & 1);            // first d_v column of the matrix this thread addresses
-                    const uint32_t row0 = vrow + (uint32_t)(d >> 6) * HALF_BYTES + (((uint32_t)((d & 63) >> 3) ^ (uint32_t)mr) << 4);
-#pragma unroll
-                    for (int t16 = 0; t16 < 8; ++t16)
-                        ldmatrix_x4_trans(row0 + (uint32_t)(t16 * 16 * 128), vt[hh][4 * t16], vt[hh][4 * t16 + 1], vt[hh][4 * t16 + 2], vt[hh][4 * t16 + 3]);
-                }
-#pragma unroll
-                for (int t16 = 0; t16 < 8; ++t16) {
-                    const uint32_t w0 = ld_shared_u32(wp + 32 * t16), w1 = ld_shared_u32(wp + 32 * t16 + 16);
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t* r = vt[hh] + 4 * t16;
-                        r[0] = hmul2_u32(r[0], w0); r[1] = hmul2_u32(r[1], w0);
-                        r[2] = hmul2_u32(r[2], w1); r[3] = hmul2_u32(r[3], w1);
-                    }
-                }
+            weighted_v(tiles + v3 * TILE_BYTES, gs, COL_SB, [&] {
                 mbar_wait_inline(&sh.ro_done, c & 1, abortp, p.status);
                 tc_fence_after();
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    tmem_st_16x128b_x8(sb_addr + ((uint32_t)(16 * hh) << 16), vt[hh]);
-                    tmem_st_16x128b_x8(sb_addr + ((uint32_t)(16 * hh) << 16) + 32, vt[hh] + 16);
-                }
-            }
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) { mbar_arrive(&sh.vt_ready[hi]); mbar_arrive(&sh.g_free[s]); }
+            });
+            if (lane == 0) { mbar_arrive(&sh.vt_ready[0]); mbar_arrive(&sh.vt_ready[1]); mbar_arrive(&sh.g_free[s]); }
             // ---- outputs, tokens 64 hi .. 64 hi + 63 of this warp's lane quadrant.  Whole chunks: token-major bf16 tile in the slot of
             // this chunk's V (stmatrix transposes the fragments of a 16x256b load), which the producer warp stores with one TMA
             // copy; 64 stores of one token's 64 bytes each held the warps up for 2400 cycles.
@@ -518,14 +647,17 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     tc_wait_ld();
 #pragma unroll
                     for (int jj = 0; jj < 16; ++jj) {
-                        if (b + jj < valid) *dst = __float2bfloat16_rn(__uint_as_float(r[jj]));
+                        if (b + jj < valid) {
+                            const __nv_bfloat16 y = __float2bfloat16_rn(__uint_as_float(r[jj]));
+                            *dst = p.accumulate ? __hadd(*dst, y) : y;
+                        }
                         dst += row;
                     }
                 }
             }
             v3 = v3 == 2 ? 0 : v3 + 1;
         }
-        if (last) {
+        if (last && nc > 0) {
             WAIT(&sh.u_full[hi], (nc - 1) & 1);
             tc_fence_after();
             if (!(p.single && hi == 1)) store_state(slot1 + (size_t)hi * state_stride, v, s_addr, 0, 4);
@@ -552,25 +684,63 @@ int sm_count() {
     return sms;
 }
 
-// Segments per sequence: enough work items (CTAs, or clusters of the pair variant) to cover the SMs when there
-// are few (sequence, head) pairs, never shorter than 256 tokens per segment.
+// The most clusters of each size (one CTA per SM) that fit on the device at once; sizes over 8 are opt-in.
+constexpr int MAX_SEG = 16;
+int resident_clusters(int size) {
+    static std::atomic<int> cached[64][MAX_SEG + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return sm_count() / size; }
+    int n = cached[dev][size].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(size * 148));
+        cfg.blockDim = dim3(NTHREADS);
+        cfg.dynamicSmemBytes = SMEM_DYN;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess ||
+            (size > 8 && cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, prefill_tc_kernel, &cfg) != cudaSuccess || n <= 0)
+            n = -1;
+        (void)cudaGetLastError();
+        cached[dev][size].store(n, std::memory_order_relaxed);
+    }
+    return n > 0 ? n : 0;
+}
+
+// Segments per sequence: the most that keep all work items resident at once (CTAs of a cluster, or clusters of the pair variant).
+// The single-CTA kernel's segments hold at least one chunk of 128 tokens, and a sequence of two chunks stays whole (summary and
+// fold cost about as much as the chunk they would save); the pair variant's at least four of 64.
 void plan(const dsla_prefill_args* a, bool pair, int* nseg, int* cps, int* skew8) {
-    const int chunk = pair ? C : CM, min_cps = pair ? 4 : 2;
+    const int chunk = pair ? C : CM;
     const int max_chunks = (a->max_seqlen + chunk - 1) / chunk;
     const long long units = (long long)a->N * a->H;
-    const int room = pair ? pair_resident_clusters() : sm_count();     // work items resident at once
     int ns = 1;
-    if (units > 0 && units < room) ns = (int)(room / units);
-    if (ns > 16) ns = 16;
-    while (ns > 1 && (max_chunks + ns - 1) / ns < min_cps) --ns;
+    *skew8 = 0;
+    if (pair) {
+        const int room = pair_resident_clusters();
+        if (units > 0 && units < room) ns = (int)(room / units);
+        if (ns > MAX_SEG) ns = MAX_SEG;
+        while (ns > 1 && (max_chunks + ns - 1) / ns < 4) --ns;
+    } else if (units > 0 && units < sm_count() && max_chunks > 2) {
+        ns = (int)(sm_count() / units);
+        if (ns > MAX_SEG) ns = MAX_SEG;
+        if (ns > max_chunks) ns = max_chunks;
+        while (ns > 1 && resident_clusters(ns) < units) --ns;
+        ns = (max_chunks + (max_chunks + ns - 1) / ns - 1) / ((max_chunks + ns - 1) / ns);      // no segment without a chunk in the longest sequence
+    }
     if (max_chunks <= 0) ns = 1;
     *nseg = ns;
     *cps = max_chunks > 0 ? (max_chunks + ns - 1) / ns : 1;
-    // later segments fold more summaries into their initial state before they start (about 50 tokens' time each):
-    // make consecutive segments about that much shorter, as far as the shortest keeps at least 192 tokens
-    int sk = ns > 1 ? (8 * (*cps - (pair ? 3 : 2))) / (ns - 1) : 0;
-    const int most = pair ? 3 : 2;
-    *skew8 = sk < 0 ? 0 : (sk > most ? most : sk);
+    // The pair variant's later segments fold more summaries into their initial state before they start (about 50 tokens' time
+    // each): make consecutive segments about that much shorter, as far as the shortest keeps at least 192 tokens.
+    if (pair && ns > 1) {
+        const int sk = (8 * (*cps - 3)) / (ns - 1);
+        *skew8 = sk < 0 ? 0 : (sk > 3 ? 3 : sk);
+    }
 }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -579,20 +749,22 @@ size_t order_bytes(const dsla_prefill_args* a) { return wants_order(a) ? up256((
 // room for the snapshot of the initial states of split sequences (used when use_initial_state is set)
 size_t snapshot_bytes(const dsla_prefill_args* a, int nseg) { return nseg > 1 ? (size_t)a->N * a->H * 2 * D * D * sizeof(float) : 0; }
 
-dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo, const TcParams& tp,
-                        bool dependent, cudaStream_t s) {
+dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo, const TcParams& tp, cudaStream_t s) {
     if (cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess) return DSLA_ERR_CUDA;
+    if (tp.nseg > 8 && cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return DSLA_ERR_CUDA;
     const long long units = (long long)tp.p.N * tp.p.H;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(units * tp.nseg));
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = SMEM_DYN;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)tp.nseg; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
+    cfg.numAttrs = tp.nseg > 1 ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, prefill_tc_kernel, mq, mk, mv, mo, tp) != cudaSuccess) return DSLA_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DSLA_OK : DSLA_ERR_CUDA;
@@ -626,7 +798,7 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
         launch_seq_order(p.cu_seqlens, p.N, order, s);
         tp.order = order;
     }
-    if (tp.nseg > 1 && p.use_initial_state) {
+    if (pair && tp.nseg > 1 && p.use_initial_state) {
         // The CTA of a sequence's last segment overwrites the slot with the final state; CTAs of earlier segments read the
         // slot as their initial state and nothing orders the two inside the grid: they read a copy taken beforehand.
         float* snap = reinterpret_cast<float*>(wsp + summaries_bytes(a, tp.nseg) + order_bytes(a));
@@ -639,13 +811,13 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
         return DSLA_ERR_CUDA;
     const long long units = (long long)p.N * p.H;
     if (2 * units * tp.nseg > 0x7fffffffLL) return DSLA_ERR_UNSUPPORTED;
-    if (tp.nseg > 1) {
+    if (pair && tp.nseg > 1) {
         CUtensorMap sk, sv;
         if (!make_tile_map(&sk, p.k, a->T_total, p.H, C) || !make_tile_map(&sv, p.v, a->T_total, p.H, C)) return DSLA_ERR_CUDA;
         const dsla_status rc = launch_summary(sk, sv, tp, s);
         if (rc != DSLA_OK) return rc;
     }
-    return pair ? launch_main_pair(mq, mk, mv, tp, tp.nseg > 1, s) : launch_main(mq, mk, mv, mo, tp, tp.nseg > 1, s);
+    return pair ? launch_main_pair(mq, mk, mv, tp, tp.nseg > 1, s) : launch_main(mq, mk, mv, mo, tp, s);
 }
 
 }  // namespace dsla
