@@ -70,6 +70,7 @@ struct alignas(16) Shared {
     uint64_t s_full[SUM_STAGES], s_empty[SUM_STAGES], sw_ready[2], sw_free[2], svt_ready[2], svt_free[2], s_done;      // summaries
     uint32_t tmem_base;
     int abort_flag;
+    float* slot;                          // the first state of this (sequence, head) in its slot: read where it is needed, not kept in registers
     GateSmem gs[2];
     float a_seg[16][2];                   // products of the gates of every segment of the cluster
 };
@@ -89,6 +90,9 @@ __device__ __forceinline__ void issue4_ts(uint32_t d, uint32_t a, uint32_t b, ui
 // ============================================================================================
 // Main kernel
 // ============================================================================================
+// SPLIT: the sequences are cut into segments (a variant of its own: with that code in it the chunk loop of whole sequences
+// ran 2 % longer).
+template <bool SPLIT>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const TcParams tp) {
@@ -99,7 +103,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the launch may overlap the tail of what precedes it in the stream
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int nseg = tp.nseg;
+    const int nseg = SPLIT ? tp.nseg : 1;
     const int g = blockIdx.x % nseg;             // rank in the cluster
     const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
     const int n = tp.order ? tp.order[rank] : rank;
@@ -117,7 +121,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int t0 = sq.t_begin + sq.c_begin * CM;  // first token of this segment
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
     const bool last = g == sq.last_seg;           // the final state is kept; other segments skip the last chunk's update
-    const bool split = nseg > 1, summarize = g < sq.last_seg;
+    const bool summarize = SPLIT && g < sq.last_seg;
 
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -132,11 +136,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         for (int i = 0; i < 2; ++i) { mbar_init(&sh.sw_ready[i], 2); mbar_init(&sh.sw_free[i], 8); mbar_init(&sh.svt_ready[i], 8); mbar_init(&sh.svt_free[i], 1); }
         mbar_init(&sh.s_done, 1);
         sh.abort_flag = 0;
+        sh.slot = slot1;
         fence_barrier_init();
     }
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
-    if (split) cluster_sync_all();      // (nothing is sent to a CTA that has not started)
+    if (SPLIT) cluster_sync_all();      // (nothing is sent to a CTA that has not started)
     else __syncthreads();
     tc_fence_after();
     const uint32_t tb = 0;      // all 512 columns are allocated: the base is column 0
@@ -155,7 +160,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int i = f >> 12, e = f & 4095;
             const uint32_t at = smem_u32(tiles + summary_off(i) + e * 16);
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p.use_initial_state && !(p.single && i == 1)) x = *reinterpret_cast<const float4*>(slot1 + (size_t)i * state_stride + (size_t)e * 4);
+            if (p.use_initial_state && !(p.single && i == 1)) x = *reinterpret_cast<const float4*>(sh.slot + (size_t)i * state_stride + (size_t)e * 4);
 #pragma unroll 1
             for (int s0 = 0; s0 <= nsum; s0 += 3) {      // three segments' loads in flight
                 float4 u[3];
@@ -179,8 +184,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     };
     // d_k rows 64 part .. 64 part + 63 of state i, one d_v lane per thread: the bf16 copy for the readout and a_0 S for the first update
     auto start_state = [&](int i, int part, uint32_t lane_addr, int v, float a) {
-        const float* src = split ? reinterpret_cast<const float*>(tiles + summary_off(i)) : slot1 + (size_t)i * state_stride;
-        init_state_pass(src, (split && g > 0) || (p.use_initial_state && !(p.single && i == 1)), nullptr, 0, i, v, a, lane_addr + COL_S + 128 * i, lane_addr + COL_SB + 64 * i,
+        const float* src = SPLIT ? reinterpret_cast<const float*>(tiles + summary_off(i)) : sh.slot + (size_t)i * state_stride;
+        init_state_pass(src, (SPLIT && g > 0) || (p.use_initial_state && !(p.single && i == 1)), nullptr, 0, i, v, a, lane_addr + COL_S + 128 * i, lane_addr + COL_SB + 64 * i,
                         2 * part, 2 * part + 2);
         tc_wait_st();
         tc_fence_before();
@@ -217,9 +222,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (nc > 0) load_kq(0, 0);
         }
         __syncwarp();
-        if (split) { cluster_sync_all(); cluster_sync_all(); }
+        if (SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         if (lane == 0 && nc > 0) {
-            if (split) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
+            if (SPLIT) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
             load_v(0, 2);
             if (nc > 1) load_kq(1, 1);
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
@@ -295,7 +300,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (nc > 0) scores(0, 0);
         }
         __syncwarp();
-        if (split) { cluster_sync_all(); cluster_sync_all(); }
+        if (SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         if (elect_one()) {
             int c3 = 0;
 #pragma unroll 1
@@ -345,7 +350,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first] : p.gamma[h]) * p.scale;
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
 
-        if (split) initial_state_from_cluster(tid - TILE_W0 * 32);
+        if (SPLIT) initial_state_from_cluster(tid - TILE_W0 * 32);
         if (nc > 0) {
             WAIT(&sh.g_ready[0], 0);
             start_state(half, 1, lane_addr, j, sh.gs[0].a[half]);
@@ -484,7 +489,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (int it = max(0, nc - 2); it < nc; ++it) WAIT(&sh.sw_free[it & 1], (it >> 1) & 1);      // the ring is reused for the chunks below
         }
         fetch(0);
-        if (nc == 0 && split) { cluster_sync_all(); cluster_sync_all(); }
+        if (nc == 0 && SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         for (int c = 0; c < nc; ++c) {
             const int s = c & 1;
             GateSmem& gs = sh.gs[s];
@@ -509,7 +514,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0) gs.a[i] = pr;
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.g_ready[s]);
-            if (c == 0 && split) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }
+            if (c == 0 && SPLIT) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }
         }
     } else {
         // ------------------------------------------------------------------ state warps 10..17
@@ -565,7 +570,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc_fence_after();
             store_state(reinterpret_cast<float*>(tiles + summary_off(hi)), v, s_addr, 0, 4);
         }
-        if (split) initial_state_from_cluster(256 + tid - STATE_W0 * 32);
+        if (SPLIT) initial_state_from_cluster(256 + tid - STATE_W0 * 32);
         int v3 = 2;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
@@ -660,7 +665,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (last && nc > 0) {
             WAIT(&sh.u_full[hi], (nc - 1) & 1);
             tc_fence_after();
-            if (!(p.single && hi == 1)) store_state(slot1 + (size_t)hi * state_stride, v, s_addr, 0, 4);
+            if (!(p.single && hi == 1)) store_state(sh.slot + (size_t)hi * state_stride, v, s_addr, 0, 4);
         }
     }
     tc_fence_before();
@@ -701,9 +706,9 @@ int resident_clusters(int size) {
         attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess ||
-            (size > 8 && cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-            cudaOccupancyMaxActiveClusters(&n, prefill_tc_kernel, &cfg) != cudaSuccess || n <= 0)
+        if (cudaFuncSetAttribute(prefill_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess ||
+            (size > 8 && cudaFuncSetAttribute(prefill_tc_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, prefill_tc_kernel<true>, &cfg) != cudaSuccess || n <= 0)
             n = -1;
         (void)cudaGetLastError();
         cached[dev][size].store(n, std::memory_order_relaxed);
@@ -750,8 +755,9 @@ size_t order_bytes(const dsla_prefill_args* a) { return wants_order(a) ? up256((
 size_t snapshot_bytes(const dsla_prefill_args* a, int nseg) { return nseg > 1 ? (size_t)a->N * a->H * 2 * D * D * sizeof(float) : 0; }
 
 dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo, const TcParams& tp, cudaStream_t s) {
-    if (cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess) return DSLA_ERR_CUDA;
-    if (tp.nseg > 8 && cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return DSLA_ERR_CUDA;
+    const auto kernel = tp.nseg > 1 ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess) return DSLA_ERR_CUDA;
+    if (tp.nseg > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return DSLA_ERR_CUDA;
     const long long units = (long long)tp.p.N * tp.p.H;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(units * tp.nseg));
@@ -765,7 +771,7 @@ dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
     attr[1].val.clusterDim.x = (unsigned)tp.nseg; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = tp.nseg > 1 ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, prefill_tc_kernel, mq, mk, mv, mo, tp) != cudaSuccess) return DSLA_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, tp) != cudaSuccess) return DSLA_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DSLA_OK : DSLA_ERR_CUDA;
 }
