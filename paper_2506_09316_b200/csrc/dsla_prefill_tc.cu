@@ -90,6 +90,21 @@ __device__ __forceinline__ void issue4_ts(uint32_t d, uint32_t a, uint32_t b, ui
 // ============================================================================================
 // Main kernel
 // ============================================================================================
+// Index of the rank-th longest of up to 64 sequences, ties by index (what seq_order_kernel computes); one warp, every lane gets it.
+__device__ __forceinline__ int longest_first(const int32_t* cu, int N, int rank, int lane) {
+    int len[2], before[2] = {0, 0};
+#pragma unroll
+    for (int x = 0; x < 2; ++x) len[x] = lane + 32 * x < N ? cu[lane + 32 * x + 1] - cu[lane + 32 * x] : -1;
+#pragma unroll 1
+    for (int j = 0; j < N; ++j) {
+        const int lj = __shfl_sync(0xffffffffu, j < 32 ? len[0] : len[1], j & 31);
+#pragma unroll
+        for (int x = 0; x < 2; ++x) before[x] += (lj > len[x] || (lj == len[x] && j < lane + 32 * x)) ? 1 : 0;
+    }
+    const unsigned lo = __ballot_sync(0xffffffffu, lane < N && before[0] == rank), hi = __ballot_sync(0xffffffffu, lane + 32 < N && before[1] == rank);
+    return lo ? __ffs(lo) - 1 : 31 + __ffs(hi);
+}
+
 // SPLIT: the sequences are cut into segments (a variant of its own: with that code in it the chunk loop of whole sequences
 // ran 2 % longer).
 template <bool SPLIT>
@@ -106,7 +121,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int nseg = SPLIT ? tp.nseg : 1;
     const int g = blockIdx.x % nseg;             // rank in the cluster
     const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
-    const int n = tp.order ? tp.order[rank] : rank;
+    const int n = tp.order ? tp.order[rank] : tp.order_here ? longest_first(p.cu_seqlens, p.N, rank, lane) : rank;
     const SeqInfo sq = seq_info(p, n, g, tp);
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (tid == 0 && g == 0 && sq.nchunks > seg_begin(tp.nseg, tp.nseg, tp.cps, tp.skew8)) atomicExch(p.status, (int)DSLA_ERR_INVALID_ARG);
@@ -117,6 +132,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (int i = tid; i < (p.single ? 1 : 2) * D * D; i += NTHREADS) slot1[(size_t)(i / (D * D)) * state_stride + i % (D * D)] = 0.f;
         return;
     }
+    if (p.use_initial_state)      // 128-byte lines of both states into L2: the loads proper wait for the first chunk's gates
+        for (int i = tid; i < (p.single ? 512 : 1024); i += NTHREADS)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(slot1 + (size_t)(i >> 9) * state_stride + (size_t)(i & 511) * 32));
     const int nc = max(0, sq.c_end - sq.c_begin);  // 0: a segment behind the end of its sequence, here only for its share of the fold
     const int t0 = sq.t_begin + sq.c_begin * CM;  // first token of this segment
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
@@ -678,6 +696,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
 namespace {
 
+// Packed batches are visited longest first; up to ORDER_HERE_MAX_N sequences the main kernel of the single-CTA variant finds its place
+// in the order by itself (a kernel for it takes 3 us of a call).
 bool wants_order(const dsla_prefill_args* a) { return a->cu_seqlens != nullptr && a->N > 1 && a->N <= ORDER_MAX_N; }
 
 int sm_count() {
@@ -798,8 +818,9 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
     char* wsp = static_cast<char*>(a->workspace);
     tp.ws = tp.nseg > 1 ? reinterpret_cast<float*>(wsp) : nullptr;
     tp.order = nullptr;
+    tp.order_here = !pair && wants_order(a) && p.N <= ORDER_HERE_MAX_N;
     tp.init = nullptr;
-    if (wants_order(a)) {
+    if (wants_order(a) && !tp.order_here) {
         int* order = reinterpret_cast<int*>(wsp + summaries_bytes(a, tp.nseg));
         launch_seq_order(p.cu_seqlens, p.N, order, s);
         tp.order = order;

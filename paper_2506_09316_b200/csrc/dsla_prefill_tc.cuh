@@ -15,6 +15,7 @@ constexpr int D = 128;                // head size
 // One summary per (sequence, head, segment): U (both states, fp32 [2][D][D]) followed by the two
 // segment decays A[2], padded to a multiple of 256 bytes.
 constexpr size_t SUMMARY_STRIDE = 2 * D * D * sizeof(float) + 256;
+constexpr int ORDER_HERE_MAX_N = 64;
 constexpr int ORDER_MAX_N = 8192;     // packed batches up to this many sequences are visited longest first
 
 struct TcParams {
@@ -28,6 +29,7 @@ struct TcParams {
     int cps;            // chunks per segment (mean)
     int skew8;          // eighths of a chunk by which consecutive segments get shorter (later segments start later: they
                         // first fold the summaries of all earlier segments into their initial state)
+    int order_here;     // the main kernel finds that order by itself (few sequences)
     const int* order;   // sequences by descending length (longest first), or nullptr for index order
 };
 

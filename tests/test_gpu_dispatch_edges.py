@@ -80,3 +80,20 @@ def test_channel_prefill_tensor(lens, H, resume, pattern):
     # states: fp32 sums of exact products (three bf16 terms of an fp32 factor); outputs: one bf16 rounding (2^-9 of the value)
     assert rel_err(S[slots], S_ref[slots]) <= 1e-5
     assert rel_err(o, o_ref) <= 4e-3
+
+
+# The order in which a packed batch is visited: found inside the kernel (up to 64 sequences, one and two per lane) and by a kernel of its
+# own (more); ties and empty sequences, whole sequences and split ones
+@pytest.mark.parametrize("N,H,top", [(2, 3, 500), (31, 5, 90), (33, 4, 200), (64, 3, 70), (65, 3, 70)])
+def test_packed_order(N, H, top):
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, gpu_prefill, oracle_prefill, rel_err
+    rng = np.random.default_rng(5400 + N)
+    lens = [int(x) for x in rng.integers(0, top, N)]
+    lens[N // 2] = lens[0]
+    inp = gen.make_packed(5401 + N, lens, H, 128, BF)
+    slots = rng.permutation(N + 1)[:N].astype(np.int32)
+    state0 = gen.make_states(5402, N + 1, H, 128, 128, std=0.5).numpy()
+    o, S = gpu_prefill(inp, num_slots=N + 1, state0=state0, slots=slots, impl="tensor")
+    o_ref, S_ref = oracle_prefill(inp, state0=state0.astype(np.float64), slots=slots)
+    assert rel_err(o, o_ref) <= TOL[BF] and rel_err(S[slots], S_ref[slots]) <= TOL[BF]
