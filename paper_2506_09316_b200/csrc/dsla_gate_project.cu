@@ -46,7 +46,7 @@ gate_project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     __shared__ uint64_t full[GP_MAX_STAGES], empty[GP_MAX_STAGES], acc_full, red_full;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* tiles = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);      // (an offset, not a rounded address: the compiler still knows that it is shared memory)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = p.split, stages = p.stages;
     const int rank = split > 1 ? (int)cluster_ctarank() : 0;

@@ -39,7 +39,7 @@ prefill_tc_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     extern __shared__ uint8_t smem_raw[];
     __shared__ SumShared sh;
     const PrefillParams& p = tp.p;
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* tiles = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);      // (an offset, not a rounded address: the compiler still knows that it is shared memory)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the main grid may be scheduled as SMs become free
     const int nsum = tp.nseg - 1;

@@ -114,7 +114,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const PrefillParams& p = tp.p;
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* tiles = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);      // (an offset, not a rounded address: the compiler still knows that it is shared memory)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the launch may overlap the tail of what precedes it in the stream
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
