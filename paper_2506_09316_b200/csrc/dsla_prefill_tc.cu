@@ -140,23 +140,68 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
     const bool last = g == sq.last_seg;           // the final state is kept; other segments skip the last chunk's update
     const bool summarize = SPLIT && g < sq.last_seg;
+    const bool zero_start = !p.use_initial_state && g == 0;      // no readout of chunk 0, its update starts from zero
 
-    if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&sh.kq_full[i], 1); mbar_init(&sh.v_full[i], 1);
-            mbar_init(&sh.sb_ready[i], 4); mbar_init(&sh.vt_ready[i], 8); mbar_init(&sh.u_full[i], 1);
-            mbar_init(&sh.g_ready[i], 2); mbar_init(&sh.g_free[i], 16);
+    // Set-up: the barriers are initialised by several warps, the TMA warp starts the first loads on its own ones, the gate warps request
+    // their first gates.  (One thread for all barriers, and everything else behind it: 2200 cycles before the first load.)
+    auto load_kq = [&](int c, int q3) {
+        mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
+        tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+        tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+    };
+    auto load_v = [&](int c, int v3) {
+        mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
+        tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
+    };
+    auto load_summary = [&](int it) {      // step it = chunk nc - 1 - it
+        const int st = it % SUM_STAGES, t = t0 + (nc - 1 - it) * CM;
+        mbar_arrive_expect_tx(&sh.s_full[st], 2 * TILE_BYTES);
+        tma_load_4d(tiles + (2 * st + 1) * TILE_BYTES, &map_v, &sh.s_full[st], 0, t, 0, h);
+        tma_load_4d(tiles + 2 * st * TILE_BYTES, &map_k, &sh.s_full[st], 0, t, 0, h);
+    };
+    if (lane == 0) {
+        if (warp == WARP_TMA) {
+            for (int i = 0; i < 2; ++i) { mbar_init(&sh.kq_full[i], 1); mbar_init(&sh.v_full[i], 1); }
+            for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_full[i], 1);
+            fence_barrier_init();
+            if (summarize) {
+                for (int it = 0; it < min(nc, SUM_STAGES); ++it) load_summary(it);
+            } else if (nc > 0) {
+                load_kq(0, 0);
+                if (!SPLIT) {
+                    load_v(0, 2);
+                    if (nc > 1) load_kq(1, 1);
+                }
+            }
+        } else if (warp == 2) {
+            mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
+            mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, 16); mbar_init(&sh.s_done, 1);
+            sh.abort_flag = 0;
+            sh.slot = slot1;
+            fence_barrier_init();
+        } else if (warp == 3 || warp == 4) {
+            const int i = warp - 3;
+            mbar_init(&sh.sb_ready[i], 4); mbar_init(&sh.vt_ready[i], 8); mbar_init(&sh.u_full[i], 1); mbar_init(&sh.g_ready[i], 2); mbar_init(&sh.g_free[i], 16);
+            fence_barrier_init();
+        } else if (SPLIT && (warp == 5 || warp == 6)) {
+            const int i = warp - 5;
+            mbar_init(&sh.sw_ready[i], 2); mbar_init(&sh.sw_free[i], 8); mbar_init(&sh.svt_ready[i], 8); mbar_init(&sh.svt_free[i], 1);
+            fence_barrier_init();
+        } else if (SPLIT && warp == 7) {
+            for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_empty[i], 9);      // eight V~ warps + the MMAs on K
+            fence_barrier_init();
         }
-        mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
-        mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8);
-        mbar_init(&sh.init_done, 16);
-        for (int i = 0; i < SUM_STAGES; ++i) { mbar_init(&sh.s_full[i], 1); mbar_init(&sh.s_empty[i], 9); }      // eight V~ warps + the MMAs on K
-        for (int i = 0; i < 2; ++i) { mbar_init(&sh.sw_ready[i], 2); mbar_init(&sh.sw_free[i], 8); mbar_init(&sh.svt_ready[i], 8); mbar_init(&sh.svt_free[i], 1); }
-        mbar_init(&sh.s_done, 1);
-        sh.abort_flag = 0;
-        sh.slot = slot1;
-        fence_barrier_init();
     }
+    float nx[4];      // gate warps: the next chunk's gates, four tokens a lane
+    auto fetch = [&](int c) {      // raw values: nothing may consume them here, or the warp would sit out the load latency in every chunk
+        const float* gsrc = warp == GATE_W0 ? p.g_hist : p.g_rec;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int j = c * CM + 4 * lane + e;
+            nx[e] = load_gate(gsrc, t0 + j, p.H, h, c >= 0 && c < nc && tok0 + j < sq.len);
+        }
+    };
+    if (warp >= GATE_W0) fetch(summarize ? nc - 1 : 0);
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
     if (SPLIT) cluster_sync_all();      // (nothing is sent to a CTA that has not started)
@@ -202,9 +247,26 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     };
     // d_k rows 64 part .. 64 part + 63 of state i, one d_v lane per thread: the bf16 copy for the readout and a_0 S for the first update
     auto start_state = [&](int i, int part, uint32_t lane_addr, int v, float a) {
-        const float* src = SPLIT ? reinterpret_cast<const float*>(tiles + summary_off(i)) : sh.slot + (size_t)i * state_stride;
-        init_state_pass(src, (SPLIT && g > 0) || (p.use_initial_state && !(p.single && i == 1)), nullptr, 0, i, v, a, lane_addr + COL_S + 128 * i, lane_addr + COL_SB + 64 * i,
-                        2 * part, 2 * part + 2);
+#pragma unroll 1
+        for (int k0 = 64 * part; k0 < 64 * part + 64; k0 += 32) {
+            float x[32];
+            if (SPLIT) {
+                const float* src = reinterpret_cast<const float*>(tiles + summary_off(i)) + (size_t)k0 * D + v;
+#pragma unroll
+                for (int k = 0; k < 32; ++k) x[k] = src[(size_t)k * D];
+            } else {
+                const float* src = sh.slot + (size_t)i * state_stride + (size_t)k0 * D + v;
+#pragma unroll
+                for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0.f : src[(size_t)k * D];
+            }
+            uint32_t pk[16], sc[32];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(x[2 * k], x[2 * k + 1]);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) sc[k] = __float_as_uint(x[k] * a);
+            tmem_st16(lane_addr + COL_SB + 64 * i + k0 / 2, pk);
+            tmem_st32(lane_addr + COL_S + 128 * i + k0, sc);
+        }
         tc_wait_st();
         tc_fence_before();
         fence_proxy_async_smem();
@@ -214,37 +276,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
     if (warp == WARP_TMA) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
-        }
-        auto load_kq = [&](int c, int q3) {
-            mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
-            tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-            tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-        };
-        auto load_v = [&](int c, int v3) {
-            mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
-            tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
-        };
-        if (lane == 0) {
-            if (summarize) {      // step it = chunk nc - 1 - it
-                for (int it = 0; it < nc; ++it) {
-                    const int st = it % SUM_STAGES, t = t0 + (nc - 1 - it) * CM;
-                    if (it >= SUM_STAGES) WAIT(&sh.s_empty[st], (it / SUM_STAGES - 1) & 1);
-                    mbar_arrive_expect_tx(&sh.s_full[st], 2 * TILE_BYTES);
-                    tma_load_4d(tiles + (2 * st + 1) * TILE_BYTES, &map_v, &sh.s_full[st], 0, t, 0, h);
-                    tma_load_4d(tiles + 2 * st * TILE_BYTES, &map_k, &sh.s_full[st], 0, t, 0, h);
-                }
-                WAIT(&sh.s_done, 0);
+        if (lane == 0 && summarize) {
+            for (int it = SUM_STAGES; it < nc; ++it) {
+                WAIT(&sh.s_empty[it % SUM_STAGES], (it / SUM_STAGES - 1) & 1);
+                load_summary(it);
             }
-            if (nc > 0) load_kq(0, 0);
+            WAIT(&sh.s_done, 0);
+            load_kq(0, 0);
         }
         __syncwarp();
         if (SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         if (lane == 0 && nc > 0) {
-            if (SPLIT) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
-            load_v(0, 2);
-            if (nc > 1) load_kq(1, 1);
+            if (SPLIT) {
+                if (!zero_start) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
+                fence_proxy_async_smem();
+                load_v(0, 2);
+                if (nc > 1) load_kq(1, 1);
+            }
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
             int c3 = 0;
 #pragma unroll 1
@@ -326,8 +374,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 const int v3 = c3 == 0 ? 2 : c3 - 1, n3 = c3 == 2 ? 0 : c3 + 1;
                 WAIT(&sh.v_full[c & 1], (c >> 1) & 1);
                 WAIT(&sh.prep_ready, c & 1);               // P read out of TMEM, P~, Q~1, Q~2 in place
+                const bool first = zero_start && c == 0;   // nothing to read out, nothing to add to
+                if (first) tc_fence_after();
 #pragma unroll 1
-                for (int i = 0; i < 2; ++i) {
+                for (int i = first ? 2 : 0; i < 2; ++i) {
                     WAIT(&sh.sb_ready[i], c & 1);
                     tc_fence_after();
                     const uint32_t a = COL_SB + 64 * i, b = i == 0 ? dq0 + (uint32_t)c3 * T_STEP : dq2;
@@ -336,7 +386,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
                 tc_commit(&sh.ro_done);
                 const uint32_t v = dv0 + (uint32_t)v3 * T_STEP;
-                issue4_ss<128, 2>(COL_R, v, dp0, ID_V128, 1u);
+                issue4_ss<128, 2>(COL_R, v, dp0, ID_V128, first ? 0u : 1u);
                 issue4_ss<128, 2>(COL_R + 64, v + 512, dp0 + H_STEP, ID_V64, 1u);     // keys 64..127 reach only the outputs of tokens 64..127
                 tc_commit(&sh.o_full);
                 const bool update = last || c + 1 < nc;
@@ -346,7 +396,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     if (update) {
                         WAIT(&sh.vt_ready[i], c & 1);
                         tc_fence_after();
-                        issue4_ts<128>(COL_S + 128 * i, COL_SB + 64 * i, bk, ID_U, 1u);
+                        issue4_ts<128>(COL_S + 128 * i, COL_SB + 64 * i, bk, ID_U, first ? 0u : 1u);
                         issue4_ts<128>(COL_S + 128 * i, COL_SB + 64 * i + 32, bk + 512, ID_U, 1u);
                         tc_commit(&sh.u_full[i]);
                     }
@@ -369,7 +419,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
 
         if (SPLIT) initial_state_from_cluster(tid - TILE_W0 * 32);
-        if (nc > 0) {
+        if (nc > 0 && !zero_start) {
             WAIT(&sh.g_ready[0], 0);
             start_state(half, 1, lane_addr, j, sh.gs[0].a[half]);
         }
@@ -456,7 +506,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // through independent exponentials.  Lane l holds tokens 4 l .. 4 l + 3.  The chunk decay that carries the state
         // is the plain product of the gates.
         const int i = warp - GATE_W0;
-        const float* gsrc = i == 0 ? p.g_hist : p.g_rec;
         const float Wi = (p.weights ? (i == 1 && p.single ? 0.f : p.weights[(size_t)h * p.n_total + p.state_first + i])
                                     : (i == 0 ? p.gamma[h] : 1.f - p.gamma[h])) * p.scale;
         auto decays = [&](const float (&x)[4], float (&L)[4], float& pr, float& incl) {      // L: inclusive from the chunk start; incl: of the lane's last token
@@ -477,17 +526,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) pr *= __shfl_xor_sync(0xffffffffu, pr, off);
         };
-        float nx[4];
-        auto fetch = [&](int c) {      // raw values: nothing may consume them here, or the warp would sit out the load latency in every chunk
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = c * CM + 4 * lane + e;
-                nx[e] = load_gate(gsrc, t0 + j, p.H, h, c >= 0 && c < nc && tok0 + j < sq.len);
-            }
-        };
         if (summarize) {      // weights to the end of the segment, chunks from the last to the first
             float after = 0.f, A = 1.f;      // log2 and product of the gates of all later chunks
-            fetch(nc - 1);
             for (int it = 0; it < nc; ++it) {
                 const int b = it & 1;
                 const float x[4] = {nx[0], nx[1], nx[2], nx[3]};
@@ -505,8 +545,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             if (lane < nseg) st_cluster_f32(map_to_cta(smem_u32(&sh.a_seg[g][i]), (uint32_t)lane), A);      // to every CTA of the cluster
             for (int it = max(0, nc - 2); it < nc; ++it) WAIT(&sh.sw_free[it & 1], (it >> 1) & 1);      // the ring is reused for the chunks below
+            fetch(0);
         }
-        fetch(0);
         if (nc == 0 && SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         for (int c = 0; c < nc; ++c) {
             const int s = c & 1;
@@ -586,7 +626,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             WAIT(&sh.s_done, 0);
             tc_fence_after();
-            store_state(reinterpret_cast<float*>(tiles + summary_off(hi)), v, s_addr, 0, 4);
+#pragma unroll 1
+            for (int k0 = 0; k0 < D; k0 += 32) {
+                uint32_t r[32];
+                tmem_ld32(s_addr + k0, r);
+                float* dst = reinterpret_cast<float*>(tiles + summary_off(hi)) + (size_t)k0 * D + v;
+                tc_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 32; ++k) dst[(size_t)k * D] = __uint_as_float(r[k]);
+            }
         }
         if (SPLIT) initial_state_from_cluster(256 + tid - STATE_W0 * 32);
         int v3 = 2;
@@ -597,8 +645,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
             const float a = gs.a[hi];
             if (c == 0) {
-                start_state(hi, 0, lane_addr, v, a);
-                WAIT(&sh.init_done, 0);     // the tile warps' half
+                if (!zero_start) {
+                    start_state(hi, 0, lane_addr, v, a);
+                    WAIT(&sh.init_done, 0);     // the tile warps' half
+                }
             } else {
                 WAIT(&sh.u_full[hi], (c - 1) & 1);
                 tc_fence_after();
