@@ -17,10 +17,12 @@
 // operands, and Q the only tile that is copied.
 //
 // A sequence may be split into segments along T so that few (sequence, head) pairs still fill the GPU.  The segments of a
-// sequence are the CTAs of a thread-block cluster: each first accumulates the state its own tokens leave behind, from
-// zero (its summary), the initial states are folded out of the summaries through distributed shared memory, then each runs
-// its chunks.  (As a kernel of its own the summaries took 21 of 68 us at T = 4096, 32 heads: launch, fill and drain of a second
-// pipeline, and 131 KB per segment through global memory and back.)
+// sequence are the CTAs of a thread-block cluster: each first accumulates the state its own tokens leave behind, from zero (its
+// summary U, with the product A of its gates), then the initial states travel down the cluster, S <- A S + U, in
+// pieces, and each segment runs its chunks.  (As a kernel of its own the summaries took 21 of 68 us at T = 4096, 32 heads: launch,
+// fill and drain of a second pipeline.  Stores into another CTA's shared memory ran at 26 bytes a cycle, loads from it at 12:
+// hence a chain that only stores.  Three hops of 128 KB cost 9 k cycles, a fold in which every CTA loads its share of all
+// summaries and stores it back took 16 k.)
 // Packed batches are visited longest sequence first.  This file also holds the host side of both tensor-core variants (segment
 // plan, workspace layout, launches).
 #include <atomic>
@@ -51,9 +53,9 @@ constexpr uint32_t COL_S = 0;      // fp32 S1^T [0,128), S2^T [128,256)
 constexpr uint32_t COL_SB = 256;   // per state 64 columns: the bf16 copy of S^T (readout), then the weighted V~^T (update)
 constexpr uint32_t COL_R = 384;    // P (scores, tokens x tokens), then O^T (d_v x tokens): 128 columns
 
-// Where the summaries of the two states (fp32 [d_k][d_v], 64 KB each) wait for the fold, and the initial states for their owner: slots
-// that the first chunk's Q and K do not land in.
-__device__ constexpr int summary_off(int i) { return i == 0 ? TILE_BYTES : OFF_K + TILE_BYTES; }
+// Where the initial states of a segment arrive (64 KB each, [d_k / 4][d_v] pieces of four d_k): slots that the first chunk's Q and K do not
+// land in.
+__device__ constexpr int initial_off(int i) { return i == 0 ? TILE_BYTES : OFF_K + TILE_BYTES; }
 constexpr int SUM_STAGES = 3;        // K and V tiles of the summaries: two slots each, in order
 
 // Per-token terms of one chunk; the first index is the state.
@@ -68,11 +70,12 @@ struct alignas(16) GateSmem {
 struct alignas(16) Shared {
     uint64_t kq_full[2], v_full[2], p_full, prep_ready, sb_ready[2], ro_done, vt_ready[2], o_full, o_free, o_staged, u_full[2], g_ready[2], g_free[2], init_done;
     uint64_t s_full[SUM_STAGES], s_empty[SUM_STAGES], sw_ready[2], sw_free[2], svt_ready[2], svt_free[2], s_done;      // summaries
+    uint64_t s_in[8][4], next_ready;      // initial state: a piece has arrived, the next segment has room for its own
     uint32_t tmem_base;
     int abort_flag;
     float* slot;                          // the first state of this (sequence, head) in its slot: read where it is needed, not kept in registers
     GateSmem gs[2];
-    float a_seg[16][2];                   // products of the gates of every segment of the cluster
+    float a_seg[2];                       // products of the segment's gates
 };
 
 // Four MMAs whose operands advance by a constant.
@@ -175,7 +178,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
         } else if (warp == 2) {
             mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
-            mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, 16); mbar_init(&sh.s_done, 1);
+            mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, SPLIT ? 8 : 16); mbar_init(&sh.s_done, 1);
+            mbar_init(&sh.next_ready, 8);
             sh.abort_flag = 0;
             sh.slot = slot1;
             fence_barrier_init();
@@ -190,6 +194,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         } else if (SPLIT && warp == 7) {
             for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_empty[i], 9);      // eight V~ warps + the MMAs on K
             fence_barrier_init();
+        } else if (SPLIT && warp >= STATE_W0 && warp < GATE_W0) {
+            for (int i = 0; i < 4; ++i) mbar_init(&sh.s_in[warp - STATE_W0][i], 1);
+            fence_barrier_init();
+            if (g > 0 && nc > 0)
+                for (int i = 0; i < 4; ++i) mbar_arrive_expect_tx(&sh.s_in[warp - STATE_W0][i], 32 * 128);      // 32 d_k x 32 d_v
         }
     }
     float nx[4];      // gate warps: the next chunk's gates, four tokens a lane
@@ -204,61 +213,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (warp >= GATE_W0) fetch(summarize ? nc - 1 : 0);
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
-    if (SPLIT) cluster_sync_all();      // (nothing is sent to a CTA that has not started)
-    else __syncthreads();
+    __syncwarp();
+    if (SPLIT) cluster_arrive_relaxed();      // (waited for before the first use of another CTA's barriers)
+    __syncthreads();
     tc_fence_after();
     const uint32_t tb = 0;      // all 512 columns are allocated: the base is column 0
     volatile int* abortp = &sh.abort_flag;
 #define WAIT(bar, ph) mbar_wait(bar, (uint32_t)(ph), abortp, p.status)
 
-    // Tile and state warps (t = 0..511): the slot (or zero) pushed through the summaries of the earlier segments.  Each CTA does this
-    // for its share of the elements and for every segment: it reads the share out of all summaries and writes the initial
-    // states over them, so that every CTA moves 1 / nseg of what a fold per segment would pull from the first ones.
-    auto initial_state_from_cluster = [&](int t) {
-        __syncwarp();
-        cluster_sync_all();       // the summaries are in place
-        const int nsum = sq.last_seg, begin = g * 8192 / nseg, end = (g + 1) * 8192 / nseg;      // 16-byte pieces of [2][D][D]
-#pragma unroll 2
-        for (int f = begin + t; f < end; f += 512) {
-            const int i = f >> 12, e = f & 4095;
-            const uint32_t at = smem_u32(tiles + summary_off(i) + e * 16);
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p.use_initial_state && !(p.single && i == 1)) x = *reinterpret_cast<const float4*>(sh.slot + (size_t)i * state_stride + (size_t)e * 4);
-#pragma unroll 1
-            for (int s0 = 0; s0 <= nsum; s0 += 3) {      // three segments' loads in flight
-                float4 u[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-                    if (s0 + k < nsum) u[k] = ld_cluster_f32x4(map_to_cta(at, (uint32_t)(s0 + k)));
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int r = s0 + k;
-                    if (r > nsum) break;
-                    if (r > 0 || p.use_initial_state) st_cluster_f32x4(map_to_cta(at, (uint32_t)r), x.x, x.y, x.z, x.w);
-                    if (r < nsum) {
-                        const float a = sh.a_seg[r][i];
-                        x.x = fmaf(a, x.x, u[k].x); x.y = fmaf(a, x.y, u[k].y); x.z = fmaf(a, x.z, u[k].z); x.w = fmaf(a, x.w, u[k].w);
-                    }
-                }
-            }
-        }
-        __syncwarp();
-        cluster_sync_all();       // the initial states are in place; every read of the slot is done
-    };
-    // d_k rows 64 part .. 64 part + 63 of state i, one d_v lane per thread: the bf16 copy for the readout and a_0 S for the first update
+    // Whole sequences: d_k rows 64 part .. 64 part + 63 of state i from the slot, one d_v lane per thread: the bf16 copy for the readout and
+    // a_0 S for the first update.
     auto start_state = [&](int i, int part, uint32_t lane_addr, int v, float a) {
 #pragma unroll 1
         for (int k0 = 64 * part; k0 < 64 * part + 64; k0 += 32) {
             float x[32];
-            if (SPLIT) {
-                const float* src = reinterpret_cast<const float*>(tiles + summary_off(i)) + (size_t)k0 * D + v;
+            const float* src = sh.slot + (size_t)i * state_stride + (size_t)k0 * D + v;
 #pragma unroll
-                for (int k = 0; k < 32; ++k) x[k] = src[(size_t)k * D];
-            } else {
-                const float* src = sh.slot + (size_t)i * state_stride + (size_t)k0 * D + v;
-#pragma unroll
-                for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0.f : src[(size_t)k * D];
-            }
+            for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0.f : src[(size_t)k * D];
             uint32_t pk[16], sc[32];
 #pragma unroll
             for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(x[2 * k], x[2 * k + 1]);
@@ -269,7 +240,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         tc_wait_st();
         tc_fence_before();
-        fence_proxy_async_smem();
         __syncwarp();
         if ((threadIdx.x & 31) == 0) mbar_arrive(&sh.init_done);
     };
@@ -284,12 +254,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             WAIT(&sh.s_done, 0);
             load_kq(0, 0);
         }
-        __syncwarp();
-        if (SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         if (lane == 0 && nc > 0) {
             if (SPLIT) {
-                if (!zero_start) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
-                fence_proxy_async_smem();
+                if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
                 load_v(0, 2);
                 if (nc > 1) load_kq(1, 1);
             }
@@ -366,7 +333,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (nc > 0) scores(0, 0);
         }
         __syncwarp();
-        if (SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         if (elect_one()) {
             int c3 = 0;
 #pragma unroll 1
@@ -418,8 +384,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first] : p.gamma[h]) * p.scale;
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
 
-        if (SPLIT) initial_state_from_cluster(tid - TILE_W0 * 32);
-        if (nc > 0 && !zero_start) {
+        if (!SPLIT && !zero_start) {
             WAIT(&sh.g_ready[0], 0);
             start_state(half, 1, lane_addr, j, sh.gs[0].a[half]);
         }
@@ -440,6 +405,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // ---- scaled copies of Q, eight 16-byte pieces per thread.  The copy for state 2 is written as soon as the readout of the
             // previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
             if (c > 0) WAIT(&sh.ro_done, (c - 1) & 1);
+            else if (SPLIT && g > 0 && c == 0) WAIT(&sh.init_done, 0);      // (the initial state arrives where Q~2 goes)
             uint4 q1[8];
 #pragma unroll
             for (int m = 0; m < 8; ++m) q1[m] = reinterpret_cast<const uint4*>(qs)[tt + 256 * m];
@@ -543,11 +509,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sh.sw_ready[b]);
             }
-            if (lane < nseg) st_cluster_f32(map_to_cta(smem_u32(&sh.a_seg[g][i]), (uint32_t)lane), A);      // to every CTA of the cluster
+            if (lane == 0) sh.a_seg[i] = A;
             for (int it = max(0, nc - 2); it < nc; ++it) WAIT(&sh.sw_free[it & 1], (it >> 1) & 1);      // the ring is reused for the chunks below
             fetch(0);
         }
-        if (nc == 0 && SPLIT) { cluster_sync_all(); cluster_sync_all(); }
         for (int c = 0; c < nc; ++c) {
             const int s = c & 1;
             GateSmem& gs = sh.gs[s];
@@ -572,7 +537,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0) gs.a[i] = pr;
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.g_ready[s]);
-            if (c == 0 && SPLIT) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }
         }
     } else {
         // ------------------------------------------------------------------ state warps 10..17
@@ -626,17 +590,60 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             WAIT(&sh.s_done, 0);
             tc_fence_after();
-#pragma unroll 1
-            for (int k0 = 0; k0 < D; k0 += 32) {
-                uint32_t r[32];
-                tmem_ld32(s_addr + k0, r);
-                float* dst = reinterpret_cast<float*>(tiles + summary_off(hi)) + (size_t)k0 * D + v;
-                tc_wait_ld();
-#pragma unroll
-                for (int k = 0; k < 32; ++k) dst[(size_t)k * D] = __uint_as_float(r[k]);
-            }
         }
-        if (SPLIT) initial_state_from_cluster(256 + tid - STATE_W0 * 32);
+        // Initial state of this warp's state and d_v lanes, in pieces of 32 d_k: from the slot (or zero) in the first segment, else from the
+        // same warp of the segment before; what the next segment starts from goes to the same warp there.
+        auto chain = [&](float a) {
+            const float A = sh.a_seg[hi];
+            const uint32_t mine = (uint32_t)(initial_off(hi) + v * 16), w = warp - STATE_W0;
+            const uint32_t next = map_to_cta(smem_u32(tiles + mine), (uint32_t)(g + 1 < nseg ? g + 1 : g));
+            const uint32_t next_bar = map_to_cta(smem_u32(&sh.s_in[w][0]), (uint32_t)(g + 1 < nseg ? g + 1 : g));
+            if (summarize) mbar_wait_cluster(&sh.next_ready, 0, abortp, p.status);
+#pragma unroll 1
+            for (int b = 0; b < 8; ++b) {      // 16 d_k at a time, handed over in pairs
+                uint32_t u[16];
+                float x[16];
+                if (summarize) tmem_ld16(s_addr + 16 * b, u);
+                if (g > 0) {
+                    if ((b & 1) == 0) mbar_wait_cluster(&sh.s_in[w][b >> 1], 0, abortp, p.status);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float4 y = *reinterpret_cast<const float4*>(tiles + mine + (4 * b + k) * (D * 16));
+                        x[4 * k] = y.x; x[4 * k + 1] = y.y; x[4 * k + 2] = y.z; x[4 * k + 3] = y.w;
+                    }
+                } else {
+                    const float* src = sh.slot + (size_t)hi * state_stride + (size_t)(16 * b) * D + v;
+                    const bool load = p.use_initial_state && !(p.single && hi == 1);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) x[k] = load ? src[(size_t)k * D] : 0.f;
+                }
+                if (summarize) {
+                    tc_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        st_async_f32x4(next + (uint32_t)((4 * b + k) * (D * 16)), fmaf(A, x[4 * k], __uint_as_float(u[4 * k])), fmaf(A, x[4 * k + 1], __uint_as_float(u[4 * k + 1])),
+                                       fmaf(A, x[4 * k + 2], __uint_as_float(u[4 * k + 2])), fmaf(A, x[4 * k + 3], __uint_as_float(u[4 * k + 3])), next_bar + 8u * (b >> 1));
+                }
+                if (!zero_start) {
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) pk[k] = pack_bf16(x[2 * k], x[2 * k + 1]);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) u[k] = __float_as_uint(x[k] * a);
+                    tmem_st8(sb_addr + 8 * b, pk);
+                    tmem_st16(s_addr + 16 * b, u);
+                }
+            }
+            tc_wait_st();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.init_done);
+        };
+        if (SPLIT) {
+            __syncwarp();
+            cluster_wait();
+            if (g > 0 && nc > 0 && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.next_ready), (uint32_t)(g - 1)));      // room for this segment's initial state
+        }
         int v3 = 2;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
@@ -645,7 +652,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
             const float a = gs.a[hi];
             if (c == 0) {
-                if (!zero_start) {
+                if (SPLIT) {
+                    chain(a);
+                } else if (!zero_start) {
                     start_state(hi, 0, lane_addr, v, a);
                     WAIT(&sh.init_done, 0);     // the tile warps' half
                 }
@@ -736,6 +745,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!(p.single && hi == 1)) store_state(sh.slot + (size_t)hi * state_stride, v, s_addr, 0, 4);
         }
     }
+    __syncwarp();
+    if (SPLIT && !(warp >= STATE_W0 && warp < GATE_W0)) cluster_wait();
     tc_fence_before();
     __syncthreads();
     if (warp == WARP_MMA) tmem_dealloc(tb, 512);

@@ -117,6 +117,10 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The two halves of it; every thread of the cluster executes both.  Relaxed: what others may use after it has to be published by a fence
+// (initialised mbarriers: fence_barrier_init).
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of the same shared-memory location in the CTA of the given rank (shared::cluster window).
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
     uint32_t r;
@@ -133,7 +137,6 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t caddr) {
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(caddr) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t caddr, float a) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(caddr), "f"(a) : "memory"); }
 __device__ __forceinline__ void st_cluster_f32x4(uint32_t caddr, float a, float b, float c, float d) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(caddr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
@@ -334,6 +337,9 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&v)[4]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%4], {%0,%1,%2,%3};" ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(taddr)
                  : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::DSLA_W8(v, 0), "r"(taddr) : "memory");
 }
 // 16 lanes x 32 columns in the 16x256b distribution (the accumulator layout of mma fragments): for each group i of 8
 // columns, thread t receives columns 8 i + 2 (t % 4) and + 1 of lane t / 4 (v[4 i], v[4 i + 1]) and of lane t / 4 + 8
