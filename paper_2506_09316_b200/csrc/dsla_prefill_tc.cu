@@ -93,19 +93,35 @@ __device__ __forceinline__ void issue4_ts(uint32_t d, uint32_t a, uint32_t b, ui
 // ============================================================================================
 // Main kernel
 // ============================================================================================
-// Index of the rank-th longest of up to 64 sequences, ties by index (what seq_order_kernel computes); one warp, every lane gets it.
-__device__ __forceinline__ int longest_first(const int32_t* cu, int N, int rank, int lane) {
-    int len[2], before[2] = {0, 0};
+// The rank-th longest of up to 64 sequences, ties by index (the order of seq_order_kernel); one warp, every lane gets the result.
+// The slots are read along with the lengths.
+struct SeqPlace {
+    int n, t_begin, t_end, slot;
+};
+__device__ __forceinline__ SeqPlace longest_first(const PrefillParams& p, int rank, int lane) {
+    int begin[2], end[2], slot[2], before[2] = {0, 0};
 #pragma unroll
-    for (int x = 0; x < 2; ++x) len[x] = lane + 32 * x < N ? cu[lane + 32 * x + 1] - cu[lane + 32 * x] : -1;
-#pragma unroll 1
-    for (int j = 0; j < N; ++j) {
-        const int lj = __shfl_sync(0xffffffffu, j < 32 ? len[0] : len[1], j & 31);
-#pragma unroll
-        for (int x = 0; x < 2; ++x) before[x] += (lj > len[x] || (lj == len[x] && j < lane + 32 * x)) ? 1 : 0;
+    for (int x = 0; x < 2; ++x) {
+        const int i = lane + 32 * x;
+        begin[x] = i < p.N ? p.cu_seqlens[i] : 0;
+        end[x] = i < p.N ? p.cu_seqlens[i + 1] : -1;
+        slot[x] = i < p.N && p.slots ? p.slots[i] : i;
     }
-    const unsigned lo = __ballot_sync(0xffffffffu, lane < N && before[0] == rank), hi = __ballot_sync(0xffffffffu, lane + 32 < N && before[1] == rank);
-    return lo ? __ffs(lo) - 1 : 31 + __ffs(hi);
+    const int len0 = end[0] - begin[0], len1 = end[1] - begin[1];
+#pragma unroll 1
+    for (int j = 0; j < p.N; ++j) {
+        const int lj = __shfl_sync(0xffffffffu, j < 32 ? len0 : len1, j & 31);
+        before[0] += (lj > len0 || (lj == len0 && j < lane)) ? 1 : 0;
+        before[1] += (lj > len1 || (lj == len1 && j < lane + 32)) ? 1 : 0;
+    }
+    const unsigned lo = __ballot_sync(0xffffffffu, lane < p.N && before[0] == rank), hi = __ballot_sync(0xffffffffu, lane + 32 < p.N && before[1] == rank);
+    const int from = lo ? __ffs(lo) - 1 : __ffs(hi) - 1;
+    SeqPlace r;
+    r.n = lo ? from : from + 32;
+    r.t_begin = __shfl_sync(0xffffffffu, lo ? begin[0] : begin[1], from);
+    r.t_end = __shfl_sync(0xffffffffu, lo ? end[0] : end[1], from);
+    r.slot = __shfl_sync(0xffffffffu, lo ? slot[0] : slot[1], from);
+    return r;
 }
 
 // SPLIT: the sequences are cut into segments (a variant of its own: with that code in it the chunk loop of whole sequences
@@ -124,8 +140,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int nseg = SPLIT ? tp.nseg : 1;
     const int g = blockIdx.x % nseg;             // rank in the cluster
     const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
-    const int n = tp.order ? tp.order[rank] : tp.order_here ? longest_first(p.cu_seqlens, p.N, rank, lane) : rank;
-    const SeqInfo sq = seq_info(p, n, g, tp);
+    SeqInfo sq;
+    if (tp.order_here) {
+        const SeqPlace at = longest_first(p, rank, lane);
+        sq = seq_info_at(at.t_begin, at.t_end, at.slot, g, tp);
+    } else {
+        sq = seq_info(p, tp.order ? tp.order[rank] : rank, g, tp);
+    }
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (tid == 0 && g == 0 && sq.nchunks > seg_begin(tp.nseg, tp.nseg, tp.cps, tp.skew8)) atomicExch(p.status, (int)DSLA_ERR_INVALID_ARG);
     float* slot1 = p.state + (((size_t)sq.slot * p.n_total + p.state_first) * p.H + h) * (size_t)(D * D);
@@ -135,9 +156,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (int i = tid; i < (p.single ? 1 : 2) * D * D; i += NTHREADS) slot1[(size_t)(i / (D * D)) * state_stride + i % (D * D)] = 0.f;
         return;
     }
-    if (p.use_initial_state)      // 128-byte lines of both states into L2: the loads proper wait for the first chunk's gates
-        for (int i = tid; i < (p.single ? 512 : 1024); i += NTHREADS)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(slot1 + (size_t)(i >> 9) * state_stride + (size_t)(i & 511) * 32));
     const int nc = max(0, sq.c_end - sq.c_begin);  // 0: a segment behind the end of its sequence, here only for its share of the fold
     const int t0 = sq.t_begin + sq.c_begin * CM;  // first token of this segment
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
@@ -201,6 +219,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int i = 0; i < 4; ++i) mbar_arrive_expect_tx(&sh.s_in[warp - STATE_W0][i], 32 * 128);      // 32 d_k x 32 d_v
         }
     }
+    if (p.use_initial_state && warp >= TILE_W0 && warp < GATE_W0)      // 128-byte lines of both states into L2
+        for (int i = tid - TILE_W0 * 32; i < (p.single ? 512 : 1024); i += 512)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(slot1 + (size_t)(i >> 9) * state_stride + (size_t)(i & 511) * 32));
     float nx[4];      // gate warps: the next chunk's gates, four tokens a lane
     auto fetch = [&](int c) {      // raw values: nothing may consume them here, or the warp would sit out the load latency in every chunk
         const float* gsrc = warp == GATE_W0 ? p.g_hist : p.g_rec;
@@ -221,22 +242,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     volatile int* abortp = &sh.abort_flag;
 #define WAIT(bar, ph) mbar_wait(bar, (uint32_t)(ph), abortp, p.status)
 
-    // Whole sequences: d_k rows 64 part .. 64 part + 63 of state i from the slot, one d_v lane per thread: the bf16 copy for the readout and
-    // a_0 S for the first update.
-    auto start_state = [&](int i, int part, uint32_t lane_addr, int v, float a) {
+    // Whole sequences: d_k rows 64 part .. 64 part + 63 of state i from the slot, one d_v lane per thread, while the first gates are on
+    // their way.
+    auto start_state = [&](int i, int part, uint32_t lane_addr, int v) {
 #pragma unroll 1
         for (int k0 = 64 * part; k0 < 64 * part + 64; k0 += 32) {
-            float x[32];
+            uint32_t x[32];
             const float* src = sh.slot + (size_t)i * state_stride + (size_t)k0 * D + v;
 #pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0.f : src[(size_t)k * D];
-            uint32_t pk[16], sc[32];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(x[2 * k], x[2 * k + 1]);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) sc[k] = __float_as_uint(x[k] * a);
-            tmem_st16(lane_addr + COL_SB + 64 * i + k0 / 2, pk);
-            tmem_st32(lane_addr + COL_S + 128 * i + k0, sc);
+            for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0u : __float_as_uint(src[(size_t)k * D]);
+            tmem_st32(lane_addr + COL_S + 128 * i + k0, x);
         }
         tc_wait_st();
         tc_fence_before();
@@ -384,10 +399,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first] : p.gamma[h]) * p.scale;
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
 
-        if (!SPLIT && !zero_start) {
-            WAIT(&sh.g_ready[0], 0);
-            start_state(half, 1, lane_addr, j, sh.gs[0].a[half]);
-        }
+        if (!SPLIT && !zero_start) start_state(half, 1, lane_addr, j);
         // The ten 32 x 32 blocks of the lower triangle: a quadrant's q + 1 blocks are split between its two warps (the second one
         // has the diagonal block).  The two blocks above the diagonal that the MMAs read are zeroed once.
         const int blk0 = half == 0 ? 0 : (q == 1 ? 1 : 2), nblk = q == 0 ? 1 - half : (q == 3 || (q == 2 && half == 0)) ? 2 : 1;
@@ -644,6 +656,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             cluster_wait();
             if (g > 0 && nc > 0 && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.next_ready), (uint32_t)(g - 1)));      // room for this segment's initial state
         }
+        if (!SPLIT && !zero_start) {
+            start_state(hi, 0, lane_addr, v);
+            WAIT(&sh.init_done, 0);     // the tile warps' half
+        }
         int v3 = 2;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
@@ -651,15 +667,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const GateSmem& gs = sh.gs[s];
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
             const float a = gs.a[hi];
-            if (c == 0) {
-                if (SPLIT) {
-                    chain(a);
-                } else if (!zero_start) {
-                    start_state(hi, 0, lane_addr, v, a);
-                    WAIT(&sh.init_done, 0);     // the tile warps' half
-                }
-            } else {
-                WAIT(&sh.u_full[hi], (c - 1) & 1);
+            if (SPLIT && c == 0) {
+                chain(a);
+            } else if (c > 0 || !zero_start) {
+                if (c > 0) WAIT(&sh.u_full[hi], (c - 1) & 1);
                 tc_fence_after();
                 // ---- one pass over the state (TMEM -> registers once): the bf16 copy of S_{c-1} that the readout of chunk c
                 // multiplies, and a_c S_{c-1} in place, onto which the update MMA of chunk c accumulates

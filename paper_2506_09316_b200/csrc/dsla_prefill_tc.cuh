@@ -65,13 +65,12 @@ struct SeqInfo {
 // chunks longer than the mean.  seg_begin(0) = 0 and seg_begin(nseg) = nseg cps.
 __host__ __device__ __forceinline__ int seg_begin(int g, int nseg, int cps, int skew8) { return g * cps + (skew8 * g * (nseg - g)) / 8; }
 
-__device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g, const TcParams& tp) {
+__device__ __forceinline__ SeqInfo seq_info_at(int t_begin, int t_end, int slot, int g, const TcParams& tp) {
     const int nseg = tp.nseg, cps = tp.cps, skew8 = tp.skew8;
     SeqInfo s;
-    s.t_begin = p.cu_seqlens ? p.cu_seqlens[n] : n * p.T;
-    const int t_end = p.cu_seqlens ? p.cu_seqlens[n + 1] : (n + 1) * p.T;
-    s.len = t_end - s.t_begin;
-    s.slot = p.slots ? p.slots[n] : n;
+    s.t_begin = t_begin;
+    s.len = t_end - t_begin;
+    s.slot = slot;
     s.nchunks = (s.len + tp.chunk - 1) / tp.chunk;
     s.c_begin = seg_begin(g, nseg, cps, skew8);
     s.c_end = min(s.nchunks, seg_begin(g + 1, nseg, cps, skew8));
@@ -79,6 +78,9 @@ __device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g
     for (int j = 1; j < nseg; ++j)
         if (seg_begin(j, nseg, cps, skew8) < s.nchunks) s.last_seg = j;
     return s;
+}
+__device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g, const TcParams& tp) {
+    return seq_info_at(p.cu_seqlens ? p.cu_seqlens[n] : n * p.T, p.cu_seqlens ? p.cu_seqlens[n + 1] : (n + 1) * p.T, p.slots ? p.slots[n] : n, g, tp);
 }
 
 // Initial state of a segment (cold path, kept out of line so the chunk loop stays small): the slot
