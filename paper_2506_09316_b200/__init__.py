@@ -15,6 +15,8 @@ def __getattr__(name):
         return importlib.import_module(f"{__name__}.{name}")
     b = importlib.import_module(f"{__name__}.binding")
     try:
-        return getattr(b, name)
+        value = getattr(b, name)
     except AttributeError:
         raise AttributeError(f"module {__name__!r} has no attribute {name!r}") from None
+    globals()[name] = value     # found without this function from now on (it costs more than the rest of a call's Python)
+    return value

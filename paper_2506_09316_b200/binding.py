@@ -225,8 +225,8 @@ def dsla_selftest_bounded_wait(st: DslaState, max_polls: int = 2000, stream=None
     _check(_lib.dsla_selftest_bounded_wait(st.handle, int(max_polls), _stream(stream)), "dsla_selftest_bounded_wait")
 
 
-def _stream_or_none(stream):
-    return stream if stream is None else stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+def _raw_stream(stream):
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _sequences(T_total, cu_seqlens, max_seqlen):
@@ -288,7 +288,7 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
     _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, int(max_seqlen), int(chunk),
                            scale, 1 if use_initial_state else 0, _IMPLS[impl] if isinstance(impl, str) else int(impl),
-                           _stream_or_none(stream)), "dsla_prefill")
+                           None if stream is None else _raw_stream(stream)), "dsla_prefill")
     return o
 
 
@@ -334,8 +334,9 @@ def dsla_decode_step(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, sl
     [B, H, d] per key channel.  ``row_mask`` (uint8 [B]): rows with 0 are not touched (state and o)."""
     if o is None:
         o = torch.empty_like(v)
-    _check(_native.decode_step(q, k, v, o, g_hist, g_rec, gamma, slots, row_mask, st.address, scale, _stream_or_none(stream)),
-           "dsla_decode_step")
+    rc = _native.decode_step(q, k, v, o, g_hist, g_rec, gamma, slots, row_mask, st.address, scale, None if stream is None else _raw_stream(stream))
+    if rc:
+        _check(rc, "dsla_decode_step")
     return o
 
 
@@ -389,7 +390,7 @@ def dsla_nstate_decode_step(q, k, v, gates, weights, st: DslaState, *, o=None, s
     """n-state decode step: gates [n, B, H] (or [n, B, H, d] per key channel) fp32, weights [H, n] fp32."""
     if o is None:
         o = torch.empty_like(v)
-    _check(_native.nstate_decode_step(q, k, v, o, gates, weights, slots, row_mask, st.address, scale, _stream_or_none(stream)),
+    _check(_native.nstate_decode_step(q, k, v, o, gates, weights, slots, row_mask, st.address, scale, None if stream is None else _raw_stream(stream)),
            "dsla_nstate_decode_step")
     return o
 
@@ -440,7 +441,7 @@ def dsla_nstate_prefill(q, k, v, gates, weights, st: DslaState, *, o=None, cu_se
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
     _check(_native.nstate_prefill(q, k, v, o, gates, weights, cu_seqlens, slots, workspace, st.address, N, T, int(longest), scale,
-                                  1 if use_initial_state else 0, _IMPLS[impl], _stream_or_none(stream)), "dsla_nstate_prefill")
+                                  1 if use_initial_state else 0, _IMPLS[impl], None if stream is None else _raw_stream(stream)), "dsla_nstate_prefill")
     return o
 
 
@@ -451,7 +452,7 @@ def dsla_gate_project(x, w, bias=None, *, g_hist=None, g_rec=None, stream=None):
         g_hist = torch.empty((x.shape[0], w.shape[0] // 2), dtype=torch.float32, device=x.device)
     if g_rec is None:
         g_rec = torch.empty((x.shape[0], w.shape[0] // 2), dtype=torch.float32, device=x.device)
-    _check(_native.gate_project(x, w, bias, g_hist, g_rec, _stream_or_none(stream)), "dsla_gate_project")
+    _check(_native.gate_project(x, w, bias, g_hist, g_rec, None if stream is None else _raw_stream(stream)), "dsla_gate_project")
     return g_hist, g_rec
 
 
