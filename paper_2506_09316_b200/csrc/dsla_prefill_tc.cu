@@ -135,8 +135,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const PrefillParams& p = tp.p;
     uint8_t* tiles = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);      // (an offset, not a rounded address: the compiler still knows that it is shared memory)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // the launch may overlap the tail of what precedes it in the stream
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // The launch may overlap the tail of what precedes it in the stream: nothing is read from or written to global memory before
+    // griddepcontrol.wait, which a dense batch reaches after its index arithmetic.
+    if (p.cu_seqlens || p.slots) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int nseg = SPLIT ? tp.nseg : 1;
     const int g = blockIdx.x % nseg;             // rank in the cluster
     const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
@@ -165,35 +166,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
     // Set-up: the barriers are initialised by several warps, the TMA warp starts the first loads on its own ones, the gate warps request
     // their first gates.  (One thread for all barriers, and everything else behind it: 2200 cycles before the first load.)
-    auto load_kq = [&](int c, int q3) {
-        mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
-        tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-        tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
-    };
-    auto load_v = [&](int c, int v3) {
-        mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
-        tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
-    };
-    auto load_summary = [&](int it) {      // step it = chunk nc - 1 - it
-        const int st = it % SUM_STAGES, t = t0 + (nc - 1 - it) * CM;
-        mbar_arrive_expect_tx(&sh.s_full[st], 2 * TILE_BYTES);
-        tma_load_4d(tiles + (2 * st + 1) * TILE_BYTES, &map_v, &sh.s_full[st], 0, t, 0, h);
-        tma_load_4d(tiles + 2 * st * TILE_BYTES, &map_k, &sh.s_full[st], 0, t, 0, h);
-    };
     if (lane == 0) {
         if (warp == WARP_TMA) {
             for (int i = 0; i < 2; ++i) { mbar_init(&sh.kq_full[i], 1); mbar_init(&sh.v_full[i], 1); }
             for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_full[i], 1);
             fence_barrier_init();
-            if (summarize) {
-                for (int it = 0; it < min(nc, SUM_STAGES); ++it) load_summary(it);
-            } else if (nc > 0) {
-                load_kq(0, 0);
-                if (!SPLIT) {
-                    load_v(0, 2);
-                    if (nc > 1) load_kq(1, 1);
-                }
-            }
         } else if (warp == 2) {
             mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
             mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, SPLIT ? 8 : 16); mbar_init(&sh.s_done, 1);
@@ -217,6 +194,34 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             fence_barrier_init();
             if (g > 0 && nc > 0)
                 for (int i = 0; i < 4; ++i) mbar_arrive_expect_tx(&sh.s_in[warp - STATE_W0][i], 32 * 128);      // 32 d_k x 32 d_v
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    auto load_kq = [&](int c, int q3) {
+        mbar_arrive_expect_tx(&sh.kq_full[c & 1], 2 * TILE_BYTES);
+        tma_load_4d(tiles + q3 * TILE_BYTES, &map_q, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+        tma_load_4d(tiles + OFF_K + (c & 1) * TILE_BYTES, &map_k, &sh.kq_full[c & 1], 0, t0 + c * CM, 0, h);
+    };
+    auto load_v = [&](int c, int v3) {
+        mbar_arrive_expect_tx(&sh.v_full[c & 1], TILE_BYTES);
+        tma_load_4d(tiles + v3 * TILE_BYTES, &map_v, &sh.v_full[c & 1], 0, t0 + c * CM, 0, h);
+    };
+    auto load_summary = [&](int it) {      // step it = chunk nc - 1 - it
+        const int st = it % SUM_STAGES, t = t0 + (nc - 1 - it) * CM;
+        mbar_arrive_expect_tx(&sh.s_full[st], 2 * TILE_BYTES);
+        tma_load_4d(tiles + (2 * st + 1) * TILE_BYTES, &map_v, &sh.s_full[st], 0, t, 0, h);
+        tma_load_4d(tiles + 2 * st * TILE_BYTES, &map_k, &sh.s_full[st], 0, t, 0, h);
+    };
+    if (warp == WARP_TMA && lane == 0) {
+        if (summarize) {
+            for (int it = 0; it < min(nc, SUM_STAGES); ++it) load_summary(it);
+        } else if (nc > 0) {
+            load_kq(0, 0);
+            if (!SPLIT) {
+                load_v(0, 2);
+                if (nc > 1) load_kq(1, 1);
+            }
         }
     }
     if (p.use_initial_state && warp >= TILE_W0 && warp < GATE_W0)      // 128-byte lines of both states into L2
