@@ -142,7 +142,7 @@ typedef struct {
                                    CUDA-core kernel.  impl TENSOR and TENSOR_PAIR take scalar gates only: DSLA_ERR_UNSUPPORTED */
 } dsla_prefill_args;
 
-/* Scratch the chosen kernel needs for these sizes (0 for the SIMT kernel): the segment summaries of
+/* Scratch to hand over for these sizes (0 for the SIMT kernel): room for the segment summaries of
  * sequences that are split along T, plus, for packed batches (cu_seqlens != NULL, N > 1), one int32 per
  * sequence for the longest-first visiting order.  Pointers in `a` are not dereferenced (cu_seqlens is
  * only compared with NULL). */
@@ -264,8 +264,7 @@ typedef struct {
  *  - TENSOR (what AUTO picks when it applies): bf16, d = 128, scalar gates (n = 1 runs as a pair whose second state
  *    has weight 0 and is never stored): the chunkwise tensor-core
  *    kernel of dsla_prefill run once per pair of states (2i, 2i + 1) with the weights (w_2i, w_2i+1); pairs after the
- *    first write their share to a scratch tensor in the workspace that is then added to o, so o is rounded to bf16 once
- *    per pair.  Needs the workspace below.
+ *    first add their share to o, so o is rounded to bf16 once per pair.  Needs the workspace below.
  * Errors as dsla_prefill; time-outs and a too small max_seqlen are reported through dsla_state_last_error. */
 size_t dsla_nstate_prefill_workspace_bytes(const dsla_nstate_prefill_args* a);
 dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* st, void* cuda_stream);

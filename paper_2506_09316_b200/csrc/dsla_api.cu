@@ -160,7 +160,7 @@ static dsla_status check_prefill_sizes(const dsla_prefill_args* a) {
     if (a->impl != DSLA_IMPL_AUTO && a->impl != DSLA_IMPL_SIMT && a->impl != DSLA_IMPL_TENSOR && a->impl != DSLA_IMPL_TENSOR_PAIR)
         return DSLA_ERR_INVALID_ARG;
     if (a->gate_layout != DSLA_GATE_SCALAR && a->gate_layout != DSLA_GATE_PER_KEY_CHANNEL) return DSLA_ERR_INVALID_ARG;
-    if (a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL) {      // the token-by-token CUDA-core kernel; chunk is ignored
+    if (a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL) {      // chunk is ignored: the kernels for vector gates have their own
         return (a->impl == DSLA_IMPL_TENSOR || a->impl == DSLA_IMPL_TENSOR_PAIR) ? DSLA_ERR_UNSUPPORTED : DSLA_OK;
     }
     const dsla_impl impl = resolve_impl(a);

@@ -157,7 +157,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (int i = tid; i < (p.single ? 1 : 2) * D * D; i += NTHREADS) slot1[(size_t)(i / (D * D)) * state_stride + i % (D * D)] = 0.f;
         return;
     }
-    const int nc = max(0, sq.c_end - sq.c_begin);  // 0: a segment behind the end of its sequence, here only for its share of the fold
+    const int nc = max(0, sq.c_end - sq.c_begin);  // 0: a segment behind the end of its sequence
     const int t0 = sq.t_begin + sq.c_begin * CM;  // first token of this segment
     const int tok0 = sq.c_begin * CM;             // its index inside the sequence
     const bool last = g == sq.last_seg;           // the final state is kept; other segments skip the last chunk's update
@@ -815,7 +815,7 @@ int resident_clusters(int size) {
 
 // Segments per sequence: the most that keep all work items resident at once (CTAs of a cluster, or clusters of the pair variant).
 // The single-CTA kernel's segments hold at least one chunk of 128 tokens, and a sequence of two chunks stays whole (summary and
-// fold cost about as much as the chunk they would save); the pair variant's at least four of 64.
+// chain cost about as much as the chunk they would save); the pair variant's at least four of 64.
 void plan(const dsla_prefill_args* a, bool pair, int* nseg, int* cps, int* skew8) {
     const int chunk = pair ? C : CM;
     const int max_chunks = (a->max_seqlen + chunk - 1) / chunk;

@@ -20,14 +20,14 @@ constexpr int ORDER_MAX_N = 8192;     // packed batches up to this many sequence
 
 struct TcParams {
     PrefillParams p;
-    float* ws;          // summaries: [(n*H + h)*nseg + g] -> {U[2][D][D], A[2]}
-    const float* init;  // initial states the segments start from: the slots themselves, or a snapshot of them
-                        // [(n*H + h)][2][D][D] taken before the main grid when a sequence is split (the CTA of the
+    float* ws;          // summaries of the pair variant: [(n*H + h)*nseg + g] -> {U[2][D][D], A[2]}
+    const float* init;  // initial states the pair variant's segments start from: the slots themselves, or a snapshot of
+                        // them [(n*H + h)][2][D][D] taken before the main grid when a sequence is split (the CTA of the
                         // last segment overwrites the slot while CTAs of earlier segments may not have read it yet)
     int chunk;          // tokens per chunk of the main grid (a multiple of C): the unit of cps
     int nseg;           // segments per sequence (grid dimension)
     int cps;            // chunks per segment (mean)
-    int skew8;          // eighths of a chunk by which consecutive segments get shorter (later segments start later: they
+    int skew8;          // pair variant: eighths of a chunk by which consecutive segments get shorter (later segments
                         // first fold the summaries of all earlier segments into their initial state)
     int order_here;     // the main kernel finds that order by itself (few sequences)
     const int* order;   // sequences by descending length (longest first), or nullptr for index order
@@ -83,7 +83,7 @@ __device__ __forceinline__ SeqInfo seq_info(const PrefillParams& p, int n, int g
     return seq_info_at(p.cu_seqlens ? p.cu_seqlens[n] : n * p.T, p.cu_seqlens ? p.cu_seqlens[n + 1] : (n + 1) * p.T, p.slots ? p.slots[n] : n, g, tp);
 }
 
-// Initial state of a segment (cold path, kept out of line so the chunk loop stays small): the slot
+// Initial state of a segment of the pair variant (cold path, kept out of line so the chunk loop stays small): the slot
 // contents (or zero) pushed through the summaries of the earlier segments, S <- A_j S + U_j; writes the bf16
 // copy for the readout and a_0 S for the first update.  One thread = one d_v lane of one state and the d_k rows
 // 32 bt_begin .. 32 bt_end - 1.  The fold is a chain of dependent rounds of loads.
