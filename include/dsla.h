@@ -263,8 +263,8 @@ typedef struct {
  *    d = 128) the states are processed in groups, each group adding its share to o.
  *  - TENSOR (what AUTO picks when it applies): bf16, d = 128, scalar gates (n = 1 runs as a pair whose second state
  *    has weight 0 and is never stored): the chunkwise tensor-core
- *    kernel of dsla_prefill run once per pair of states (2i, 2i + 1) with the weights (w_2i, w_2i+1); pairs after the
- *    first add their share to o, so o is rounded to bf16 once per pair.  Needs the workspace below.
+ *    kernel of dsla_prefill once per pair of states (2i, 2i + 1) with the weights (w_2i, w_2i+1), one launch per pair or, with
+ *    few (sequence, head) pairs, several side by side; pairs after the first add their share to o in order, so o is rounded to bf16 once per pair.  Needs the workspace below.
  * Errors as dsla_prefill; time-outs and a too small max_seqlen are reported through dsla_state_last_error. */
 size_t dsla_nstate_prefill_workspace_bytes(const dsla_nstate_prefill_args* a);
 dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* st, void* cuda_stream);

@@ -353,7 +353,10 @@ dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* s
         p.scale = a->scale; p.use_initial_state = a->use_initial_state ? 1 : 0;
         p.weights = a->weights; p.n_total = a->n_states;
         const size_t gs = (size_t)a->T_total * a->H;
-        for (int first = 0; first < a->n_states; first += 2) {      // one pass of the dual-state kernel per pair of states
+        // the dual-state kernel once per pair of states, or for several pairs at a time
+        p.pairs = a->n_states > 2 ? prefill_tc_pairs(&b, a->n_states / 2) : 1;
+        p.pair_stride = 2 * gs;
+        for (int first = 0; first < a->n_states; first += 2 * p.pairs) {
             p.g_hist = a->gates + (size_t)first * gs;
             p.single = a->n_states == 1;
             p.g_rec = a->gates + (size_t)(p.single ? first : first + 1) * gs;

@@ -36,6 +36,8 @@ struct PrefillParams {
     int accumulate;             // o += instead of o = (pairs of states after the first)
     int single;                 // only state_first exists (n = 1): the second state of the kernel runs with weight 0 on the first
                                 // state's gates, starts from zero and is never loaded from or stored to the slot
+    int pairs;                  // pairs of states in this call (0 counts as 1), consecutive from state_first; the gates of pair j are
+    size_t pair_stride;         // pair_stride values behind those of pair j - 1
 };
 
 struct DecodeParams {
@@ -86,6 +88,7 @@ void launch_bounded_wait_selftest(int* status, unsigned max_polls, cudaStream_t 
 // dsla_prefill_tc.cu (pair = the cluster variant of dsla_prefill_tc_pair.cu)
 bool prefill_tc_available();
 size_t prefill_tc_workspace_bytes(const dsla_prefill_args* a, bool pair);
+int prefill_tc_pairs(const dsla_prefill_args* a, int npairs);      // how many of npairs pairs of states one launch should take
 dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a, bool pair, cudaStream_t s);
 
 __device__ __forceinline__ float to_f32(float x) { return x; }

@@ -76,6 +76,8 @@ struct alignas(16) Shared {
     float* slot;                          // the first state of this (sequence, head) in its slot: read where it is needed, not kept in registers
     GateSmem gs[2];
     float a_seg[2];                       // products of the segment's gates
+    uint64_t o_tail;                      // the pair of states before this one has written a ragged last chunk's outputs
+    uint32_t o_turn;                      // and the first o_turn whole chunks'
 };
 
 // Four MMAs whose operands advance by a constant.
@@ -125,8 +127,8 @@ __device__ __forceinline__ SeqPlace longest_first(const PrefillParams& p, int ra
 }
 
 // SPLIT: the sequences are cut into segments (a variant of its own: with that code in it the chunk loop of whole sequences
-// ran 2 % longer).
-template <bool SPLIT>
+// ran 2 % longer).  PAIRS: the pairs of states of the n-state form side by side in the cluster (a variant for the same reason).
+template <bool SPLIT, bool PAIRS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const TcParams tp) {
@@ -139,8 +141,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // griddepcontrol.wait, which a dense batch reaches after its index arithmetic.
     if (p.cu_seqlens || p.slots) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int nseg = SPLIT ? tp.nseg : 1;
-    const int g = blockIdx.x % nseg;             // rank in the cluster
-    const int unit = blockIdx.x / nseg, h = unit % p.H, rank = unit / p.H;
+    const int pairs = PAIRS ? tp.pairs : 1;
+    const int cta = blockIdx.x % (nseg * pairs);      // rank in the cluster
+    const int pr = PAIRS ? cta / nseg : 0, g = cta - pr * nseg;
+    const int unit = blockIdx.x / (nseg * pairs), h = unit % p.H, rank = unit / p.H;
+    // (read where they are needed, not kept in registers)
+    auto first = [&] { return p.state_first + 2 * pr; };
+    auto accumulate = [&] { return PAIRS && pr > 0 ? true : p.accumulate != 0; };
     SeqInfo sq;
     if (tp.order_here) {
         const SeqPlace at = longest_first(p, rank, lane);
@@ -150,7 +157,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     }
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (tid == 0 && g == 0 && sq.nchunks > seg_begin(tp.nseg, tp.nseg, tp.cps, tp.skew8)) atomicExch(p.status, (int)DSLA_ERR_INVALID_ARG);
-    float* slot1 = p.state + (((size_t)sq.slot * p.n_total + p.state_first) * p.H + h) * (size_t)(D * D);
+    float* slot1 = p.state + (((size_t)sq.slot * p.n_total + first()) * p.H + h) * (size_t)(D * D);
     const size_t state_stride = (size_t)p.H * D * D;
     if (sq.len <= 0) {  // empty sequence: a fresh start leaves zero states, a resume leaves the slot alone
         if (g == 0 && !p.use_initial_state)
@@ -175,6 +182,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
             mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, SPLIT ? 8 : 16); mbar_init(&sh.s_done, 1);
             mbar_init(&sh.next_ready, 8);
+            if (PAIRS) {
+                mbar_init(&sh.o_tail, 8);
+                sh.o_turn = 0;
+                __threadfence();      // before the cluster barrier, behind which another CTA writes it
+            }
             sh.abort_flag = 0;
             sh.slot = slot1;
             fence_barrier_init();
@@ -229,7 +241,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             asm volatile("prefetch.global.L2 [%0];" ::"l"(slot1 + (size_t)(i >> 9) * state_stride + (size_t)(i & 511) * 32));
     float nx[4];      // gate warps: the next chunk's gates, four tokens a lane
     auto fetch = [&](int c) {      // raw values: nothing may consume them here, or the warp would sit out the load latency in every chunk
-        const float* gsrc = warp == GATE_W0 ? p.g_hist : p.g_rec;
+        const float* gsrc = (warp == GATE_W0 ? p.g_hist : p.g_rec) + (PAIRS ? (size_t)pr * p.pair_stride : 0);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int j = c * CM + 4 * lane + e;
@@ -274,7 +286,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             WAIT(&sh.s_done, 0);
             load_kq(0, 0);
         }
+        if (PAIRS) {
+            __syncwarp();
+            cluster_wait();
+        }
         if (lane == 0 && nc > 0) {
+            const uint32_t next_turn = PAIRS && pr + 1 < pairs ? map_to_cta(smem_u32(&sh.o_turn), (uint32_t)(cta + nseg)) : 0u;
             if (SPLIT) {
                 if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
                 load_v(0, 2);
@@ -293,7 +310,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
                 if (c < nfull) {
                     WAIT(&sh.o_staged, c & 1);             // the outputs of chunk c are in the slot of its V
-                    if (p.accumulate) tma_add_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);      // bf16 sums, one rounding each
+                    if (PAIRS && pr > 0) {                 // behind the pair of states before this one: sums in a fixed order
+                        wait_count_cluster(&sh.o_turn, (uint32_t)(c + 1), abortp, p.status);
+                        fence_proxy_async_global();
+                    }
+                    if (accumulate()) tma_add_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);      // bf16 sums, one rounding each
                     else tma_store_4d(&map_o, tiles + v3 * TILE_BYTES, 0, t0 + c * CM, 0, h);
                     bulk_commit();
                     bulk_wait_read();
@@ -305,6 +326,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         tma_prefetch_4d(&map_q, 0, t0 + (c + 3) * CM, 0, h);
                         tma_prefetch_4d(&map_k, 0, t0 + (c + 3) * CM, 0, h);
                     }
+                }
+                if (PAIRS && pr + 1 < pairs && c < nfull) {
+                    bulk_wait_all();
+                    st_release_cluster(next_turn, (uint32_t)(c + 1));
                 }
                 c3 = c3 == 2 ? 0 : c3 + 1;
             }
@@ -401,8 +426,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const int half = (warp - TILE_W0) >> 2;           // column half: keys 64 half .. 64 half + 63
         const uint32_t lane_addr = tb + ((uint32_t)(32 * q) << 16);
         const int j = 32 * q + lane;
-        const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first] : p.gamma[h]) * p.scale;
-        const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + p.state_first + 1] : 1.f - p.gamma[h]) * p.scale;
+        const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + first()] : p.gamma[h]) * p.scale;
+        const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + first() + 1] : 1.f - p.gamma[h]) * p.scale;
 
         if (!SPLIT && !zero_start) start_state(half, 1, lane_addr, j);
         // The ten 32 x 32 blocks of the lower triangle: a quadrant's q + 1 blocks are split between its two warps (the second one
@@ -489,7 +514,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // through independent exponentials.  Lane l holds tokens 4 l .. 4 l + 3.  The chunk decay that carries the state
         // is the plain product of the gates.
         const int i = warp - GATE_W0;
-        const float Wi = (p.weights ? (i == 1 && p.single ? 0.f : p.weights[(size_t)h * p.n_total + p.state_first + i])
+        const float Wi = (p.weights ? (i == 1 && p.single ? 0.f : p.weights[(size_t)h * p.n_total + first() + i])
                                     : (i == 0 ? p.gamma[h] : 1.f - p.gamma[h])) * p.scale;
         auto decays = [&](const float (&x)[4], float (&L)[4], float& pr, float& incl) {      // L: inclusive from the chunk start; incl: of the lane's last token
             float run = 0.f;
@@ -613,8 +638,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         auto chain = [&](float a) {
             const float A = sh.a_seg[hi];
             const uint32_t mine = (uint32_t)(initial_off(hi) + v * 16), w = warp - STATE_W0;
-            const uint32_t next = map_to_cta(smem_u32(tiles + mine), (uint32_t)(g + 1 < nseg ? g + 1 : g));
-            const uint32_t next_bar = map_to_cta(smem_u32(&sh.s_in[w][0]), (uint32_t)(g + 1 < nseg ? g + 1 : g));
+            const uint32_t next = map_to_cta(smem_u32(tiles + mine), (uint32_t)(g + 1 < nseg ? cta + 1 : cta));
+            const uint32_t next_bar = map_to_cta(smem_u32(&sh.s_in[w][0]), (uint32_t)(g + 1 < nseg ? cta + 1 : cta));
             if (summarize) mbar_wait_cluster(&sh.next_ready, 0, abortp, p.status);
 #pragma unroll 1
             for (int b = 0; b < 8; ++b) {      // 16 d_k at a time, handed over in pairs
@@ -659,7 +684,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (SPLIT) {
             __syncwarp();
             cluster_wait();
-            if (g > 0 && nc > 0 && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.next_ready), (uint32_t)(g - 1)));      // room for this segment's initial state
+            if (g > 0 && nc > 0 && lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.next_ready), (uint32_t)(cta - 1)));      // room for this segment's initial state
         }
         if (!SPLIT && !zero_start) {
             start_state(hi, 0, lane_addr, v);
@@ -738,6 +763,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             } else {      // the sequence's ragged last chunk: each thread owns one d_v lane of O^T
                 __nv_bfloat16* dst = og + ((size_t)(t0 + c * CM + 64 * hi) * p.H + h) * D + v;
                 const size_t row = (size_t)p.H * D;
+                if (PAIRS && pr > 0) mbar_wait_cluster(&sh.o_tail, 0, abortp, p.status);
 #pragma unroll 1
                 for (int b = 64 * hi; b < 64 * hi + 64; b += 16) {
                     uint32_t r[16];
@@ -747,10 +773,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     for (int jj = 0; jj < 16; ++jj) {
                         if (b + jj < valid) {
                             const __nv_bfloat16 y = __float2bfloat16_rn(__uint_as_float(r[jj]));
-                            *dst = p.accumulate ? __hadd(*dst, y) : y;
+                            *dst = accumulate() ? __hadd(*dst, y) : y;
                         }
                         dst += row;
                     }
+                }
+                if (PAIRS && pr + 1 < pairs) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.o_tail), (uint32_t)(cta + nseg)));
                 }
             }
             v3 = v3 == 2 ? 0 : v3 + 1;
@@ -762,7 +792,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
     }
     __syncwarp();
-    if (SPLIT && !(warp >= STATE_W0 && warp < GATE_W0)) cluster_wait();
+    if (SPLIT && !(PAIRS && warp == WARP_TMA) && !(warp >= STATE_W0 && warp < GATE_W0)) cluster_wait();
     tc_fence_before();
     __syncthreads();
     if (warp == WARP_MMA) tmem_dealloc(tb, 512);
@@ -803,9 +833,9 @@ int resident_clusters(int size) {
         attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(prefill_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess ||
-            (size > 8 && cudaFuncSetAttribute(prefill_tc_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-            cudaOccupancyMaxActiveClusters(&n, prefill_tc_kernel<true>, &cfg) != cudaSuccess || n <= 0)
+        if (cudaFuncSetAttribute(prefill_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess ||
+            (size > 8 && cudaFuncSetAttribute(prefill_tc_kernel<true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, prefill_tc_kernel<true, false>, &cfg) != cudaSuccess || n <= 0)
             n = -1;
         (void)cudaGetLastError();
         cached[dev][size].store(n, std::memory_order_relaxed);
@@ -816,7 +846,9 @@ int resident_clusters(int size) {
 // Segments per sequence: the most that keep all work items resident at once (CTAs of a cluster, or clusters of the pair variant).
 // The single-CTA kernel's segments hold at least one chunk of 128 tokens, and a sequence of two chunks stays whole (summary and
 // chain cost about as much as the chunk they would save); the pair variant's at least four of 64.
-void plan(const dsla_prefill_args* a, bool pair, int* nseg, int* cps, int* skew8) {
+// Several pairs of states of the n-state form in one launch: the CTAs of all of them and of all segments form one cluster; *nseg = 0 if
+// they cannot all be resident.
+void plan(const dsla_prefill_args* a, bool pair, int pairs, int* nseg, int* cps, int* skew8) {
     const int chunk = pair ? C : CM;
     const int max_chunks = (a->max_seqlen + chunk - 1) / chunk;
     const long long units = (long long)a->N * a->H;
@@ -827,6 +859,12 @@ void plan(const dsla_prefill_args* a, bool pair, int* nseg, int* cps, int* skew8
         if (units > 0 && units < room) ns = (int)(room / units);
         if (ns > MAX_SEG) ns = MAX_SEG;
         while (ns > 1 && (max_chunks + ns - 1) / ns < 4) --ns;
+    } else if (pairs > 1) {
+        ns = units > 0 ? (int)(sm_count() / (units * pairs)) : 1;
+        if (ns > MAX_SEG / pairs) ns = MAX_SEG / pairs;
+        if (ns > 1 && (ns > max_chunks || max_chunks <= 2)) ns = max_chunks <= 2 ? 1 : max_chunks;
+        while (ns > 0 && resident_clusters(ns * pairs) < units) --ns;
+        if (ns > 1) ns = (max_chunks + (max_chunks + ns - 1) / ns - 1) / ((max_chunks + ns - 1) / ns);
     } else if (units > 0 && units < sm_count() && max_chunks > 2) {
         ns = (int)(sm_count() / units);
         if (ns > MAX_SEG) ns = MAX_SEG;
@@ -836,7 +874,7 @@ void plan(const dsla_prefill_args* a, bool pair, int* nseg, int* cps, int* skew8
     }
     if (max_chunks <= 0) ns = 1;
     *nseg = ns;
-    *cps = max_chunks > 0 ? (max_chunks + ns - 1) / ns : 1;
+    *cps = max_chunks > 0 && ns > 0 ? (max_chunks + ns - 1) / ns : 1;
     // The pair variant's later segments fold more summaries into their initial state before they start (about 50 tokens' time
     // each): make consecutive segments about that much shorter, as far as the shortest keeps at least 192 tokens.
     if (pair && ns > 1) {
@@ -852,12 +890,13 @@ size_t order_bytes(const dsla_prefill_args* a) { return wants_order(a) ? up256((
 size_t snapshot_bytes(const dsla_prefill_args* a, int nseg) { return nseg > 1 ? (size_t)a->N * a->H * 2 * D * D * sizeof(float) : 0; }
 
 dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo, const TcParams& tp, cudaStream_t s) {
-    const auto kernel = tp.nseg > 1 ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
+    const int size = tp.nseg * tp.pairs;      // CTAs of a cluster
+    const auto kernel = tp.pairs > 1 ? prefill_tc_kernel<true, true> : size > 1 ? prefill_tc_kernel<true, false> : prefill_tc_kernel<false, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN) != cudaSuccess) return DSLA_ERR_CUDA;
-    if (tp.nseg > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return DSLA_ERR_CUDA;
+    if (size > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return DSLA_ERR_CUDA;
     const long long units = (long long)tp.p.N * tp.p.H;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(units * tp.nseg));
+    cfg.gridDim = dim3((unsigned)(units * size));
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = SMEM_DYN;
     cfg.stream = s;
@@ -865,9 +904,9 @@ dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)tp.nseg; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = (unsigned)size; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = tp.nseg > 1 ? 2 : 1;
+    cfg.numAttrs = size > 1 ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, tp) != cudaSuccess) return DSLA_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? DSLA_OK : DSLA_ERR_CUDA;
@@ -877,9 +916,26 @@ dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
 
 bool prefill_tc_available() { return true; }
 
+// Pairs of states side by side need fewer segments per sequence, so shorter chains of initial states, and read Q, K and V from L2
+// the second time (four states, T = 4096, 32 heads: 116 us as two launches, 97 as one; eight: 224 and 163); but SMs may be left over,
+// or the sequences be cut less than a launch for each pair would.  Times in eighths of a chunk's (7.2 k cycles): a chunk 8, set-up and
+// drain 5, a summary 2 per chunk, a hop of the initial states 3.
+int prefill_tc_pairs(const dsla_prefill_args* a, int npairs) {
+    int best = 1;
+    long long least = 0;
+    for (int k = 1; k <= npairs; k *= 2) {
+        int nseg, cps, skew8;
+        plan(a, false, k, &nseg, &cps, &skew8);
+        if (nseg < 1) break;
+        const long long cost = (npairs / k) * (8ll * cps + 5 + (nseg > 1 ? 2ll * cps + 3 * (nseg - 1) : 0));
+        if (k == 1 || cost < least) { best = k; least = cost; }
+    }
+    return best;
+}
+
 size_t prefill_tc_workspace_bytes(const dsla_prefill_args* a, bool pair) {
     int nseg, cps, skew8;
-    plan(a, pair, &nseg, &cps, &skew8);
+    plan(a, pair, 1, &nseg, &cps, &skew8);
     return summaries_bytes(a, nseg) + order_bytes(a) + snapshot_bytes(a, nseg);     // each a multiple of 256
 }
 
@@ -891,7 +947,8 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
     TcParams tp;
     tp.p = p;
     tp.chunk = pair ? C : CM;
-    plan(a, pair, &tp.nseg, &tp.cps, &tp.skew8);
+    tp.pairs = p.pairs > 1 ? p.pairs : 1;
+    plan(a, pair, tp.pairs, &tp.nseg, &tp.cps, &tp.skew8);
     char* wsp = static_cast<char*>(a->workspace);
     tp.ws = tp.nseg > 1 ? reinterpret_cast<float*>(wsp) : nullptr;
     tp.order = nullptr;

@@ -26,6 +26,7 @@ struct TcParams {
                         // last segment overwrites the slot while CTAs of earlier segments may not have read it yet)
     int chunk;          // tokens per chunk of the main grid (a multiple of C): the unit of cps
     int nseg;           // segments per sequence (grid dimension)
+    int pairs;          // pairs of states (n-state form), side by side in a cluster
     int cps;            // chunks per segment (mean)
     int skew8;          // pair variant: eighths of a chunk by which consecutive segments get shorter (later segments
                         // first fold the summaries of all earlier segments into their initial state)

@@ -145,6 +145,26 @@ __device__ __forceinline__ void st_cluster_f32x4(uint32_t caddr, float a, float 
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
 }
+// A counter in the shared memory of another CTA of the cluster: written there with a release, polled by its owner (bounded like the
+// barrier waits) with an acquire.
+__device__ __forceinline__ void st_release_cluster(uint32_t caddr, uint32_t v) {
+    asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
+}
+__device__ __forceinline__ bool wait_count_cluster(const uint32_t* count, uint32_t at_least, volatile int* abort_flag, int* status) {
+    const uint64_t t0 = global_timer_ns();
+    for (uint32_t i = 0; i < MBAR_WAIT_LIMIT; ++i) {
+        uint32_t v;
+        asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(count)) : "memory");
+        if (v >= at_least) return true;
+        if ((i & 63u) == 63u) {
+            if (*abort_flag) return false;
+            if (global_timer_ns() - t0 > 1000000000ull) break;
+        }
+    }
+    *abort_flag = 1;
+    atomicExch(status, 5 /* DSLA_ERR_TIMEOUT */);
+    return false;
+}
 // Asynchronous 16-byte store into another CTA's shared memory; its completion is counted (16 bytes) on an mbarrier
 // of that CTA, so the sender needs no fence and no separate arrive: the receiver arms the barrier with the number of
 // bytes it expects and waits on it.
@@ -177,6 +197,7 @@ __device__ __forceinline__ uint32_t ld_shared_u32(uint32_t saddr) {
 }
 __device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- TMA (tile mode, 4-D, destination in this CTA's shared memory) ------------------------

@@ -97,3 +97,33 @@ def test_packed_order(N, H, top):
     o, S = gpu_prefill(inp, num_slots=N + 1, state0=state0, slots=slots, impl="tensor")
     o_ref, S_ref = oracle_prefill(inp, state0=state0.astype(np.float64), slots=slots)
     assert rel_err(o, o_ref) <= TOL[BF] and rel_err(S[slots], S_ref[slots]) <= TOL[BF]
+
+
+# Pairs of states side by side in a cluster: two and four pairs, with one segment per sequence and with several (clusters of up to 16),
+# whole chunks and ragged ones, a batch of which one sequence is empty and one shorter than a segment; 75 heads: one pair at a time
+@pytest.mark.parametrize("n,lens,H,resume", [(4, (100,), 3, False), (8, (128,), 2, True), (4, (129,), 74, True), (4, (1500, 0, 64, 777), 2, True),
+                                             (8, (1153,), 3, False), (8, (640, 300), 5, True), (4, (1024,), 32, False), (4, (257,), 75, False)])
+def test_nstate_pairs_in_one_cluster(n, lens, H, resume):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, rel_err
+    rng = np.random.default_rng(5500 + n + sum(lens))
+    inp = gen.make_packed(5501 + H, lens, H, 128, BF)
+    gates = (1.0 / (1.0 + np.exp(-rng.normal(3.0, 1.5, size=(n, inp.T_total, H))))).astype(np.float32)
+    gates[:, 60, :] = 0.0
+    w = rng.normal(size=(H, n)).astype(np.float32)
+    st0 = (rng.normal(size=(len(lens), n, H, 128, 128)) * 0.3).astype(np.float32)
+    dv, g, wd = inp.to("cuda"), torch.from_numpy(gates).cuda(), torch.from_numpy(w).cuda()
+    st, outs = dsla.dsla_state_alloc_n(len(lens), n, H, 128, 128), []
+    for _ in range(2):          # back to back; the order in which the pairs add to o is fixed, so the second run gives the same bits
+        st.tensor.copy_(torch.from_numpy(st0))
+        outs.append(dsla.dsla_nstate_prefill(dv.q, dv.k, dv.v, g, wd, st, cu_seqlens=dv.cu_seqlens, max_seqlen=max(lens),
+                                             use_initial_state=resume, scale=0.8))
+    torch.cuda.synchronize()
+    assert dsla.dsla_state_last_error(st) == dsla.DSLA_OK
+    assert torch.equal(outs[0], outs[1])
+    f = inp.as_f64()
+    start = st0.astype(np.float64) if resume else np.zeros(st0.shape)
+    o_ref, S_ref = orc.prefill_n(f["q"], f["k"], f["v"], gates, w, f["cu_seqlens"], scale=0.8, state=start)
+    assert rel_err(outs[0].double().cpu().numpy(), o_ref) <= TOL[BF] * (1.5 if n == 8 else 1.0)
+    assert rel_err(st.tensor.double().cpu().numpy(), S_ref) <= TOL[BF]
