@@ -235,72 +235,8 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) s[a][b] = 0.f;
-    bool staged = false;      // the segment's only chunk is in shared memory already
-    if (segs > 1) {
-        // ---- summary of this segment, left in Ss and a_seg for the later segments
-        if (c_end < nchunks) {
-            const bool only = c_end - c_begin == 1;      // then Q is staged with it and the second pass starts from there
-            float as = 1.f;
-            fetch(c_begin, only);
-            for (int c = c_begin; c < c_end; ++c) {
-                stage(only);
-                __syncthreads();
-                if (c + 1 < c_end) fetch(c + 1, false);
-                update();
-                as *= a_dec[si];
-                __syncthreads();
-            }
-            staged = only;
-            publish();
-            if (tid % (2 * D) == 0) a_seg[si] = as;
-        }
-        tc::cluster_sync_all();
-        // ---- initial states: the slot (or zero) pushed through the earlier segments.  Each CTA does this for its share of the
-        // elements and for every segment: it reads the share out of all summaries and writes the initial states over them, so
-        // every CTA reads and writes 1 / segs of what a fold per segment would pull from the first CTAs of the cluster.
-        for (int f = seg * (2 * D * 8 / segs) + tid; f < (seg + 1) * (2 * D * 8 / segs); f += NT) {
-            const int fi = f / (D * 8), k = (f / 8) % D, c = (f & 7) * 4;
-            const float* slot_at = p.state + (((size_t)slot * 2 + fi) * p.H + h) * (size_t)(D * D) + (size_t)k * D + col0 + c;
-            float4 x = p.use_initial_state ? *reinterpret_cast<const float4*>(slot_at) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const uint32_t at = tc::smem_u32(Ss + (fi * D + k) * VP + c), a_at = tc::smem_u32(&a_seg[fi]);
-            float4 u[7];
-            float as[7];
-#pragma unroll
-            for (int e = 0; e < 7; ++e)
-                if (e < segs - 1) {
-                    u[e] = tc::ld_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e));
-                    as[e] = tc::ld_cluster_f32(tc::map_to_cta(a_at, (uint32_t)e));
-                }
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (e < segs) {
-                    tc::st_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e), x.x, x.y, x.z, x.w);
-                    // (segments behind the sequence's last chunk have no summary, and nobody uses what they would start from)
-                    if (e < 7) { x.x = fmaf(as[e], x.x, u[e].x); x.y = fmaf(as[e], x.y, u[e].y); x.z = fmaf(as[e], x.z, u[e].z); x.w = fmaf(as[e], x.w, u[e].w); }
-                }
-        }
-        tc::cluster_sync_all();      // the initial states are in place; every read of the slot is done
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float4 x = *reinterpret_cast<const float4*>(Sme + a * VP);
-            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
-        }
-        if (c_begin >= c_end && !(seg == 0 && nchunks == 0)) return;
-    } else if (p.use_initial_state) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float4 x = *reinterpret_cast<const float4*>(G + (size_t)a * D);
-            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
-        }
-    }
-    if (!staged && c_begin < c_end) fetch(c_begin, true);
-    for (int c = c_begin; c < c_end; ++c) {
-        const int c0 = c * C, valid = min(C, len - c0);
-        publish();
-        if (!staged) stage(true);
-        __syncthreads();
-        if (c + 1 < c_end) fetch(c + 1, true);
-        // ---- masked scores: 4 x 4 tiles of the lower triangle, tile t of row group r is number r (r + 1) / 2 + t
+    // ---- masked scores: 4 x 4 tiles of the lower triangle, tile t of row group r is number r (r + 1) / 2 + t
+    auto scores = [&]() {
         constexpr int TILES = (C / 4) * (C / 4 + 1) / 2;
         for (int it = tid; it < ((TILES * SPLIT + 31) & ~31); it += NT) {
             const int tile = min(it / SPLIT, TILES - 1), part = it % SPLIT;
@@ -339,8 +275,9 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
                 if (part == 0) *reinterpret_cast<float4*>(Ps + (j0 + a) * CP + s0) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
             }
         }
-        __syncthreads();
-        // ---- decay mask, one element per thread and round (the tiles above keep half of the threads busy, this all of them)
+    };
+    // ---- decay mask, one element per thread and round (the tiles above keep half of the threads busy, this all of them)
+    auto mask = [&]() {
 #pragma unroll 2
         for (int idx = tid; idx < C * C; idx += NT) {
             const int j = idx / C, t = idx % C;
@@ -354,6 +291,91 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
                 Ps[j * CP + t] *= m;
             }
         }
+    };
+    bool ahead = false;       // the segment's first chunk is in shared memory, its masked scores too
+    if (segs > 1) {
+        // ---- summary of this segment, left in Ss and a_seg for the later segments.  The first chunk's scores need no state: they and
+        // their mask are computed while the cluster barriers on both sides of the fold complete.
+        ahead = c_begin < c_end;
+        const bool only = c_end - c_begin == 1;      // the summary's last chunk is the first of the second pass
+        if (c_end < nchunks) {
+            float as = 1.f;
+            fetch(c_begin, only);
+            for (int c = c_begin; c < c_end; ++c) {
+                stage(only);
+                __syncthreads();
+                if (c + 1 < c_end) fetch(c + 1, false);
+                else if (!only) fetch(c_begin, true);
+                update();
+                as *= a_dec[si];
+                __syncthreads();
+            }
+            publish();
+            if (tid % (2 * D) == 0) a_seg[si] = as;
+        } else if (ahead) {
+            fetch(c_begin, true);
+        }
+        tc::cluster_arrive();
+        if (ahead) {
+            if (!only || c_end == nchunks) { stage(true); __syncthreads(); }
+            if (!only) fetch(c_begin + 1, true);
+            scores();
+            __syncthreads();
+        }
+        tc::cluster_wait();
+        // ---- initial states: the slot (or zero) pushed through the earlier segments.  Each CTA does this for its share of the
+        // elements and for every segment: it reads the share out of all summaries and writes the initial states over them, so
+        // every CTA reads and writes 1 / segs of what a fold per segment would pull from the first CTAs of the cluster.
+        for (int f = seg * (2 * D * 8 / segs) + tid; f < (seg + 1) * (2 * D * 8 / segs); f += NT) {
+            const int fi = f / (D * 8), k = (f / 8) % D, c = (f & 7) * 4;
+            const float* slot_at = p.state + (((size_t)slot * 2 + fi) * p.H + h) * (size_t)(D * D) + (size_t)k * D + col0 + c;
+            float4 x = p.use_initial_state ? *reinterpret_cast<const float4*>(slot_at) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const uint32_t at = tc::smem_u32(Ss + (fi * D + k) * VP + c), a_at = tc::smem_u32(&a_seg[fi]);
+            float4 u[7];
+            float as[7];
+#pragma unroll
+            for (int e = 0; e < 7; ++e)
+                if (e < segs - 1) {
+                    u[e] = tc::ld_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e));
+                    as[e] = tc::ld_cluster_f32(tc::map_to_cta(a_at, (uint32_t)e));
+                }
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e < segs) {
+                    tc::st_cluster_f32x4(tc::map_to_cta(at, (uint32_t)e), x.x, x.y, x.z, x.w);
+                    // (segments behind the sequence's last chunk have no summary, and nobody uses what they would start from)
+                    if (e < 7) { x.x = fmaf(as[e], x.x, u[e].x); x.y = fmaf(as[e], x.y, u[e].y); x.z = fmaf(as[e], x.z, u[e].z); x.w = fmaf(as[e], x.w, u[e].w); }
+                }
+        }
+        tc::cluster_arrive();
+        if (ahead) mask();
+        tc::cluster_wait();      // the initial states are in place; every read of the slot is done
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 x = *reinterpret_cast<const float4*>(Sme + a * VP);
+            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
+        }
+        if (c_begin >= c_end && !(seg == 0 && nchunks == 0)) return;
+    } else if (p.use_initial_state) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 x = *reinterpret_cast<const float4*>(G + (size_t)a * D);
+            s[a][0] = x.x; s[a][1] = x.y; s[a][2] = x.z; s[a][3] = x.w;
+        }
+    }
+    if (!ahead && c_begin < c_end) fetch(c_begin, true);
+    for (int c = c_begin; c < c_end; ++c) {
+        const int c0 = c * C, valid = min(C, len - c0);
+        if (!ahead) {
+            publish();
+            stage(true);
+            __syncthreads();
+            if (c + 1 < c_end) fetch(c + 1, true);
+            scores();
+            __syncthreads();
+            mask();
+        }
+        ahead = false;
         __syncthreads();
         // ---- outputs: 4 rows x 2 columns; with SPLIT = 2 lane `part` reads out state `part` and takes every other 4 columns of P
         for (int it = tid; it < (C / 4) * (DVS / 2) * SPLIT; it += NT) {

@@ -120,6 +120,7 @@ __device__ __forceinline__ void cluster_sync_all() {
 // The two halves of it; every thread of the cluster executes both.  Relaxed: what others may use after it has to be published by a fence
 // (initialised mbarriers: fence_barrier_init).
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of the same shared-memory location in the CTA of the given rank (shared::cluster window).
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
