@@ -15,8 +15,9 @@
 // first accumulates its own state from zero (K and V only) and leaves it, with the product of its gates, in its
 // shared memory; after a cluster barrier the initial states are folded out of the summaries through distributed
 // shared memory and every CTA runs its chunks.  No scratch in global memory, no second launch.
-// 4 heads of 64, T = 512, fp32: 21 us, 106 us with one CTA per slab.  Bound by shared-memory wavefronts: the 4 x 4 tiles of
-// the update (2.6 us), the scores and their mask (5.8) and the outputs (3.0) do two FMAs per float read.
+// 4 heads of 64, T = 512, fp32: 17 us, 106 us with one CTA per slab.  Bound by shared-memory reads, FMA issue and the barriers between
+// the steps of a chunk: the 4 x 4 tiles of the update, the scores and the outputs do 8 packed FMAs (two products each) per two
+// 16-byte reads.  Scalar FMAs, and output tiles of 4 x 2, took 18; scores behind the fold instead of under its barriers 21.
 #include "dsla_internal.cuh"
 #include "tc_utils.cuh"
 
@@ -42,10 +43,17 @@ template <> struct Vec4<__nv_bfloat16> {
     }
 };
 
-__device__ __forceinline__ void store2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
-__device__ __forceinline__ void store2(__nv_bfloat16* p, float a, float b) {
-    *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
+__device__ __forceinline__ void store_row(float* p, const float2 (&y)[1]) { *reinterpret_cast<float2*>(p) = y[0]; }
+__device__ __forceinline__ void store_row(float* p, const float2 (&y)[2]) { *reinterpret_cast<float4*>(p) = make_float4(y[0].x, y[0].y, y[1].x, y[1].y); }
+__device__ __forceinline__ void store_row(__nv_bfloat16* p, const float2 (&y)[1]) { *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(y[0].x, y[0].y); }
+__device__ __forceinline__ void store_row(__nv_bfloat16* p, const float2 (&y)[2]) {
+    const __nv_bfloat162 z[2] = {__floats2bfloat162_rn(y[0].x, y[0].y), __floats2bfloat162_rn(y[1].x, y[1].y)};
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&z[0]), *reinterpret_cast<const uint32_t*>(&z[1]));
 }
+// Operands of __ffma2_rn: one instruction for two fp32 FMAs, each rounded as fmaf rounds it.
+__device__ __forceinline__ float2 lo(const float4& x) { return make_float2(x.x, x.y); }
+__device__ __forceinline__ float2 hi(const float4& x) { return make_float2(x.z, x.w); }
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
 
 constexpr int DVS = 32;      // d_v columns per CTA
 
@@ -65,15 +73,33 @@ template <int D, int C> struct Layout {
 
 }  // namespace
 
+// acc[a][columns] += sum_e x[a][e] y[e][columns], tiles of 4 rows and 2 NB columns
+template <int NB> __device__ __forceinline__ void tile_fma(float2 (&acc)[4][NB], const float4 (&x)[4], const float2 (&y)[4][NB]) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const float xe[4] = {x[a].x, x[a].y, x[a].z, x[a].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) acc[a][b] = __ffma2_rn(both(xe[e]), y[e][b], acc[a][b]);
+    }
+}
+__device__ __forceinline__ void load_row(const float* p, float2 (&y)[1]) { y[0] = *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ void load_row(const float* p, float2 (&y)[2]) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    y[0] = lo(x); y[1] = hi(x);
+}
+
 // 4 D threads.  In the state update a thread owns a 4 x 4 tile of one state (in registers across the chunk loop, with a
-// copy in shared memory for the readout); in the readout two neighbouring lanes share 4 rows x 2 columns of the
-// output, one lane per state when D = 128.  Q K^T is recomputed per slab (D / 32 times).
+// copy in shared memory for the readout); in the readout two neighbouring lanes share a tile of the output, one
+// per state.  Q K^T is recomputed per slab (D / 32 times).
 template <int D, int C, typename T>
 __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams p, const int segs) {
     using L = Layout<D, C>;
     using V4 = Vec4<T>;
     constexpr int SLABS = D / DVS, VP = L::VP, CP = L::CP, NT = 4 * D;
-    constexpr int SPLIT = D / 64;            // lanes that share a score tile or an output tile
+    constexpr int SPLIT = D / 64;            // lanes that share a score tile
+    constexpr int NB = 2 / SPLIT, MW = 2 * NB;      // columns of an output tile, in pairs and in all
     extern __shared__ __align__(16) float smem[];
     float *Qs = smem + L::Q, *Ks = smem + L::K, *Vs = smem + L::V, *Ps = smem + L::P, *Ss = smem + L::S;
     float *bb = smem + L::BB, *rowf = smem + L::ROWF, *ww = smem + L::WW;
@@ -202,29 +228,31 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
     };
     // S <- a S + (K (.) w)^T V on this thread's tile
     auto update = [&]() {
-        float u[4][4];
+        float2 u[4][2];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) u[a][b] = 0.f;
+        for (int a = 0; a < 4; ++a) u[a][0] = u[a][1] = both(0.f);
         const float* w = ww + si * C;
-#pragma unroll 4
-        for (int t = 0; t < C; ++t) {
-            const float4 kv = *reinterpret_cast<const float4*>(Ks + L::qk(t, k0));
-            const float4 vv = *reinterpret_cast<const float4*>(Vs + t * VP + n0);
-            const float wt = w[t];
-            const float ka[4] = {kv.x * wt, kv.y * wt, kv.z * wt, kv.w * wt};
-            const float va[4] = {vv.x, vv.y, vv.z, vv.w};
+#pragma unroll 2
+        for (int t0 = 0; t0 < C; t0 += 4) {
+            const float4 w4 = *reinterpret_cast<const float4*>(w + t0);
+            const float we[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int e = 0; e < 4; ++e) {
+                const float4 kv = *reinterpret_cast<const float4*>(Ks + L::qk(t0 + e, k0));
+                const float4 vv = *reinterpret_cast<const float4*>(Vs + (t0 + e) * VP + n0);
+                const float ka[4] = {kv.x * we[e], kv.y * we[e], kv.z * we[e], kv.w * we[e]};
 #pragma unroll
-                for (int b = 0; b < 4; ++b) u[a][b] = fmaf(ka[a], va[b], u[a][b]);
+                for (int a = 0; a < 4; ++a) {
+                    u[a][0] = __ffma2_rn(both(ka[a]), lo(vv), u[a][0]);
+                    u[a][1] = __ffma2_rn(both(ka[a]), hi(vv), u[a][1]);
+                }
+            }
         }
         const float ad = a_dec[si];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) s[a][b] = fmaf(ad, s[a][b], u[a][b]);
+            for (int b = 0; b < 4; ++b) s[a][b] = fmaf(ad, s[a][b], (b & 1) ? u[a][b >> 1].y : u[a][b >> 1].x);
     };
     auto publish = [&]() {      // the tile -> its place in shared memory
 #pragma unroll
@@ -244,11 +272,12 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
             if (r * (r + 1) / 2 > tile) --r;
             if ((r + 1) * (r + 2) / 2 <= tile) ++r;
             const int j0 = 4 * r, s0 = 4 * (tile - r * (r + 1) / 2);
+            float2 acc2[4][4];      // sums over even and odd columns
             float acc[4][4];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+                for (int b = 0; b < 4; ++b) acc2[a][b] = both(0.f);
 #pragma unroll 2
             for (int kk = 4 * part; kk < D; kk += 4 * SPLIT) {
                 float4 qv[4], kv[4];
@@ -260,12 +289,14 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        acc[a][b] = fmaf(qv[a].x, kv[b].x, acc[a][b]);
-                        acc[a][b] = fmaf(qv[a].y, kv[b].y, acc[a][b]);
-                        acc[a][b] = fmaf(qv[a].z, kv[b].z, acc[a][b]);
-                        acc[a][b] = fmaf(qv[a].w, kv[b].w, acc[a][b]);
+                        acc2[a][b] = __ffma2_rn(lo(qv[a]), lo(kv[b]), acc2[a][b]);
+                        acc2[a][b] = __ffma2_rn(hi(qv[a]), hi(kv[b]), acc2[a][b]);
                     }
             }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] = acc2[a][b].x + acc2[a][b].y;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
                 if (SPLIT > 1) {
@@ -377,66 +408,49 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
         }
         ahead = false;
         __syncthreads();
-        // ---- outputs: 4 rows x 2 columns; with SPLIT = 2 lane `part` reads out state `part` and takes every other 4 columns of P
-        for (int it = tid; it < (C / 4) * (DVS / 2) * SPLIT; it += NT) {
-            const int part = it % SPLIT, tile = it / SPLIT;
-            const int j0 = (tile / (DVS / 2)) * 4, m0 = (tile % (DVS / 2)) * 2;
-            float acc[4][2];
+        // ---- outputs: tiles of 4 rows x 4 columns (x 2 when D = 128), shared by two lanes, one per state, which also take turns in the
+        // columns of P
+        for (int it = tid; it < (C / 4) * (DVS / MW) * 2; it += NT) {
+            const int st = it & 1, tile = it >> 1;
+            const int j0 = (tile / (DVS / MW)) * 4, m0 = (tile % (DVS / MW)) * MW;
+            float2 acc[4][NB];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = 0.f;
+            for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int i = 0; i < 2 / SPLIT; ++i) {
-                const int st = SPLIT > 1 ? part : i;
-                const float* S = Ss + st * D * VP + m0;
-                float r[4][2];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) r[a][0] = r[a][1] = 0.f;
+                for (int b = 0; b < NB; ++b) acc[a][b] = both(0.f);
+            const float* S = Ss + st * D * VP + m0;
 #pragma unroll 2
-                for (int kk = 0; kk < D; kk += 4) {
-                    float4 qv[4];
-                    float2 x[4];
+            for (int kk = 0; kk < D; kk += 4) {
+                float4 qv[4];
+                float2 x[4][NB];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + L::qk(j0 + a, kk));
+                for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + L::qk(j0 + a, kk));
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float2*>(S + (kk + e) * VP);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) {
-                        r[a][0] = fmaf(qv[a].x, x[0].x, r[a][0]); r[a][1] = fmaf(qv[a].x, x[0].y, r[a][1]);
-                        r[a][0] = fmaf(qv[a].y, x[1].x, r[a][0]); r[a][1] = fmaf(qv[a].y, x[1].y, r[a][1]);
-                        r[a][0] = fmaf(qv[a].z, x[2].x, r[a][0]); r[a][1] = fmaf(qv[a].z, x[2].y, r[a][1]);
-                        r[a][0] = fmaf(qv[a].w, x[3].x, r[a][0]); r[a][1] = fmaf(qv[a].w, x[3].y, r[a][1]);
-                    }
-                }
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float f = rowf[st * C + j0 + a];
-                    acc[a][0] = fmaf(f, r[a][0], acc[a][0]); acc[a][1] = fmaf(f, r[a][1], acc[a][1]);
-                }
+                for (int e = 0; e < 4; ++e) load_row(S + (kk + e) * VP, x[e]);
+                tile_fma(acc, qv, x);
             }
-            for (int t = 4 * part; t < j0 + 4; t += 4 * SPLIT) {  // masked scores are 0 beyond the diagonal tile
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < NB; ++b) acc[a][b] = __fmul2_rn(both(rowf[st * C + j0 + a]), acc[a][b]);
+            for (int t = 4 * st; t < j0 + 4; t += 8) {  // masked scores are 0 beyond the diagonal tile
                 float4 pv[4];
-                float2 vv[4];
+                float2 x[4][NB];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) pv[a] = *reinterpret_cast<const float4*>(Ps + (j0 + a) * CP + t);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) vv[e] = *reinterpret_cast<const float2*>(Vs + (t + e) * VP + m0);
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    acc[a][0] = fmaf(pv[a].x, vv[0].x, acc[a][0]); acc[a][1] = fmaf(pv[a].x, vv[0].y, acc[a][1]);
-                    acc[a][0] = fmaf(pv[a].y, vv[1].x, acc[a][0]); acc[a][1] = fmaf(pv[a].y, vv[1].y, acc[a][1]);
-                    acc[a][0] = fmaf(pv[a].z, vv[2].x, acc[a][0]); acc[a][1] = fmaf(pv[a].z, vv[2].y, acc[a][1]);
-                    acc[a][0] = fmaf(pv[a].w, vv[3].x, acc[a][0]); acc[a][1] = fmaf(pv[a].w, vv[3].y, acc[a][1]);
-                }
+                for (int e = 0; e < 4; ++e) load_row(Vs + (t + e) * VP + m0, x[e]);
+                tile_fma(acc, pv, x);
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                if (SPLIT > 1) {
-                    acc[a][0] += __shfl_xor_sync(0xffffffffu, acc[a][0], 1);
-                    acc[a][1] += __shfl_xor_sync(0xffffffffu, acc[a][1], 1);
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    acc[a][b].x += __shfl_xor_sync(0xffffffffu, acc[a][b].x, 1);
+                    acc[a][b].y += __shfl_xor_sync(0xffffffffu, acc[a][b].y, 1);
                 }
                 const int j = j0 + a;
-                if (a / (4 / SPLIT) == part && j < valid)
-                    store2(og + ((size_t)(t_begin + c0 + j) * p.H + h) * D + col0 + m0, acc[a][0], acc[a][1]);
+                if (a / 2 == st && j < valid) store_row(og + ((size_t)(t_begin + c0 + j) * p.H + h) * D + col0 + m0, acc[a]);
             }
         }
         if (c_end < nchunks && c + 1 == c_end) break;      // not the last segment: its final state is nobody's
@@ -449,11 +463,12 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
     }
 }
 
-// Segments per sequence: while a doubling still fits the SMs twice over (the extra pass over K and V for the summaries costs
-// less than idle SMs) and leaves every segment a chunk of the longest sequence.
-static int plan_segments(long long units, int max_chunks) {
+// Segments per sequence: while a doubling still fits on the device at once (two CTAs per SM with D = 64, one with 128) (the extra pass over K and V for the summaries costs
+// less than idle SMs) and some segment has more than one chunk of the longest sequence (three chunks take four segments,
+// one of them empty: T = 130, 2 heads of 64: 34 us with two).
+static int plan_segments(long long units, int max_chunks, int per_sm) {
     int segs = 1;
-    while (segs < 8 && units * segs * 2 <= 2 * 148 && segs * 2 <= max_chunks) segs *= 2;
+    while (segs < 8 && units * segs * 2 <= per_sm * 148 && segs < max_chunks) segs *= 2;
     return segs;
 }
 
@@ -462,7 +477,7 @@ static dsla_status launch_one(const PrefillParams& p, cudaStream_t s) {
     constexpr size_t smem = sizeof(float) * Layout<D, C>::END;
     if (cudaFuncSetAttribute(prefill_simt_kernel<D, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DSLA_ERR_CUDA;
     const long long units = (long long)p.N * p.H * (D / DVS);
-    const int segs = plan_segments(units, p.max_chunks);
+    const int segs = plan_segments(units, p.max_chunks, D == 64 ? 2 : 1);
     if (units * segs > 0x7fffffffLL) return DSLA_ERR_UNSUPPORTED;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(units * segs));
