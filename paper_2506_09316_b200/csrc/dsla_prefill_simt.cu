@@ -15,7 +15,7 @@
 // first accumulates its own state from zero (K and V only) and leaves it, with the product of its gates, in its
 // shared memory; after a cluster barrier the initial states are folded out of the summaries through distributed
 // shared memory and every CTA runs its chunks.  No scratch in global memory, no second launch.
-// 4 heads of 64, T = 512, fp32: 17 us, 106 us with one CTA per slab.  Bound by shared-memory reads, FMA issue and the barriers between
+// 4 heads of 64, T = 512, fp32: 16 us, 106 us with one CTA per slab.  Bound by shared-memory reads, FMA issue and the barriers between
 // the steps of a chunk: the 4 x 4 tiles of the update, the scores and the outputs do 8 packed FMAs (two products each) per two
 // 16-byte reads.  Scalar FMAs, and output tiles of 4 x 2, took 18; scores behind the fold instead of under its barriers 21.
 #include "dsla_internal.cuh"
@@ -92,9 +92,9 @@ __device__ __forceinline__ void load_row(const float* p, float2 (&y)[2]) {
 
 // 4 D threads.  In the state update a thread owns a 4 x 4 tile of one state (in registers across the chunk loop, with a
 // copy in shared memory for the readout); in the readout two neighbouring lanes share a tile of the output, one
-// per state.  Q K^T is recomputed per slab (D / 32 times).
+// per state.  Q K^T is recomputed per slab (D / 32 times).  D = 64: two CTAs per SM (16 heads, T = 512: 45 us with one).
 template <int D, int C, typename T>
-__global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams p, const int segs) {
+__global__ void __launch_bounds__(4 * D, D == 64 ? 2 : 1) prefill_simt_kernel(const PrefillParams p, const int segs) {
     using L = Layout<D, C>;
     using V4 = Vec4<T>;
     constexpr int SLABS = D / DVS, VP = L::VP, CP = L::CP, NT = 4 * D;
@@ -307,19 +307,29 @@ __global__ void __launch_bounds__(4 * D) prefill_simt_kernel(const PrefillParams
             }
         }
     };
-    // ---- decay mask, one element per thread and round (the tiles above keep half of the threads busy, this all of them)
+    // ---- decay mask: a thread keeps to one column, four rows at a time, so that the loads and exponentials of four elements overlap
+    // (one element after the other: 6800 cycles)
     auto mask = [&]() {
-#pragma unroll 2
-        for (int idx = tid; idx < C * C; idx += NT) {
-            const int j = idx / C, t = idx % C;
-            if (t <= (j | 3)) {
-                float m = 0.f;
-                if (t <= j) {
-                    const float d1 = (zc[j] == zc[t]) ? expf(bb[j] - bb[t]) : 0.f;
-                    const float d2 = (zc[C + j] == zc[C + t]) ? expf(bb[C + j] - bb[C + t]) : 0.f;
-                    m = W1 * d1 + W2 * d2;
-                }
-                Ps[j * CP + t] *= m;
+        constexpr int JS = NT / C;      // rows apart
+        const int t = tid % C;
+        const float b1 = bb[t], b2 = bb[C + t];
+        const int z1 = zc[t], z2 = zc[C + t];
+#pragma unroll 1
+        for (int j0 = tid / C; j0 < C; j0 += 4 * JS) {
+            if (t > ((j0 + 3 * JS) | 3)) continue;
+            float x[4], m[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = min(j0 + e * JS, C - 1);
+                x[e] = Ps[j * CP + t];
+                const float d1 = zc[j] == z1 ? expf(bb[j] - b1) : 0.f;
+                const float d2 = zc[C + j] == z2 ? expf(bb[C + j] - b2) : 0.f;
+                m[e] = t <= j ? W1 * d1 + W2 * d2 : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = j0 + e * JS;
+                if (j < C && t <= (j | 3)) Ps[j * CP + t] = x[e] * m[e];
             }
         }
     };
