@@ -221,7 +221,12 @@ static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cu
     }
     const dsla_impl impl = resolve_impl(a);
     if (impl != DSLA_IMPL_SIMT) return launch_prefill_tc(p, a, impl == DSLA_IMPL_TENSOR_PAIR, s);
-    return launch_prefill_simt(p, a->d_k, chunk, a->dtype, s);
+    // A batch of sequences that fit in half a chunk takes shorter chunks (the kernel computes whole ones: T = 32, 2 heads of 64, 13.4 us
+    // with chunks of 64).
+    int fit = chunk;
+    while (fit > 16 && a->max_seqlen <= fit / 2) fit /= 2;
+    p.max_chunks = (a->max_seqlen + fit - 1) / fit;
+    return launch_prefill_simt(p, a->d_k, fit, a->dtype, s);
 }
 
 }  // extern "C"

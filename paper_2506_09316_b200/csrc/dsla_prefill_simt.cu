@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(4 * D, D == 64 ? 2 : 1) prefill_simt_kernel(co
 #pragma unroll
         for (int a = 0; a < 4; ++a) u[a][0] = u[a][1] = both(0.f);
         const float* w = ww + si * C;
-#pragma unroll 2
+#pragma unroll 4
         for (int t0 = 0; t0 < C; t0 += 4) {
             const float4 w4 = *reinterpret_cast<const float4*>(w + t0);
             const float we[4] = {w4.x, w4.y, w4.z, w4.w};

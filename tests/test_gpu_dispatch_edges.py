@@ -54,6 +54,20 @@ def test_simt_prefill_segments(lens, H, d, dtype, chunk, resume):
     assert rel_err(o, o_ref) <= TOL[dtype] and rel_err(S[slots], S_ref[slots]) <= TOL[torch.float32]
 
 
+# Short sequences take chunks of 16 and 32 tokens: both sides of each line, a packed batch whose longest sequence decides
+@pytest.mark.parametrize("lens,H,d", [((1,), 2, 64), ((16,), 3, 64), ((17,), 2, 128), ((32,), 4, 128), ((33,), 2, 64), ((9, 0, 31), 2, 64)])
+def test_simt_prefill_short(lens, H, d):
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, gpu_prefill, oracle_prefill, rel_err
+    inp = gen.make_packed(5600 + sum(lens) + d, lens, H, d, torch.float32)
+    inp.g_rec[5::7] = 0.0
+    slots = np.arange(len(lens), dtype=np.int32)
+    state0 = gen.make_states(5601, len(lens), H, d, d, std=0.5).numpy()
+    o, S = gpu_prefill(inp, num_slots=len(lens), state0=state0, slots=slots, scale=0.8)
+    o_ref, S_ref = oracle_prefill(inp, state0=state0.astype(np.float64), slots=slots, scale=0.8)
+    assert rel_err(o, o_ref) <= TOL[torch.float32] and rel_err(S, S_ref) <= TOL[torch.float32]
+
+
 # Gates per key channel on the tensor cores: whole and ragged chunks of 32 tokens, one token past a block, several segments (with the
 # workspace dsla_prefill brings) and one (impl="auto" without room), exact zeros and ones, sequences shorter than a segment
 @pytest.mark.parametrize("lens,H,resume", [((1,), 2, False), ((16,), 1, True), ((17,), 3, False), ((32,), 2, True), ((33, 31, 0, 64), 2, True),
