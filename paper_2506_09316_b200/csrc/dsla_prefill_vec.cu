@@ -12,15 +12,19 @@
 // 16-token block are fp32 on CUDA cores, those between the chunk's two blocks are products of two-term operands scaled
 // to the block boundary.
 //
+// The tensor core cuts its fp32 sums off instead of rounding them: every MMA onto a state would move it by up to an ulp, always
+// towards zero (six per chunk: states off by 1.5e-6 after 4096 tokens, 3.4e-7 token by token).  So what a chunk adds to a
+// state, V^T (s_i (.) K), is a sum of its own from zero, smallest terms first, and is added on CUDA cores.
+//
 // CTA = (sequence, head, segment), 16 warps in step: each step takes one state through its pass (two bf16 terms of it for the
 // readout, then S_i diag(A_i)) and its MMAs, and meanwhile builds the operands of the other state for its next turn, so
 // nothing but the raw inputs is double-buffered.  Bound by instruction issue: 7000 warp instructions per chunk and SM
-// sub-partition, half of them for the operands, a quarter for the scores; 15.8 k cycles per chunk.
+// sub-partition, half of them for the operands, a quarter for the scores; 16.7 k cycles per chunk.
 //
 // A sequence is split into segments when there are few (sequence, head) pairs and the caller's workspace has room: a first
 // grid accumulates each segment's state from zero, walking the chunks backwards with the product of all later gates (no pass
 // over the states), and the main grid folds the summaries of the earlier segments into its initial states.
-// T = 4096, 32 heads: 280 us (of them 60 for the summaries); 2490 us with the token-by-token kernel.
+// T = 4096, 32 heads: 300 us (of them 64 for the summaries; 280 with the MMAs onto the states); 2490 us with the token-by-token kernel.
 #include "dsla_prefill_tc.cuh"
 
 namespace dsla {
@@ -50,8 +54,9 @@ constexpr int OFF_SKT = 2 * V_TILE;
 constexpr int OFF_SG = OFF_SKT + 12 * V_TILE;        // gates [parity][state][32][128] fp32
 constexpr int OFF_SK = OFF_SG + 2 * V_GBYTES;        // raw K [parity]
 constexpr int V_SMEM_SUM = OFF_SK + 2 * V_TILE + 1024;
-// TMEM columns
-constexpr uint32_t VCOL_S = 0, VCOL_SB = 256, VCOL_O = 384;      // fp32 states 2 x 128, bf16 terms of one state 2 x 64, O^T 32
+// TMEM columns: fp32 states 2 x 128; the bf16 terms of one state, per 32 key channels 16 columns of high ones, then 16 of low ones, and when the
+// readout has read them what the chunk adds to that state, fp32 (so that each warp overwrites only columns it has read); O^T 32
+constexpr uint32_t VCOL_S = 0, VCOL_SB = 256, VCOL_O = 384;
 constexpr size_t VEC_STRIDE = (2 * D * D + 2 * D) * sizeof(float);      // one summary: U[2][d][d], A[2][d]
 
 struct VecParams {
@@ -61,7 +66,7 @@ struct VecParams {
 };
 
 struct alignas(16) VecShared {
-    uint64_t raw_full[2], done[2];
+    uint64_t raw_full[2], done[2], ro;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -311,6 +316,7 @@ __device__ __forceinline__ void build_operands(uint8_t* tiles, int i, int buf, f
 __device__ __forceinline__ void vec_setup(VecShared& sh, int tid, int warp, int mma_warp) {
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) { mbar_init(&sh.raw_full[i], 1); mbar_init(&sh.done[i], 1); }
+        mbar_init(&sh.ro, 1);
         sh.abort_flag = 0;
         fence_barrier_init();
     }
@@ -380,9 +386,24 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             if (((tid >> 3) & (VC - 1)) >= valid) reinterpret_cast<uint4*>(tiles + OFF_V + b * V_TILE)[tid] = zero;
         }
     };
-    // S_i -> two bf16 terms for the readout, then S_i diag(A_i); 32 columns (key channels) of one lane quadrant per warp
-    auto pass = [&](int i) {
-        uint32_t r[32], hi[16], lo[16];
+    // S_i += d, which its last chunk added; 32 columns (key channels) of one lane quadrant per warp
+    auto merge = [&](int i, const uint32_t (&d)[32]) {
+        uint32_t r[32];
+        tmem_ld32(lane_addr + VCOL_S + 128 * i + 32 * cg, r);
+        tc_wait_ld();
+#pragma unroll
+        for (int k = 0; k < 32; k += 2) {
+            const float2 x = __fadd2_rn(make_float2(__uint_as_float(r[k]), __uint_as_float(r[k + 1])), make_float2(__uint_as_float(d[k]), __uint_as_float(d[k + 1])));
+            r[k] = __float_as_uint(x.x); r[k + 1] = __float_as_uint(x.y);
+        }
+        tmem_st32(lane_addr + VCOL_S + 128 * i + 32 * cg, r);
+        tc_wait_st();
+        tc_fence_before();
+    };
+    // S_i -> two bf16 terms for the readout, over the other state's sum (which moves into d), then S_i diag(A_i)
+    auto pass = [&](int i, bool sum, uint32_t (&d)[32]) {
+        uint32_t r[32], hl[32];
+        if (sum) tmem_ld32(lane_addr + VCOL_SB + 32 * cg, d);
         tmem_ld32(lane_addr + VCOL_S + 128 * i + 32 * cg, r);
         const float4* A = reinterpret_cast<const float4*>(tiles + OFF_A) + i * (D / 4) + 8 * cg;
         tc_wait_ld();
@@ -391,12 +412,11 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             const float4 a = A[k];
             float2 x = make_float2(__uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1])), y = make_float2(__uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
             const float2 xs = __fmul2_rn(x, make_float2(a.x, a.y)), ys = __fmul2_rn(y, make_float2(a.z, a.w));
-            hi[2 * k] = take_term(x); lo[2 * k] = pack_bf16(x.x, x.y);
-            hi[2 * k + 1] = take_term(y); lo[2 * k + 1] = pack_bf16(y.x, y.y);
+            hl[2 * k] = take_term(x); hl[16 + 2 * k] = pack_bf16(x.x, x.y);
+            hl[2 * k + 1] = take_term(y); hl[17 + 2 * k] = pack_bf16(y.x, y.y);
             r[4 * k] = __float_as_uint(xs.x); r[4 * k + 1] = __float_as_uint(xs.y); r[4 * k + 2] = __float_as_uint(ys.x); r[4 * k + 3] = __float_as_uint(ys.y);
         }
-        tmem_st16(lane_addr + VCOL_SB + 16 * cg, hi);
-        tmem_st16(lane_addr + VCOL_SB + 64 + 16 * cg, lo);
+        tmem_st32(lane_addr + VCOL_SB + 32 * cg, hl);
         tmem_st32(lane_addr + VCOL_S + 128 * i + 32 * cg, r);
         tc_wait_st();
     };
@@ -411,22 +431,27 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             if (j < valid) dst[(size_t)j * p.H * D] = __float2bfloat16_rn(__uint_as_float(r[j]));
     };
     const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    auto issue = [&](int i, int buf) {      // by one thread
-        constexpr uint32_t ID_RO = idesc_bf16(128, VC, 0, 0), ID_PV = idesc_bf16(128, VC, 1, 0), ID_U = idesc_bf16(128, 128, 1, 1);
-        const uint32_t vd = smem_desc_lo(sa + OFF_V + buf * V_TILE, V_HALF), qd = smem_desc_lo(sa + OFF_QT + 2 * i * V_TILE, 16);
-        const uint32_t kd = smem_desc_lo(sa + OFF_KT + 3 * i * V_TILE, V_HALF), pd = smem_desc_lo(sa + OFF_PT, 16);
+    auto readout = [&](int i, int buf) {      // by one thread
+        constexpr uint32_t ID_RO = idesc_bf16(128, VC, 0, 0), ID_PV = idesc_bf16(128, VC, 1, 0);
+        const uint32_t vd = smem_desc_lo(sa + OFF_V + buf * V_TILE, V_HALF), qd = smem_desc_lo(sa + OFF_QT + 2 * i * V_TILE, 16), pd = smem_desc_lo(sa + OFF_PT, 16);
 #pragma unroll 1
         for (int m = 0; m < 3; ++m) {       // low x high, high x low, high x high terms
-            const uint32_t a = VCOL_SB + (m == 0 ? 64 : 0), b = qd + (m == 1 ? V_TILE >> 4 : 0);
+            const uint32_t a = VCOL_SB + (m == 0 ? 16 : 0), b = qd + (m == 1 ? V_TILE >> 4 : 0);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) mma_ts_lo(VCOL_O, a + 8 * kk, b + (uint32_t)((kk >> 2) * (V_HALF >> 4) + 2 * (kk & 3)), ID_RO, (i | m | kk) ? 1u : 0u);
+            for (int kk = 0; kk < 8; ++kk)
+                mma_ts_lo(VCOL_O, a + 32 * (kk >> 1) + 8 * (kk & 1), b + (uint32_t)((kk >> 2) * (V_HALF >> 4) + 2 * (kk & 3)), ID_RO, (i | m | kk) ? 1u : 0u);
         }
         if (i == 1) {
 #pragma unroll
             for (int m = 0; m < 4; ++m) mma_ss_lo(VCOL_O, vd + (m & 1) * 128, pd + (uint32_t)((m >> 1) * (VC * 128 >> 4) + 2 * (m & 1)), ID_PV, 1u);
         }
+        tc_commit(&sh.ro);
+    };
+    auto update = [&](int i, int buf) {       // by one thread, behind the readout: over the terms that it has read
+        constexpr uint32_t ID_U = idesc_bf16(128, 128, 1, 1);
+        const uint32_t vd = smem_desc_lo(sa + OFF_V + buf * V_TILE, V_HALF), kd = smem_desc_lo(sa + OFF_KT + 3 * i * V_TILE, V_HALF);
 #pragma unroll
-        for (int m = 0; m < 6; ++m) mma_ss_lo(VCOL_S + 128 * i, vd + (m & 1) * 128, kd + (uint32_t)((m >> 1) * (V_TILE >> 4) + (m & 1) * 128), ID_U, 1u);
+        for (int m = 0; m < 6; ++m) mma_ss_lo(VCOL_SB, vd + (m & 1) * 128, kd + (uint32_t)((2 - (m >> 1)) * (V_TILE >> 4) + (m & 1) * 128), ID_U, m ? 1u : 0u);
         tc_commit(&sh.done[i]);
     };
 
@@ -495,18 +520,28 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
                 *reinterpret_cast<uint32_t*>(at + VC * 128) = pack_bf16(z.x, z.y);
                 fence_proxy_async_smem();
             }
-            pass(i);
+            uint32_t d[32];
+            pass(i, hs > 0, d);
             tc_fence_before();
             if (warp == 1) {      // only the issuing warp waits for the others
                 asm volatile("bar.sync 2, 512;" ::: "memory");
                 if (elect_one()) {
                     tc_fence_after();
-                    issue(i, b);
+                    readout(i, b);
                 }
                 __syncwarp();
             } else {
                 asm volatile("bar.arrive 2, 512;" ::: "memory");
             }
+            if (hs > 0) merge(i ^ 1, d);
+        }
+        if (hs >= 0 && warp == 12) {      // (one of the warps with the least to build; behind its build: 1 % of the kernel's time more)
+            WAIT(&sh.ro, hs & 1);
+            if (elect_one()) {
+                tc_fence_after();
+                update(i, b);
+            }
+            __syncwarp();
         }
         if (hs + 1 < 2 * nc) build_operands(tiles, i ^ 1, i == 0 ? b : b ^ 1, W1, W2, warp, lane);
         if (i == 0 && c + 1 < nc) {
@@ -519,6 +554,13 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
     WAIT(&sh.done[1], (nc - 1) & 1);
     tc_fence_after();
     outputs(nc - 1);
+    {
+        uint32_t d[32];
+        tmem_ld32(lane_addr + VCOL_SB + 32 * cg, d);
+        merge(1, d);
+    }
+    __syncthreads();
+    tc_fence_after();
     if (last) store_state(slot1 + (size_t)(warp >> 3) * state_stride, v, lane_addr + VCOL_S + 128 * (warp >> 3), 2 * ((warp >> 2) & 1), 2 * ((warp >> 2) & 1) + 2);
     tc_fence_before();
     __syncthreads();
@@ -529,7 +571,7 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
 // Segment summaries
 // ============================================================================================
 // U_g (both states, accumulated from zero) and A_g (products of the segment's gates) of a segment that has a successor.  Warps 0..15
-// build K~ (state, channel half, eight rows each), warp 16 loads and issues.  The first segment of a sequence that continues
+// build K~ (state, channel half, eight rows each) and add up U in registers, warp 16 loads and issues.  The first segment of a sequence that continues
 // from its slot also pushes that through its summary, and leaves a copy of it in the entry of the last segment.
 constexpr int VS_NTHREADS = 17 * 32;
 __global__ void __launch_bounds__(VS_NTHREADS, 1)
@@ -555,6 +597,23 @@ prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gr
     const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int i = warp >> 3, hh = warp & 1, rows = 8 * ((warp >> 1) & 3);
     float2 after = make_float2(1.f, 1.f);
+    // U of state warp / 8, key channels 64 ((warp / 4) % 2) .. + 63, one d_v lane per thread.  What a chunk adds to both states is a sum of
+    // its own in the TMEM columns of its parity.
+    const int q = warp & 3, ch0 = 64 * ((warp >> 2) & 1);
+    float2 U[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) U[k] = make_float2(0.f, 0.f);
+    auto merge = [&](int par) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            uint32_t r[16];
+            tmem_ld16(((uint32_t)(32 * q) << 16) + 256 * par + 128 * i + ch0 + 16 * b, r);
+            tc_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 8; ++k) U[8 * b + k] = __fadd2_rn(U[8 * b + k], make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1])));
+        }
+        tc_fence_before();
+    };
     // step it = chunk nc - 1 - it; buffers by the parity of it
     auto load = [&](int it) {      // by one thread
         const int par = it & 1, t = t0 + (nc - 1 - it) * VC;
@@ -576,7 +635,11 @@ prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gr
         } else {
             if (it > 0) after = carries[par][i][32 * hh + lane];
             WAIT(&sh.raw_full[par], (it >> 1) & 1);
-            if (it >= 2) WAIT(&sh.done[par], ((it >> 1) - 1) & 1);              // ... and those of step it - 2 this K~
+            if (it >= 2) {                                                      // ... and those of step it - 2 this K~
+                WAIT(&sh.done[par], ((it >> 1) - 1) & 1);
+                tc_fence_after();
+                merge(par);
+            }
             const float2 a = build_k<8, true>(tiles + OFF_SKT + (par * 6 + 3 * i) * V_TILE, tiles + OFF_SK + par * V_TILE + hh * 128 + lane * 4,
                                               tiles + OFF_SG + par * V_GBYTES + i * (V_GBYTES / 2) + hh * 256 + lane * 8, hh, rows, after, lane);
             if (rows == 0) carries[par ^ 1][i][32 * hh + lane] = a;
@@ -589,36 +652,37 @@ prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gr
             const uint32_t vd = smem_desc_lo(sa + OFF_V + par * V_TILE, V_HALF), kd = smem_desc_lo(sa + OFF_SKT + par * 6 * V_TILE, V_HALF);
             WAIT(&sh.raw_full[par], (it >> 1) & 1);
 #pragma unroll
-            for (int m = 0; m < 6; ++m) {       // (state, term)
-                const uint32_t d = VCOL_S + (m >= 3 ? 128 : 0), k = kd + (uint32_t)(m * (V_TILE >> 4)), fresh = (it == 0 && (m == 0 || m == 3)) ? 0u : 1u;
-                mma_ss_lo(d, vd, k, ID_U, fresh);
+            for (int m = 5; m >= 0; --m) {      // (state, term), smallest terms first
+                const uint32_t d = 256 * par + (m >= 3 ? 128 : 0), k = kd + (uint32_t)(m * (V_TILE >> 4));
+                mma_ss_lo(d, vd, k, ID_U, m % 3 == 2 ? 0u : 1u);
                 mma_ss_lo(d, vd + 128, k + 128, ID_U, 1u);
             }
             tc_commit(&sh.done[par]);
         }
         __syncwarp();
     }
+    if (nc > 1) WAIT(&sh.done[nc & 1], ((nc - 2) >> 1) & 1);
     WAIT(&sh.done[(nc - 1) & 1], ((nc - 1) >> 1) & 1);
     tc_fence_after();
     if (warp < 16) {
+        if (nc > 1) merge(nc & 1);
+        merge((nc - 1) & 1);
         const float* A = reinterpret_cast<const float*>(carries[nc & 1][i]);
-        const int q = warp & 3, v = 32 * q + lane;
+        const int v = 32 * q + lane;
         const bool from_slot = u.g == 0 && p.use_initial_state;
         const float* slot = p.state + (((size_t)u.slot * 2 + i) * p.H + u.h) * (size_t)(D * D) + v;
         float* copy = unit + (size_t)(vp.nseg - 1) * (VEC_STRIDE / 4) + (size_t)i * D * D + v;
         float* dst = out + (size_t)i * D * D + v;
-#pragma unroll 1
-        for (int k0 = 64 * ((warp >> 2) & 1), end = k0 + 64; k0 < end; k0 += 32) {
-            uint32_t r[32];
-            float x[32];
-            tmem_ld32(((uint32_t)(32 * q) << 16) + VCOL_S + 128 * i + k0, r);
 #pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = from_slot ? slot[(size_t)(k0 + k) * D] : 0.f;
-            tc_wait_ld();
+        for (int b = 0; b < 8; ++b) {
+            const int k0 = ch0 + 8 * b;
+            float x[8];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
+            for (int k = 0; k < 8; ++k) x[k] = from_slot ? slot[(size_t)(k0 + k) * D] : 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
                 if (from_slot) copy[(size_t)(k0 + k) * D] = x[k];
-                dst[(size_t)(k0 + k) * D] = fmaf(A[k0 + k], x[k], __uint_as_float(r[k]));
+                dst[(size_t)(k0 + k) * D] = fmaf(A[k0 + k], x[k], (k & 1) ? U[4 * b + (k >> 1)].y : U[4 * b + (k >> 1)].x);
             }
         }
         if (tid < 64) reinterpret_cast<float4*>(out + 2 * D * D)[tid] = reinterpret_cast<const float4*>(&carries[nc & 1][0][0])[tid];

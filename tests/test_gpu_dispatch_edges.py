@@ -96,6 +96,27 @@ def test_channel_prefill_tensor(lens, H, resume, pattern):
     assert rel_err(o, o_ref) <= 4e-3
 
 
+# The states of the tensor-core kernel for vector gates are fp32 sums like those of the token-by-token kernel, and no further from the
+# exact ones: 260 tokens in one segment, 2000 in several.
+@pytest.mark.parametrize("T,H", [(260, 4), (1100, 40), (2000, 4)])
+def test_channel_prefill_state_precision(T, H):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    from util import oracle_prefill
+    inp = gen.make_packed(5350 + T, [T], H, 128, BF)
+    rng = np.random.default_rng(5351)
+    for name, mu in (("g_hist", 6.0), ("g_rec", 1.0)):
+        g = 1.0 / (1.0 + np.exp(-rng.normal(mu, 0.5, size=(T, H, 128))))
+        setattr(inp, name, torch.from_numpy(g.astype(np.float32)))
+    dv, st = inp.to("cuda"), dsla.dsla_state_alloc(1, H, 128, 128)
+    _, S_ref = oracle_prefill(inp, state0=np.zeros((1, 2, H, 128, 128)))
+    off = {}
+    for impl in ("auto", "simt"):
+        dsla.dsla_prefill(dv.q, dv.k, dv.v, dv.g_hist, dv.g_rec, dv.gamma, st, impl=impl)
+        off[impl] = np.linalg.norm(st.tensor.double().cpu().numpy() - S_ref) / np.linalg.norm(S_ref)
+    assert off["auto"] <= off["simt"], off
+
+
 # The order in which a packed batch is visited: found inside the kernel (up to 64 sequences, one and two per lane) and by a kernel of its
 # own (more); ties and empty sequences, whole sequences and split ones
 @pytest.mark.parametrize("N,H,top", [(2, 3, 500), (31, 5, 90), (33, 4, 200), (64, 3, 70), (65, 3, 70)])
