@@ -117,6 +117,22 @@ def test_channel_prefill_state_precision(T, H):
     assert off["auto"] <= off["simt"], off
 
 
+# What a token adds to a state, w k^T v, is rounded to bf16 once (w v; the weight itself has 16 bits): at most 2^-9 of it, whether the
+# sequence is one chunk, one segment or several.
+@pytest.mark.parametrize("T,H", [(64, 8), (128, 8), (777, 4), (1500, 150)])
+def test_tensor_prefill_state_precision(T, H):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    from util import oracle_prefill
+    inp = gen.make_packed(5360 + T, [T], H, 128, BF)
+    dv, st = inp.to("cuda"), dsla.dsla_state_alloc(1, H, 128, 128)
+    dsla.dsla_prefill(dv.q, dv.k, dv.v, dv.g_hist, dv.g_rec, dv.gamma, st, impl="tensor")
+    _, S_ref = oracle_prefill(inp, state0=np.zeros((1, 2, H, 128, 128)))
+    for i in range(2):
+        S, ref = st.tensor[:, i].double().cpu().numpy(), S_ref[:, i]
+        assert np.linalg.norm(S - ref) <= 2.0 ** -9 * np.linalg.norm(ref)
+
+
 # The order in which a packed batch is visited: found inside the kernel (up to 64 sequences, one and two per lane) and by a kernel of its
 # own (more); ties and empty sequences, whole sequences and split ones
 @pytest.mark.parametrize("N,H,top", [(2, 3, 500), (31, 5, 90), (33, 4, 200), (64, 3, 70), (65, 3, 70)])
