@@ -254,7 +254,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncwarp();
-    if (SPLIT) cluster_arrive_relaxed();      // (waited for before the first use of another CTA's barriers)
+    // Cluster barrier, phase 1: every CTA's barriers are initialised (waited for before the first use of another CTA's).  Phase 2: this
+    // warp writes nothing more into other CTAs.  No CTA leaves before it is complete: a wait that gave up would otherwise let a CTA go that
+    // its neighbours still write into.  Each warp arrives as early as it can, so that nobody waits for it at the end.
+    if (SPLIT) cluster_arrive_relaxed();
+    auto started_alone = [&] {      // a warp that keeps to its own CTA: both at once
+        __syncwarp();
+        cluster_wait();
+        cluster_arrive_relaxed();
+    };
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = 0;      // all 512 columns are allocated: the base is column 0
@@ -291,6 +299,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (PAIRS) {
             __syncwarp();
             cluster_wait();
+        } else if (SPLIT) {
+            started_alone();
         }
         if (lane == 0 && nc > 0) {
             const uint32_t next_turn = PAIRS && pr + 1 < pairs ? map_to_cta(smem_u32(&sh.o_turn), (uint32_t)(cta + nseg)) : 0u;
@@ -337,6 +347,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             bulk_wait_all();
         }
+        if (PAIRS) {
+            __syncwarp();
+            cluster_arrive_relaxed();
+        }
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issuer
         // Per chunk:  O^T = S1^T Q~1^T + S2^T Q~2^T,  O^T += V^T P~^T,  S1^T += V~1^T K,  P of the next chunk,  S2^T += V~2^T K.
@@ -380,6 +394,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (nc > 0) scores(0, 0);
         }
         __syncwarp();
+        if (SPLIT) started_alone();
         if (elect_one()) {
             int c3 = 0;
 #pragma unroll 1
@@ -438,6 +453,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (half == 0 && (q == 0 || q == 2))
             for (int m4 = 0; m4 < 4; ++m4)
                 *reinterpret_cast<uint4*>(tiles + OFF_PT + (q == 2 ? HALF_BYTES - 64 * 128 : 0) + sw128_offset(j, 32 + 8 * m4)) = make_uint4(0u, 0u, 0u, 0u);
+        if (SPLIT) started_alone();
         int c3 = 0;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
@@ -587,7 +603,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0) gs.a[i] = pr;
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.g_ready[s]);
+            if (SPLIT && c == 0) started_alone();
         }
+        if (SPLIT && nc == 0) started_alone();
     } else {
         // ------------------------------------------------------------------ state warps 10..17
         const int q = warp & 3, hi = (warp - STATE_W0) >> 2;   // TMEM lane quadrant, state index
@@ -711,6 +729,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const float a = gs.a[hi];
             if (SPLIT && c == 0) {
                 chain(a);
+                __syncwarp();
+                if (!PAIRS) cluster_arrive_relaxed();
             } else if (c > 0 || !zero_start) {
                 if (c > 0) WAIT(&sh.u_full[hi], (c - 1) & 1);
                 tc_fence_after();
@@ -797,6 +817,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             v3 = v3 == 2 ? 0 : v3 + 1;
         }
+        if (SPLIT && (PAIRS || nc == 0)) {
+            __syncwarp();
+            cluster_arrive_relaxed();
+        }
         if (last && nc > 0) {
             WAIT(&sh.u_full[hi], (nc - 1) & 1);
             tc_fence_after();
@@ -804,7 +828,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
     }
     __syncwarp();
-    if (SPLIT && !(PAIRS && warp == WARP_TMA) && !(warp >= STATE_W0 && warp < GATE_W0)) cluster_wait();
+    if (SPLIT) cluster_wait();      // phase 2
     tc_fence_before();
     __syncthreads();
     if (warp == WARP_MMA) tmem_dealloc(tb, 512);

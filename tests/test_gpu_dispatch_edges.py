@@ -150,6 +150,29 @@ def test_packed_order(N, H, top):
     assert rel_err(o, o_ref) <= TOL[BF] and rel_err(S[slots], S_ref[slots]) <= TOL[BF]
 
 
+# Segments on the CTAs of a cluster, all of which leave together: batches in which segments have no chunk, one chunk or several, and a
+# sequence none at all, one launch behind the other; every run gives the same bits.
+@pytest.mark.parametrize("lens,H", [((1500, 0, 64, 777, 130), 2), ((257,), 1), ((4096, 1), 3), ((385, 2000), 17)])
+@pytest.mark.parametrize("resume", [False, True])
+def test_split_clusters_leave_together(lens, H, resume):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    from util import TOL, oracle_prefill, rel_err
+    inp = gen.make_packed(5450 + sum(lens), lens, H, 128, BF)
+    state0 = gen.make_states(5451, len(lens), H, 128, 128, std=0.5)
+    dv, st, runs = inp.to("cuda"), dsla.dsla_state_alloc(len(lens), H, 128, 128), []
+    for _ in range(20):
+        st.tensor.copy_(state0)
+        o = dsla.dsla_prefill(dv.q, dv.k, dv.v, dv.g_hist, dv.g_rec, dv.gamma, st, cu_seqlens=dv.cu_seqlens, max_seqlen=max(lens),
+                              use_initial_state=resume, impl="tensor")
+        runs.append((o, st.tensor.clone()))
+    assert dsla.dsla_state_last_error(st) == dsla.DSLA_OK
+    assert all(torch.equal(o, runs[0][0]) and torch.equal(S, runs[0][1]) for o, S in runs[1:])
+    o_ref, S_ref = oracle_prefill(inp, state0=state0.double().numpy() if resume else np.zeros(tuple(state0.shape)))
+    assert rel_err(runs[0][0].double().cpu().numpy(), o_ref) <= TOL[BF]
+    assert rel_err(runs[0][1].double().cpu().numpy(), S_ref) <= TOL[BF]
+
+
 # Pairs of states side by side in a cluster: two and four pairs, with one segment per sequence and with several (clusters of up to 16),
 # whole chunks and ragged ones, a batch of which one sequence is empty and one shorter than a segment; 75 heads: one pair at a time
 @pytest.mark.parametrize("n,lens,H,resume", [(4, (100,), 3, False), (8, (128,), 2, True), (4, (129,), 74, True), (4, (1500, 0, 64, 777), 2, True),
