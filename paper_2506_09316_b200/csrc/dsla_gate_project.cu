@@ -173,6 +173,7 @@ gate_project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     tc_fence_before();
     if (split > 1) cluster_sync_all();      // a rank's shared memory stays up until its copies have been received
     else __syncthreads();
+    settle_after_timeout(abortp);           // (behind the barrier every thread sees the flag: each stays, and with it the CTA)
     if (warp == 1) tmem_dealloc(tb, ncols);
 }
 

@@ -197,6 +197,7 @@ prefill_tc_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         tc_fence_after();
         store_state(out + (size_t)hi * D * D, 32 * q + lane, lane_addr + 128 * hi, 0, 4);
     }
+    settle_after_timeout(abortp);
     tc_fence_before();
     __syncthreads();
     if (warp == 9) tmem_dealloc(tb, 512);
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(32) bounded_wait_selftest_kernel(int* status, 
     __syncwarp();
     // a wait that starts after the abort flag is up returns on its first poll
     mbar_wait(&bar, 0, abortp, status, MBAR_WAIT_LIMIT);
+    settle_after_timeout(abortp);
 }
 
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,

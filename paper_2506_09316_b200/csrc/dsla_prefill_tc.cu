@@ -291,6 +291,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (lane == 0 && summarize) {
             for (int it = SUM_STAGES; it < nc; ++it) {
                 WAIT(&sh.s_empty[it % SUM_STAGES], (it / SUM_STAGES - 1) & 1);
+                if (*abortp) break;
                 load_summary(it);
             }
             WAIT(&sh.s_done, 0);
@@ -312,7 +313,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
             int c3 = 0;
 #pragma unroll 1
-            for (int c = 0; c < nc; ++c) {
+            for (int c = 0; c < nc && !*abortp; ++c) {
                 const int v3 = c3 == 0 ? 2 : c3 - 1;
                 if (c + 1 < nc) {
                     WAIT(&sh.ro_done, c & 1);              // Q of chunk c has been read: its slot takes V of chunk c + 1
@@ -829,6 +830,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     }
     __syncwarp();
     if (SPLIT) cluster_wait();      // phase 2
+    settle_after_timeout(abortp);
     tc_fence_before();
     __syncthreads();
     if (warp == WARP_MMA) tmem_dealloc(tb, 512);

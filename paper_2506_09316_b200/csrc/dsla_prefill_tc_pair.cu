@@ -615,6 +615,7 @@ prefill_tc_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();        // the peer may still be sending to this CTA's shared memory until it gets here too
+    settle_after_timeout(abortp);
     if (warp == WARP_Y) tmem_dealloc(tb, 512);
 }
 

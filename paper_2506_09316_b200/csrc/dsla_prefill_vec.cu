@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
                 tc_fence_after();
             }
             if (i == 0) {
-                if (warp == 15 && lane == 0 && c + 1 < nc) load_raw(c + 1);
+                if (warp == 15 && lane == 0 && c + 1 < nc && !*abortp) load_raw(c + 1);
                 __syncwarp();
                 if (c > 0) outputs(c - 1);
             } else {      // P~: two columns of one row per thread
@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
     __syncthreads();
     tc_fence_after();
     if (last) store_state(slot1 + (size_t)(warp >> 3) * state_stride, v, lane_addr + VCOL_S + 128 * (warp >> 3), 2 * ((warp >> 2) & 1), 2 * ((warp >> 2) & 1) + 2);
+    settle_after_timeout(abortp);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(0, 512);
@@ -630,7 +631,7 @@ prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gr
         if (warp == 16) {
             if (it + 1 < nc) {
                 if (it >= 1) WAIT(&sh.done[par ^ 1], ((it - 1) >> 1) & 1);      // the MMAs of step it - 1 have read V
-                if (lane == 0) load(it + 1);
+                if (lane == 0 && !*abortp) load(it + 1);
             }
         } else {
             if (it > 0) after = carries[par][i][32 * hh + lane];
@@ -687,6 +688,7 @@ prefill_vec_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gr
         }
         if (tid < 64) reinterpret_cast<float4*>(out + 2 * D * D)[tid] = reinterpret_cast<const float4*>(&carries[nc & 1][0][0])[tid];
     }
+    settle_after_timeout(abortp);
     tc_fence_before();
     __syncthreads();
     if (warp == 16) tmem_dealloc(0, 512);

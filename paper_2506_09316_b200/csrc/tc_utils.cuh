@@ -106,6 +106,15 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     return mbar_wait_slow<true>(bar, parity, abort_flag, status, limit);
 }
 
+// Before a CTA in which a wait gave up frees TMEM and leaves: copies and MMAs that are still in flight towards it land within microseconds
+// of their issue.  Every thread calls this behind its last instruction that starts one, before or behind the CTA's
+// last barrier.
+static __device__ __noinline__ void settle_after_timeout(volatile int* abort_flag) {
+    if (!*abort_flag) return;
+    const uint64_t t0 = global_timer_ns();
+    for (uint32_t i = 0; i < (1u << 20) && global_timer_ns() - t0 < 200000ull; ++i) {}
+}
+
 // ---- thread-block cluster: ranks, barrier, the peer CTA's shared memory ---------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
