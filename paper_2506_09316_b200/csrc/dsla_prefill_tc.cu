@@ -94,6 +94,16 @@ __device__ __forceinline__ void issue4_ts(uint32_t d, uint32_t a, uint32_t b, ui
     for (uint32_t k = 0; k < 4; ++k) mma_ts_lo(d, a + 8 * k, b + k * BSTEP, idesc, k ? 1u : acc);
 }
 
+// Rows valid .. CM - 1 of a K and a V tile, by 256 threads (cold path, out of line).
+__device__ __noinline__ void zero_rows(uint8_t* kt, uint8_t* vt, int valid, int t) {
+#pragma unroll 1
+    for (int i = 16 * valid + t; i < 16 * CM; i += 256) {
+        const int at = (i & 8 ? HALF_BYTES : 0) + (i >> 4) * 128 + (i & 7) * 16;
+        *reinterpret_cast<uint4*>(kt + at) = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(vt + at) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
 // ============================================================================================
 // Main kernel
 // ============================================================================================
@@ -454,6 +464,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (half == 0 && (q == 0 || q == 2))
             for (int m4 = 0; m4 < 4; ++m4)
                 *reinterpret_cast<uint4*>(tiles + OFF_PT + (q == 2 ? HALF_BYTES - 64 * 128 : 0) + sw128_offset(j, 32 + 8 * m4)) = make_uint4(0u, 0u, 0u, 0u);
+        const int nfull = (sq.len - tok0) / CM;           // index of the ragged chunk, if there is one
         if (SPLIT) started_alone();
         int c3 = 0;
 #pragma unroll 1
@@ -463,6 +474,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             uint8_t* qs = tiles + c3 * TILE_BYTES;
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
             WAIT(&sh.kq_full[s], (c >> 1) & 1);           // the TMA writes of Q are visible to this thread
+            // Rows of K and V past the end of the sequence belong to the next one.  They would meet only zero weights, but 0 * inf is not 0.  (The
+            // scores, which may be reading K, meet them only in columns that no row of this sequence uses; V~ and the other MMAs wait for
+            // prep_ready.  Here, under the scores; ahead of prep_ready it took 1 % of a packed batch's time.)
+            if (c == nfull) {
+                WAIT(&sh.v_full[s], (c >> 1) & 1);
+                zero_rows(tiles + OFF_K + s * TILE_BYTES, tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES, sq.len - tok0 - c * CM, tt);
+            }
             // ---- scaled copies of Q, eight 16-byte pieces per thread.  The copy for state 2 is written as soon as the readout of the
             // previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
             if (c > 0) WAIT(&sh.ro_done, (c - 1) & 1);

@@ -173,6 +173,43 @@ def test_split_clusters_leave_together(lens, H, resume):
     assert rel_err(runs[0][1].double().cpu().numpy(), S_ref) <= TOL[BF]
 
 
+# The tiles of a sequence's last chunk also hold the first tokens of the next sequence, which may be anything: with infinities and NaN in q, k
+# and v of every other sequence, a sequence comes out as it does alone.
+@pytest.mark.parametrize("lens,H", [((64, 90), 2), ((100, 1), 3), ((5, 700, 129), 2), ((300, 40), 150), ((1, 200), 1)])
+@pytest.mark.parametrize("form", ["dual", "four", "channel", "f32"])
+def test_neighbour_sequences_do_not_leak(lens, H, form):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    inp = gen.make_packed(5470 + sum(lens), lens, H, 128, torch.float32 if form == "f32" else BF)
+    if form == "channel":
+        rng = np.random.default_rng(5471)
+        for name in ("g_hist", "g_rec"):
+            setattr(inp, name, torch.from_numpy(rng.uniform(0.3, 1.0, size=(inp.T_total, H, 128)).astype(np.float32)))
+    d = inp.to("cuda")
+    gates, w = torch.stack([d.g_hist, d.g_rec, d.g_hist, d.g_rec]), torch.full((H, 4), 0.25, device="cuda")
+    cu = [0] + list(np.cumsum(lens))
+
+    def run(q, k, v):
+        st = dsla.dsla_state_alloc_n(len(lens), 4, H, 128, 128) if form == "four" else dsla.dsla_state_alloc(len(lens), H, 128, 128)
+        kw = dict(cu_seqlens=d.cu_seqlens, max_seqlen=max(lens))
+        if form == "four":
+            o = dsla.dsla_nstate_prefill(q, k, v, gates, w, st, **kw)
+        else:
+            o = dsla.dsla_prefill(q, k, v, d.g_hist, d.g_rec, d.gamma, st, **kw)
+        assert dsla.dsla_state_last_error(st) == dsla.DSLA_OK
+        return o, st.tensor
+
+    o0, S0 = run(d.q, d.k, d.v)
+    assert bool(torch.isfinite(o0).all()) and bool(torch.isfinite(S0).all())
+    for keep in range(len(lens)):
+        dirty = [x.clone() for x in (d.q, d.k, d.v)]
+        for x, bad in zip(dirty, (float("nan"), float("inf"), float("nan"))):
+            x[:cu[keep]] = bad
+            x[cu[keep + 1]:] = bad
+        o, S = run(*dirty)
+        assert torch.equal(o[cu[keep]:cu[keep + 1]], o0[cu[keep]:cu[keep + 1]]) and torch.equal(S[keep], S0[keep])
+
+
 # Pairs of states side by side in a cluster: two and four pairs, with one segment per sequence and with several (clusters of up to 16),
 # whole chunks and ragged ones, a batch of which one sequence is empty and one shorter than a segment; 75 heads: one pair at a time
 @pytest.mark.parametrize("n,lens,H,resume", [(4, (100,), 3, False), (8, (128,), 2, True), (4, (129,), 74, True), (4, (1500, 0, 64, 777), 2, True),
