@@ -69,6 +69,7 @@ struct alignas(16) VecShared {
     uint64_t raw_full[2], done[2], ro;
     uint32_t tmem_base;
     int abort_flag;
+    int inf_in_v[4];     // [chunk % 4]: chunk + 1 if V of the chunk holds an infinity or NaN
 };
 
 // bf16 terms of a pair of fp32 values; x is left with what the term does not hold
@@ -313,10 +314,31 @@ __device__ __forceinline__ void build_operands(uint8_t* tiles, int i, int buf, f
     }
 }
 
+// Outputs of a chunk whose V holds an infinity or NaN (cold path, out of line).  A product with P~ would carry that to the tokens before
+// it, whose weight for it is 0: O^T from the states alone, and V of the tokens up to each one added here.
+__device__ __noinline__ void outputs_by_hand(const uint8_t* tiles, int buf, __nv_bfloat16* o, int H, int valid, int warp, int lane) {
+    const int v = 32 * (warp & 3) + lane, j0 = 8 * (warp >> 2);
+    const float* sc = reinterpret_cast<const float*>(tiles + OFF_SC) + buf * VC * VC;
+    const uint8_t* vt = tiles + OFF_V + buf * V_TILE + (v >> 6) * V_HALF + (v & 7) * 2;
+    uint32_t r[8];
+    tmem_ld8(((uint32_t)(32 * (warp & 3)) << 16) + VCOL_O + j0, r);
+    tc_wait_ld();
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int j = j0 + e;
+        float x = __uint_as_float(r[e]);
+#pragma unroll 1
+        for (int s = 0; s <= j; ++s)
+            x = fmaf(sc[j * VC + s], __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(vt + s * 128 + ((((v & 63) >> 3) ^ (s & 7)) << 4))), x);
+        if (j < valid) o[(size_t)j * H * D + v] = __float2bfloat16_rn(x);
+    }
+}
+
 __device__ __forceinline__ void vec_setup(VecShared& sh, int tid, int warp, int mma_warp) {
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) { mbar_init(&sh.raw_full[i], 1); mbar_init(&sh.done[i], 1); }
         mbar_init(&sh.ro, 1);
+        for (int i = 0; i < 4; ++i) sh.inf_in_v[i] = 0;
         sh.abort_flag = 0;
         fence_barrier_init();
     }
@@ -385,6 +407,8 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             }
             if (((tid >> 3) & (VC - 1)) >= valid) reinterpret_cast<uint4*>(tiles + OFF_V + b * V_TILE)[tid] = zero;
         }
+        const uint4 y = reinterpret_cast<const uint4*>(tiles + OFF_V + b * V_TILE)[tid];      // (this thread's own piece in both cases)
+        if (hfma2_u32(y.x, 0u, hfma2_u32(y.y, 0u, hfma2_u32(y.z, 0u, hmul2_u32(y.w, 0u)))) & 0x7fff7fffu) sh.inf_in_v[c & 3] = c + 1;
     };
     // S_i += d, which its last chunk added; 32 columns (key channels) of one lane quadrant per warp
     auto merge = [&](int i, const uint32_t (&d)[32]) {
@@ -431,7 +455,8 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             if (j < valid) dst[(size_t)j * p.H * D] = __float2bfloat16_rn(__uint_as_float(r[j]));
     };
     const uint32_t sa = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    auto readout = [&](int i, int buf) {      // by one thread
+    auto inf_in_v = [&](int c) { return sh.inf_in_v[c & 3] == c + 1; };
+    auto readout = [&](int i, int buf, bool with_v) {      // by one thread
         constexpr uint32_t ID_RO = idesc_bf16(128, VC, 0, 0), ID_PV = idesc_bf16(128, VC, 1, 0);
         const uint32_t vd = smem_desc_lo(sa + OFF_V + buf * V_TILE, V_HALF), qd = smem_desc_lo(sa + OFF_QT + 2 * i * V_TILE, 16), pd = smem_desc_lo(sa + OFF_PT, 16);
 #pragma unroll 1
@@ -441,7 +466,7 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
             for (int kk = 0; kk < 8; ++kk)
                 mma_ts_lo(VCOL_O, a + 32 * (kk >> 1) + 8 * (kk & 1), b + (uint32_t)((kk >> 2) * (V_HALF >> 4) + 2 * (kk & 3)), ID_RO, (i | m | kk) ? 1u : 0u);
         }
-        if (i == 1) {
+        if (i == 1 && with_v) {
 #pragma unroll
             for (int m = 0; m < 4; ++m) mma_ss_lo(VCOL_O, vd + (m & 1) * 128, pd + (uint32_t)((m >> 1) * (VC * 128 >> 4) + 2 * (m & 1)), ID_PV, 1u);
         }
@@ -508,9 +533,14 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
                 tc_fence_after();
             }
             if (i == 0) {
+                const bool by_hand = c > 0 && inf_in_v(c - 1);
+                if (by_hand) {      // before the next V takes the place of that one
+                    outputs_by_hand(tiles, b ^ 1, og + ((size_t)(t0 + (c - 1) * VC) * p.H + u.h) * D, p.H, VC, warp, lane);
+                    __syncthreads();
+                }
                 if (warp == 15 && lane == 0 && c + 1 < nc && !*abortp) load_raw(c + 1);
                 __syncwarp();
-                if (c > 0) outputs(c - 1);
+                if (c > 0 && !by_hand) outputs(c - 1);
             } else {      // P~: two columns of one row per thread
                 const int j = tid >> 4, s = (tid & 15) * 2;
                 const float2 x = *reinterpret_cast<const float2*>(tiles + OFF_SC + (b * VC * VC + j * VC + s) * 4);
@@ -527,7 +557,7 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
                 asm volatile("bar.sync 2, 512;" ::: "memory");
                 if (elect_one()) {
                     tc_fence_after();
-                    readout(i, b);
+                    readout(i, b, !inf_in_v(c));
                 }
                 __syncwarp();
             } else {
@@ -553,7 +583,8 @@ __global__ void __launch_bounds__(V_NTHREADS, 1) prefill_vec_kernel(const __grid
     }
     WAIT(&sh.done[1], (nc - 1) & 1);
     tc_fence_after();
-    outputs(nc - 1);
+    if (inf_in_v(nc - 1)) outputs_by_hand(tiles, (nc - 1) & 1, og + ((size_t)(t0 + (nc - 1) * VC) * p.H + u.h) * D, p.H, u.len - tok0 - (nc - 1) * VC, warp, lane);
+    else outputs(nc - 1);
     {
         uint32_t d[32];
         tmem_ld32(lane_addr + VCOL_SB + 32 * cg, d);

@@ -210,6 +210,41 @@ def test_neighbour_sequences_do_not_leak(lens, H, form):
         assert torch.equal(o[cu[keep]:cu[keep + 1]], o0[cu[keep]:cu[keep + 1]]) and torch.equal(S[keep], S0[keep])
 
 
+# Token by token, an infinity or NaN in v reaches no output before it.  Its chunk's products are matrix products with zeros for the tokens
+# before it, and 0 * inf is not 0: at the first and last rows of a chunk of 32 and of its blocks of 16, in the ragged last chunk, in the
+# last one but one, in a later segment; o before it and every other column as without it, the states non-finite in that column alone.
+@pytest.mark.parametrize("T,H,at", [(40, 2, (0,)), (64, 3, (31, 40)), (97, 1, (16, 47, 96)), (700, 2, (350, 699)), (333, 160, (200,))])
+@pytest.mark.parametrize("bad", [float("nan"), float("-inf")])
+def test_channel_prefill_is_causal_in_v(T, H, at, bad):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    inp = gen.make_packed(5480 + T, [T], H, 128, BF)
+    rng = np.random.default_rng(5481)
+    for name in ("g_hist", "g_rec"):
+        setattr(inp, name, torch.from_numpy(rng.uniform(0.3, 1.0, size=(T, H, 128)).astype(np.float32)))
+    d = inp.to("cuda")
+
+    def run(v):
+        st = dsla.dsla_state_alloc(1, H, 128, 128)
+        o = dsla.dsla_prefill(d.q, d.k, v, d.g_hist, d.g_rec, d.gamma, st)
+        assert dsla.dsla_state_last_error(st) == dsla.DSLA_OK
+        return o, st.tensor
+
+    o0, S0 = run(d.v)
+    for t in at:
+        v, col = d.v.clone(), (37 * t) % 128
+        v[t, H - 1, col] = bad
+        o, S = run(v)
+        hit = torch.zeros_like(o, dtype=torch.bool)
+        hit[t:, H - 1, col] = True
+        assert not bool(torch.isfinite(o[hit]).any())
+        # the chunk's other outputs add fp32 scores instead of two bf16 terms of them: one rounding of the output apart
+        assert bool(torch.isfinite(o[~hit]).all())
+        assert float((o.float() - o0.float())[~hit].abs().max()) <= 2.0 ** -8 * float(o0.float().abs().max())
+        rest = [c for c in range(128) if c != col]
+        assert torch.equal(S[:, :, :, :, rest], S0[:, :, :, :, rest]) and not bool(torch.isfinite(S[0, :, H - 1, :, col]).any())
+
+
 # Pairs of states side by side in a cluster: two and four pairs, with one segment per sequence and with several (clusters of up to 16),
 # whole chunks and ragged ones, a batch of which one sequence is empty and one shorter than a segment; 75 heads: one pair at a time
 @pytest.mark.parametrize("n,lens,H,resume", [(4, (100,), 3, False), (8, (128,), 2, True), (4, (129,), 74, True), (4, (1500, 0, 64, 777), 2, True),
