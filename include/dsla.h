@@ -137,15 +137,16 @@ typedef struct {
     size_t workspace_bytes;
     dsla_gate_layout gate_layout; /* SCALAR (0): g_hist, g_rec are [T_total, H].  PER_KEY_CHANNEL: [T_total, H, d_k];
                                    impl AUTO takes the tensor-core kernel for vector gates (bf16, d = 128, gates on 16-byte
-                                   boundaries; it needs no workspace, but with one -- the size dsla_prefill_workspace_bytes
-                                   gives for scalar gates -- it splits long sequences), else, and for impl SIMT, a token-by-token
-                                   CUDA-core kernel.  impl TENSOR and TENSOR_PAIR take scalar gates only: DSLA_ERR_UNSUPPORTED */
+                                   boundaries), else, and for impl SIMT, a token-by-token CUDA-core kernel.  The former has a use
+                                   for dsla_prefill_workspace_bytes(), 16-byte aligned, but needs none: it cuts long sequences of few
+                                   heads into as many segments as there is room for (T = 4096, 32 heads: 297 us, 903 without).    impl TENSOR and TENSOR_PAIR take scalar gates only: DSLA_ERR_UNSUPPORTED */
 } dsla_prefill_args;
 
 /* Scratch to hand over for these sizes (0 for the SIMT kernel): room for the segment summaries of
  * sequences that are split along T, plus, for packed batches (cu_seqlens != NULL, N > 1), one int32 per
- * sequence for the longest-first visiting order.  Pointers in `a` are not dereferenced (cu_seqlens is
- * only compared with NULL). */
+ * sequence for the longest-first visiting order.  A call with scalar gates is refused without it, one with
+ * vector gates is not (see gate_layout).  Pointers in `a` are not dereferenced (cu_seqlens is
+ * only compared with NULL, the gates' alignment is looked at). */
 size_t dsla_prefill_workspace_bytes(const dsla_prefill_args* a);
 
 /* Writes o for every token and the final states of every sequence into its slot.  A sequence of
@@ -167,9 +168,10 @@ dsla_status dsla_prefill(const dsla_prefill_args* a, dsla_state* st, void* cuda_
  *
  * It computes exactly what dsla_prefill computes for the same arguments (a->workspace and
  * a->workspace_bytes are ignored) and allocates nothing: no cudaMalloc, no cudaFree, no allocating
- * library call.  If the arguments would need more scratch than the array holds
+ * library call.  If the arguments need more scratch than the array holds
  * (dsla_prefill_workspace_bytes(a) > DSLA_STATIC_SCRATCH_BYTES) nothing is launched and
- * DSLA_ERR_SCRATCH_LIMIT is returned; use dsla_prefill with your own workspace then.
+ * DSLA_ERR_SCRATCH_LIMIT is returned; use dsla_prefill with your own workspace then.  (Vector gates need
+ * none: a call whose summaries do not fit is cut into fewer segments.)
  *
  * The first call on each device looks up the array's device address (one cudaGetSymbolAddress with that
  * device current); make that first call outside any CUDA stream capture.  Every call on a device shares the

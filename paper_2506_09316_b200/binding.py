@@ -257,13 +257,18 @@ def _prefill_args(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, N, T, max
 
 
 def dsla_prefill_workspace_bytes(T_total, N, max_seqlen, H, d, dtype=torch.bfloat16, chunk=64, impl="auto",
-                                 dense_T=None) -> int:
+                                 dense_T=None, gate_layout=None) -> int:
+    """Workspace bytes for these sizes; ``gate_layout`` None: enough for either layout."""
+    if gate_layout is None:
+        layouts = (DSLA_GATE_SCALAR, DSLA_GATE_PER_KEY_CHANNEL)
+        return max(dsla_prefill_workspace_bytes(T_total, N, max_seqlen, H, d, dtype, chunk, impl, dense_T, x) for x in layouts)
     a = dsla_prefill_args()
     a.N, a.T, a.T_total, a.max_seqlen = int(N), int(dense_T or 0), int(T_total), int(max_seqlen)
     a.H, a.d_k, a.d_v, a.chunk = int(H), int(d), int(d), int(chunk)
     a.dtype = _DTYPES[dtype]
     a.impl = _IMPLS[impl]
     a.scale = 1.0
+    a.gate_layout = gate_layout
     if dense_T is None:
         a.cu_seqlens = c_void_p(8)  # only tested for NULL, never dereferenced
     return int(_lib.dsla_prefill_workspace_bytes(byref(a)))
@@ -283,7 +288,8 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
     if workspace is None:
         need = dsla_prefill_workspace_bytes(T_total, N, max_seqlen, q.shape[1], q.shape[2], q.dtype, chunk,
                                             impl if isinstance(impl, str) else "auto",
-                                            dense_T=T if cu_seqlens is None else None)
+                                            dense_T=T if cu_seqlens is None else None,
+                                            gate_layout=DSLA_GATE_PER_KEY_CHANNEL if g_hist is not None and g_hist.dim() == 3 else DSLA_GATE_SCALAR)
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
     _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, int(max_seqlen), int(chunk),

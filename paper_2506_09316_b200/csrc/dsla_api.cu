@@ -173,10 +173,15 @@ static dsla_status check_prefill_sizes(const dsla_prefill_args* a) {
     return DSLA_OK;
 }
 
-size_t dsla_prefill_workspace_bytes(const dsla_prefill_args* a) {
+static size_t required_bytes(const dsla_prefill_args* a) {
     if (check_prefill_sizes(a) != DSLA_OK) return 0;
     const dsla_impl impl = resolve_impl(a);
     return impl == DSLA_IMPL_SIMT ? 0 : prefill_tc_workspace_bytes(a, impl == DSLA_IMPL_TENSOR_PAIR);
+}
+
+size_t dsla_prefill_workspace_bytes(const dsla_prefill_args* a) {
+    if (check_prefill_sizes(a) != DSLA_OK) return 0;
+    return a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL && a->impl == DSLA_IMPL_AUTO ? prefill_vec_workspace_bytes(a) : required_bytes(a);
 }
 
 static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cudaStream_t s) {
@@ -193,7 +198,7 @@ static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cu
         if (!aligned(a->q, 16) || !aligned(a->k, 16) || !aligned(a->v, 16) || !aligned(a->o, 16)) return DSLA_ERR_INVALID_ARG;
         if (!aligned(a->g_hist, 4) || !aligned(a->g_rec, 4)) return DSLA_ERR_INVALID_ARG;
     }
-    const size_t need = dsla_prefill_workspace_bytes(a);
+    const size_t need = required_bytes(a);
     if (need > 0 && (!a->workspace || a->workspace_bytes < need || !aligned(a->workspace, 256))) return DSLA_ERR_INVALID_ARG;
     if (!(a->scale == a->scale)) return DSLA_ERR_INVALID_ARG;
 
@@ -232,6 +237,7 @@ static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cu
 }  // extern "C"
 namespace dsla {
 dsla_status prefill_checked(const dsla_prefill_args* a, dsla_state* st, cudaStream_t s) { return prefill_device(a, st, s); }
+size_t prefill_required_bytes(const dsla_prefill_args* a) { return required_bytes(a); }
 }
 extern "C" {
 

@@ -70,6 +70,7 @@ void count_launch(int n = 1);
 
 // dsla_api.cu: argument checks + dispatch shared by the prefill entry points
 dsla_status prefill_checked(const dsla_prefill_args* a, dsla_state* st, cudaStream_t s);
+size_t prefill_required_bytes(const dsla_prefill_args* a);      // the part of dsla_prefill_workspace_bytes that a call is refused without
 // dsla_decode.cu
 dsla_status launch_decode(const DecodeParams& p, int d, dsla_dtype dt, cudaStream_t s);
 // dsla_gate_project.cu
@@ -80,6 +81,7 @@ dsla_status launch_prefill_recurrent(const RecurrentParams& p, const float* cons
                                      cudaStream_t s);
 // dsla_prefill_vec.cu: gates per key channel on the tensor cores
 bool prefill_vec_applies(const dsla_prefill_args* a);
+size_t prefill_vec_workspace_bytes(const dsla_prefill_args* a);    // what it has a use for; it needs none
 dsla_status launch_prefill_vec(const PrefillParams& p, const dsla_prefill_args* a, cudaStream_t s);
 // dsla_prefill_simt.cu
 dsla_status launch_prefill_simt(const PrefillParams& p, int d, int chunk, dsla_dtype dt, cudaStream_t s);

@@ -743,17 +743,28 @@ bool prefill_vec_applies(const dsla_prefill_args* a) {
            reinterpret_cast<uintptr_t>(a->g_rec) % 16 == 0;
 }
 
+// Segments per sequence: as many as keep every SM at one CTA, at least eight chunks each (below that the extra launch costs more than the
+// shorter chains save), and no more than there is room for (these calls need none: without any a sequence is one segment).
+static int plan_segments(const dsla_prefill_args* a, size_t room) {
+    const long long units = (long long)a->N * a->H;
+    const int max_chunks = (a->max_seqlen + VC - 1) / VC;
+    int ns = units > 0 ? (int)(148 / units) : 1;
+    if (ns > 16) ns = 16;
+    while (ns > 1 && ((max_chunks + ns - 1) / ns < 8 || (size_t)units * ns * VEC_STRIDE > room)) --ns;
+    return ns < 1 ? 1 : ns;
+}
+
+size_t prefill_vec_workspace_bytes(const dsla_prefill_args* a) {
+    const int ns = prefill_vec_applies(a) ? plan_segments(a, SIZE_MAX) : 1;
+    return ns > 1 ? (size_t)a->N * a->H * ns * VEC_STRIDE : 0;
+}
+
 dsla_status launch_prefill_vec(const PrefillParams& p, const dsla_prefill_args* a, cudaStream_t s) {
     VecParams vp;
     vp.p = p;
     const long long units = (long long)p.N * p.H;
     const int max_chunks = (a->max_seqlen + VC - 1) / VC;
-    // Segments: as many as keep every SM at one CTA, at least eight chunks each (below that the extra launch costs more than the
-    // shorter chains save), and no more than the workspace holds (these calls need none: without one a sequence is one segment).
-    int ns = (int)(148 / units);
-    if (ns > 16) ns = 16;
-    while (ns > 1 && ((max_chunks + ns - 1) / ns < 8 || (size_t)units * ns * VEC_STRIDE > a->workspace_bytes)) --ns;
-    if (ns < 1 || !a->workspace || reinterpret_cast<uintptr_t>(a->workspace) % 16 != 0) ns = 1;
+    const int ns = a->workspace && reinterpret_cast<uintptr_t>(a->workspace) % 16 == 0 ? plan_segments(a, a->workspace_bytes) : 1;
     vp.nseg = ns;
     vp.cps = ns > 1 ? (max_chunks + ns - 1) / ns : max_chunks;
     vp.ws = ns > 1 ? static_cast<float*>(a->workspace) : nullptr;

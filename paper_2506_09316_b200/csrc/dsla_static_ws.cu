@@ -40,9 +40,8 @@ extern "C" dsla_status dsla_prefill_static_ws(const dsla_prefill_args* a, dsla_s
     dsla_prefill_args b = *a;
     b.workspace = nullptr;
     b.workspace_bytes = 0;
-    const size_t need = dsla_prefill_workspace_bytes(&b);   // 0 for invalid sizes; those are rejected below
-    if (need > (size_t)DSLA_STATIC_SCRATCH_BYTES) return DSLA_ERR_SCRATCH_LIMIT;
-    if (need > 0) {
+    if (dsla::prefill_required_bytes(&b) > (size_t)DSLA_STATIC_SCRATCH_BYTES) return DSLA_ERR_SCRATCH_LIMIT;
+    if (dsla_prefill_workspace_bytes(&b) > 0) {             // 0 for invalid sizes; those are rejected below
         void* ptr = nullptr;
         const dsla_status rc = static_scratch(&ptr);
         if (rc != DSLA_OK) return rc;

@@ -86,3 +86,17 @@ def test_product_package_does_not_import_the_checker():
             if fn.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dirpath, fn)).read()
                 assert "oracle" not in text, f"{fn} mentions the checker"
+
+
+def test_workspace_query_knows_the_gate_layout(lib):
+    """What dsla_prefill_workspace_bytes reports is what the kernel of that layout can use: with vector gates the summaries of the
+    segments (fp32 [2][128][128] and [2][128] each), also through the C structure; without a layout, enough for either."""
+    import torch
+    from paper_2506_09316_b200 import binding as b
+    entry = (2 * 128 * 128 + 2 * 128) * 4
+    sizes = dict(T_total=4096, N=1, max_seqlen=4096, H=32, d=128, dense_T=4096)
+    vec = b.dsla_prefill_workspace_bytes(gate_layout=b.DSLA_GATE_PER_KEY_CHANNEL, **sizes)
+    assert vec == 32 * 4 * entry <= b.DSLA_STATIC_SCRATCH_BYTES
+    assert b.dsla_prefill_workspace_bytes(**sizes) >= vec
+    for other in (dict(dtype=torch.float32), dict(impl="simt"), dict(impl="tensor"), dict(d=64)):      # forms that kernel does not serve
+        assert b.dsla_prefill_workspace_bytes(gate_layout=b.DSLA_GATE_PER_KEY_CHANNEL, **{**sizes, **other}) == 0

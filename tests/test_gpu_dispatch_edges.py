@@ -68,8 +68,8 @@ def test_simt_prefill_short(lens, H, d):
     assert rel_err(o, o_ref) <= TOL[torch.float32] and rel_err(S, S_ref) <= TOL[torch.float32]
 
 
-# Gates per key channel on the tensor cores: whole and ragged chunks of 32 tokens, one token past a block, several segments (with the
-# workspace dsla_prefill brings) and one (impl="auto" without room), exact zeros and ones, sequences shorter than a segment
+# Gates per key channel on the tensor cores: whole and ragged chunks of 32 tokens, one token past a block, several segments and one (too few
+# chunks or too many heads), exact zeros and ones, sequences shorter than a segment
 @pytest.mark.parametrize("lens,H,resume", [((1,), 2, False), ((16,), 1, True), ((17,), 3, False), ((32,), 2, True), ((33, 31, 0, 64), 2, True),
                                            ((257,), 2, False), ((515, 40, 260), 1, True), ((1030,), 37, False), ((300,), 80, True)])
 @pytest.mark.parametrize("pattern", ["mix", "zeros", "ones"])
@@ -94,6 +94,42 @@ def test_channel_prefill_tensor(lens, H, resume, pattern):
     # states: fp32 sums of exact products (three bf16 terms of an fp32 factor); outputs: one bf16 rounding (2^-9 of the value)
     assert rel_err(S[slots], S_ref[slots]) <= 1e-5
     assert rel_err(o, o_ref) <= 4e-3
+
+
+# Vector gates cut a sequence into as many segments as the workspace has room for: none, a misaligned one, room for two, for all that
+# dsla_prefill_workspace_bytes gives (four here), and the array inside the library; fresh and continued (the slot pushed through the first summary).
+@pytest.mark.parametrize("resume", [False, True])
+def test_channel_prefill_workspaces(resume):
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import inputs as gen
+    from util import oracle_prefill, rel_err
+    T, H, stride = 1100, 2, (2 * 128 * 128 + 2 * 128) * 4
+    inp = gen.make_packed(5390, [T], H, 128, BF)
+    rng = np.random.default_rng(5391)
+    for name, mu in (("g_hist", 6.0), ("g_rec", 1.0)):
+        setattr(inp, name, torch.from_numpy((1.0 / (1.0 + np.exp(-rng.normal(mu, 0.5, size=(T, H, 128))))).astype(np.float32)))
+    state0 = gen.make_states(5392, 1, H, 128, 128, std=0.5)
+    o_ref, S_ref = oracle_prefill(inp, state0=state0.double().numpy() if resume else np.zeros(tuple(state0.shape)))
+    dv, st = inp.to("cuda"), dsla.dsla_state_alloc(1, H, 128, 128)
+    full = dsla.dsla_prefill_workspace_bytes(T, 1, T, H, 128, dense_T=T, gate_layout=dsla.DSLA_GATE_PER_KEY_CHANNEL)
+    assert full == 4 * H * stride
+    room = torch.empty(full + 256, dtype=torch.uint8, device="cuda")
+    forms = [("none", room[:0], 1), ("too small", room[:2 * H * stride - 1], 1), ("misaligned", room[8:], 1), ("two", room[:2 * H * stride], 2),
+             ("full", room[:full], 2), ("the binding's", None, 2), ("static", None, 2)]
+    results = {}
+    for name, ws, launches in forms:
+        st.tensor.copy_(state0)
+        before = dsla.dsla_launch_count()
+        if name == "static":
+            o = dsla.dsla_prefill_static_ws(dv.q, dv.k, dv.v, dv.g_hist, dv.g_rec, dv.gamma, st, use_initial_state=resume)
+        else:
+            o = dsla.dsla_prefill(dv.q, dv.k, dv.v, dv.g_hist, dv.g_rec, dv.gamma, st, use_initial_state=resume, workspace=ws)
+        assert dsla.dsla_launch_count() - before == launches, name
+        assert dsla.dsla_state_last_error(st) == dsla.DSLA_OK
+        assert rel_err(o.double().cpu().numpy(), o_ref) <= 4e-3 and rel_err(st.tensor.double().cpu().numpy(), S_ref) <= 1e-5, name
+        results[name] = (o, st.tensor.clone())
+    for name in ("the binding's", "static"):
+        assert all(torch.equal(x, y) for x, y in zip(results[name], results["full"])), name
 
 
 # The states of the tensor-core kernel for vector gates are fp32 sums like those of the token-by-token kernel, and no further from the
