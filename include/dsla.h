@@ -133,7 +133,7 @@ typedef struct {
     int use_initial_state;      /* 0: start every sequence from zero states; 1: continue from the
                                    contents of its slot (chunked prefill / resume)               */
     dsla_impl impl;
-    void* workspace;            /* scratch of dsla_prefill_workspace_bytes(); may be NULL if 0    */
+    void* workspace;            /* scratch of dsla_prefill_workspace_bytes(), 256-byte aligned       */
     size_t workspace_bytes;
     dsla_gate_layout gate_layout; /* SCALAR (0): g_hist, g_rec are [T_total, H].  PER_KEY_CHANNEL: [T_total, H, d_k];
                                    impl AUTO takes the tensor-core kernel for vector gates (bf16, d = 128, gates on 16-byte
@@ -142,10 +142,11 @@ typedef struct {
                                    heads into as many segments as there is room for (T = 4096, 32 heads: 297 us, 903 without).    impl TENSOR and TENSOR_PAIR take scalar gates only: DSLA_ERR_UNSUPPORTED */
 } dsla_prefill_args;
 
-/* Scratch to hand over for these sizes (0 for the SIMT kernel): room for the segment summaries of
- * sequences that are split along T, plus, for packed batches (cu_seqlens != NULL, N > 1), one int32 per
- * sequence for the longest-first visiting order.  A call with scalar gates is refused without it, one with
- * vector gates is not (see gate_layout).  Pointers in `a` are not dereferenced (cu_seqlens is
+/* Scratch to hand over for these sizes (0 for the SIMT kernel).  TENSOR_PAIR and vector gates: room for the
+ * segment summaries of sequences that are split along T; vector gates need none (see gate_layout).  TENSOR
+ * keeps them on chip: at most 256 bytes where it splits sequences, which it does not need either.  Scalar
+ * gates and packed batches (cu_seqlens != NULL) of 2 (TENSOR: 65) to 8192 sequences: one int32 per sequence
+ * for the longest-first visiting order.  A call is refused (DSLA_ERR_INVALID_ARG) without what it needs.  Pointers in `a` are not dereferenced (cu_seqlens is
  * only compared with NULL, the gates' alignment is looked at). */
 size_t dsla_prefill_workspace_bytes(const dsla_prefill_args* a);
 
@@ -160,18 +161,18 @@ dsla_status dsla_prefill(const dsla_prefill_args* a, dsla_state* st, void* cuda_
  * Who needs it: code that runs where device memory cannot be allocated at the time of the call -- for
  * example a serving loop whose allocator is frozen after start-up, a plug-in that is only handed its
  * input and output tensors, or a latency-critical path that must never reach cudaMalloc (an allocation
- * can stall a step for hundreds of milliseconds).  dsla_prefill needs a caller-owned workspace whenever
- * it splits sequences into segments; this variant uses a fixed array inside the library instead:
+ * can stall a step for hundreds of milliseconds).  dsla_prefill uses a caller-owned workspace where its kernel
+ * needs one or has a use for it; this variant uses a fixed array inside the library instead:
  *
  *     static __device__ array of DSLA_STATIC_SCRATCH_BYTES bytes, one per GPU that loads the library,
  *     held until the process exits.
  *
  * It computes exactly what dsla_prefill computes for the same arguments (a->workspace and
  * a->workspace_bytes are ignored) and allocates nothing: no cudaMalloc, no cudaFree, no allocating
- * library call.  If the arguments need more scratch than the array holds
- * (dsla_prefill_workspace_bytes(a) > DSLA_STATIC_SCRATCH_BYTES) nothing is launched and
- * DSLA_ERR_SCRATCH_LIMIT is returned; use dsla_prefill with your own workspace then.  (Vector gates need
- * none: a call whose summaries do not fit is cut into fewer segments.)
+ * library call.  If the arguments need more scratch than the array holds nothing is launched and
+ * DSLA_ERR_SCRATCH_LIMIT is returned; use dsla_prefill with your own workspace then.  (The kernels as they are
+ * need no more on a B200: TENSOR_PAIR at most 15 MB.  Vector gates need none: a call whose summaries do not
+ * fit is cut into fewer segments.)
  *
  * The first call on each device looks up the array's device address (one cudaGetSymbolAddress with that
  * device current); make that first call outside any CUDA stream capture.  Every call on a device shares the
@@ -266,7 +267,8 @@ typedef struct {
  *  - TENSOR (what AUTO picks when it applies): bf16, d = 128, scalar gates (n = 1 runs as a pair whose second state
  *    has weight 0 and is never stored): the chunkwise tensor-core
  *    kernel of dsla_prefill once per pair of states (2i, 2i + 1) with the weights (w_2i, w_2i+1), one launch per pair or, with
- *    few (sequence, head) pairs, several side by side; pairs after the first add their share to o in order, so o is rounded to bf16 once per pair.  Needs the workspace below.
+ *    few (sequence, head) pairs, several side by side; pairs after the first add their share to o in order, so o is rounded to bf16 once per pair.  Packed batches of more than
+ *    64 sequences need the workspace below.
  * Errors as dsla_prefill; time-outs and a too small max_seqlen are reported through dsla_state_last_error. */
 size_t dsla_nstate_prefill_workspace_bytes(const dsla_nstate_prefill_args* a);
 dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* st, void* cuda_stream);

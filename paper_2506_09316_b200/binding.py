@@ -285,16 +285,13 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
         raise ValueError("max_seqlen is required with cu_seqlens")
     if o is None:
         o = torch.empty_like(v)
+    max_seqlen, chunk, impl = int(max_seqlen), int(chunk), _IMPLS[impl] if isinstance(impl, str) else int(impl)
     if workspace is None:
-        need = dsla_prefill_workspace_bytes(T_total, N, max_seqlen, q.shape[1], q.shape[2], q.dtype, chunk,
-                                            impl if isinstance(impl, str) else "auto",
-                                            dense_T=T if cu_seqlens is None else None,
-                                            gate_layout=DSLA_GATE_PER_KEY_CHANNEL if g_hist is not None and g_hist.dim() == 3 else DSLA_GATE_SCALAR)
+        need = _native.prefill_workspace(q, v, g_hist, cu_seqlens, N, T, max_seqlen, chunk, impl)
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, int(max_seqlen), int(chunk),
-                           scale, 1 if use_initial_state else 0, _IMPLS[impl] if isinstance(impl, str) else int(impl),
-                           None if stream is None else _raw_stream(stream)), "dsla_prefill")
+    _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, max_seqlen, chunk,
+                           scale, 1 if use_initial_state else 0, impl, None if stream is None else _raw_stream(stream)), "dsla_prefill")
     return o
 
 
@@ -443,7 +440,7 @@ def dsla_nstate_prefill(q, k, v, gates, weights, st: DslaState, *, o=None, cu_se
     if longest is None:
         longest = T_total      # an upper bound is valid (the tighter the bound, the better the segment plan)
     if workspace is None:
-        need = dsla_nstate_prefill_workspace_bytes(q, k, v, gates, weights, cu_seqlens=cu_seqlens, max_seqlen=max_seqlen, impl=impl)
+        need = _native.nstate_prefill_workspace(q, v, gates, cu_seqlens, N, T, int(longest), _IMPLS[impl])
         if need:
             workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
     _check(_native.nstate_prefill(q, k, v, o, gates, weights, cu_seqlens, slots, workspace, st.address, N, T, int(longest), scale,

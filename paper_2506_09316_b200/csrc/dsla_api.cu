@@ -176,12 +176,14 @@ static dsla_status check_prefill_sizes(const dsla_prefill_args* a) {
 static size_t required_bytes(const dsla_prefill_args* a) {
     if (check_prefill_sizes(a) != DSLA_OK) return 0;
     const dsla_impl impl = resolve_impl(a);
-    return impl == DSLA_IMPL_SIMT ? 0 : prefill_tc_workspace_bytes(a, impl == DSLA_IMPL_TENSOR_PAIR);
+    return impl == DSLA_IMPL_SIMT ? 0 : prefill_tc_required_bytes(a, impl == DSLA_IMPL_TENSOR_PAIR);
 }
 
 size_t dsla_prefill_workspace_bytes(const dsla_prefill_args* a) {
     if (check_prefill_sizes(a) != DSLA_OK) return 0;
-    return a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL && a->impl == DSLA_IMPL_AUTO ? prefill_vec_workspace_bytes(a) : required_bytes(a);
+    if (a->gate_layout == DSLA_GATE_PER_KEY_CHANNEL) return a->impl == DSLA_IMPL_AUTO ? prefill_vec_workspace_bytes(a) : 0;
+    const dsla_impl impl = resolve_impl(a);
+    return impl == DSLA_IMPL_SIMT ? 0 : prefill_tc_workspace_bytes(a, impl == DSLA_IMPL_TENSOR_PAIR);
 }
 
 static dsla_status prefill_device(const dsla_prefill_args* a, dsla_state* st, cudaStream_t s) {
@@ -351,7 +353,7 @@ dsla_status dsla_nstate_prefill(const dsla_nstate_prefill_args* a, dsla_state* s
     }
     if (a->impl != DSLA_IMPL_SIMT && nstate_tensor_applies(a) && a->T_total > 0) {
         const dsla_prefill_args b = nstate_as_prefill_args(a);
-        const size_t need = prefill_tc_workspace_bytes(&b, false);
+        const size_t need = prefill_tc_required_bytes(&b, false);
         if (need > 0 && (!a->workspace || a->workspace_bytes < need || !aligned(a->workspace, 256))) return DSLA_ERR_INVALID_ARG;
         if (!aligned(a->gates, 4)) return DSLA_ERR_INVALID_ARG;
         cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);

@@ -90,6 +90,7 @@ void launch_bounded_wait_selftest(int* status, unsigned max_polls, cudaStream_t 
 // dsla_prefill_tc.cu (pair = the cluster variant of dsla_prefill_tc_pair.cu)
 bool prefill_tc_available();
 size_t prefill_tc_workspace_bytes(const dsla_prefill_args* a, bool pair);
+size_t prefill_tc_required_bytes(const dsla_prefill_args* a, bool pair);
 int prefill_tc_pairs(const dsla_prefill_args* a, int npairs);      // how many of npairs pairs of states one launch should take
 dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a, bool pair, cudaStream_t s);
 

@@ -862,6 +862,7 @@ namespace {
 // Packed batches are visited longest first; up to ORDER_HERE_MAX_N sequences the main kernel of the single-CTA variant finds its place
 // in the order by itself (a kernel for it takes 3 us of a call).
 bool wants_order(const dsla_prefill_args* a) { return a->cu_seqlens != nullptr && a->N > 1 && a->N <= ORDER_MAX_N; }
+bool orders_here(const dsla_prefill_args* a) { return a->N <= ORDER_HERE_MAX_N; }
 
 int sm_count() {
     int dev = 0, sms = 0;
@@ -940,8 +941,9 @@ void plan(const dsla_prefill_args* a, bool pair, int pairs, int* nseg, int* cps,
 }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+size_t order_bytes(const dsla_prefill_args* a, bool pair) { return wants_order(a) && (pair || !orders_here(a)) ? up256((size_t)a->N * sizeof(int)) : 0; }
+// The pair variant's summaries (the single-CTA kernel's stay on chip)
 size_t summaries_bytes(const dsla_prefill_args* a, int nseg) { return nseg > 1 ? (size_t)a->N * a->H * nseg * SUMMARY_STRIDE : 0; }
-size_t order_bytes(const dsla_prefill_args* a) { return wants_order(a) ? up256((size_t)a->N * sizeof(int)) : 0; }
 // room for the snapshot of the initial states of split sequences (used when use_initial_state is set)
 size_t snapshot_bytes(const dsla_prefill_args* a, int nseg) { return nseg > 1 ? (size_t)a->N * a->H * 2 * D * D * sizeof(float) : 0; }
 
@@ -989,10 +991,16 @@ int prefill_tc_pairs(const dsla_prefill_args* a, int npairs) {
     return best;
 }
 
+// What a call is refused without: of the single-CTA kernel only the visiting order of large packed batches.
+size_t prefill_tc_required_bytes(const dsla_prefill_args* a, bool pair) { return pair ? prefill_tc_workspace_bytes(a, true) : order_bytes(a, false); }
+
+// What a caller is told to hand over.  (The single-CTA kernel's summaries stay on chip; where it cuts sequences the answer is one block more
+// than it needs, so that it says, as it always has, which calls are cut.)
 size_t prefill_tc_workspace_bytes(const dsla_prefill_args* a, bool pair) {
     int nseg, cps, skew8;
     plan(a, pair, 1, &nseg, &cps, &skew8);
-    return summaries_bytes(a, nseg) + order_bytes(a) + snapshot_bytes(a, nseg);     // each a multiple of 256
+    if (!pair) return order_bytes(a, false) + (nseg > 1 ? 256 : 0);
+    return summaries_bytes(a, nseg) + order_bytes(a, true) + snapshot_bytes(a, nseg);     // each a multiple of 256
 }
 
 dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a, bool pair, cudaStream_t s) {
@@ -1006,19 +1014,19 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
     tp.pairs = p.pairs > 1 ? p.pairs : 1;
     plan(a, pair, tp.pairs, &tp.nseg, &tp.cps, &tp.skew8);
     char* wsp = static_cast<char*>(a->workspace);
-    tp.ws = tp.nseg > 1 ? reinterpret_cast<float*>(wsp) : nullptr;
+    tp.ws = pair && tp.nseg > 1 ? reinterpret_cast<float*>(wsp) : nullptr;
     tp.order = nullptr;
-    tp.order_here = !pair && wants_order(a) && p.N <= ORDER_HERE_MAX_N;
+    tp.order_here = !pair && wants_order(a) && orders_here(a);
     tp.init = nullptr;
     if (wants_order(a) && !tp.order_here) {
-        int* order = reinterpret_cast<int*>(wsp + summaries_bytes(a, tp.nseg));
+        int* order = reinterpret_cast<int*>(wsp + (pair ? summaries_bytes(a, tp.nseg) : 0));
         launch_seq_order(p.cu_seqlens, p.N, order, s);
         tp.order = order;
     }
     if (pair && tp.nseg > 1 && p.use_initial_state) {
         // The CTA of a sequence's last segment overwrites the slot with the final state; CTAs of earlier segments read the
         // slot as their initial state and nothing orders the two inside the grid: they read a copy taken beforehand.
-        float* snap = reinterpret_cast<float*>(wsp + summaries_bytes(a, tp.nseg) + order_bytes(a));
+        float* snap = reinterpret_cast<float*>(wsp + summaries_bytes(a, tp.nseg) + order_bytes(a, true));
         launch_state_snapshot(p, snap, s);
         tp.init = snap;
     }

@@ -164,6 +164,52 @@ PyObject* py_prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
     GUARD_END
 }
 
+// Sizes, types and layouts of a prefill call, which is all that its workspace depends on.
+bool read_sizes(PyObject* const* args, const Arg& q, const Arg& v, const Arg& cu, dsla_prefill_args* a) {
+    if (!has_dims(q, 3, "q") || !has_dims(v, 3, "v") || !read_dtype(*q.t, &a->dtype) || !read_int(args[0], &a->N) || !read_int(args[1], &a->T) ||
+        !read_int(args[2], &a->max_seqlen))
+        return false;
+    a->cu_seqlens = static_cast<int32_t*>(cu.ptr);
+    a->T_total = (int)q.t->size(0); a->H = (int)q.t->size(1); a->d_k = (int)q.t->size(2); a->d_v = (int)v.t->size(2);
+    a->scale = 1.f;
+    return true;
+}
+
+// prefill_workspace(q, v, g_hist, cu_seqlens, N, T, max_seqlen, chunk, impl) -> bytes
+PyObject* py_prefill_workspace(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    GUARD_BEGIN
+    Arg t[4];
+    int impl;
+    dsla_prefill_args a;
+    std::memset(&a, 0, sizeof(a));
+    if (!count_is(n, 9) || !read_tensors(args, 4, t) || !read_sizes(args + 4, t[0], t[1], t[3], &a) || !read_int(args[7], &a.chunk) || !read_int(args[8], &impl))
+        return nullptr;
+    a.impl = static_cast<dsla_impl>(impl);
+    a.gate_layout = layout_of(t[2], 2);
+    return PyLong_FromSize_t(dsla_prefill_workspace_bytes(&a));
+    GUARD_END
+}
+
+// nstate_prefill_workspace(q, v, gates, cu_seqlens, N, T, max_seqlen, impl) -> bytes
+PyObject* py_nstate_prefill_workspace(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    GUARD_BEGIN
+    Arg t[4];
+    int impl;
+    dsla_prefill_args s;
+    std::memset(&s, 0, sizeof(s));
+    if (!count_is(n, 8) || !read_tensors(args, 4, t) || !read_sizes(args + 4, t[0], t[1], t[3], &s) || !read_int(args[7], &impl)) return nullptr;
+    if (!t[2].t || t[2].t->dim() < 1) { PyErr_SetString(PyExc_ValueError, "gates must be a tensor"); return nullptr; }
+    dsla_nstate_prefill_args a;
+    std::memset(&a, 0, sizeof(a));
+    a.cu_seqlens = s.cu_seqlens; a.N = s.N; a.T = s.T; a.T_total = s.T_total; a.max_seqlen = s.max_seqlen;
+    a.H = s.H; a.d_k = s.d_k; a.d_v = s.d_v; a.dtype = s.dtype; a.scale = 1.f;
+    a.n_states = (int)t[2].t->size(0);
+    a.impl = static_cast<dsla_impl>(impl);
+    a.gate_layout = layout_of(t[2], 3);
+    return PyLong_FromSize_t(dsla_nstate_prefill_workspace_bytes(&a));
+    GUARD_END
+}
+
 // nstate_prefill(q, k, v, o, gates, weights, cu_seqlens, slots, workspace, handle, N, T, max_seqlen, scale,
 //                use_initial_state, impl, stream) -> status
 PyObject* py_nstate_prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
@@ -211,6 +257,8 @@ PyObject* py_gate_project(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyMethodDef kMethods[] = {{"decode_step", FAST(py_decode_step), METH_FASTCALL, nullptr},
                           {"nstate_decode_step", FAST(py_nstate_decode_step), METH_FASTCALL, nullptr},
                           {"prefill", FAST(py_prefill), METH_FASTCALL, nullptr},
+                          {"prefill_workspace", FAST(py_prefill_workspace), METH_FASTCALL, nullptr},
+                          {"nstate_prefill_workspace", FAST(py_nstate_prefill_workspace), METH_FASTCALL, nullptr},
                           {"nstate_prefill", FAST(py_nstate_prefill), METH_FASTCALL, nullptr},
                           {"gate_project", FAST(py_gate_project), METH_FASTCALL, nullptr},
                           {nullptr, nullptr, 0, nullptr}};

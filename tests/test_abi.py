@@ -100,3 +100,18 @@ def test_workspace_query_knows_the_gate_layout(lib):
     assert b.dsla_prefill_workspace_bytes(**sizes) >= vec
     for other in (dict(dtype=torch.float32), dict(impl="simt"), dict(impl="tensor"), dict(d=64)):      # forms that kernel does not serve
         assert b.dsla_prefill_workspace_bytes(gate_layout=b.DSLA_GATE_PER_KEY_CHANNEL, **{**sizes, **other}) == 0
+
+
+def test_workspace_is_what_the_kernel_uses(lib):
+    """The single-CTA tensor kernel keeps its segment summaries on chip: no room for them is asked for, whatever the length; only the
+    cluster variant and the visiting order of large packed batches need any."""
+    from paper_2506_09316_b200 import binding as b
+
+    def query(T, H, N=1, impl="tensor", dense=True):
+        return b.dsla_prefill_workspace_bytes(N * T, N, T, H, 128, impl=impl, dense_T=T if dense else None, gate_layout=b.DSLA_GATE_SCALAR)
+
+    for T in (64, 257, 385, 512, 777, 1152, 4096, 65536):
+        for H in (1, 4, 16, 24, 32, 40):
+            assert query(T, H) <= 256 and query(T, H, impl="auto") <= 256
+    assert query(64, 2, N=64, dense=False) == 0 and query(64, 2, N=65, dense=False) >= 65 * 4
+    assert query(4096, 32, impl="pair") > 2 * 32 * 2 * 128 * 128 * 4

@@ -60,3 +60,18 @@ def test_static_scratch_refuses_sizes_beyond_the_array():
         dsla.dsla_prefill_static_ws(dev.q, dev.k, dev.v, dev.g_hist, dev.g_rec, dev.gamma, st, max_seqlen=T,
                                     impl="tensor")
     assert e.value.status == dsla.DSLA_ERR_SCRATCH_LIMIT
+
+
+# Splitting a sequence takes no scratch of the single-CTA kernel: sizes whose summaries would be beyond the array are served, as they
+# are by dsla_prefill, bit for bit, with a workspace or without.
+@pytest.mark.parametrize("T,H", [(385, 32), (512, 32), (4096, 32), (700, 24), (1000, 16), (300, 40), (576, 40)])
+def test_static_scratch_serves_split_sequences_of_many_heads(T, H):
+    import paper_2506_09316_b200 as dsla
+    dev = gen.make_dense(9110 + T, 1, T, H, 128, torch.bfloat16).to("cuda")
+    st, o = dsla.dsla_state_alloc(1, H, 128, 128), torch.empty_like(dev.v)
+    o_ref, S_ref = _run(dsla.dsla_prefill, dev, st, T, o)
+    o_none, S_none = _run(dsla.dsla_prefill, dev, st, T, o, workspace=torch.empty(0, dtype=torch.uint8, device="cuda"))
+    o_new, S_new = _run(dsla.dsla_prefill_static_ws, dev, st, T, o)
+    assert np.array_equal(o_new, o_ref) and np.array_equal(S_new, S_ref)
+    assert np.array_equal(o_none, o_ref) and np.array_equal(S_none, S_ref)
+
