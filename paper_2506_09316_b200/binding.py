@@ -234,7 +234,7 @@ def _sequences(T_total, cu_seqlens, max_seqlen):
     if cu_seqlens is None:
         T = int(max_seqlen) if max_seqlen is not None else T_total
         return (T_total // T if T > 0 else 0), T, T
-    return cu_seqlens.shape[0] - 1, 0, max_seqlen
+    return cu_seqlens.numel() - 1, 0, max_seqlen
 
 
 def _prefill_args(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, N, T, max_seqlen, chunk, scale,

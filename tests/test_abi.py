@@ -115,3 +115,12 @@ def test_workspace_is_what_the_kernel_uses(lib):
             assert query(T, H) <= 256 and query(T, H, impl="auto") <= 256
     assert query(64, 2, N=64, dense=False) == 0 and query(64, 2, N=65, dense=False) >= 65 * 4
     assert query(4096, 32, impl="pair") > 2 * 32 * 2 * 128 * 128 * 4
+
+
+def test_sequence_count_of_any_cu_seqlens_shape(lib):
+    import torch
+    from paper_2506_09316_b200 import binding as b
+    cu = torch.tensor([0, 3, 3, 10], dtype=torch.int32)
+    for shape in ((4,), (1, 4), (4, 1), (2, 2)):
+        assert b._sequences(10, cu.view(shape), 7) == (3, 0, 7)
+    assert b._sequences(12, None, 4) == (3, 4, 4) and b._sequences(12, None, None) == (1, 12, 12) and b._sequences(0, None, None)[0] == 0
