@@ -42,6 +42,11 @@ bool has_dims(const Arg& a, int dims, const char* name) {
     PyErr_Format(PyExc_ValueError, "%s must be a tensor of %d dimensions", name, dims);
     return false;
 }
+bool has_dims_from(const Arg& a, int dims, const char* name) {      // further dimensions are the caller's business: only size(dims - 1) is read
+    if (a.t && a.t->dim() >= dims) return true;
+    PyErr_Format(PyExc_ValueError, "%s must be a tensor of at least %d dimensions", name, dims);
+    return false;
+}
 bool read_dtype(const at::Tensor& t, dsla_dtype* out) {
     if (t.scalar_type() == at::kBFloat16) { *out = DSLA_BF16; return true; }
     if (t.scalar_type() == at::kFloat) { *out = DSLA_F32; return true; }
@@ -104,7 +109,7 @@ PyObject* py_decode_step(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void* stream;
     dsla_decode_args a;
     std::memset(&a, 0, sizeof(a));
-    if (!count_is(n, 12) || !read_tensors(args, 9, t) || !has_dims(t[0], 3, "q") || !has_dims(t[2], 3, "v") ||
+    if (!count_is(n, 12) || !read_tensors(args, 9, t) || !has_dims(t[0], 3, "q") || !has_dims_from(t[2], 3, "v") ||
         !read_dtype(*t[0].t, &a.dtype) || !read_handle(args[9], &st) || !read_float(args[10], &a.scale) || !read_stream(args[11], &stream))
         return nullptr;
     a.q = t[0].ptr; a.k = t[1].ptr; a.v = t[2].ptr; a.o = t[3].ptr;
@@ -124,7 +129,7 @@ PyObject* py_nstate_decode_step(PyObject*, PyObject* const* args, Py_ssize_t n) 
     void* stream;
     dsla_nstate_decode_args a;
     std::memset(&a, 0, sizeof(a));
-    if (!count_is(n, 11) || !read_tensors(args, 8, t) || !has_dims(t[0], 3, "q") || !has_dims(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
+    if (!count_is(n, 11) || !read_tensors(args, 8, t) || !has_dims(t[0], 3, "q") || !has_dims_from(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
         !read_handle(args[8], &st) || !read_float(args[9], &a.scale) || !read_stream(args[10], &stream))
         return nullptr;
     if (!t[4].t || t[4].t->dim() < 1) { PyErr_SetString(PyExc_ValueError, "gates must be a tensor"); return nullptr; }
@@ -148,7 +153,7 @@ PyObject* py_prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
     int impl;
     dsla_prefill_args a;
     std::memset(&a, 0, sizeof(a));
-    if (!count_is(n, 19) || !read_tensors(args, 10, t) || !has_dims(t[0], 3, "q") || !has_dims(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
+    if (!count_is(n, 19) || !read_tensors(args, 10, t) || !has_dims(t[0], 3, "q") || !has_dims_from(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
         !read_handle(args[10], &st) || !read_int(args[11], &a.N) || !read_int(args[12], &a.T) || !read_int(args[13], &a.max_seqlen) ||
         !read_int(args[14], &a.chunk) || !read_float(args[15], &a.scale) || !read_int(args[16], &a.use_initial_state) ||
         !read_int(args[17], &impl) || !read_stream(args[18], &stream))
@@ -166,7 +171,7 @@ PyObject* py_prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
 
 // Sizes, types and layouts of a prefill call, which is all that its workspace depends on.
 bool read_sizes(PyObject* const* args, const Arg& q, const Arg& v, const Arg& cu, dsla_prefill_args* a) {
-    if (!has_dims(q, 3, "q") || !has_dims(v, 3, "v") || !read_dtype(*q.t, &a->dtype) || !read_int(args[0], &a->N) || !read_int(args[1], &a->T) ||
+    if (!has_dims(q, 3, "q") || !has_dims_from(v, 3, "v") || !read_dtype(*q.t, &a->dtype) || !read_int(args[0], &a->N) || !read_int(args[1], &a->T) ||
         !read_int(args[2], &a->max_seqlen))
         return false;
     a->cu_seqlens = static_cast<int32_t*>(cu.ptr);
@@ -220,7 +225,7 @@ PyObject* py_nstate_prefill(PyObject*, PyObject* const* args, Py_ssize_t n) {
     int impl;
     dsla_nstate_prefill_args a;
     std::memset(&a, 0, sizeof(a));
-    if (!count_is(n, 17) || !read_tensors(args, 9, t) || !has_dims(t[0], 3, "q") || !has_dims(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
+    if (!count_is(n, 17) || !read_tensors(args, 9, t) || !has_dims(t[0], 3, "q") || !has_dims_from(t[2], 3, "v") || !read_dtype(*t[0].t, &a.dtype) ||
         !read_handle(args[9], &st) || !read_int(args[10], &a.N) || !read_int(args[11], &a.T) || !read_int(args[12], &a.max_seqlen) ||
         !read_float(args[13], &a.scale) || !read_int(args[14], &a.use_initial_state) || !read_int(args[15], &impl) ||
         !read_stream(args[16], &stream))
@@ -245,7 +250,7 @@ PyObject* py_gate_project(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void* stream;
     dsla_gate_project_args a;
     std::memset(&a, 0, sizeof(a));
-    if (!count_is(n, 6) || !read_tensors(args, 5, t) || !has_dims(t[0], 2, "x") || !has_dims(t[1], 2, "w") || !read_stream(args[5], &stream)) return nullptr;
+    if (!count_is(n, 6) || !read_tensors(args, 5, t) || !has_dims(t[0], 2, "x") || !has_dims_from(t[1], 1, "w") || !read_stream(args[5], &stream)) return nullptr;
     a.x = t[0].ptr; a.w = t[1].ptr; a.bias = static_cast<float*>(t[2].ptr);
     a.g_hist = static_cast<float*>(t[3].ptr); a.g_rec = static_cast<float*>(t[4].ptr);
     a.T = (int)t[0].t->size(0); a.D_model = (int)t[0].t->size(1); a.H = (int)(t[1].t->size(0) / 2);

@@ -124,3 +124,24 @@ def test_sequence_count_of_any_cu_seqlens_shape(lib):
     for shape in ((4,), (1, 4), (4, 1), (2, 2)):
         assert b._sequences(10, cu.view(shape), 7) == (3, 0, 7)
     assert b._sequences(12, None, 4) == (3, 4, 4) and b._sequences(12, None, None) == (1, 12, 12) and b._sequences(0, None, None)[0] == 0
+
+
+def test_extension_module_reads_only_the_sizes_it_needs(lib):
+    """v may have dimensions behind the head size and w any behind its first; q and x have exactly three and two.  No store is passed, so
+    the C entry points refuse every call before they touch a device."""
+    import torch
+    from paper_2506_09316_b200 import _native, binding as b
+    q, g, gamma = torch.zeros(4, 2, 64), torch.zeros(4, 2), torch.zeros(2)
+    v, w = q.view(4, 2, 64, 1), torch.zeros(2, 4)
+    gates = torch.stack([g, g])
+    dense, steps = (None, 1, 4, 4, 64, 1.0, 0, 0, 0), (None, 1.0, 0)
+    assert _native.prefill(q, q, v, v, g, g, gamma, None, None, None, *dense) == b.DSLA_ERR_INVALID_ARG
+    assert _native.decode_step(q, q, v, v, g, g, gamma, None, None, *steps) == b.DSLA_ERR_INVALID_ARG
+    assert _native.nstate_decode_step(q, q, v, v, gates, w, None, None, *steps) == b.DSLA_ERR_INVALID_ARG
+    assert _native.nstate_prefill(q, q, v, v, gates, w, None, None, None, None, 1, 4, 4, 1.0, 0, 0, 0) == b.DSLA_ERR_INVALID_ARG
+    assert _native.prefill_workspace(q, v, g, None, 1, 4, 4, 64, 0) == 0 and _native.nstate_prefill_workspace(q, v, gates, None, 1, 4, 4, 0) == 0
+    x = torch.zeros(4, 64, dtype=torch.bfloat16)
+    assert _native.gate_project(x, torch.zeros(6, 64, 1, dtype=torch.bfloat16), None, g, g, 0) == b.DSLA_ERR_UNSUPPORTED      # H = 3
+    for bad in (lambda: _native.decode_step(v, q, v, v, g, g, gamma, None, None, *steps), lambda: _native.gate_project(q, x, None, g, g, 0)):
+        with pytest.raises(ValueError):
+            bad()
