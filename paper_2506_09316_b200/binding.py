@@ -229,6 +229,18 @@ def _raw_stream(stream):
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _scratch(need, device, stream):
+    """Workspace of one call.  It is freed when the call returns, and the allocator may hand it out again on the current stream
+    at once: a call on another stream has to be recorded."""
+    workspace = torch.empty(need, dtype=torch.uint8, device=device)
+    if stream is not None:
+        if not isinstance(stream, torch.cuda.Stream):
+            raw = _raw_stream(stream)
+            stream = torch.cuda.ExternalStream(raw, device=device) if raw else torch.cuda.default_stream(device)
+        workspace.record_stream(stream)
+    return workspace
+
+
 def _sequences(T_total, cu_seqlens, max_seqlen):
     """(N, T, max_seqlen) of the C interface: dense batches have T tokens per sequence, packed ones T = 0."""
     if cu_seqlens is None:
@@ -289,7 +301,7 @@ def dsla_prefill(q, k, v, g_hist, g_rec, gamma, st: DslaState, *, o=None, cu_seq
     if workspace is None:
         need = _native.prefill_workspace(q, v, g_hist, cu_seqlens, N, T, max_seqlen, chunk, impl)
         if need:
-            workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+            workspace = _scratch(need, q.device, stream)
     _check(_native.prefill(q, k, v, o, g_hist, g_rec, gamma, cu_seqlens, slots, workspace, st.address, N, T, max_seqlen, chunk,
                            scale, 1 if use_initial_state else 0, impl, None if stream is None else _raw_stream(stream)), "dsla_prefill")
     return o
@@ -442,7 +454,7 @@ def dsla_nstate_prefill(q, k, v, gates, weights, st: DslaState, *, o=None, cu_se
     if workspace is None:
         need = _native.nstate_prefill_workspace(q, v, gates, cu_seqlens, N, T, int(longest), _IMPLS[impl])
         if need:
-            workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+            workspace = _scratch(need, q.device, stream)
     _check(_native.nstate_prefill(q, k, v, o, gates, weights, cu_seqlens, slots, workspace, st.address, N, T, int(longest), scale,
                                   1 if use_initial_state else 0, _IMPLS[impl], None if stream is None else _raw_stream(stream)), "dsla_nstate_prefill")
     return o

@@ -73,3 +73,39 @@ def test_split_prefill_with_initial_state_next_to_a_busy_stream(tc_impl):
         o, S = gpu_prefill(inp, state0=st0, impl=tc_impl)
         side.synchronize()
         assert rel_err(o, o_ref) <= TOL[BF] and rel_err(S, S_ref) <= TOL[BF], f"attempt {attempt}"
+
+
+@pytest.mark.parametrize("form", ["stream", "raw", "default"])
+def test_workspace_of_a_call_on_another_stream_is_not_handed_out_again(form, monkeypatch):
+    """The binding allocates a workspace for the duration of the call.  While the call's stream is still busy the allocator must not give
+    the same memory to the next tensor of the current stream."""
+    import types
+    import paper_2506_09316_b200 as dsla
+    from paper_2506_09316_b200 import binding
+    T, H = 1100, 2
+    inp = gen.make_dense(9905, 1, T, H, 128, BF)
+    rng = np.random.default_rng(9906)
+    for name in ("g_hist", "g_rec"):
+        setattr(inp, name, torch.from_numpy(rng.uniform(0.3, 1.0, size=(T, H, 128)).astype(np.float32)))
+    d, st = inp.to("cuda"), dsla.dsla_state_alloc(1, H, 128, 128)
+    o, seen = torch.empty_like(d.v), []
+
+    def prefill(*args):
+        seen.append((args[9].data_ptr(), args[9].numel()))
+        return native.prefill(*args)
+
+    native = binding._native
+    monkeypatch.setattr(binding, "_native", types.SimpleNamespace(prefill=prefill, prefill_workspace=native.prefill_workspace))
+    side, here = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    busy = torch.cuda.default_stream() if form == "default" else side
+    with torch.cuda.stream(busy):
+        torch.cuda._sleep(100_000_000)                # about 50 ms
+    with torch.cuda.stream(here):
+        dsla.dsla_prefill(d.q, d.k, d.v, d.g_hist, d.g_rec, d.gamma, st, o=o,
+                          stream={"stream": side, "raw": side.cuda_stream, "default": 0}[form])
+        again = torch.empty(seen[0][1], dtype=torch.uint8, device="cuda")
+        assert again.data_ptr() != seen[0][0]
+    torch.cuda.synchronize()
+    o_ref, _ = oracle_prefill(inp)
+    assert rel_err(o.double().cpu().numpy(), o_ref) <= 4e-3
