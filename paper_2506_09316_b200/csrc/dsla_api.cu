@@ -9,6 +9,14 @@
 
 namespace dsla {
 static std::atomic<uint64_t> g_launches{0};
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
+        (void)cudaGetLastError();
+        return 148;      // a B200, when there is no device to ask (sizing a workspace on a build machine)
+    }
+    return sms;
+}
 void count_launch(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
 __global__ void zero_slots_kernel(float* data, const int32_t* slots, int num_slots, size_t slot_elems) {

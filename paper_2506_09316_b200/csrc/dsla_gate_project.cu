@@ -214,8 +214,7 @@ dsla_status launch_gate_project(const dsla_gate_project_args* a, cudaStream_t s)
     // Split K over a cluster while the token tiles alone leave SMs idle, each rank keeps at least four K steps and the partial
     // tiles fit behind the stages.  Clusters: as many stages as fit (one CTA per SM, the loads of the whole K share in flight);
     // (four to eight stages are within 3 % of each other at T = 4096, three are 10 % slower); otherwise four (two CTAs per SM at H = 32, the epilogue of one under the loads of the other).
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { (void)cudaGetLastError(); sms = 148; }
+    const int sms = sm_count();
     const size_t red = (size_t)GP_M * n_out * 4;
     int split = 1;
     for (int c = 8; c >= 2; c >>= 1)

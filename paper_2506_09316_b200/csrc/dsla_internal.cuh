@@ -67,6 +67,7 @@ struct RecurrentParams {
 };
 
 void count_launch(int n = 1);
+int sm_count();      // of the current device
 
 // dsla_api.cu: argument checks + dispatch shared by the prefill entry points
 dsla_status prefill_checked(const dsla_prefill_args* a, dsla_state* st, cudaStream_t s);

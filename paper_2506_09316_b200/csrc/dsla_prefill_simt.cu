@@ -477,8 +477,9 @@ __global__ void __launch_bounds__(4 * D, D == 64 ? 2 : 1) prefill_simt_kernel(co
 // less than idle SMs) and some segment has more than one chunk of the longest sequence (three chunks take four segments,
 // one of them empty: T = 130, 2 heads of 64: 34 us with two).
 static int plan_segments(long long units, int max_chunks, int per_sm) {
+    const int room = per_sm * sm_count();
     int segs = 1;
-    while (segs < 8 && units * segs * 2 <= per_sm * 148 && segs < max_chunks) segs *= 2;
+    while (segs < 8 && units * segs * 2 <= room && segs < max_chunks) segs *= 2;
     return segs;
 }
 

@@ -864,15 +864,6 @@ namespace {
 bool wants_order(const dsla_prefill_args* a) { return a->cu_seqlens != nullptr && a->N > 1 && a->N <= ORDER_MAX_N; }
 bool orders_here(const dsla_prefill_args* a) { return a->N <= ORDER_HERE_MAX_N; }
 
-int sm_count() {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
-        (void)cudaGetLastError();
-        return 148;      // a B200, when there is no device to ask (sizing a workspace on a build machine)
-    }
-    return sms;
-}
-
 // The most clusters of each size (one CTA per SM) that fit on the device at once; sizes over 8 are opt-in.
 constexpr int MAX_SEG = 16;
 int resident_clusters(int size) {
@@ -882,7 +873,7 @@ int resident_clusters(int size) {
     int n = cached[dev][size].load(std::memory_order_relaxed);
     if (n == 0) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(size * 148));
+        cfg.gridDim = dim3((unsigned)(size * sm_count()));
         cfg.blockDim = dim3(NTHREADS);
         cfg.dynamicSmemBytes = SMEM_DYN;
         cudaLaunchAttribute attr[1];

@@ -748,7 +748,7 @@ bool prefill_vec_applies(const dsla_prefill_args* a) {
 static int plan_segments(const dsla_prefill_args* a, size_t room) {
     const long long units = (long long)a->N * a->H;
     const int max_chunks = (a->max_seqlen + VC - 1) / VC;
-    int ns = units > 0 ? (int)(148 / units) : 1;
+    int ns = units > 0 ? (int)(sm_count() / units) : 1;
     if (ns > 16) ns = 16;
     while (ns > 1 && ((max_chunks + ns - 1) / ns < 8 || (size_t)units * ns * VEC_STRIDE > room)) --ns;
     return ns < 1 ? 1 : ns;
