@@ -443,7 +443,7 @@ def dsla_nstate_prefill_workspace_bytes(q, k, v, gates, weights, *, cu_seqlens=N
 def dsla_nstate_prefill(q, k, v, gates, weights, st: DslaState, *, o=None, cu_seqlens=None, slots=None, max_seqlen=None,
                         scale=1.0, use_initial_state=False, impl="auto", workspace=None, stream=None):
     """n-state prefill: gates [n, T_total, H] (or [n, T_total, H, d] per key channel), weights [H, n].  bf16, d = 128
-    with scalar gates runs on the chunkwise tensor-core kernel, one pass per pair of states (``impl="simt"`` forces the
+    with scalar gates runs on the chunkwise tensor-core kernel, its pairs of states one after the other or side by side (``impl="simt"`` forces the
     token-by-token CUDA-core kernel, which serves everything else)."""
     if o is None:
         o = torch.empty_like(v)

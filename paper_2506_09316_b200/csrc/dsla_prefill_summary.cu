@@ -1,5 +1,5 @@
-// Helper kernels of the tensor-core prefill: the state summaries of the segments a sequence is split
-// into, the longest-first visiting order of a packed batch, and the snapshot of the initial states.
+// Helper kernels of the tensor-core prefill: of the cluster variant the state summaries of the segments a sequence is split
+// into and the snapshot of the initial states; of both variants the longest-first visiting order of a large packed batch.
 //
 // Segment summaries: U_g (both states, accumulated from zero) and A_g (product of the segment's gates)
 // for every segment but a sequence's last, so that a later segment can start from
@@ -50,8 +50,8 @@ prefill_tc_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const SeqInfo sq = seq_info(p, n, g, tp);
     if (sq.slot < 0 || sq.slot >= p.num_slots) return;
     if (sq.len <= 0 || g >= sq.last_seg) return;      // only segments that have a successor
-    const int nc = (sq.c_end - sq.c_begin) * (tp.chunk / C);      // full chunks only (not the sequence's last segment)
-    const int t0 = sq.t_begin + sq.c_begin * tp.chunk;
+    const int nc = sq.c_end - sq.c_begin;             // full chunks only (not the sequence's last segment)
+    const int t0 = sq.t_begin + sq.c_begin * C;
     float* out = tp.ws + ((size_t)(n * p.H + h) * tp.nseg + g) * (SUMMARY_STRIDE / 4);
 
     if (tid == 0) {

@@ -966,9 +966,10 @@ dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
 bool prefill_tc_available() { return true; }
 
 // Pairs of states side by side need fewer segments per sequence, so shorter chains of initial states, and read Q, K and V from L2
-// the second time (four states, T = 4096, 32 heads: 116 us as two launches, 97 as one; eight: 224 and 163); but SMs may be left over,
+// the second time (four states, T = 4096, 32 heads: 114 us as two launches, 101 as one; eight: 228 and 162); but SMs may be left over,
 // or the sequences be cut less than a launch for each pair would.  Times in eighths of a chunk's (7.2 k cycles): a chunk 8, set-up and
-// drain 5, a summary 2 per chunk, a hop of the initial states 3.
+// drain 5, a summary 2 per chunk (2.3 k cycles while all SMs read K and V, nearer to 3; with 2.5 here 97 of 100 shapes come out the same), a hop
+// of the initial states 3.
 int prefill_tc_pairs(const dsla_prefill_args* a, int npairs) {
     int best = 1;
     long long least = 0;
@@ -1023,14 +1024,12 @@ dsla_status launch_prefill_tc(const PrefillParams& p, const dsla_prefill_args* a
     }
     CUtensorMap mq, mk, mv, mo;
     if (!make_tile_map(&mq, p.q, a->T_total, p.H, tp.chunk) || !make_tile_map(&mk, p.k, a->T_total, p.H, tp.chunk) ||
-        !make_tile_map(&mv, p.v, a->T_total, p.H, tp.chunk) || !make_tile_map(&mo, p.o, a->T_total, p.H, tp.chunk))
+        !make_tile_map(&mv, p.v, a->T_total, p.H, tp.chunk) || (!pair && !make_tile_map(&mo, p.o, a->T_total, p.H, tp.chunk)))
         return DSLA_ERR_CUDA;
     const long long units = (long long)p.N * p.H;
     if (2 * units * tp.nseg > 0x7fffffffLL) return DSLA_ERR_UNSUPPORTED;
     if (pair && tp.nseg > 1) {
-        CUtensorMap sk, sv;
-        if (!make_tile_map(&sk, p.k, a->T_total, p.H, C) || !make_tile_map(&sv, p.v, a->T_total, p.H, C)) return DSLA_ERR_CUDA;
-        const dsla_status rc = launch_summary(sk, sv, tp, s);
+        const dsla_status rc = launch_summary(mk, mv, tp, s);
         if (rc != DSLA_OK) return rc;
     }
     return pair ? launch_main_pair(mq, mk, mv, tp, tp.nseg > 1, s) : launch_main(mq, mk, mv, mo, tp, s);
