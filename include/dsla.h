@@ -53,7 +53,8 @@ typedef enum { DSLA_GATE_SCALAR = 0, DSLA_GATE_PER_KEY_CHANNEL = 1 } dsla_gate_l
  *   SIMT        : CUDA cores, fp32 arithmetic; any supported dtype and head size, chunk 16 / 32 / 64.
  *   TENSOR      : tcgen05 tensor cores, bf16 with d = 128, chunk 64; one CTA holds both states of a (sequence, head) pair.
  *   TENSOR_PAIR : same mathematics and limits, one state per CTA in a cluster of two CTAs that exchange partial
- *                 outputs through distributed shared memory.
+ *                 outputs through distributed shared memory.  (An infinity or NaN in the first tokens of a packed sequence may
+ *                 turn results of the sequence before it into NaN here: chunk tiles are not cleared past a sequence's end.)
  *   AUTO        : TENSOR for bf16 with d = 128 (the faster of the two tensor variants on the measured shapes), else SIMT
  *                 -- in particular bf16 with d = 64 and everything fp32 run on CUDA cores, an order of magnitude slower. */
 typedef enum { DSLA_IMPL_AUTO = 0, DSLA_IMPL_SIMT = 1, DSLA_IMPL_TENSOR = 2, DSLA_IMPL_TENSOR_PAIR = 3 } dsla_impl;

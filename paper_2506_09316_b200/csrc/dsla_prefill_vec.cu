@@ -15,11 +15,13 @@
 // The tensor core cuts its fp32 sums off instead of rounding them: every MMA onto a state would move it by up to an ulp, always
 // towards zero (six per chunk: states off by 1.5e-6 after 4096 tokens, 3.4e-7 token by token).  So what a chunk adds to a
 // state, V^T (s_i (.) K), is a sum of its own from zero, smallest terms first, and is added on CUDA cores.
+// An infinity or NaN in V would reach the tokens before it through the zeros of P~: the outputs of such a chunk are finished on CUDA cores.
 //
 // CTA = (sequence, head, segment), 16 warps in step: each step takes one state through its pass (two bf16 terms of it for the
 // readout, then S_i diag(A_i)) and its MMAs, and meanwhile builds the operands of the other state for its next turn, so
-// nothing but the raw inputs is double-buffered.  Bound by instruction issue: 7000 warp instructions per chunk and SM
-// sub-partition, half of them for the operands, a quarter for the scores; 16.7 k cycles per chunk.
+// nothing but the raw inputs is double-buffered.  16.7 k cycles per chunk, of which 7600 issue a warp instruction on each SM
+// sub-partition (57 %; half of the instructions for the operands, a quarter for the scores): the warps have unequal shares and wait for
+// the longest one at the barriers of every step.
 //
 // A sequence is split into segments when there are few (sequence, head) pairs and the caller's workspace has room: a first
 // grid accumulates each segment's state from zero, walking the chunks backwards with the product of all later gates (no pass
