@@ -34,10 +34,10 @@ namespace dsla {
 
 namespace {
 
-// Warp roles of the main kernel: 0 = TMA producer, 1 = MMA issuer, 2..9 = tile warps (masked scores, scaled copies of Q),
-// 10..17 = state warps (state rescale + bf16 copy, weighted V^T, outputs, initial/final state), 18, 19 = gate warps.
+// Warp roles of the main kernel: 0 = TMA producer, 1 = MMA issuer, 2, 3 = gate warps, 4..11 = tile warps (masked scores, scaled copies
+// of Q), 12..19 = state warps (state rescale + bf16 copy, weighted V^T, outputs, initial/final state).
 // A warp may touch only the 32 TMEM lanes of its quadrant (warp index mod 4).
-constexpr int WARP_TMA = 0, WARP_MMA = 1, TILE_W0 = 2, STATE_W0 = 10, GATE_W0 = 18;
+constexpr int WARP_TMA = 0, WARP_MMA = 1, GATE_W0 = 2, TILE_W0 = 4, STATE_W0 = 12;
 constexpr int NTHREADS = 20 * 32;
 constexpr int CM = 128;                      // tokens per chunk of this kernel
 // Shared memory, tiles of 128 tokens x 128 elements (32 KB, two halves of 64 elements, 128-byte swizzle).  Q of chunk c lands in
@@ -63,7 +63,7 @@ constexpr int SUM_STAGES = 3;        // K and V tiles of the summaries: two slot
 struct alignas(16) GateSmem {
     float L[2][CM];                  // cumulative log2-gate from the chunk start, inclusive
     uint32_t rowf[2][CM];            // weight_i * (decay from the chunk start through the token), bf16 in both halves
-    __nv_bfloat16 E[2][CM];          // decay from the token to the end of its block of 32 tokens
+    float E[2][CM];                  // decay from the token to the end of its block of 32 tokens
     __nv_bfloat16 w[2][CM];          // decay from the token to the end of the chunk, and what its rounding left; 0 past the end of the sequence
     __nv_bfloat16 w_rest[2][CM];
     float a[2];                      // product of the chunk's gates
@@ -190,7 +190,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (int i = 0; i < 2; ++i) { mbar_init(&sh.kq_full[i], 1); mbar_init(&sh.v_full[i], 1); }
             for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_full[i], 1);
             fence_barrier_init();
-        } else if (warp == 2) {
+        } else if (warp == TILE_W0) {
             mbar_init(&sh.p_full, 1); mbar_init(&sh.prep_ready, 8); mbar_init(&sh.ro_done, 1);
             mbar_init(&sh.o_full, 1); mbar_init(&sh.o_free, 8); mbar_init(&sh.o_staged, 8); mbar_init(&sh.init_done, SPLIT ? 8 : 16); mbar_init(&sh.s_done, 1);
             mbar_init(&sh.next_ready, 8);
@@ -202,18 +202,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             sh.abort_flag = 0;
             sh.slot = slot1;
             fence_barrier_init();
-        } else if (warp == 3 || warp == 4) {
-            const int i = warp - 3;
+        } else if (warp == TILE_W0 + 1 || warp == TILE_W0 + 2) {
+            const int i = warp - TILE_W0 - 1;
             mbar_init(&sh.sb_ready[i], 4); mbar_init(&sh.vt_ready[i], 8); mbar_init(&sh.u_full[i], 1); mbar_init(&sh.g_ready[i], 2); mbar_init(&sh.g_free[i], 16);
             fence_barrier_init();
-        } else if (SPLIT && (warp == 5 || warp == 6)) {
-            const int i = warp - 5;
+        } else if (SPLIT && (warp == TILE_W0 + 3 || warp == TILE_W0 + 4)) {
+            const int i = warp - TILE_W0 - 3;
             mbar_init(&sh.sw_ready[i], 2); mbar_init(&sh.sw_free[i], 8); mbar_init(&sh.svt_ready[i], 8); mbar_init(&sh.svt_free[i], 1);
             fence_barrier_init();
-        } else if (SPLIT && warp == 7) {
+        } else if (SPLIT && warp == TILE_W0 + 5) {
             for (int i = 0; i < SUM_STAGES; ++i) mbar_init(&sh.s_empty[i], 9);      // eight V~ warps + the MMAs on K
             fence_barrier_init();
-        } else if (SPLIT && warp >= STATE_W0 && warp < GATE_W0) {
+        } else if (SPLIT && warp >= STATE_W0) {
             for (int i = 0; i < 4; ++i) mbar_init(&sh.s_in[warp - STATE_W0][i], 1);
             fence_barrier_init();
             if (g > 0 && nc > 0)
@@ -248,7 +248,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
         }
     }
-    if (p.use_initial_state && warp >= TILE_W0 && warp < GATE_W0)      // 128-byte lines of both states into L2
+    if (p.use_initial_state && warp >= TILE_W0)      // 128-byte lines of both states into L2
         for (int i = tid - TILE_W0 * 32; i < (p.single ? 512 : 1024); i += 512)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(slot1 + (size_t)(i >> 9) * state_stride + (size_t)(i & 511) * 32));
     float nx[4];      // gate warps: the next chunk's gates, four tokens a lane
@@ -260,7 +260,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             nx[e] = load_gate(gsrc, t0 + j, p.H, h, c >= 0 && c < nc && tok0 + j < sq.len);
         }
     };
-    if (warp >= GATE_W0) fetch(summarize ? nc - 1 : 0);
+    if (warp >= GATE_W0 && warp < TILE_W0) fetch(summarize ? nc - 1 : 0);
     if (warp == WARP_MMA) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncwarp();
@@ -447,8 +447,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 c3 = n3;
             }
         }
-    } else if (warp < STATE_W0) {
-        // ------------------------------------------------------------------ tile warps 2..9
+    } else if (warp >= TILE_W0 && warp < STATE_W0) {
+        // ------------------------------------------------------------------ tile warps 4..11
         const int tt = tid - TILE_W0 * 32;                // 0..255
         const int q = warp & 3;                           // TMEM lane quadrant: rows (tokens) 32 q .. 32 q + 31
         const int half = (warp - TILE_W0) >> 2;           // column half: keys 64 half .. 64 half + 63
@@ -458,13 +458,25 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + first() + 1] : 1.f - p.gamma[h]) * p.scale;
 
         if (!SPLIT && !zero_start) start_state(half, 1, lane_addr, j);
-        // The ten 32 x 32 blocks of the lower triangle: a quadrant's q + 1 blocks are split between its two warps (the second one
-        // has the diagonal block).  The two blocks above the diagonal that the MMAs read are zeroed once.
-        const int blk0 = half == 0 ? 0 : (q == 1 ? 1 : 2), nblk = q == 0 ? 1 - half : (q == 3 || (q == 2 && half == 0)) ? 2 : 1;
+        // The ten 32 x 32 blocks of the lower triangle: a quadrant's q + 1 blocks are split between its two warps, the second one
+        // takes the diagonal block first.  The decays of a warp's first block are computed ahead of the scores.  The two blocks above the
+        // diagonal that the MMAs read are zeroed once.
+        const int blk0 = half == 0 ? 0 : q, blk1 = half == 0 ? (q >= 2 ? 1 : -1) : (q == 3 ? 2 : -1);
         if (half == 0 && (q == 0 || q == 2))
             for (int m4 = 0; m4 < 4; ++m4)
                 *reinterpret_cast<uint4*>(tiles + OFF_PT + (q == 2 ? HALF_BYTES - 64 * 128 : 0) + sw128_offset(j, 32 + 8 * m4)) = make_uint4(0u, 0u, 0u, 0u);
         const int nfull = (sq.len - tok0) / CM;           // index of the ragged chunk, if there is one
+        // a block left of the diagonal: its decays factor through its last token
+        auto block_decays = [&](const GateSmem& gs, int blk, float L1, float L2, float2 (&mk)[16]) {
+            const float R1 = W1 * ex2(L1 - gs.L[0][32 * blk + 31]), R2 = W2 * ex2(L2 - gs.L[1][32 * blk + 31]);
+            const float2 RR1 = make_float2(R1, R1), RR2 = make_float2(R2, R2);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 E1 = *reinterpret_cast<const float4*>(&gs.E[0][32 * blk + 4 * e]), E2 = *reinterpret_cast<const float4*>(&gs.E[1][32 * blk + 4 * e]);
+                mk[2 * e] = __ffma2_rn(RR2, make_float2(E2.x, E2.y), __fmul2_rn(RR1, make_float2(E1.x, E1.y)));
+                mk[2 * e + 1] = __ffma2_rn(RR2, make_float2(E2.z, E2.w), __fmul2_rn(RR1, make_float2(E1.z, E1.w)));
+            }
+        };
         if (SPLIT) started_alone();
         int c3 = 0;
 #pragma unroll 1
@@ -473,6 +485,19 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const GateSmem& gs = sh.gs[s];
             uint8_t* qs = tiles + c3 * TILE_BYTES;
             WAIT(&sh.g_ready[s], (c >> 1) & 1);
+            // ---- decays of this warp's first block, ahead of the scores that they multiply
+            const float L1 = gs.L[0][j], L2 = gs.L[1][j];
+            float2 mk[16];
+            if (half == 0) {
+                if (q > 0) block_decays(gs, 0, L1, L2, mk);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float4 K1 = *reinterpret_cast<const float4*>(&gs.L[0][32 * q + 4 * e]), K2 = *reinterpret_cast<const float4*>(&gs.L[1][32 * q + 4 * e]);
+                    mk[2 * e].x = fmaf(W2, ex2(L2 - K2.x), W1 * ex2(L1 - K1.x)); mk[2 * e].y = fmaf(W2, ex2(L2 - K2.y), W1 * ex2(L1 - K1.y));
+                    mk[2 * e + 1].x = fmaf(W2, ex2(L2 - K2.z), W1 * ex2(L1 - K1.z)); mk[2 * e + 1].y = fmaf(W2, ex2(L2 - K2.w), W1 * ex2(L1 - K1.w));
+                }
+            }
             WAIT(&sh.kq_full[s], (c >> 1) & 1);           // the TMA writes of Q are visible to this thread
             // Rows of K and V past the end of the sequence belong to the next one.  They would meet only zero weights, but 0 * inf is not 0.  (The
             // scores, which may be reading K, meet them only in columns that no row of this sequence uses; V~ and the other MMAs wait for
@@ -498,44 +523,25 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc_fence_after();
 #pragma unroll
             for (int m = 0; m < 8; ++m) reinterpret_cast<uint4*>(qs)[tt + 256 * m] = q1[m];
-            // ---- P~ = P (.) M; the decays of a block left of the diagonal factor through the block's last token
-            const float L1 = gs.L[0][j], L2 = gs.L[1][j];
-#pragma unroll 1
-            for (int blk = blk0; blk < blk0 + nblk; ++blk) {
+            // ---- P~ = P (.) M
+            auto store_masked = [&](int blk, const float2 (&m)[16], int upto) {      // keys later than `upto` carry nothing
                 uint8_t* at = tiles + OFF_PT + (blk >= 2 ? HALF_BYTES - 64 * 128 : 0);
                 uint32_t r[32], pk[16];
                 tmem_ld32(lane_addr + COL_R + 32 * blk, r);
-                if (blk < q) {
-                    const float R1 = W1 * ex2(L1 - gs.L[0][32 * blk + 31]), R2 = W2 * ex2(L2 - gs.L[1][32 * blk + 31]);
-                    const float2 RR1 = make_float2(R1, R1), RR2 = make_float2(R2, R2);
-                    uint4 E1[4], E2[4];
+                tc_wait_ld();
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        E1[e] = *reinterpret_cast<const uint4*>(&gs.E[0][32 * blk + 8 * e]);
-                        E2[e] = *reinterpret_cast<const uint4*>(&gs.E[1][32 * blk + 8 * e]);
-                    }
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const float2 m = __ffma2_rn(RR2, unpack_bf16(word_of(E2[e >> 2], e & 3)), __fmul2_rn(RR1, unpack_bf16(word_of(E1[e >> 2], e & 3))));
-                        const float2 y = __fmul2_rn(m, make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])));
-                        pk[e] = pack_bf16(y.x, y.y);
-                    }
-                } else {
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e4 = 0; e4 < 8; ++e4) {
-                        const float4 K1 = *reinterpret_cast<const float4*>(&gs.L[0][32 * blk + 4 * e4]), K2 = *reinterpret_cast<const float4*>(&gs.L[1][32 * blk + 4 * e4]);
-                        const float m0 = fmaf(W2, ex2(L2 - K2.x), W1 * ex2(L1 - K1.x)), m1 = fmaf(W2, ex2(L2 - K2.y), W1 * ex2(L1 - K1.y));
-                        const float m2 = fmaf(W2, ex2(L2 - K2.z), W1 * ex2(L1 - K1.z)), m3 = fmaf(W2, ex2(L2 - K2.w), W1 * ex2(L1 - K1.w));
-                        const int e = 4 * e4;      // keys later than the row's token carry nothing
-                        pk[2 * e4] = pack_bf16(e <= lane ? __uint_as_float(r[e]) * m0 : 0.f, e + 1 <= lane ? __uint_as_float(r[e + 1]) * m1 : 0.f);
-                        pk[2 * e4 + 1] = pack_bf16(e + 2 <= lane ? __uint_as_float(r[e + 2]) * m2 : 0.f, e + 3 <= lane ? __uint_as_float(r[e + 3]) * m3 : 0.f);
-                    }
+                for (int e = 0; e < 16; ++e) {
+                    const float2 y = __fmul2_rn(m[e], make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])));
+                    pk[e] = pack_bf16(2 * e <= upto ? y.x : 0.f, 2 * e + 1 <= upto ? y.y : 0.f);
                 }
 #pragma unroll
                 for (int m4 = 0; m4 < 4; ++m4)
                     *reinterpret_cast<uint4*>(at + sw128_offset(j, 32 * (blk & 1) + 8 * m4)) = make_uint4(pk[4 * m4], pk[4 * m4 + 1], pk[4 * m4 + 2], pk[4 * m4 + 3]);
+            };
+            if (half == 1 || q > 0) store_masked(blk0, mk, half == 0 ? 31 : lane);
+            if (blk1 >= 0) {
+                block_decays(gs, blk1, L1, L2, mk);
+                store_masked(blk1, mk, 31);
             }
             tc_fence_before();
             fence_proxy_async_smem();
@@ -543,8 +549,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (lane == 0) { mbar_arrive(&sh.prep_ready); mbar_arrive(&sh.g_free[s]); }
             c3 = c3 == 2 ? 0 : c3 + 1;
         }
-    } else if (warp >= GATE_W0) {
-        // ------------------------------------------------------------------ gate warps: 18 = state 1, 19 = state 2
+    } else if (warp < TILE_W0) {
+        // ------------------------------------------------------------------ gate warps: 2 = state 1, 3 = state 2
         // Everything the chunk needs from the gates comes from the cumulative log-gates
         //     L_j = sum_{t <= j} log2 g_t        (inclusive, from the chunk start; a zero gate counts as -130, so any product
         //                                         that contains one flushes to an exact zero)
@@ -617,7 +623,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             *reinterpret_cast<float4*>(&gs.L[i][4 * lane]) = make_float4(L[0], L[1], L[2], L[3]);
             *reinterpret_cast<uint4*>(&gs.rowf[i][4 * lane]) = make_uint4(dup_bf16(f[0]), dup_bf16(f[1]), dup_bf16(f[2]), dup_bf16(f[3]));
-            *reinterpret_cast<uint2*>(&gs.E[i][4 * lane]) = make_uint2(pack_bf16(E[0], E[1]), pack_bf16(E[2], E[3]));
+            *reinterpret_cast<float4*>(&gs.E[i][4 * lane]) = make_float4(E[0], E[1], E[2], E[3]);
             store_weights(gs, w);
             if (lane == 0) gs.a[i] = pr;
             __syncwarp();
@@ -626,7 +632,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         if (SPLIT && nc == 0) started_alone();
     } else {
-        // ------------------------------------------------------------------ state warps 10..17
+        // ------------------------------------------------------------------ state warps 12..19
         const int q = warp & 3, hi = (warp - STATE_W0) >> 2;   // TMEM lane quadrant, state index
         const uint32_t lane_addr = tb + ((uint32_t)(32 * q) << 16);
         const uint32_t s_addr = lane_addr + COL_S + 128 * hi;
