@@ -62,7 +62,6 @@ constexpr int SUM_STAGES = 3;        // K and V tiles of the summaries: two slot
 // Per-token terms of one chunk; the first index is the state.
 struct alignas(16) GateSmem {
     float L[2][CM];                  // cumulative log2-gate from the chunk start, inclusive
-    uint32_t rowf[2][CM];            // weight_i * (decay from the chunk start through the token), bf16 in both halves
     float E[2][CM];                  // decay from the token to the end of its block of 32 tokens
     __nv_bfloat16 w[2][CM];          // decay from the token to the end of the chunk, and what its rounding left; 0 past the end of the sequence
     __nv_bfloat16 w_rest[2][CM];
@@ -454,6 +453,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const int half = (warp - TILE_W0) >> 2;           // column half: keys 64 half .. 64 half + 63
         const uint32_t lane_addr = tb + ((uint32_t)(32 * q) << 16);
         const int j = 32 * q + lane;
+        const uint32_t row_at = (uint32_t)(j * 128 + ((j & 7) << 4));      // row j of a swizzled half tile: piece m is at row_at ^ (m << 4)
         const float W1 = (p.weights ? p.weights[(size_t)h * p.n_total + first()] : p.gamma[h]) * p.scale;
         const float W2 = p.single ? 0.f : (p.weights ? p.weights[(size_t)h * p.n_total + first() + 1] : 1.f - p.gamma[h]) * p.scale;
 
@@ -506,23 +506,25 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 WAIT(&sh.v_full[s], (c >> 1) & 1);
                 zero_rows(tiles + OFF_K + s * TILE_BYTES, tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES, sq.len - tok0 - c * CM, tt);
             }
-            // ---- scaled copies of Q, eight 16-byte pieces per thread.  The copy for state 2 is written as soon as the readout of the
-            // previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
+            // ---- scaled copies of Q, eight 16-byte pieces (half a row) per thread: one factor per state for all of them.  (Consecutive pieces per
+            // thread needed the factors of eight rows from shared memory, which the loop is bound by.)  The copy for state 2 is written as soon as the readout
+            // of the previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
             if (c > 0) WAIT(&sh.ro_done, (c - 1) & 1);
             else if (SPLIT && g > 0 && c == 0) WAIT(&sh.init_done, 0);      // (the initial state arrives where Q~2 goes)
+            uint8_t* qh = qs + half * HALF_BYTES;
+            const uint32_t f1 = dup_bf16(W1 * ex2(L1)), f2 = dup_bf16(W2 * ex2(L2));      // weight * decay from the chunk start through the token
             uint4 q1[8];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) q1[m] = reinterpret_cast<const uint4*>(qs)[tt + 256 * m];
+            for (int m = 0; m < 8; ++m) q1[m] = *reinterpret_cast<const uint4*>(qh + (row_at ^ (m << 4)));
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
-                const int idx = tt + 256 * m, row = (idx >> 3) & 127;
-                reinterpret_cast<uint4*>(tiles + OFF_Q2)[idx] = scale8(q1[m], gs.rowf[1][row]);
-                q1[m] = scale8(q1[m], gs.rowf[0][row]);
+                *reinterpret_cast<uint4*>(tiles + OFF_Q2 + half * HALF_BYTES + (row_at ^ (m << 4))) = scale8(q1[m], f2);
+                q1[m] = scale8(q1[m], f1);
             }
             mbar_wait_inline(&sh.p_full, c & 1, abortp, p.status);
             tc_fence_after();
 #pragma unroll
-            for (int m = 0; m < 8; ++m) reinterpret_cast<uint4*>(qs)[tt + 256 * m] = q1[m];
+            for (int m = 0; m < 8; ++m) *reinterpret_cast<uint4*>(qh + (row_at ^ (m << 4))) = q1[m];
             // ---- P~ = P (.) M
             auto store_masked = [&](int blk, const float2 (&m)[16], int upto) {      // keys later than `upto` carry nothing
                 uint8_t* at = tiles + OFF_PT + (blk >= 2 ? HALF_BYTES - 64 * 128 : 0);
@@ -536,7 +538,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
 #pragma unroll
                 for (int m4 = 0; m4 < 4; ++m4)
-                    *reinterpret_cast<uint4*>(at + sw128_offset(j, 32 * (blk & 1) + 8 * m4)) = make_uint4(pk[4 * m4], pk[4 * m4 + 1], pk[4 * m4 + 2], pk[4 * m4 + 3]);
+                    *reinterpret_cast<uint4*>(at + (row_at ^ ((4 * (blk & 1) + m4) << 4))) = make_uint4(pk[4 * m4], pk[4 * m4 + 1], pk[4 * m4 + 2], pk[4 * m4 + 3]);
             };
             if (half == 1 || q > 0) store_masked(blk0, mk, half == 0 ? 31 : lane);
             if (blk1 >= 0) {
@@ -557,8 +559,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // through independent exponentials.  Lane l holds tokens 4 l .. 4 l + 3.  The chunk decay that carries the state
         // is the plain product of the gates.
         const int i = warp - GATE_W0;
-        const float Wi = (p.weights ? (i == 1 && p.single ? 0.f : p.weights[(size_t)h * p.n_total + first() + i])
-                                    : (i == 0 ? p.gamma[h] : 1.f - p.gamma[h])) * p.scale;
         auto decays = [&](const float (&x)[4], float (&L)[4], float& pr, float& incl) {      // L: inclusive from the chunk start; incl: of the lane's last token
             float run = 0.f;
             pr = 1.f;
@@ -614,15 +614,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const float block_end = __shfl_sync(0xffffffffu, incl, lane | 7), end = __shfl_sync(0xffffffffu, incl, 31);
             const int valid = min(CM, sq.len - tok0 - c * CM);
             if (c >= 2) WAIT(&sh.g_free[s], ((c >> 1) - 1) & 1);
-            float f[4], E[4], w[4];
+            float E[4], w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                f[e] = Wi * ex2(L[e]);
                 E[e] = ex2(block_end - L[e]);
                 w[e] = 4 * lane + e < valid ? ex2(end - L[e]) : 0.f;
             }
             *reinterpret_cast<float4*>(&gs.L[i][4 * lane]) = make_float4(L[0], L[1], L[2], L[3]);
-            *reinterpret_cast<uint4*>(&gs.rowf[i][4 * lane]) = make_uint4(dup_bf16(f[0]), dup_bf16(f[1]), dup_bf16(f[2]), dup_bf16(f[3]));
             *reinterpret_cast<float4*>(&gs.E[i][4 * lane]) = make_float4(E[0], E[1], E[2], E[3]);
             store_weights(gs, w);
             if (lane == 0) gs.a[i] = pr;
@@ -641,34 +639,40 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         __nv_bfloat16* og = reinterpret_cast<__nv_bfloat16*>(p.o);
         // ldmatrix: this thread addresses row mr of matrix mk; matrices (tokens 0..7 | 8..15) x (d_v 0..7 | 8..15)
         const int mk = lane >> 3, mr = lane & 7;
-        // V~_i^T[v][s] = w^i_s V[s][v] of both states, for the 16 lanes 16 hi .. of this quadrant: ldmatrix.trans hands out the element
-        // pairs a 16x128b TMEM store takes.  `wait` runs between the arithmetic and the stores.  The weights have two bf16 terms, so that the
-        // product is rounded once: with one term, over chunks of 128 tokens, states were 2.11e-3 from the exact ones, now 1.65e-3 (T = 4096,
-        // 59.3 to 59.7 us; other sizes lose up to 2 %).
+        // V~_i^T[v][s] = w^i_s V[s][v] of both states, for the 32 d_v lanes of this quadrant and tokens 64 hi .. 64 hi + 63 (16 lanes and all tokens
+        // took twice the loads of weights): ldmatrix.trans hands out the element pairs a 16x128b TMEM store takes.  `wait` runs between the
+        // arithmetic and the stores.  The weights have two bf16 terms, so that the product is rounded once: with one term, over chunks of 128 tokens,
+        // states were 2.11e-3 from the exact ones, now 1.65e-3 (T = 4096, 59.3 to 59.7 us; other sizes lose up to 2 %).
         auto weighted_v = [&](const uint8_t* vtile, const GateSmem& gs, uint32_t col, auto wait) {
-            const int d = 32 * q + 16 * hi + 8 * (mk & 1);            // first d_v column of the matrix this thread addresses
-            const uint32_t row0 = smem_u32(vtile) + (uint32_t)((8 * (mk >> 1) + mr) * 128) + (uint32_t)(d >> 6) * HALF_BYTES +
+            const int d = 32 * q + 8 * (mk & 1);                      // first d_v column of the matrix this thread addresses, lanes 0..15 of the quadrant
+            const uint32_t row0 = smem_u32(vtile) + (uint32_t)((64 * hi + 8 * (mk >> 1) + mr) * 128) + (uint32_t)(d >> 6) * HALF_BYTES +
                                   (((uint32_t)((d & 63) >> 3) ^ (uint32_t)mr) << 4);
-            uint32_t r[32], y[32];
+            uint32_t r[32], y[32];      // [lanes 0..15 | 16..31][16 tokens][4]
 #pragma unroll
-            for (int t16 = 0; t16 < 8; ++t16) ldmatrix_x4_trans(row0 + (uint32_t)(t16 * 16 * 128), r[4 * t16], r[4 * t16 + 1], r[4 * t16 + 2], r[4 * t16 + 3]);
+            for (int t16 = 0; t16 < 8; ++t16) {
+                const uint32_t at = (t16 < 4 ? row0 : row0 ^ 32u) + (uint32_t)((t16 & 3) * 16 * 128);
+                ldmatrix_x4_trans(at, r[4 * t16], r[4 * t16 + 1], r[4 * t16 + 2], r[4 * t16 + 3]);
+            }
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 constexpr uint32_t REST = (uint32_t)(offsetof(GateSmem, w_rest) - offsetof(GateSmem, w));
-                const uint32_t wp = smem_u32(&gs.w[i][2 * (lane & 3)]);
+                const uint32_t wp = smem_u32(&gs.w[i][64 * hi + 2 * (lane & 3)]);
                 uint32_t* o = i == 0 ? y : r;
 #pragma unroll
-                for (int t16 = 0; t16 < 8; ++t16) {
-                    const uint32_t w0 = ld_shared_u32(wp + 32 * t16), w1 = ld_shared_u32(wp + 32 * t16 + 16);
-                    const uint32_t l0 = ld_shared_u32(wp + REST + 32 * t16), l1 = ld_shared_u32(wp + REST + 32 * t16 + 16);
-                    o[4 * t16] = hfma2_u32(r[4 * t16], w0, hmul2_u32(r[4 * t16], l0)); o[4 * t16 + 1] = hfma2_u32(r[4 * t16 + 1], w0, hmul2_u32(r[4 * t16 + 1], l0));
-                    o[4 * t16 + 2] = hfma2_u32(r[4 * t16 + 2], w1, hmul2_u32(r[4 * t16 + 2], l1)); o[4 * t16 + 3] = hfma2_u32(r[4 * t16 + 3], w1, hmul2_u32(r[4 * t16 + 3], l1));
+                for (int t = 0; t < 4; ++t) {
+                    const uint32_t w0 = ld_shared_u32(wp + 32 * t), w1 = ld_shared_u32(wp + 32 * t + 16);
+                    const uint32_t l0 = ld_shared_u32(wp + REST + 32 * t), l1 = ld_shared_u32(wp + REST + 32 * t + 16);
+#pragma unroll
+                    for (int x = 4 * t; x < 32; x += 16) {
+                        o[x] = hfma2_u32(r[x], w0, hmul2_u32(r[x], l0)); o[x + 1] = hfma2_u32(r[x + 1], w0, hmul2_u32(r[x + 1], l0));
+                        o[x + 2] = hfma2_u32(r[x + 2], w1, hmul2_u32(r[x + 2], l1)); o[x + 3] = hfma2_u32(r[x + 3], w1, hmul2_u32(r[x + 3], l1));
+                    }
                 }
             }
             wait();
-            const uint32_t at = lane_addr + ((uint32_t)(16 * hi) << 16) + col;
-            tmem_st_16x128b_x8(at, y); tmem_st_16x128b_x8(at + 32, y + 16);
-            tmem_st_16x128b_x8(at + 64, r); tmem_st_16x128b_x8(at + 96, r + 16);
+            const uint32_t at = lane_addr + col + 32 * hi, at16 = at + (16u << 16);
+            tmem_st_16x128b_x8(at, y); tmem_st_16x128b_x8(at16, y + 16);
+            tmem_st_16x128b_x8(at + 64, r); tmem_st_16x128b_x8(at16 + 64, r + 16);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
