@@ -54,8 +54,9 @@ constexpr uint32_t COL_S = 0;      // fp32 S1^T [0,128), S2^T [128,256)
 constexpr uint32_t COL_SB = 256;   // per state 64 columns: the bf16 copy of S^T (readout), then the weighted V~^T (update)
 constexpr uint32_t COL_R = 384;    // P (scores, tokens x tokens), then O^T (d_v x tokens): 128 columns
 
-// Where the initial states of a segment arrive (64 KB each, [d_k / 4][d_v] pieces of four d_k): slots that the first chunk's Q and K do not
-// land in.
+// Where the initial states of a segment arrive: per state a ring of two pieces of 32 d_k (16 KB each, [d_k / 4][d_v] of four d_k), in slots that
+// nothing of the first chunk uses, so that its tiles are loaded and its scores masked meanwhile (with room for whole states, over V and
+// Q~2 of that chunk, its outputs came 3 k cycles later).
 __device__ constexpr int initial_off(int i) { return i == 0 ? TILE_BYTES : OFF_K + TILE_BYTES; }
 constexpr int SUM_STAGES = 3;        // K and V tiles of the summaries: two slots each, in order
 
@@ -71,7 +72,7 @@ struct alignas(16) GateSmem {
 struct alignas(16) Shared {
     uint64_t kq_full[2], v_full[2], p_full, prep_ready, sb_ready[2], ro_done, vt_ready[2], o_full, o_free, o_staged, u_full[2], g_ready[2], g_free[2], init_done;
     uint64_t s_full[SUM_STAGES], s_empty[SUM_STAGES], sw_ready[2], sw_free[2], svt_ready[2], svt_free[2], s_done;      // summaries
-    uint64_t s_in[8][4], next_ready;      // initial state: a piece has arrived, the next segment has room for its own
+    uint64_t s_in[8][4], s_taken[8][2], next_ready;      // initial state: a piece has arrived, the next segment has taken its one, has room for it
     uint32_t tmem_base;
     int abort_flag;
     float* slot;                          // the first state of this (sequence, head) in its slot: read where it is needed, not kept in registers
@@ -214,6 +215,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             fence_barrier_init();
         } else if (SPLIT && warp >= STATE_W0) {
             for (int i = 0; i < 4; ++i) mbar_init(&sh.s_in[warp - STATE_W0][i], 1);
+            for (int i = 0; i < 2; ++i) mbar_init(&sh.s_taken[warp - STATE_W0][i], 1);
             fence_barrier_init();
             if (g > 0 && nc > 0)
                 for (int i = 0; i < 4; ++i) mbar_arrive_expect_tx(&sh.s_in[warp - STATE_W0][i], 32 * 128);      // 32 d_k x 32 d_v
@@ -315,8 +317,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (lane == 0 && nc > 0) {
             const uint32_t next_turn = PAIRS && pr + 1 < pairs ? map_to_cta(smem_u32(&sh.o_turn), (uint32_t)(cta + nseg)) : 0u;
             if (SPLIT) {
-                if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
                 load_v(0, 2);
+                if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
                 if (nc > 1) load_kq(1, 1);
             }
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
@@ -510,7 +512,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // thread needed the factors of eight rows from shared memory, which the loop is bound by.)  The copy for state 2 is written as soon as the readout
             // of the previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
             if (c > 0) WAIT(&sh.ro_done, (c - 1) & 1);
-            else if (SPLIT && g > 0 && c == 0) WAIT(&sh.init_done, 0);      // (the initial state arrives where Q~2 goes)
             uint8_t* qh = qs + half * HALF_BYTES;
             const uint32_t f1 = dup_bf16(W1 * ex2(L1)), f2 = dup_bf16(W2 * ex2(L2));      // weight * decay from the chunk start through the token
             uint4 q1[8];
@@ -709,7 +710,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     if ((b & 1) == 0) mbar_wait_cluster(&sh.s_in[w][b >> 1], 0, abortp, p.status);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const float4 y = *reinterpret_cast<const float4*>(tiles + mine + (4 * b + k) * (D * 16));
+                        const float4 y = *reinterpret_cast<const float4*>(tiles + mine + (4 * (b & 3) + k) * (D * 16));
                         x[4 * k] = y.x; x[4 * k + 1] = y.y; x[4 * k + 2] = y.z; x[4 * k + 3] = y.w;
                     }
                 } else {
@@ -720,9 +721,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
                 if (summarize) {
                     tc_wait_ld();
+                    if (b == 4 || b == 6) mbar_wait_cluster(&sh.s_taken[w][(b >> 1) - 2], 0, abortp, p.status);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        st_async_f32x4(next + (uint32_t)((4 * b + k) * (D * 16)), fmaf(A, x[4 * k], __uint_as_float(u[4 * k])), fmaf(A, x[4 * k + 1], __uint_as_float(u[4 * k + 1])),
+                        st_async_f32x4(next + (uint32_t)((4 * (b & 3) + k) * (D * 16)), fmaf(A, x[4 * k], __uint_as_float(u[4 * k])), fmaf(A, x[4 * k + 1], __uint_as_float(u[4 * k + 1])),
                                        fmaf(A, x[4 * k + 2], __uint_as_float(u[4 * k + 2])), fmaf(A, x[4 * k + 3], __uint_as_float(u[4 * k + 3])), next_bar + 8u * (b >> 1));
                 }
                 if (!zero_start) {
@@ -733,6 +735,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     for (int k = 0; k < 16; ++k) u[k] = __float_as_uint(x[k] * a);
                     tmem_st8(sb_addr + 8 * b, pk);
                     tmem_st16(s_addr + 16 * b, u);
+                }
+                if (g > 0 && (b == 1 || b == 3)) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&sh.s_taken[w][b >> 1]), (uint32_t)(cta - 1)));
                 }
             }
             tc_wait_st();
