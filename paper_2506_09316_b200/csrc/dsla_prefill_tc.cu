@@ -245,7 +245,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             load_kq(0, 0);
             if (!SPLIT) {
                 load_v(0, 2);
-                if (nc > 1) load_kq(1, 1);
+                if (nc > 1 && zero_start) load_kq(1, 1);
             }
         }
     }
@@ -283,14 +283,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // Whole sequences: d_k rows 64 part .. 64 part + 63 of state i from the slot, one d_v lane per thread, while the first gates are on
     // their way.
     auto start_state = [&](int i, int part, uint32_t lane_addr, int v) {
-#pragma unroll 1
-        for (int k0 = 64 * part; k0 < 64 * part + 64; k0 += 32) {
-            uint32_t x[32];
-            const float* src = sh.slot + (size_t)i * state_stride + (size_t)k0 * D + v;
+        uint32_t x[2][32];
+        const float* src = sh.slot + (size_t)i * state_stride + (size_t)(64 * part) * D + v;
 #pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = p.single && i == 1 ? 0u : __float_as_uint(src[(size_t)k * D]);
-            tmem_st32(lane_addr + COL_S + 128 * i + k0, x);
-        }
+        for (int k = 0; k < 64; ++k) x[k >> 5][k & 31] = p.single && i == 1 ? 0u : __float_as_uint(src[(size_t)k * D]);
+        tmem_st32(lane_addr + COL_S + 128 * i + 64 * part, x[0]);
+        tmem_st32(lane_addr + COL_S + 128 * i + 64 * part + 32, x[1]);
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -320,6 +318,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 load_v(0, 2);
                 if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
                 if (nc > 1) load_kq(1, 1);
+            }
+            if (!SPLIT && !zero_start && nc > 1) {
+                WAIT(&sh.init_done, 0);      // behind the initial state, which is needed first
+                load_kq(1, 1);
             }
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
             int c3 = 0;
