@@ -94,8 +94,8 @@ __device__ __forceinline__ void issue4_ts(uint32_t d, uint32_t a, uint32_t b, ui
     for (uint32_t k = 0; k < 4; ++k) mma_ts_lo(d, a + 8 * k, b + k * BSTEP, idesc, k ? 1u : acc);
 }
 
-// Rows valid .. CM - 1 of a K and a V tile, by 256 threads (cold path, out of line).
-__device__ __noinline__ void zero_rows(uint8_t* kt, uint8_t* vt, int valid, int t) {
+// Rows valid .. CM - 1 of a K and a V tile, by 256 threads.
+__device__ __forceinline__ void zero_rows(uint8_t* kt, uint8_t* vt, int valid, int t) {
 #pragma unroll 1
     for (int i = 16 * valid + t; i < 16 * CM; i += 256) {
         const int at = (i & 8 ? HALF_BYTES : 0) + (i >> 4) * 128 + (i & 7) * 16;
@@ -103,6 +103,8 @@ __device__ __noinline__ void zero_rows(uint8_t* kt, uint8_t* vt, int valid, int 
         *reinterpret_cast<uint4*>(vt + at) = make_uint4(0u, 0u, 0u, 0u);
     }
 }
+// (the same as a call: in the variants with more code it spills less)
+__device__ __noinline__ void zero_rows_call(uint8_t* kt, uint8_t* vt, int valid, int t) { zero_rows(kt, vt, valid, t); }
 
 // ============================================================================================
 // Main kernel
@@ -469,7 +471,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (half == 0 && (q == 0 || q == 2))
             for (int m4 = 0; m4 < 4; ++m4)
                 *reinterpret_cast<uint4*>(tiles + OFF_PT + (q == 2 ? HALF_BYTES - 64 * 128 : 0) + sw128_offset(j, 32 + 8 * m4)) = make_uint4(0u, 0u, 0u, 0u);
-        const int nfull = (sq.len - tok0) / CM;           // index of the ragged chunk, if there is one
         // a block left of the diagonal: its decays factor through its last token
         auto block_decays = [&](const GateSmem& gs, int blk, float L1, float L2, float2 (&mk)[16]) {
             const float R1 = W1 * ex2(L1 - gs.L[0][32 * blk + 31]), R2 = W2 * ex2(L2 - gs.L[1][32 * blk + 31]);
@@ -482,13 +483,36 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
         };
         if (SPLIT) started_alone();
+        // The decays of a block (32 registers) and the scaled Q (32) are alive across the waits of this loop, where a call costs spills.  Whole
+        // sequences: waits for what has long arrived come before the decays, the cleared rows without a call (16 prompts of 335K tokens 2780 to
+        // 2720 us, 8 x 512 tokens 49.6 to 48.2, pieces of one chunk 15.3 to 15.0).  Segments: decays first, since the tiles come late, and waits without
+        // a call (777 tokens 20.9 to 20.6; with the other order 21.8).  Pairs of states keep the calls (eight states 156 us, without them 170).
+        auto tile_wait = [&](uint64_t* bar, int ph) {
+            if (SPLIT && !PAIRS) mbar_wait_inline(bar, (uint32_t)ph, abortp, p.status);
+            else WAIT(bar, ph);
+        };
         int c3 = 0;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
             const int s = c & 1;
             const GateSmem& gs = sh.gs[s];
             uint8_t* qs = tiles + c3 * TILE_BYTES;
-            WAIT(&sh.g_ready[s], (c >> 1) & 1);
+            // Q and K have landed (the TMA writes of Q are visible to this thread).  Rows of K and V past the end of the sequence belong to the next one.
+            // They would meet only zero weights, but 0 * inf is not 0.  (The scores, which may be reading K, meet them only in columns that no
+            // row of this sequence uses; V~ and the other MMAs wait for prep_ready.  Here, under the scores; ahead of prep_ready it took 1 % of a
+            // packed batch's time.)
+            auto landed = [&] {
+                tile_wait(&sh.kq_full[s], (c >> 1) & 1);
+                const int valid = sq.len - tok0 - c * CM;
+                if (valid < CM) {
+                    tile_wait(&sh.v_full[s], (c >> 1) & 1);
+                    uint8_t *kt = tiles + OFF_K + s * TILE_BYTES, *vt = tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES;
+                    if (SPLIT) zero_rows_call(kt, vt, valid, tt);
+                    else zero_rows(kt, vt, valid, tt);
+                }
+            };
+            tile_wait(&sh.g_ready[s], (c >> 1) & 1);
+            if (!SPLIT) landed();
             // ---- decays of this warp's first block, ahead of the scores that they multiply
             const float L1 = gs.L[0][j], L2 = gs.L[1][j];
             float2 mk[16];
@@ -502,18 +526,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     mk[2 * e + 1].x = fmaf(W2, ex2(L2 - K2.z), W1 * ex2(L1 - K1.z)); mk[2 * e + 1].y = fmaf(W2, ex2(L2 - K2.w), W1 * ex2(L1 - K1.w));
                 }
             }
-            WAIT(&sh.kq_full[s], (c >> 1) & 1);           // the TMA writes of Q are visible to this thread
-            // Rows of K and V past the end of the sequence belong to the next one.  They would meet only zero weights, but 0 * inf is not 0.  (The
-            // scores, which may be reading K, meet them only in columns that no row of this sequence uses; V~ and the other MMAs wait for
-            // prep_ready.  Here, under the scores; ahead of prep_ready it took 1 % of a packed batch's time.)
-            if (c == nfull) {
-                WAIT(&sh.v_full[s], (c >> 1) & 1);
-                zero_rows(tiles + OFF_K + s * TILE_BYTES, tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES, sq.len - tok0 - c * CM, tt);
-            }
+            if (SPLIT) landed();
             // ---- scaled copies of Q, eight 16-byte pieces (half a row) per thread: one factor per state for all of them.  (Consecutive pieces per
             // thread needed the factors of eight rows from shared memory, which the loop is bound by.)  The copy for state 2 is written as soon as the readout
             // of the previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
-            if (c > 0) WAIT(&sh.ro_done, (c - 1) & 1);
+            if (c > 0) tile_wait(&sh.ro_done, (c - 1) & 1);
             uint8_t* qh = qs + half * HALF_BYTES;
             const uint32_t f1 = dup_bf16(W1 * ex2(L1)), f2 = dup_bf16(W2 * ex2(L2));      // weight * decay from the chunk start through the token
             uint4 q1[8];

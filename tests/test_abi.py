@@ -145,3 +145,18 @@ def test_extension_module_reads_only_the_sizes_it_needs(lib):
     for bad in (lambda: _native.decode_step(v, q, v, v, g, g, gamma, None, None, *steps), lambda: _native.gate_project(q, x, None, g, g, 0)):
         with pytest.raises(ValueError):
             bad()
+
+
+def test_prefill_of_whole_sequences_spills_no_registers(tmp_path):
+    """The chunk loop of the tensor-core prefill keeps two 32-register sets alive at 96 registers a thread; ptxas reports what does not fit."""
+    import shutil
+    import subprocess
+    from paper_2506_09316_b200 import build
+    nvcc = shutil.which(build._nvcc())
+    if nvcc is None:
+        pytest.skip("no nvcc")
+    out = subprocess.run([nvcc, *build.NVCC_FLAGS, "-Xptxas", "-v", "-c", os.path.join(build.CSRC, "dsla_prefill_tc.cu"), "-o",
+                          str(tmp_path / "x.o")], capture_output=True, text=True, check=True)
+    entry = [s for s in re.split("Compiling entry function", out.stderr + out.stdout)[1:] if "prefill_tc_kernelILb0ELb0E" in s]
+    assert len(entry) == 1
+    assert re.search(r"(\d+) bytes spill stores, (\d+) bytes spill loads", entry[0]).groups() == ("0", "0")
