@@ -25,7 +25,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 // Bounded wait.  The fast path (phase already complete) is a single inlined test; otherwise a
 // non-inlined loop parks the thread on the barrier (mbarrier.try_wait) again and again.  It gives up
 // after `limit` rounds or about a second, raises *abort_flag (shared) and *status (global) and returns false.  Once the abort flag is up every
-// later wait returns on its first poll, so a CTA that lost a signal still runs to its end, frees its
+// later wait returns from its first parked poll (0.13 ms), so a CTA that lost a signal still runs to its end, frees its
 // TMEM and exits instead of hanging.  CLUSTER = true makes the successful test an acquire at
 // cluster scope (data another CTA of the cluster wrote into this CTA's shared memory before its
 // remote arrive is then visible).
@@ -78,10 +78,8 @@ __device__ __forceinline__ bool mbar_wait_loop(uint64_t* bar, uint32_t parity, v
     const uint64_t t0 = global_timer_ns();
     for (uint32_t i = 0; i < limit; ++i) {
         if (mbar_try_wait_t<CLUSTER>(bar, parity)) return true;
-        if ((i & 7u) == 7u) {
-            if (*abort_flag) return false;
-            if (global_timer_ns() - t0 > 1000000000ull) break;
-        }
+        if (*abort_flag) return false;
+        if (global_timer_ns() - t0 > 1000000000ull) break;
     }
     *abort_flag = 1;
     atomicExch(status, 5 /* DSLA_ERR_TIMEOUT */);

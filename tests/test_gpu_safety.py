@@ -25,6 +25,28 @@ def test_bounded_wait_gives_up_and_the_device_stays_usable():
     assert rel_err(o, o_ref) <= TOL[BF] and rel_err(S, S_ref) <= TOL[BF]
 
 
+def test_waits_behind_one_that_gave_up_end_on_their_first_poll():
+    """The self-test is one wait of `max_polls` polls, one that starts with the abort flag up, and the 0.2 ms in which copies land."""
+    import paper_2506_09316_b200 as dsla
+    st = dsla.dsla_state_alloc(1, 2, 128, 128)
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+
+    def ms(polls):
+        times = []
+        for _ in range(5):
+            torch.cuda.synchronize()
+            begin.record()
+            dsla.dsla_selftest_bounded_wait(st, polls)
+            end.record()
+            end.synchronize()
+            times.append(begin.elapsed_time(end))
+        return min(times)
+
+    one, many = ms(1), ms(101)
+    poll = (many - one) / 100
+    assert one <= 0.2 + 0.1 + 4 * poll      # two polls, the 0.2 ms and a launch; nine polls where the flag is read on every eighth
+
+
 def test_selftest_rejects_unbounded_limits():
     import paper_2506_09316_b200 as dsla
     st = dsla.dsla_state_alloc(1, 2, 128, 128)
