@@ -306,7 +306,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 load_summary(it);
             }
             WAIT(&sh.s_done, 0);
-            load_kq(0, 0);
+            if (!*abortp) load_kq(0, 0);
         }
         if (PAIRS) {
             __syncwarp();
@@ -317,13 +317,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (lane == 0 && nc > 0) {
             const uint32_t next_turn = PAIRS && pr + 1 < pairs ? map_to_cta(smem_u32(&sh.o_turn), (uint32_t)(cta + nseg)) : 0u;
             if (SPLIT) {
-                load_v(0, 2);
+                if (!*abortp) load_v(0, 2);
                 if (g > 0) WAIT(&sh.init_done, 0);      // the initial state is in TMEM, its place free
-                if (nc > 1) load_kq(1, 1);
+                if (nc > 1 && !*abortp) load_kq(1, 1);      // (not onto pieces that may still arrive, where a wait for them gave up)
             }
             if (!SPLIT && !zero_start && nc > 1) {
                 WAIT(&sh.init_done, 0);      // behind the initial state, which is needed first
-                load_kq(1, 1);
+                if (!*abortp) load_kq(1, 1);
             }
             const int nfull = (sq.len - tok0) / CM;         // whole chunks leave through shared memory and a tile store
             int c3 = 0;
