@@ -21,8 +21,8 @@
 // summary U, with the product A of its gates), then the initial states travel down the cluster, S <- A S + U, in
 // pieces, and each segment runs its chunks.  (As a kernel of its own the summaries took 21 of 68 us at T = 4096, 32 heads: launch,
 // fill and drain of a second pipeline.  Stores into another CTA's shared memory ran at 26 bytes a cycle, loads from it at 12:
-// hence a chain that only stores.  Three hops of 128 KB cost 9 k cycles, a fold in which every CTA loads its share of all
-// summaries and stores it back took 16 k.)
+// hence a chain that only stores.  Its last of four CTAs has its initial state 13 to 15 k cycles after the first began to send, of which the
+// first hop takes 9 to 11 k and a further one 2 k; a fold in which every CTA loads its share of all summaries and stores it back took 16 k.)
 // Packed batches are visited longest sequence first.  This file also holds the host side of both tensor-core variants (segment
 // plan, workspace layout, launches).
 #include <atomic>
@@ -928,7 +928,8 @@ int resident_clusters(int size) {
 
 // Segments per sequence: the most that keep all work items resident at once (CTAs of a cluster, or clusters of the pair variant).
 // The single-CTA kernel's segments hold at least one chunk of 128 tokens, and a sequence of two chunks stays whole (summary and
-// chain cost about as much as the chunk they would save); the pair variant's at least four of 64.
+// chain cost more than the chunk they would save: 256 tokens, 8 heads 11.6 us whole, 13.8 in two segments; 74 heads 12.7 and 16.9); the pair
+// variant's at least four of 64.
 // Several pairs of states of the n-state form in one launch: the CTAs of all of them and of all segments form one cluster; *nseg = 0 if
 // they cannot all be resident.
 void plan(const dsla_prefill_args* a, bool pair, int pairs, int* nseg, int* cps, int* skew8) {
@@ -1001,10 +1002,11 @@ dsla_status launch_main(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
 bool prefill_tc_available() { return true; }
 
 // Pairs of states side by side need fewer segments per sequence, so shorter chains of initial states, and read Q, K and V from L2
-// the second time (four states, T = 4096, 32 heads: 114 us as two launches, 101 as one; eight: 228 and 162); but SMs may be left over,
-// or the sequences be cut less than a launch for each pair would.  Times in eighths of a chunk's (7.2 k cycles): a chunk 8, set-up and
-// drain 5, a summary 2 per chunk (2.3 k cycles while all SMs read K and V, nearer to 3; with 2.5 here 97 of 100 shapes come out the same), a hop
-// of the initial states 3.
+// the second time (four states, T = 4096, 32 heads: 112 us as two launches, 89 as one; eight: 221 and 152); but SMs may be left over,
+// or the sequences be cut less than a launch for each pair would.  Weights: a chunk 8, set-up and drain 5, a summary 2 per chunk, a hop of the
+// initial states 3.  (Stamped now, a chunk is 6.6 to 7.1 k cycles, a summary 1.9 to 2.5 k, the first hop 9 k and further ones 2 k.  With these
+// weights the choice is within 3 % of the best of 1, 2 and 4 on 272 of 278 shapes of four and eight states; the worst are eight states of
+// 3000 tokens, 16 heads, 141 us where all pairs in one launch take 128, and of 2048 tokens, 40 heads, 168 and 159.)
 int prefill_tc_pairs(const dsla_prefill_args* a, int npairs) {
     int best = 1;
     long long least = 0;
