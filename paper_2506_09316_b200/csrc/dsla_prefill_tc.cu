@@ -484,8 +484,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         };
         if (SPLIT) started_alone();
         // The decays of a block (32 registers) and the scaled Q (32) are alive across the waits of this loop, where a call costs spills.  Whole
-        // sequences: waits for what has long arrived come before the decays, the cleared rows without a call (16 prompts of 335K tokens 2780 to
-        // 2720 us, 8 x 512 tokens 49.6 to 48.2, pieces of one chunk 15.3 to 15.0).  Segments: decays first, since the tiles come late, and waits without
+        // sequences: the wait for Q and K comes before the decays, rows are cleared without a call (16 prompts of 335K tokens 2791 to
+        // 2756 us, 8 x 512 tokens 50.0 to 48.7, pieces of one chunk 14.9 to 14.7, 232 tokens 13.0 to 12.8).  Segments: decays first, since the tiles come late, and waits without
         // a call (777 tokens 20.9 to 20.6; with the other order 21.8).  Pairs of states keep the calls (eight states 156 us, without them 170).
         auto tile_wait = [&](uint64_t* bar, int ph) {
             if (SPLIT && !PAIRS) mbar_wait_inline(bar, (uint32_t)ph, abortp, p.status);
@@ -497,22 +497,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int s = c & 1;
             const GateSmem& gs = sh.gs[s];
             uint8_t* qs = tiles + c3 * TILE_BYTES;
-            // Q and K have landed (the TMA writes of Q are visible to this thread).  Rows of K and V past the end of the sequence belong to the next one.
-            // They would meet only zero weights, but 0 * inf is not 0.  (The scores, which may be reading K, meet them only in columns that no
-            // row of this sequence uses; V~ and the other MMAs wait for prep_ready.  Here, under the scores; ahead of prep_ready it took 1 % of a
-            // packed batch's time.)
-            auto landed = [&] {
-                tile_wait(&sh.kq_full[s], (c >> 1) & 1);
-                const int valid = sq.len - tok0 - c * CM;
-                if (valid < CM) {
-                    tile_wait(&sh.v_full[s], (c >> 1) & 1);
-                    uint8_t *kt = tiles + OFF_K + s * TILE_BYTES, *vt = tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES;
-                    if (SPLIT) zero_rows_call(kt, vt, valid, tt);
-                    else zero_rows(kt, vt, valid, tt);
-                }
-            };
             tile_wait(&sh.g_ready[s], (c >> 1) & 1);
-            if (!SPLIT) landed();
+            if (!SPLIT) tile_wait(&sh.kq_full[s], (c >> 1) & 1);      // the TMA writes of Q are visible to this thread
             // ---- decays of this warp's first block, ahead of the scores that they multiply
             const float L1 = gs.L[0][j], L2 = gs.L[1][j];
             float2 mk[16];
@@ -526,7 +512,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     mk[2 * e + 1].x = fmaf(W2, ex2(L2 - K2.z), W1 * ex2(L1 - K1.z)); mk[2 * e + 1].y = fmaf(W2, ex2(L2 - K2.w), W1 * ex2(L1 - K1.w));
                 }
             }
-            if (SPLIT) landed();
+            if (SPLIT) tile_wait(&sh.kq_full[s], (c >> 1) & 1);
+            // Rows of K and V past the end of the sequence belong to the next one.  They would meet only zero weights, but 0 * inf is not 0.  (The
+            // scores, which may be reading K, meet them only in columns that no row of this sequence uses; V~ and the other MMAs wait for
+            // prep_ready.  Here, under the scores; ahead of prep_ready it took 1 % of a packed batch's time, ahead of the decays 2 % of a call of
+            // 129 tokens.)
+            const int valid = sq.len - tok0 - c * CM;
+            if (valid < CM) {
+                tile_wait(&sh.v_full[s], (c >> 1) & 1);
+                uint8_t *kt = tiles + OFF_K + s * TILE_BYTES, *vt = tiles + (c3 == 0 ? 2 : c3 - 1) * TILE_BYTES;
+                if (SPLIT) zero_rows_call(kt, vt, valid, tt);
+                else zero_rows(kt, vt, valid, tt);
+            }
             // ---- scaled copies of Q, eight 16-byte pieces (half a row) per thread: one factor per state for all of them.  (Consecutive pieces per
             // thread needed the factors of eight rows from shared memory, which the loop is bound by.)  The copy for state 2 is written as soon as the readout
             // of the previous chunk is done with its buffer, the one for state 1 waits in registers until the scores have read the raw Q.
